@@ -451,10 +451,24 @@ typedef enum {
                                        inside the sweep and the device accepts the
                                        cooperative launch, else one launch per operator
                                        (0 always) */
-    SV_OPT_SWEEP_BLOCKS_PER_SM = 18 /* launch geometry of the whole-sweep launches: at most
+    SV_OPT_SWEEP_BLOCKS_PER_SM = 18,/* launch geometry of the whole-sweep launches: at most
                                        this many blocks per SM, no more than can be
                                        resident (1..64, default 2; sv_autotune times
                                        1, 2, 4, 8) */
+    SV_OPT_FULL_VECTOR = 19         /* 0 (default): the path runs on the sector's amplitudes
+                                       alone, in real arithmetic where the reference is
+                                       real (a determinant, or a stored state without
+                                       imaginary parts: integrals, generators and angles
+                                       are real, so the state stays real), and the handle's
+                                       vector is written from them before each call
+                                       returns; 1: every kernel works on the handle's own
+                                       vector in its own type (dense storage: rotations and
+                                       adjoint steps over all 2^n amplitudes), as the
+                                       library does by itself under SV_OPT_MAX_BYTES, with
+                                       the record-scan expectation or 1-RDM, and, but for
+                                       sv_energy_grad, once the state's address has been
+                                       given out (sv_state_device_ptr,
+                                       sv_create_with_buffers) */
 } sv_option;
 
 /* Options change launch choices or summation order only: results agree within the

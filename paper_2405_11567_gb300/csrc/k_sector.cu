@@ -605,7 +605,63 @@ __global__ void k_gather_c(const A *__restrict__ psi, const uint32_t *__restrict
         out[i] = idx[i] == 0xFFFFFFFFu ? mka<A>(0, 0) : psi[idx[i]];
 }
 
+// A handle's vector from its compute core's compact amplitudes (Out the handle's type, In the
+// core's: the same, or its real one).  sa / sb: the strings' storage-space spreads (dense
+// storage, the sector's addresses of the 2^n vector), or NULL (sector storage, same order).
+// Bound: dense, one partly written 32-byte DRAM sector per scattered amplitude.
+template <typename Out, typename In>
+__global__ void __launch_bounds__(kThreads) k_core_publish(const In *__restrict__ C, Out *__restrict__ psi,
+                                                           const uint32_t *__restrict__ sa,
+                                                           const uint32_t *__restrict__ sb, int Da, int Db) {
+    using R = real_of<Out>;
+    for (int Ib = blockIdx.x; Ib < Db; Ib += gridDim.x) {
+        const size_t row = (size_t)Ib * Da;
+        const uint32_t xb = sb ? sb[Ib] : 0u;
+        for (int Ia = blockIdx.y * kThreads + threadIdx.x; Ia < Da; Ia += gridDim.y * kThreads) {
+            const In c = C[row + Ia];
+            psi[sa ? (size_t)(sa[Ia] | xb) : row + Ia] = mka<Out>((R)re(c), (R)im(c));
+        }
+    }
+}
+
+// The other way: the compact amplitudes (their real parts for a real core) of a stored reference.
+template <typename Out, typename In>
+__global__ void __launch_bounds__(kThreads) k_core_gather(const In *__restrict__ psi, Out *__restrict__ C,
+                                                          const uint32_t *__restrict__ sa,
+                                                          const uint32_t *__restrict__ sb, int Da, int Db) {
+    using R = real_of<Out>;
+    for (int Ib = blockIdx.x; Ib < Db; Ib += gridDim.x) {
+        const size_t row = (size_t)Ib * Da;
+        const uint32_t xb = sb ? sb[Ib] : 0u;
+        for (int Ia = blockIdx.y * kThreads + threadIdx.x; Ia < Da; Ia += gridDim.y * kThreads) {
+            const In c = psi[sa ? (size_t)(sa[Ia] | xb) : row + Ia];
+            C[row + Ia] = mka<Out>((R)re(c), (R)im(c));
+        }
+    }
+}
+
 // ---------------------------------------------------------------- launchers
+
+// publish: core (core_dtype) -> handle (dtype); else the handle's vector -> core.
+cudaError_t launch_core_move(void *handle_vec, int dtype, void *core_vec, int core_dtype, bool publish,
+                             const uint32_t *sa, const uint32_t *sb, int Da, int Db, int sm_count, cudaStream_t st) {
+    if (Da <= 0 || Db <= 0) return cudaSuccess;
+    // rows over the grid's x, a row's columns over its y: enough blocks for few long or many short rows
+    const int gy = (Da + kThreads - 1) / kThreads, cap = sm_count * 16;
+    const dim3 grid(Db < cap ? Db : cap, gy < 8 ? gy : 8);
+    if (dtype == core_dtype) {
+        SV_DISPATCH_AMP(dtype,
+                        if (publish) k_core_publish<A, A><<<grid, kThreads, 0, st>>>((const A *)core_vec, (A *)handle_vec, sa, sb, Da, Db);
+                        else k_core_gather<A, A><<<grid, kThreads, 0, st>>>((const A *)handle_vec, (A *)core_vec, sa, sb, Da, Db));
+    } else {  // a complex handle with a real core of the same precision
+        SV_DISPATCH_AMP(dtype, if constexpr (AmpT<A>::kCplx) {
+            using B = real_of<A>;
+            if (publish) k_core_publish<A, B><<<grid, kThreads, 0, st>>>((const B *)core_vec, (A *)handle_vec, sa, sb, Da, Db);
+            else k_core_gather<B, A><<<grid, kThreads, 0, st>>>((const A *)handle_vec, (B *)core_vec, sa, sb, Da, Db);
+        });
+    }
+    return cudaGetLastError();
+}
 
 static SectTabs tabs(const uint32_t *sa, const uint32_t *sb, const uint16_t *stra, const uint16_t *strb,
                      const uint16_t *ra, const uint16_t *rb, int Da, int Db) {

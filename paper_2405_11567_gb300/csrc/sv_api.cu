@@ -74,6 +74,8 @@ cudaError_t launch_rdm_rows(const void *C, int dtype, int ff_form, int n, const 
                             int Db, int grid, const uint32_t *alist, const int *ainfo, double *partial,
                             cudaStream_t st);
 cudaError_t launch_gather_c(const void *psi, int dtype, const uint32_t *idx, int count, void *out, cudaStream_t st);
+cudaError_t launch_core_move(void *handle_vec, int dtype, void *core_vec, int core_dtype, bool publish,
+                             const uint32_t *sa, const uint32_t *sb, int Da, int Db, int sm_count, cudaStream_t st);
 
 struct RowTables {
     const uint32_t *sa, *sb, *sa_s, *sb_s;
@@ -557,14 +559,15 @@ static sv_status check_ready(sv_handle h) {
     return SV_OK;
 }
 
+// Masks in the storage layout `perm` (the handle's own where NULL).
 static sv_status build_ops(sv_handle h, const sv_excitation *ops, int n_ops, const double *theta,
-                           std::vector<OpDesc> &out) {
+                           std::vector<OpDesc> &out, const int *perm = nullptr) {
     if (n_ops < 0) return fail(h, SV_ERR_ARG, "n_ops < 0");
     if (n_ops > 0 && (!ops || !theta)) return fail(h, SV_ERR_ARG, "NULL ops or theta");
     out.resize(n_ops);
     for (int k = 0; k < n_ops; ++k) {
         std::string why;
-        if (!make_op(ops[k], h->n, h->perm, out[k], why)) {
+        if (!make_op(ops[k], h->n, perm ? perm : h->perm, out[k], why)) {
             char buf[64];
             snprintf(buf, sizeof buf, "op %d: ", k);
             return fail(h, SV_ERR_ARG, buf + why);
@@ -613,6 +616,7 @@ static sv_status prepare_reference(sv_handle h) {
     } else {
         return fail(h, SV_ERR_STATE, "no reference state recorded");
     }
+    h->psi_clean = h->storage == 0;
     return SV_OK;
 }
 
@@ -1188,6 +1192,132 @@ static bool is_identity(sv_handle h) {
     return true;
 }
 
+// ---------------------------------------------------------------- compute core
+
+// A dense handle stores 2^n amplitudes of which only its sector's are ever non-zero (0.84%
+// at 30 qubits), and a complex handle whose reference is real stores zeros in every
+// imaginary part: the integrals, the generators T - T^dagger and the angles are real.  The
+// path runs on what remains, a sector-storage handle in real amplitudes (the core), and
+// psi is written from it: at 30 qubits energy + gradient + 1-RDM of a complex64 dense
+// handle took 254 ms over the full vector and 7.6 ms here; of a complex128 one, 647
+// and 46 ms.  The handle's own vector serves where the caller's bytes, form or writes
+// decide (SV_OPT_FULL_VECTOR lists them).
+static sv_status create_common(int n_qubits, sv_dtype dtype, void *cuda_stream, void *psi_dev, void *lam_dev,
+                               sv_handle *out, int sect_na, int sect_nb);
+static void destroy_handle(sv_handle h);
+
+static const int kIdentity[32] = {0,  1,  2,  3,  4,  5,  6,  7,  8,  9,  10, 11, 12, 13, 14, 15,
+                                  16, 17, 18, 19, 20, 21, 22, 23, 24, 25, 26, 27, 28, 29, 30, 31};
+
+static bool core_wanted(sv_handle h) {
+    if (h->outer || h->full_vector || h->max_bytes > 0 || h->ref_kind == 0) return false;
+    if (h->storage == 0) return !(is_complex(h->dtype) && (h->expect_variant == 1 || h->rdm_variant == 1));
+    return is_complex(h->dtype) && h->ref_real;
+}
+
+static void drop_core(sv_handle h) {
+    if (!h->core) return;
+    h->launches += h->core->launches;
+    destroy_handle(h->core);
+    h->core = nullptr;
+    h->core_cur = 0;
+    h->core_ref = false;
+}
+
+// The storage-space spreads of the handle's strings (NULL in sector storage: same order).
+static sv_status core_spreads(sv_handle h, const uint32_t **sa, const uint32_t **sb) {
+    *sa = *sb = nullptr;
+    if (h->storage == 1) return SV_OK;
+    SV_TRY(ensure_strings(h));
+    *sa = h->str_sa_s;
+    *sb = h->str_sb_s;
+    return SV_OK;
+}
+
+// The core for the handle's reference, with the handle's options and that reference.
+static sv_status ensure_core(sv_handle h) {
+    const sv_dtype cd = h->ref_real ? real_dtype(h->dtype) : h->dtype;
+    if (h->core && (h->core->dtype != cd || h->core->na != h->na || h->core->nb != h->nb)) {
+        const int cur = h->core_cur;
+        drop_core(h);
+        h->core_cur = cur == 1 ? 1 : 0;
+    }
+    if (!h->core) {
+        sv_handle c = nullptr;
+        SV_TRY(create_common(h->n, cd, h->stream, nullptr, nullptr, &c, h->na, h->nb));
+        c->outer = h;
+        h->core = c;
+        h->core_ref = false;
+    }
+    sv_handle c = h->core;
+    c->expect_variant = h->expect_variant;
+    c->ab_chunk = h->ab_chunk * (c->dtype == h->dtype ? 1 : 2);  // rows of half the bytes: twice as many per chunk
+    c->sect_bps = h->sect_bps;
+    c->sweep_bps = h->sweep_bps;
+    c->rdm_bps = h->rdm_bps;
+    c->rdm_variant = h->rdm_variant;
+    c->pool_variant = h->pool_variant;
+    c->wait_polls = h->wait_polls;
+    c->test_stall = h->test_stall;
+    c->sweep_mode = h->sweep_mode;
+    c->ckpt_interval = h->ckpt_interval;
+    c->profile = h->profile;
+    c->ref_kind = h->ref_kind;
+    c->ref_det = h->ref_det;
+    if (h->ref_kind == 2 && !h->core_ref) {
+        SV_TRY(ensure_strings(c));
+        if (!c->ref_vec) SV_TRY(dev_alloc(c, &c->ref_vec, vec_bytes(c), "reference copy"));
+        const uint32_t *sa, *sb;
+        SV_TRY(core_spreads(h, &sa, &sb));
+        SV_CUDA(c, launch_core_move(h->ref_vec, h->dtype, c->ref_vec, c->dtype, false, sa, sb, c->Da, c->Db, c->sm_count,
+                                    h->stream));
+        c->launches++;
+        h->core_ref = true;
+    }
+    return SV_OK;
+}
+
+// psi from the core's state.
+static sv_status core_publish(sv_handle h) {
+    sv_handle c = h->core;
+    const uint32_t *sa, *sb;
+    SV_TRY(core_spreads(h, &sa, &sb));
+    if (h->storage == 0 && (!h->psi_clean || h->exposed))
+        SV_CUDA(h, cudaMemsetAsync(h->psi, 0, vec_bytes(h), h->stream));
+    SV_CUDA(h, launch_core_move(h->psi, h->dtype, c->psi, c->dtype, true, sa, sb, c->Da, c->Db, h->sm_count, h->stream));
+    h->launches++;
+    h->psi_clean = h->storage == 0;
+    h->core_cur = 2;
+    h->prepared = true;
+    return SV_OK;
+}
+
+// A status of the core as the handle's own.
+static sv_status core_status(sv_handle h, sv_status st) {
+    if (st != SV_OK && h->core) {
+        h->err = h->core->err;
+        if (h->core->failed) h->failed = true;
+    }
+    return st;
+}
+
+// The handle that holds the current state for a call that only reads it: the core where it
+// has it (prepared first where it is still the reference), else the handle itself.
+static sv_status reader(sv_handle h, sv_handle *out) {
+    *out = h;
+    if (h->exposed || h->core_cur == 0 || !core_wanted(h)) return SV_OK;
+    if (ensure_core(h) != SV_OK) {
+        cudaGetLastError();
+        return SV_OK;
+    }
+    if (h->core_cur == 0) return SV_OK;  // another core, without the state
+    if (h->core_cur == 1) SV_TRY(core_status(h, prepare_reference(h->core)));
+    h->core->prepared = true;
+    h->core_cur = 2;
+    *out = h->core;
+    return SV_OK;
+}
+
 // ---------------------------------------------------------------- autotuning
 
 // Fastest of `reps` runs of fn (launches on the handle's stream), in ms, timed with
@@ -1379,7 +1509,9 @@ uint32_t sv_check_status(void) {
 
 const char *sv_last_error(sv_handle h) { return h ? h->err.c_str() : g_err.c_str(); }
 
-uint64_t sv_launch_count(sv_handle h) { return h ? h->launches : 0; }
+uint64_t sv_launch_count(sv_handle h) { return h ? h->launches + (h->core ? h->core->launches : 0) : 0; }
+
+}  // extern "C"
 
 static uint64_t binom(int n, int k) {
     if (k < 0 || k > n) return 0;
@@ -1390,7 +1522,7 @@ static uint64_t binom(int n, int k) {
 
 // sect_na < 0: dense storage; otherwise sector storage of (sect_na, sect_nb).
 static sv_status create_common(int n_qubits, sv_dtype dtype, void *cuda_stream, void *psi_dev, void *lam_dev,
-                               sv_handle *out, int sect_na = -1, int sect_nb = -1) {
+                               sv_handle *out, int sect_na, int sect_nb) {
     if (!out) return fail(nullptr, SV_ERR_ARG, "NULL output handle pointer");
     *out = nullptr;
     if (n_qubits < 2 || n_qubits > SV_MAX_QUBITS || (n_qubits & 1))
@@ -1427,6 +1559,7 @@ static sv_status create_common(int n_qubits, sv_dtype dtype, void *cuda_stream, 
     if (psi_dev) {
         h->psi = psi_dev;
         h->own_psi = false;
+        h->exposed = true;
     } else {
         sv_status s = dev_alloc(h, &h->psi, vec_bytes(h), "state vector");
         if (s != SV_OK) {
@@ -1442,29 +1575,7 @@ static sv_status create_common(int n_qubits, sv_dtype dtype, void *cuda_stream, 
     return SV_OK;
 }
 
-sv_status sv_create(int n_qubits, sv_dtype dtype, void *cuda_stream, sv_handle *out) {
-    return create_common(n_qubits, dtype, cuda_stream, nullptr, nullptr, out);
-}
-
-sv_status sv_create_sector(int n_qubits, int n_alpha, int n_beta, sv_dtype dtype, void *cuda_stream, sv_handle *out) {
-    if (out) *out = nullptr;
-    if (n_qubits < 2 || n_qubits > SV_MAX_QUBITS || (n_qubits & 1))
-        return fail(nullptr, SV_ERR_ARG, "n_qubits must be even and in [2, 32]");
-    const int N = n_qubits / 2;
-    if (n_alpha < 0 || n_beta < 0 || n_alpha > N || n_beta > N)
-        return fail(nullptr, SV_ERR_ARG, "electron counts must be in [0, n_qubits / 2]");
-    return create_common(n_qubits, dtype, cuda_stream, nullptr, nullptr, out, n_alpha, n_beta);
-}
-
-sv_status sv_create_with_buffers(int n_qubits, sv_dtype dtype, void *cuda_stream, void *psi_dev, void *lam_dev,
-                                 sv_handle *out) {
-    if (!psi_dev) return fail(nullptr, SV_ERR_ARG, "psi_dev is required");
-    return create_common(n_qubits, dtype, cuda_stream, psi_dev, lam_dev, out);
-}
-
-sv_status sv_destroy(sv_handle h) {
-    if (!h) return SV_OK;
-    DeviceGuard g(h->device);
+static void destroy_handle(sv_handle h) {
     cudaStreamSynchronize(h->stream);
     cudaGetLastError();
     if (h->own_psi) dev_free(h, h->psi, vec_bytes(h));
@@ -1497,9 +1608,49 @@ sv_status sv_destroy(sv_handle h) {
     for (cudaEvent_t e : h->tcev)
         if (e) cudaEventDestroy(e);
     delete h;
+}
+
+extern "C" {
+
+sv_status sv_create(int n_qubits, sv_dtype dtype, void *cuda_stream, sv_handle *out) {
+    return create_common(n_qubits, dtype, cuda_stream, nullptr, nullptr, out, -1, -1);
+}
+
+sv_status sv_create_sector(int n_qubits, int n_alpha, int n_beta, sv_dtype dtype, void *cuda_stream, sv_handle *out) {
+    if (out) *out = nullptr;
+    if (n_qubits < 2 || n_qubits > SV_MAX_QUBITS || (n_qubits & 1))
+        return fail(nullptr, SV_ERR_ARG, "n_qubits must be even and in [2, 32]");
+    const int N = n_qubits / 2;
+    if (n_alpha < 0 || n_beta < 0 || n_alpha > N || n_beta > N)
+        return fail(nullptr, SV_ERR_ARG, "electron counts must be in [0, n_qubits / 2]");
+    return create_common(n_qubits, dtype, cuda_stream, nullptr, nullptr, out, n_alpha, n_beta);
+}
+
+sv_status sv_create_with_buffers(int n_qubits, sv_dtype dtype, void *cuda_stream, void *psi_dev, void *lam_dev,
+                                 sv_handle *out) {
+    if (!psi_dev) return fail(nullptr, SV_ERR_ARG, "psi_dev is required");
+    return create_common(n_qubits, dtype, cuda_stream, psi_dev, lam_dev, out, -1, -1);
+}
+
+sv_status sv_destroy(sv_handle h) {
+    if (!h) return SV_OK;
+    DeviceGuard g(h->device);
+    cudaStreamSynchronize(h->stream);
+    cudaGetLastError();
+    drop_core(h);
+    destroy_handle(h);
     return SV_OK;
 }
 
+
+
+// A new reference: nothing that the core holds is current.
+static void reference_changed(sv_handle h) {
+    h->core_cur = 0;
+    h->core_ref = false;
+    h->psi_clean = false;
+    if (h->core) h->core->failed = false;
+}
 
 sv_status sv_prepare_hf(sv_handle h, const int32_t *occ, int n_occ) {
     if (!h) return fail(nullptr, SV_ERR_ARG, "NULL handle");
@@ -1520,11 +1671,14 @@ sv_status sv_prepare_hf(sv_handle h, const int32_t *occ, int n_occ) {
     h->prepared = false;
     h->ref_kind = 1;
     h->ref_det = x;
+    h->ref_real = true;
     h->na = na;
     h->nb = nb;
+    reference_changed(h);
     SV_TRY(prepare_reference(h));
     h->prepared = true;
     h->at_ref = true;
+    h->core_cur = 1;
     return SV_OK;
 }
 
@@ -1538,6 +1692,7 @@ sv_status sv_prepare_state(sv_handle h, const void *amplitudes_host, int n_alpha
     const uint32_t even = 0x55555555u, odd = 0xAAAAAAAAu;
     double best = -1.0;
     uint32_t best_x = 0;
+    bool real = true;
     for (uint64_t x = 0; x < h->dim; ++x) {
         double re = 0.0, im = 0.0;
         switch (h->dtype) {
@@ -1548,16 +1703,21 @@ sv_status sv_prepare_state(sv_handle h, const void *amplitudes_host, int n_alpha
         }
         if (!std::isfinite(re) || !std::isfinite(im)) return fail(h, SV_ERR_ARG, "non-finite amplitude");
         double w = re * re + im * im;
-        if (w == 0.0) continue;
+        if (w == 0.0) {
+            real = real && im == 0.0;  // (an imaginary part whose square underflows)
+            continue;
+        }
         if (__builtin_popcount((uint32_t)x & even) != n_alpha || __builtin_popcount((uint32_t)x & odd) != n_beta)
             return fail(h, SV_ERR_ARG, "amplitude outside the (n_alpha, n_beta) sector");
         if (w > best) { best = w; best_x = (uint32_t)x; }
+        real = real && im == 0.0;
     }
     if (best <= 0.0) return fail(h, SV_ERR_ARG, "zero state");
     DeviceGuard g(h->device);
     h->failed = false;
     h->prepared = false;
     h->at_ref = false;
+    reference_changed(h);
     if (!h->ref_vec) SV_TRY(dev_alloc(h, &h->ref_vec, vec_bytes(h), "reference copy"));
     if (h->storage == 1) {
         // host order is the dense qubit-order vector: keep its sector entries in C[rank(b)][rank(a)] order
@@ -1586,10 +1746,12 @@ sv_status sv_prepare_state(sv_handle h, const void *amplitudes_host, int n_alpha
     SV_CUDA(h, cudaStreamSynchronize(h->stream));
     h->ref_kind = 2;
     h->ref_det = best_x;
+    h->ref_real = real;
     h->na = n_alpha;
     h->nb = n_beta;
     SV_TRY(prepare_reference(h));
     h->prepared = true;
+    h->core_cur = 1;
     return SV_OK;
 }
 
@@ -1663,6 +1825,7 @@ sv_status sv_get_amplitudes(sv_handle h, const uint64_t *basis, int count, void 
 sv_status sv_state_device_ptr(sv_handle h, void **psi_dev) {
     if (!h || !psi_dev) return fail(h, SV_ERR_ARG, "NULL argument");
     h->at_ref = false;  // the caller may write the state through the pointer
+    h->exposed = true;
     *psi_dev = h->psi;
     return SV_OK;
 }
@@ -1710,33 +1873,46 @@ sv_status sv_ham_destroy(sv_ham_handle ham) {
 sv_status sv_apply_ansatz(sv_handle h, const sv_excitation *ops, int n_ops, const double *theta) {
     SV_TRY(check_ready(h));
     std::vector<OpDesc> d;
-    SV_TRY(build_ops(h, ops, n_ops, theta, d));
+    const bool core = core_wanted(h) && !h->exposed && h->core_cur != 0;
+    SV_TRY(build_ops(h, ops, n_ops, theta, d, core ? kIdentity : nullptr));
     DeviceGuard g(h->device);
-    L2FetchScope l2(h);
+    int np[32];
+    bool move = false;  // a fresh determinant takes the layout that the operator list prefers
     if (h->layout_auto && n_ops > 0 && h->storage == 0 && h->at_ref && h->ref_kind == 1) {
-        // the state is still the HF determinant: take the layout the operator list prefers
-        // (as sv_energy_grad does) by writing the determinant anew in it, one store
-        int np[32];
         layout_from_ops(h->n, ops, n_ops, np);
-        bool same = true;
-        for (int q = 0; q < h->n; ++q) same = same && np[q] == h->perm[q];
-        if (!same) {
+        for (int q = 0; q < h->n; ++q) move = move || np[q] != h->perm[q];
+    }
+    if (core && ensure_core(h) == SV_OK && h->core_cur != 0) {
+        sv_handle c = h->core;
+        if (h->core_cur == 1) SV_TRY(core_status(h, prepare_reference(c)));
+        h->core_cur = 0;  // until psi is written
+        c->prepared = true;
+        SV_TRY(core_status(h, forward(c, d, false)));
+        h->at_ref = false;
+        if (move) {
             for (int q = 0; q < 32; ++q) h->perm[q] = q < h->n ? np[q] : q;
             drop_layout_caches(h);
-            SV_TRY(prepare_reference(h));
-            SV_TRY(build_ops(h, ops, n_ops, theta, d));
+            h->psi_clean = false;
         }
+        return core_publish(h);
+    }
+    cudaGetLastError();
+    if (core) SV_TRY(build_ops(h, ops, n_ops, theta, d));
+    L2FetchScope l2(h);
+    if (move) {
+        // as sv_energy_grad does, by writing the determinant anew in the layout, one store
+        for (int q = 0; q < 32; ++q) h->perm[q] = q < h->n ? np[q] : q;
+        drop_layout_caches(h);
+        SV_TRY(prepare_reference(h));
+        SV_TRY(build_ops(h, ops, n_ops, theta, d));
     }
     h->at_ref = false;
+    h->core_cur = 0;
     SV_TRY(forward(h, d, false));
     return SV_OK;
 }
 
-sv_status sv_energy(sv_handle h, sv_ham_handle ham, double *e_out) {
-    SV_TRY(check_ready(h));
-    SV_TRY(check_ham(h, ham));
-    if (!e_out) return fail(h, SV_ERR_ARG, "NULL e_out");
-    DeviceGuard g(h->device);
+static sv_status energy_run(sv_handle h, sv_ham_handle ham, double *e_out) {
     DevTables *T;
     SV_TRY(get_tables(h, ham, &T));
     SV_TRY(ensure_out(h, 2));
@@ -1749,23 +1925,21 @@ sv_status sv_energy(sv_handle h, sv_ham_handle ham, double *e_out) {
     return SV_OK;
 }
 
-sv_status sv_energy_grad(sv_handle h, sv_ham_handle ham, const sv_excitation *ops, int n_ops, const double *theta,
-                         double *e_out, double *grad_out) {
-    if (!h) return fail(nullptr, SV_ERR_ARG, "NULL handle");
-    if (h->ref_kind == 0) return fail(h, SV_ERR_STATE, "no reference state recorded");
+sv_status sv_energy(sv_handle h, sv_ham_handle ham, double *e_out) {
+    SV_TRY(check_ready(h));
     SV_TRY(check_ham(h, ham));
-    std::vector<OpDesc> d;
-    SV_TRY(build_ops(h, ops, n_ops, theta, d));  // validates in any layout
-    h->at_ref = false;
+    if (!e_out) return fail(h, SV_ERR_ARG, "NULL e_out");
     DeviceGuard g(h->device);
-    L2FetchScope l2(h);
+    sv_handle r;
+    SV_TRY(reader(h, &r));
+    if (r != h) return core_status(h, energy_run(r, ham, e_out));
+    return energy_run(h, ham, e_out);
+}
+
+// sv_energy_grad on the handle's own storage, operators in its layout.
+static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vector<OpDesc> &d, double *e_out,
+                                 double *grad_out) {
     NvtxClose nvtx_close{h};
-    if (h->layout_auto && n_ops > 0 && h->storage == 0) {
-        int np[32];
-        layout_from_ops(h->n, ops, n_ops, np);
-        SV_TRY(relayout(h, np));
-        SV_TRY(build_ops(h, ops, n_ops, theta, d));
-    }
     const size_t L = d.size();
     DevTables *T;
     SV_TRY(get_tables(h, ham, &T));
@@ -1801,6 +1975,7 @@ sv_status sv_energy_grad(sv_handle h, sv_ham_handle ham, const sv_excitation *op
     SV_TRY(mark(h, 1, "sv_energy_grad: forward sweep"));
     SV_TRY(forward(h, d, true));
     SV_TRY(mark(h, 2, "sv_energy_grad: working copy"));
+    if (h->outer) SV_TRY(core_publish(h->outer));
     // The reverse sweep un-applies the ops to a working copy of psi(theta), so that psi
     // keeps psi(theta): in sector storage without checkpoint resynchronisation, the
     // interleaved (psi, lambda) matrix; else the saved-state buffer.  Where neither can be
@@ -1898,7 +2073,7 @@ sv_status sv_energy_grad(sv_handle h, sv_ham_handle ham, const sv_excitation *op
         h->phase_ms[1] = elapsed(h, 1, 2);
         h->phase_ms[2] = elapsed(h, 3, 4);
         h->phase_ms[3] = elapsed(h, 4, 5);
-        h->phase_ms[4] = elapsed(h, 5, 6);
+        h->phase_ms[4] = elapsed(h, 5, 6) + (h->outer ? elapsed(h, 2, 3) : 0.f);  // a core: writing its handle's psi
         h->phase_ms[6] = (h->tc_timed & 1) ? elapsed_ev(h->tcev[0], h->tcev[1]) : 0.0;
         h->phase_ms[7] = (h->tc_timed & 2) ? elapsed_ev(h->tcev[2], h->tcev[3]) : 0.0;
     }
@@ -1909,13 +2084,50 @@ sv_status sv_energy_grad(sv_handle h, sv_ham_handle ham, const sv_excitation *op
     return SV_OK;
 }
 
-sv_status sv_pool_gradients(sv_handle h, sv_ham_handle ham, const sv_excitation *pool, int n_pool, double *e_out,
-                            double *grad_out) {
-    SV_TRY(check_ready(h));
+sv_status sv_energy_grad(sv_handle h, sv_ham_handle ham, const sv_excitation *ops, int n_ops, const double *theta,
+                         double *e_out, double *grad_out) {
+    if (!h) return fail(nullptr, SV_ERR_ARG, "NULL handle");
+    if (h->ref_kind == 0) return fail(h, SV_ERR_STATE, "no reference state recorded");
     SV_TRY(check_ham(h, ham));
-    if (n_pool < 0 || (n_pool > 0 && (!pool || !grad_out))) return fail(h, SV_ERR_ARG, "bad pool arguments");
-    const int ident[32] = {0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15,
-                           16, 17, 18, 19, 20, 21, 22, 23, 24, 25, 26, 27, 28, 29, 30, 31};
+    std::vector<OpDesc> d;
+    const bool core = core_wanted(h);
+    SV_TRY(build_ops(h, ops, n_ops, theta, d, core ? kIdentity : nullptr));  // validates in any layout
+    h->at_ref = false;
+    DeviceGuard g(h->device);
+    int np[32];
+    const bool lay = h->layout_auto && n_ops > 0 && h->storage == 0;
+    if (lay) layout_from_ops(h->n, ops, n_ops, np);
+    if (core && ensure_core(h) == SV_OK) {
+        bool same = true;
+        for (int q = 0; lay && q < h->n; ++q) same = same && np[q] == h->perm[q];
+        h->core_cur = 0;  // until psi is written
+        if (!same) {
+            h->prepared = false;  // psi is written anew in the layout, not moved to it
+            if (h->ref_kind == 2) {
+                SV_TRY(relayout(h, np));
+            } else {
+                for (int q = 0; q < 32; ++q) h->perm[q] = q < h->n ? np[q] : q;
+                drop_layout_caches(h);
+            }
+            h->psi_clean = false;
+        }
+        const sv_status st = core_status(h, energy_grad_run(h->core, ham, d, e_out, grad_out));
+        for (int i = 0; i < SV_PHASES; ++i) h->phase_ms[i] = h->core->phase_ms[i];
+        return st;
+    }
+    cudaGetLastError();
+    if (core) SV_TRY(build_ops(h, ops, n_ops, theta, d));
+    h->core_cur = 0;
+    L2FetchScope l2(h);
+    if (lay) {
+        SV_TRY(relayout(h, np));
+        SV_TRY(build_ops(h, ops, n_ops, theta, d));
+    }
+    return energy_grad_run(h, ham, d, e_out, grad_out);
+}
+
+static sv_status pool_run(sv_handle h, sv_ham_handle ham, const sv_excitation *pool, int n_pool, double *e_out,
+                          double *grad_out) {
     const bool use_lists = h->pool_variant != 1;
     const size_t ob = pool_op_bytes();
     std::vector<uint8_t> host_ops(use_lists ? 0 : (size_t)n_pool * ob);
@@ -1924,7 +2136,7 @@ sv_status sv_pool_gradients(sv_handle h, sv_ham_handle ham, const sv_excitation 
     for (int k = 0; k < n_pool; ++k) {
         OpDesc d;
         std::string why;
-        if (!make_op(pool[k], h->n, ident, d, why)) {
+        if (!make_op(pool[k], h->n, kIdentity, d, why)) {
             char buf[64];
             snprintf(buf, sizeof buf, "pool op %d: ", k);
             return fail(h, SV_ERR_ARG, buf + why);
@@ -1932,7 +2144,6 @@ sv_status sv_pool_gradients(sv_handle h, sv_ham_handle ham, const sv_excitation 
         if (use_lists) descs.push_back(d);
         else pool_op_from(d, h->n / 2, host_ops.data() + (size_t)k * ob);
     }
-    DeviceGuard g(h->device);
     DevTables *T;
     SV_TRY(get_tables(h, ham, &T));
     SV_TRY(ensure_strings(h));
@@ -1979,10 +2190,19 @@ sv_status sv_pool_gradients(sv_handle h, sv_ham_handle ham, const sv_excitation 
     return SV_OK;
 }
 
-sv_status sv_rdm1(sv_handle h, double *re_out, double *im_out) {
+sv_status sv_pool_gradients(sv_handle h, sv_ham_handle ham, const sv_excitation *pool, int n_pool, double *e_out,
+                            double *grad_out) {
     SV_TRY(check_ready(h));
-    if (!re_out) return fail(h, SV_ERR_ARG, "NULL re_out");
+    SV_TRY(check_ham(h, ham));
+    if (n_pool < 0 || (n_pool > 0 && (!pool || !grad_out))) return fail(h, SV_ERR_ARG, "bad pool arguments");
     DeviceGuard g(h->device);
+    sv_handle r;
+    SV_TRY(reader(h, &r));
+    if (r != h) return core_status(h, pool_run(r, ham, pool, n_pool, e_out, grad_out));
+    return pool_run(h, ham, pool, n_pool, e_out, grad_out);
+}
+
+static sv_status rdm1_run(sv_handle h, double *re_out, double *im_out) {
     NvtxClose nvtx_close{h};
     if (h->storage == 1 || h->rdm_variant != 1 || !is_complex(h->dtype)) {
         // string rows: on the state itself (sector storage) or on its compact copy
@@ -2060,13 +2280,28 @@ sv_status sv_rdm1(sv_handle h, double *re_out, double *im_out) {
     return SV_OK;
 }
 
+sv_status sv_rdm1(sv_handle h, double *re_out, double *im_out) {
+    SV_TRY(check_ready(h));
+    if (!re_out) return fail(h, SV_ERR_ARG, "NULL re_out");
+    DeviceGuard g(h->device);
+    sv_handle r;
+    SV_TRY(reader(h, &r));
+    if (r == h) return rdm1_run(h, re_out, im_out);
+    const sv_status st = core_status(h, rdm1_run(r, re_out, im_out));
+    h->phase_ms[5] = r->phase_ms[5];
+    return st;
+}
+
 sv_status sv_autotune(sv_handle h, sv_ham_handle ham, const sv_excitation *ops, int n_ops, const double *theta) {
     SV_TRY(check_ready(h));
     SV_TRY(check_ham(h, ham));
     std::vector<OpDesc> d;
     SV_TRY(build_ops(h, ops, n_ops, theta, d));
     DeviceGuard g(h->device);
-    L2FetchScope l2(h);
+    sv_handle r;
+    SV_TRY(reader(h, &r));
+    if (r != h) SV_TRY(build_ops(r, ops, n_ops, theta, d));
+    L2FetchScope l2(r);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     SV_CUDA(h, cudaEventCreate(&e0));
     if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -2075,9 +2310,16 @@ sv_status sv_autotune(sv_handle h, sv_ham_handle ham, const sv_excitation *ops, 
         return fail(h, SV_ERR_CUDA, "autotune: event creation failed");
     }
     h->at_ref = false;
-    const sv_status st = autotune_impl(h, ham, d, e0, e1);
+    const sv_status st = r == h ? autotune_impl(h, ham, d, e0, e1) : core_status(h, autotune_impl(r, ham, d, e0, e1));
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    if (r != h && st == SV_OK) {  // the choices are the handle's
+        h->expect_variant = r->expect_variant;
+        h->ab_chunk = r->ab_chunk / (r->dtype == h->dtype ? 1 : 2);
+        h->sect_bps = r->sect_bps;
+        h->sweep_bps = r->sweep_bps;
+        h->rdm_bps = r->rdm_bps;
+    }
     return st;
 }
 
@@ -2101,6 +2343,7 @@ sv_status sv_get_option(sv_handle h, sv_option opt, int64_t *value) {
         case SV_OPT_SECTOR_SWEEP: *value = h->sweep_mode; return SV_OK;
         case SV_OPT_SWEEP_BLOCKS_PER_SM: *value = h->sweep_bps; return SV_OK;
         case SV_OPT_TEST_STALL: *value = h->test_stall; return SV_OK;
+        case SV_OPT_FULL_VECTOR: *value = h->full_vector; return SV_OK;
     }
     return fail(h, SV_ERR_ARG, "unknown option");
 }
@@ -2147,6 +2390,14 @@ sv_status sv_set_option(sv_handle h, sv_option opt, int64_t value) {
         case SV_OPT_MAX_BYTES:
             if (value < 0) return fail(h, SV_ERR_ARG, "max bytes < 0");
             h->max_bytes = value;
+            if (value > 0) {  // the cap counts what the handle itself plans
+                DeviceGuard g(h->device);
+                drop_core(h);
+            }
+            return SV_OK;
+        case SV_OPT_FULL_VECTOR:
+            if (value != 0 && value != 1) return fail(h, SV_ERR_ARG, "full vector must be 0 or 1");
+            h->full_vector = (int)value;
             return SV_OK;
         case SV_OPT_EXPECT_VARIANT:
             if (value < 0 || value > 6) return fail(h, SV_ERR_ARG, "expect variant must be 0 to 6");

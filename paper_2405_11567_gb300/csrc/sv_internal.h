@@ -29,6 +29,7 @@ namespace svk {
 inline size_t amp_size(int dtype) { return dtype == SV_C64 ? 8 : dtype == SV_C128 ? 16 : dtype == SV_R32 ? 4 : 8; }
 inline bool single_prec(int dtype) { return dtype == SV_C64 || dtype == SV_R32; }
 inline bool is_complex(int dtype) { return dtype == SV_C64 || dtype == SV_C128; }
+inline sv_dtype real_dtype(sv_dtype dtype) { return dtype == SV_C64 ? SV_R32 : dtype == SV_C128 ? SV_R64 : dtype; }
 
 // ---------------------------------------------------------------- excitation ops
 
@@ -238,6 +239,16 @@ struct sv_ctx {
     uint32_t ref_det = 0;      // HF determinant (ref_kind 1)
     void *ref_vec = nullptr;   // device copy of the reference (ref_kind 2)
     double ref_shift = 0.0;    // c in lambda = (H - c) psi
+    bool ref_real = false;     // the reference's amplitudes are real (a determinant always)
+    // The compute core: a sector-storage handle of this handle's sector, in real amplitudes
+    // where the reference is real, that runs the path for a dense or complex handle; psi is
+    // written from it before a call returns.
+    sv_ctx *core = nullptr, *outer = nullptr;  // outer: the handle a core serves
+    int core_cur = 0;          // what the core holds of the state in psi: 0 nothing, 1 that it is the reference, 2 psi
+    bool core_ref = false;     // the core's copy of a stored reference is current
+    bool exposed = false;      // psi's address is known outside the library: it may be written there
+    bool psi_clean = false;    // dense psi is zero outside the (na, nb) sector in layout perm
+    int full_vector = 0;       // SV_OPT_FULL_VECTOR
     // sector list (basis indices of the (na, nb) sector, ascending) for gather kernels
     uint32_t *sector = nullptr;
     uint64_t sector_len = 0;

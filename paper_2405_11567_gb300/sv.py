@@ -38,6 +38,7 @@ SV_OPT_WAIT_POLLS = 15
 SV_OPT_TEST_STALL = 16
 SV_OPT_SECTOR_SWEEP = 17
 SV_OPT_SWEEP_BLOCKS_PER_SM = 18
+SV_OPT_FULL_VECTOR = 19
 SV_PHASES = 8
 PHASE_NAMES = ("reference", "forward", "expectation", "reverse", "restore", "rdm1", "same_products", "ab_products")
 STATUS = {0: "SV_OK", 1: "SV_ERR_ARG", 2: "SV_ERR_OOM", 3: "SV_ERR_CUDA", 4: "SV_ERR_TIMEOUT", 5: "SV_ERR_STATE"}
