@@ -443,14 +443,17 @@ typedef enum {
                                        producer).  No fault and no hang: the call reports
                                        SV_ERR_CUDA */
     SV_OPT_SECTOR_SWEEP = 17,       /* sector storage: 1 (default) each forward and reverse
-                                       sweep is one cooperative launch that walks the
-                                       operators in order with a grid-wide barrier
-                                       between them (every barrier wait bounded by
-                                       SV_OPT_WAIT_POLLS: past it the call fails with
-                                       SV_ERR_CUDA); used where no checkpoint copy falls
-                                       inside the sweep and the device accepts the
-                                       cooperative launch, else one launch per operator
-                                       (0 always) */
+                                       sweep is one launch that walks the operators in
+                                       order, two to a step: in one block's shared memory
+                                       (small sectors), on a cluster of sixteen blocks, or
+                                       on every SM, launched cooperatively, with a
+                                       grid-wide barrier between the steps (every barrier
+                                       wait bounded by SV_OPT_WAIT_POLLS: past it the call
+                                       fails with SV_ERR_CUDA; with a limit below 1024
+                                       this form runs at every size); used where no
+                                       checkpoint copy falls inside the sweep and the
+                                       device accepts the launch, else one launch per
+                                       operator (0 always) */
     SV_OPT_SWEEP_BLOCKS_PER_SM = 18,/* launch geometry of the whole-sweep launches: at most
                                        this many blocks per SM, no more than can be
                                        resident (1..64, default 2; sv_autotune times

@@ -121,24 +121,6 @@ struct PairWalk {
 
 constexpr int kPairBatch = 4;
 
-// The list entries of a thread's next kPairBatch pairs (ok[v]: pair v exists).  The lists
-// are read-only during a sweep, so the whole-sweep kernels load a batch's entries ahead:
-// the first batch of an operator before its grid barrier, each next batch while the
-// current batch's amplitudes are in flight.
-struct PairBatch {
-    uint32_t ea[kPairBatch], eb[kPairBatch];
-    bool ok[kPairBatch];
-    __device__ __forceinline__ void load(PairWalk &w, const uint32_t *al, const uint32_t *bl, int nb_l) {
-        #pragma unroll
-        for (int v = 0; v < kPairBatch; ++v) {
-            ok[v] = w.r < nb_l;
-            eb[v] = ok[v] ? bl[w.r] : 0u;  // 0: rank 0, in bounds
-            ea[v] = ok[v] ? al[w.i] : 0u;
-            w.next();
-        }
-    }
-};
-
 // psi <- exp(theta G) psi over the op's pairs.
 template <typename A>
 __global__ void __launch_bounds__(kThreads) k_rotate_l(A *__restrict__ psi, const uint32_t *__restrict__ al,
@@ -284,171 +266,6 @@ __global__ void __launch_bounds__(kThreads) k_adjoint_li(A *__restrict__ CL, con
     }
     const double s = block_sum(acc, red);
     if (threadIdx.x == 0) partial[blockIdx.x] = s;
-}
-
-// ---------------------------------------------------------------- whole sweeps in one launch
-
-// The forward and reverse sweeps as one persistent launch each: the grid walks the
-// operators in order, every block taking its share of an operator's pairs exactly as
-// k_rotate_l / k_adjoint_li do, with a grid-wide barrier between operators (an
-// operator reads amplitudes the previous one wrote in other blocks).  The per-operator
-// launches of sector storage are latency bound (a few microseconds of work each on
-// L2-resident data): one launch replaces their launch gaps and ramp-ups with barriers.
-// Launched cooperatively, so every block is resident and every barrier can complete;
-// each wait is still bounded -- past the limit the block sets *err and stops, and the
-// call reports the failure.
-struct SweepArgs {
-    const uint32_t *lists;   // the ops' pair lists (k_build_lists)
-    const int4 *info;        // per op: alpha offset, alpha length, beta offset, beta length
-    const double2 *cs;       // per op: (cos theta, sin theta)
-    int n_ops, Da, Db;
-    unsigned int *bar;       // barrier arrivals, zero at launch
-    int *err;                // set to 1 when a barrier wait runs out
-    uint32_t spins;          // polls of a barrier wait
-    double *partial;         // reverse sweep: [n_ops][gridDim.x] gradient partials
-};
-
-// Grid-wide barrier number `gen` (0, 1, ...): every block arrives once per barrier.
-__device__ __forceinline__ bool sweep_barrier(const SweepArgs &g, unsigned int gen, volatile int *s_ok) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(g.bar, 1u);
-        const unsigned int target = (gen + 1u) * gridDim.x;
-        bool ok = true;
-        for (uint32_t it = 0; *(volatile unsigned int *)g.bar < target; ++it) {
-            if (it >= g.spins) {
-                ok = false;
-                atomicExch(g.err, 1);
-                break;
-            }
-            __nanosleep(32);
-        }
-        __threadfence();
-        *s_ok = ok;
-    }
-    __syncthreads();
-    return *s_ok;
-}
-
-template <typename A>
-__global__ void __launch_bounds__(kThreads) k_sweep_rotate_l(A *__restrict__ psi, SweepArgs g) {
-    using R = real_of<A>;
-    __shared__ volatile int s_ok;
-    unsigned int gen = 0;
-    for (int k = 0; k < g.n_ops; ++k) {
-        const int4 li = g.info[k];
-        const int na_l = li.y, nb_l = li.w;
-        if (na_l <= 0 || nb_l <= 0) continue;  // no pair in the sector: nothing written, no barrier
-        const uint32_t *al = g.lists + li.x, *bl = g.lists + li.z;
-        PairWalk w(na_l);
-        bool more = w.r < nb_l;
-        PairBatch cur;
-        cur.load(w, al, bl, nb_l);
-        if (gen > 0 && !sweep_barrier(g, gen - 1, &s_ok)) return;
-        ++gen;
-        const R c = (R)g.cs[k].x, sn = (R)g.cs[k].y;
-        while (more) {
-            size_t I[kPairBatch], J[kPairBatch];
-            R ss[kPairBatch];
-            #pragma unroll
-            for (int v = 0; v < kPairBatch; ++v) {
-                I[v] = (size_t)(cur.eb[v] & 0x7FFFu) * g.Da + (cur.ea[v] & 0x7FFFu);
-                J[v] = (size_t)(cur.eb[v] >> 16) * g.Da + (cur.ea[v] >> 16);
-                ss[v] = ((cur.ea[v] ^ cur.eb[v]) & 0x8000u) ? -sn : sn;
-                if (!(SV_IN_RANGE(I[v], (size_t)g.Da * g.Db, kChkPair) && SV_IN_RANGE(J[v], (size_t)g.Da * g.Db, kChkPair))) {
-                    cur.ok[v] = false;  // checked build: skip the pair
-                    I[v] = J[v] = 0;
-                }
-            }
-            A u[kPairBatch], x[kPairBatch];
-            #pragma unroll
-            for (int v = 0; v < kPairBatch; ++v) {
-                u[v] = psi[I[v]];
-                x[v] = psi[J[v]];
-            }
-            more = w.r < nb_l;
-            PairBatch nxt;
-            if (more) nxt.load(w, al, bl, nb_l);
-            #pragma unroll
-            for (int v = 0; v < kPairBatch; ++v) {
-                if (!cur.ok[v]) continue;
-                psi[I[v]] = lin2<A>(c, u[v], -ss[v], x[v]);
-                psi[J[v]] = lin2<A>(c, x[v], ss[v], u[v]);
-            }
-            if (more) cur = nxt;
-        }
-    }
-}
-
-// Reverse sweep on the interleaved (psi, lambda) matrix, ops n_ops - 1 down to 0; the
-// arithmetic of k_adjoint_li, one float64 partial per block and op (fixed order).
-template <typename A>
-__global__ void __launch_bounds__(kThreads) k_sweep_adjoint_li(A *__restrict__ CL, SweepArgs g) {
-    using R = real_of<A>;
-    __shared__ double red[kThreads / 32];
-    __shared__ volatile int s_ok;
-    AmpPair<A> *P = reinterpret_cast<AmpPair<A> *>(CL);
-    unsigned int gen = 0;
-    for (int k = g.n_ops - 1; k >= 0; --k) {
-        const int4 li = g.info[k];
-        const int na_l = li.y, nb_l = li.w;
-        double acc = 0.0;
-        if (na_l > 0 && nb_l > 0) {
-            const uint32_t *al = g.lists + li.x, *bl = g.lists + li.z;
-            PairWalk w(na_l);
-            bool more = w.r < nb_l;
-            PairBatch cur;
-            cur.load(w, al, bl, nb_l);
-            if (gen > 0 && !sweep_barrier(g, gen - 1, &s_ok)) return;
-            ++gen;
-            const R c = (R)g.cs[k].x, sn = (R)g.cs[k].y;
-            while (more) {
-                size_t I[kPairBatch], J[kPairBatch];
-                bool neg[kPairBatch];
-                #pragma unroll
-                for (int v = 0; v < kPairBatch; ++v) {
-                    I[v] = (size_t)(cur.eb[v] & 0x7FFFu) * g.Da + (cur.ea[v] & 0x7FFFu);
-                    J[v] = (size_t)(cur.eb[v] >> 16) * g.Da + (cur.ea[v] >> 16);
-                    neg[v] = ((cur.ea[v] ^ cur.eb[v]) & 0x8000u) != 0u;
-                    if (!(SV_IN_RANGE(I[v], (size_t)g.Da * g.Db, kChkPair) &&
-                          SV_IN_RANGE(J[v], (size_t)g.Da * g.Db, kChkPair))) {
-                        cur.ok[v] = false;  // checked build: skip the pair
-                        I[v] = J[v] = 0;
-                    }
-                }
-                AmpPair<A> pu[kPairBatch], px[kPairBatch];
-                #pragma unroll
-                for (int v = 0; v < kPairBatch; ++v) {
-                    pu[v] = P[I[v]];
-                    px[v] = P[J[v]];
-                }
-                more = w.r < nb_l;
-                PairBatch nxt;
-                if (more) nxt.load(w, al, bl, nb_l);
-                R t = 0;
-                #pragma unroll
-                for (int v = 0; v < kPairBatch; ++v) {
-                    if (!cur.ok[v]) continue;
-                    const A u = pu[v].c, x = px[v].c, lu = pu[v].l, lx = px[v].l;
-                    const R ti = re_dot(lx, u) - re_dot(lu, x);
-                    t += neg[v] ? -ti : ti;
-                    const R ss = neg[v] ? -sn : sn;
-                    AmpPair<A> ou, ox;
-                    ou.c = lin2<A>(c, u, ss, x);
-                    ox.c = lin2<A>(c, x, -ss, u);
-                    ou.l = lin2<A>(c, lu, ss, lx);
-                    ox.l = lin2<A>(c, lx, -ss, lu);
-                    P[I[v]] = ou;
-                    P[J[v]] = ox;
-                }
-                acc += (double)t;
-                if (more) cur = nxt;
-            }
-        }
-        const double s = block_sum(acc, red);
-        if (threadIdx.x == 0) g.partial[(size_t)k * gridDim.x + blockIdx.x] = s;
-    }
 }
 
 // The row sums' arithmetic: float32 or float64 for those states, float-float (hi + lo
@@ -606,20 +423,20 @@ __global__ void k_gather_c(const A *__restrict__ psi, const uint32_t *__restrict
 }
 
 // A handle's vector from its compute core's compact amplitudes (Out the handle's type, In the
-// core's: the same, or its real one).  sa / sb: the strings' storage-space spreads (dense
-// storage, the sector's addresses of the 2^n vector), or NULL (sector storage, same order).
+// core's: the same, or its real one): string pair (a, b) of the core, at ca[a] + cb[b] of the
+// vector (dense storage: the storage-space spreads; sector storage: the ranks in its order).
 // Bound: dense, one partly written 32-byte DRAM sector per scattered amplitude.
 template <typename Out, typename In>
 __global__ void __launch_bounds__(kThreads) k_core_publish(const In *__restrict__ C, Out *__restrict__ psi,
-                                                           const uint32_t *__restrict__ sa,
-                                                           const uint32_t *__restrict__ sb, int Da, int Db) {
+                                                           const uint32_t *__restrict__ ca,
+                                                           const uint32_t *__restrict__ cb, int Da, int Db) {
     using R = real_of<Out>;
     for (int Ib = blockIdx.x; Ib < Db; Ib += gridDim.x) {
         const size_t row = (size_t)Ib * Da;
-        const uint32_t xb = sb ? sb[Ib] : 0u;
+        const uint32_t xb = cb[Ib];
         for (int Ia = blockIdx.y * kThreads + threadIdx.x; Ia < Da; Ia += gridDim.y * kThreads) {
             const In c = C[row + Ia];
-            psi[sa ? (size_t)(sa[Ia] | xb) : row + Ia] = mka<Out>((R)re(c), (R)im(c));
+            psi[xb + ca[Ia]] = mka<Out>((R)re(c), (R)im(c));
         }
     }
 }
@@ -627,14 +444,14 @@ __global__ void __launch_bounds__(kThreads) k_core_publish(const In *__restrict_
 // The other way: the compact amplitudes (their real parts for a real core) of a stored reference.
 template <typename Out, typename In>
 __global__ void __launch_bounds__(kThreads) k_core_gather(const In *__restrict__ psi, Out *__restrict__ C,
-                                                          const uint32_t *__restrict__ sa,
-                                                          const uint32_t *__restrict__ sb, int Da, int Db) {
+                                                          const uint32_t *__restrict__ ca,
+                                                          const uint32_t *__restrict__ cb, int Da, int Db) {
     using R = real_of<Out>;
     for (int Ib = blockIdx.x; Ib < Db; Ib += gridDim.x) {
         const size_t row = (size_t)Ib * Da;
-        const uint32_t xb = sb ? sb[Ib] : 0u;
+        const uint32_t xb = cb[Ib];
         for (int Ia = blockIdx.y * kThreads + threadIdx.x; Ia < Da; Ia += gridDim.y * kThreads) {
-            const In c = psi[sa ? (size_t)(sa[Ia] | xb) : row + Ia];
+            const In c = psi[xb + ca[Ia]];
             C[row + Ia] = mka<Out>((R)re(c), (R)im(c));
         }
     }
@@ -644,20 +461,20 @@ __global__ void __launch_bounds__(kThreads) k_core_gather(const In *__restrict__
 
 // publish: core (core_dtype) -> handle (dtype); else the handle's vector -> core.
 cudaError_t launch_core_move(void *handle_vec, int dtype, void *core_vec, int core_dtype, bool publish,
-                             const uint32_t *sa, const uint32_t *sb, int Da, int Db, int sm_count, cudaStream_t st) {
+                             const uint32_t *ca, const uint32_t *cb, int Da, int Db, int sm_count, cudaStream_t st) {
     if (Da <= 0 || Db <= 0) return cudaSuccess;
     // rows over the grid's x, a row's columns over its y: enough blocks for few long or many short rows
     const int gy = (Da + kThreads - 1) / kThreads, cap = sm_count * 16;
     const dim3 grid(Db < cap ? Db : cap, gy < 8 ? gy : 8);
     if (dtype == core_dtype) {
         SV_DISPATCH_AMP(dtype,
-                        if (publish) k_core_publish<A, A><<<grid, kThreads, 0, st>>>((const A *)core_vec, (A *)handle_vec, sa, sb, Da, Db);
-                        else k_core_gather<A, A><<<grid, kThreads, 0, st>>>((const A *)handle_vec, (A *)core_vec, sa, sb, Da, Db));
+                        if (publish) k_core_publish<A, A><<<grid, kThreads, 0, st>>>((const A *)core_vec, (A *)handle_vec, ca, cb, Da, Db);
+                        else k_core_gather<A, A><<<grid, kThreads, 0, st>>>((const A *)handle_vec, (A *)core_vec, ca, cb, Da, Db));
     } else {  // a complex handle with a real core of the same precision
         SV_DISPATCH_AMP(dtype, if constexpr (AmpT<A>::kCplx) {
             using B = real_of<A>;
-            if (publish) k_core_publish<A, B><<<grid, kThreads, 0, st>>>((const B *)core_vec, (A *)handle_vec, sa, sb, Da, Db);
-            else k_core_gather<B, A><<<grid, kThreads, 0, st>>>((const A *)handle_vec, (B *)core_vec, sa, sb, Da, Db);
+            if (publish) k_core_publish<A, B><<<grid, kThreads, 0, st>>>((const B *)core_vec, (A *)handle_vec, ca, cb, Da, Db);
+            else k_core_gather<B, A><<<grid, kThreads, 0, st>>>((const A *)handle_vec, (B *)core_vec, ca, cb, Da, Db);
         });
     }
     return cudaGetLastError();
@@ -748,50 +565,6 @@ cudaError_t launch_adjoint_li(void *CL, int dtype, const uint32_t *al, int na_l,
     SV_DISPATCH_AMP(dtype, k_adjoint_li<A><<<grid, kThreads, 0, st>>>((A *)CL, al, na_l, bl, nb_l, Da,
                                                                        (real_of<A>)c, (real_of<A>)s, partial));
     return cudaGetLastError();
-}
-
-// Blocks of a whole-sweep launch: at most bps per SM (8 by default) and no more than
-// can be resident at once (a cooperative launch needs every block resident).
-template <typename K>
-static int sweep_grid_for(K kernel, int Db, int sm_count, int bps) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    const int want = bps > 0 ? bps : 8;
-    if (per_sm > want) per_sm = want;
-    const int cap = per_sm * sm_count;
-    return Db < cap ? Db : cap;
-}
-
-int sweep_grid(int dtype, bool adjoint, int Db, int sm_count, int bps) {
-    int grid = 0;
-    SV_DISPATCH_AMP(dtype, grid = adjoint ? sweep_grid_for(k_sweep_adjoint_li<A>, Db, sm_count, bps)
-                                          : sweep_grid_for(k_sweep_rotate_l<A>, Db, sm_count, bps));
-    return grid;
-}
-
-// One cooperative launch of the forward (adjoint = false: ops 0 .. n_ops-1 on psi) or the
-// reverse sweep (adjoint = true: ops n_ops-1 .. 0 on the interleaved matrix, gradient
-// partials [n_ops][grid] into partial).  info: the ops' int4 list records (device), cs
-// their (cos, sin) (device), bar a zeroed device counter, err the device error flag.
-// A refused cooperative launch returns its error (the caller falls back to one launch
-// per op).
-cudaError_t launch_sweep_l(void *buf, int dtype, bool adjoint, const uint32_t *lists, const int *info,
-                           const double *cs, int n_ops, int Da, int Db, int grid, unsigned int *bar, int *err,
-                           uint32_t spins, double *partial, cudaStream_t st) {
-    if (n_ops <= 0) return cudaSuccess;
-    if (grid <= 0) return cudaErrorInvalidValue;
-    SweepArgs g;
-    g.lists = lists; g.info = (const int4 *)info; g.cs = (const double2 *)cs; g.n_ops = n_ops; g.Da = Da; g.Db = Db;
-    g.bar = bar; g.err = err; g.spins = spins; g.partial = partial;
-    void *args[] = {&buf, &g};
-    cudaError_t e = cudaErrorInvalidValue;
-    SV_DISPATCH_AMP(dtype, e = cudaLaunchCooperativeKernel(
-                               adjoint ? (const void *)k_sweep_adjoint_li<A> : (const void *)k_sweep_rotate_l<A>,
-                               dim3(grid), dim3(kThreads), args, 0, st));
-    return e;
 }
 
 int rdm_rows_elements(int n) { return 1 + n + (n / 2) * (n / 2 - 1); }

@@ -58,10 +58,21 @@ cudaError_t launch_build_lists(const void *ops, int n_ops, const uint32_t *sa, c
                                int Da, int Db, uint32_t *out, cudaStream_t st);
 cudaError_t launch_rotate_l(void *psi, int dtype, const uint32_t *al, int na_l, const uint32_t *bl, int nb_l, int Da,
                             double c, double s, int grid, cudaStream_t st);
-int sweep_grid(int dtype, bool adjoint, int Db, int sm_count, int bps);
-cudaError_t launch_sweep_l(void *buf, int dtype, bool adjoint, const uint32_t *lists, const int *info,
-                           const double *cs, int n_ops, int Da, int Db, int grid, unsigned int *bar, int *err,
-                           uint32_t spins, double *partial, cudaStream_t st);
+// whole sector sweeps (k_sweep.cu)
+size_t sweep_stage_bytes(int dtype, uint64_t words, int n_groups, int n_ops);
+size_t sweep_angle_bytes(int dtype);
+void sweep_angles(const OpDesc *ops, int n_ops, int dtype, void *out);
+int plan_groups(const OpDesc *ops, int n_ops, int N, int na, int nb, std::vector<uint8_t> &plans, std::vector<uint8_t> &groups,
+                uint64_t *words, long long *most, long long *all);
+cudaError_t launch_build_groups(const void *plans, int n_groups, const uint32_t *sa, const uint32_t *sb, const uint16_t *stra,
+                                const uint16_t *strb, const uint16_t *ra, const uint16_t *rb, int Da, int Db, int sorted, void *out,
+                                cudaStream_t st);
+size_t sweep_block_smem(int dtype, bool adjoint, int Da, int Db);
+int sweep_grid_blocks(int dtype, bool adjoint, int sm_count, int bps);
+cudaError_t launch_sweep(void *psi, const void *lam, int dtype, bool adjoint, int form, int blocks, int threads, uint32_t words,
+                         const void *lists, const void *groups, int n_groups, const void *angles, int n_ops, int Da, int Db,
+                         long long init, void *work, unsigned int *bar, int *err, uint32_t spins, double *partial, cudaStream_t st);
+cudaError_t launch_sweep_grad(const double *partial, int dtype, int n_ops, int warps, double *out, cudaStream_t st);
 cudaError_t launch_adjoint_li(void *CL, int dtype, const uint32_t *al, int na_l, const uint32_t *bl, int nb_l, int Da,
                               double c, double s, int grid, double *partial, cudaStream_t st);
 cudaError_t launch_adjoint_l(void *psi, void *lam, int dtype, const uint32_t *al, int na_l, const uint32_t *bl,
@@ -123,6 +134,7 @@ namespace svk {
 void set_thread_error(const std::string &m) { g_err = m; }
 // the check words of the kernel units (sv_check.cuh)
 uint32_t check_word_sector();
+uint32_t check_word_sweep();
 uint32_t check_word_rows();
 uint32_t check_word_abtc();
 uint32_t check_word_pool();
@@ -389,14 +401,26 @@ static sv_status ensure_strings(sv_handle h) {
         h->str_sa = h->str_sb = h->str_sa_s = h->str_sb_s = nullptr;
     }
     const int N = h->n / 2;
+    // Ascending (the documented order of sector storage), but in a core with orbital 0 as the most
+    // significant: an excitation p -> q touches runs of strings that agree on every orbital down to
+    // the less significant of the two, longer where that is a virtual (high) orbital.  At 30 qubits
+    // its doubles touch 0.35 32-byte sectors per float32 amplitude instead of 0.54.  For
+    // float32 sectors of at least 2^21 determinants, whose sweeps L2's bandwidth bounds
+    // (30 qubits: 0.82 / 1.19 ms ascending, 0.69 / 0.97 ms so; 26 qubits, 1.7 million: no change).
+    const bool reversed = h->outer && single_prec(h->dtype) && h->elems >= (1u << 21);
     auto strings = [&](int k, std::vector<uint16_t> &str, std::vector<uint16_t> &rank) {
         rank.assign((size_t)1 << N, 0xFFFFu);
         str.clear();
-        for (uint32_t s = 0; s < (1u << N); ++s)
-            if (__builtin_popcount(s) == k) {
-                rank[s] = (uint16_t)str.size();
-                str.push_back((uint16_t)s);
+        for (uint32_t v = 0; v < (1u << N); ++v) {
+            if (__builtin_popcount(v) != k) continue;
+            uint32_t s = v;
+            if (reversed) {
+                s = 0;
+                for (int p = 0; p < N; ++p) s |= ((v >> p) & 1u) << (N - 1 - p);
             }
+            rank[s] = (uint16_t)str.size();
+            str.push_back((uint16_t)s);
+        }
     };
     std::vector<uint16_t> sa16, sb16, ra, rb;
     strings(h->na, sa16, ra);
@@ -731,10 +755,10 @@ static sv_status ensure_rdm_lists(sv_handle h) {
     return ensure_op_lists(h, ops, h->rdm_lists);
 }
 
-// Sector storage: the ops' (cos, sin) on the device for whole-sweep launches (uploaded
-// once per call; the reverse sweep reuses them).
+// Sector storage: the ops' angles on the device for whole-sweep launches (uploaded once per
+// call; the reverse sweep reuses them), after 256 bytes for the grid form's barrier.
 static sv_status upload_sweep_angles(sv_handle h, const std::vector<OpDesc> &ops) {
-    const size_t need = 256 + 2 * std::max<size_t>(ops.size(), 1) * sizeof(double);
+    const size_t one = sweep_angle_bytes(h->dtype), need = 256 + one * std::max<size_t>(ops.size(), 1);
     if (h->sweep_bytes < need) {
         dev_free(h, h->sweep_buf, h->sweep_bytes);
         h->sweep_buf = nullptr;
@@ -742,52 +766,141 @@ static sv_status upload_sweep_angles(sv_handle h, const std::vector<OpDesc> &ops
         SV_TRY(dev_alloc(h, &h->sweep_buf, need, "sweep angles"));
         h->sweep_bytes = need;
     }
-    h->sweep_host.resize(2 * ops.size());
-    for (size_t k = 0; k < ops.size(); ++k) {
-        h->sweep_host[2 * k] = ops[k].c;
-        h->sweep_host[2 * k + 1] = ops[k].s;
-    }
+    h->sweep_host.resize((one * ops.size() + 7) / 8);
+    sweep_angles(ops.data(), (int)ops.size(), h->dtype, h->sweep_host.data());
     if (!ops.empty())
-        SV_CUDA(h, cudaMemcpyAsync((uint8_t *)h->sweep_buf + 256, h->sweep_host.data(), 2 * ops.size() * sizeof(double),
+        SV_CUDA(h, cudaMemcpyAsync((uint8_t *)h->sweep_buf + 256, h->sweep_host.data(), one * ops.size(),
                                    cudaMemcpyHostToDevice, h->stream));
     return SV_OK;
 }
 
-// One launch for a whole sector sweep (forward on psi, or reverse on the interleaved
-// matrix with gradient partials [L][grid]); false (nothing launched) where the
-// cooperative launch is refused or the option is off: the caller then launches per op.
-static bool sweep_once(sv_handle h, bool adjoint, void *buf, size_t L, int grid, double *partial) {
-    if (!h->sweep_mode || L == 0 || grid <= 0 || !h->sweep_buf || !h->kerr) return false;
-    if (cudaMemsetAsync(h->sweep_buf, 0, sizeof(unsigned int), h->stream) != cudaSuccess) {
+// Sector storage: the steps of the ops' whole sweeps (k_build_groups), kept on the device and
+// rebuilt only when the ops' masks (or the sector) change.
+static sv_status ensure_groups(sv_handle h, const std::vector<OpDesc> &ops) {
+    SV_TRY(ensure_strings(h));
+    SweepGroups &c = h->groups;
+    std::vector<uint32_t> key;
+    key.reserve(3 * ops.size() + 2);
+    key.push_back((uint32_t)h->na);
+    key.push_back((uint32_t)h->nb);
+    for (const OpDesc &d : ops) {
+        key.push_back(d.m);
+        key.push_back(d.from);
+        key.push_back(d.sm);
+    }
+    if (c.buf && key == c.key) return SV_OK;
+    std::vector<uint8_t> plans, groups;
+    uint64_t words = 0;
+    long long most = 0, all = 0;
+    const int n = plan_groups(ops.data(), (int)ops.size(), h->n / 2, h->na, h->nb, plans, groups, &words, &most, &all);
+    if (words > (uint64_t)UINT32_MAX) return fail(h, SV_ERR_ARG, "operator pair lists exceed 2^32 entries");
+    auto r16 = [](size_t x) { return (x + 15) / 16 * 16; };
+    const size_t lb = r16((size_t)words * 8 + 16), pb = r16(plans.size()), need = lb + pb + groups.size();
+    if (c.bytes < need) {
+        dev_free(h, c.buf, c.bytes);
+        c.buf = nullptr;
+        c.bytes = 0;
+        c.key.clear();
+        SV_TRY(dev_alloc(h, &c.buf, need, "sweep steps"));
+        c.bytes = need;
+    }
+    uint8_t *dp = (uint8_t *)c.buf + lb;
+    SV_CUDA(h, cudaMemcpyAsync(dp, plans.data(), plans.size(), cudaMemcpyHostToDevice, h->stream));
+    SV_CUDA(h, cudaMemcpyAsync(dp + pb, groups.data(), groups.size(), cudaMemcpyHostToDevice, h->stream));
+    SV_CUDA(h, launch_build_groups(dp, n, h->str_sa, h->str_sb, h->str_a, h->str_b, h->rank_a, h->rank_b, h->Da, h->Db,
+                                   single_prec(h->dtype) ? 0 : 1, c.buf,
+                                   h->stream));
+    h->launches++;
+    SV_CUDA(h, cudaStreamSynchronize(h->stream));  // the host staging vectors go out of scope
+    c.key = key;
+    c.dgroups = dp + pb;
+    c.n_groups = n;
+    c.n_ops = (int)ops.size();
+    c.words = words;
+    c.most = most;
+    c.all = all;
+    return SV_OK;
+}
+
+// Form and geometry of a whole sweep over h->groups (k_sweep): -1 where none runs.
+struct SweepShape {
+    int form = -1, blocks = 0, threads = 0;
+    uint32_t words = 0;
+    int warps() const { return blocks * threads / 32; }
+};
+
+static SweepShape sweep_shape(sv_handle h, bool adjoint, size_t n_ops) {
+    SweepShape s;
+    if (h->storage != 1 || !h->sweep_mode || n_ops == 0) return s;
+    // Pairs of an operator on average: what a step has to move.  Measured, forward / reverse ms:
+    // 16 qubits (100 pairs, float64) block 0.115 / 0.199, cluster 0.19 / 0.28; 18 qubits (600)
+    // block 0.094 / 0.18, cluster 0.072 / 0.115, grid 0.097 / 0.130; 20 qubits (800, float32)
+    // cluster 0.037 / 0.044, grid 0.055 / 0.069; 20 qubits (4,300, complex float64) cluster
+    // 0.136 / 0.204, grid 0.147 / 0.198; 22 qubits (14,000) cluster 0.18 / 0.25, grid 0.127 / 0.170.
+    const long long avg = h->groups.all / (long long)n_ops;
+    // the block and cluster forms wait on hardware barriers: a caller who wants waits given up
+    // after a few polls gets the grid form, whose waits SV_OPT_WAIT_POLLS bounds
+    const bool hw = h->wait_polls >= 1024;
+    const size_t bs = sweep_block_smem(h->dtype, adjoint, h->Da, h->Db), cap = 226 * 1024;
+    s.form = hw && bs <= cap && avg <= 300 ? 0 : hw && avg <= 4000 ? 1 : 2;
+    if (s.form == 0) {
+        s.blocks = 1;
+        s.threads = (int)std::min<long long>(512, std::max<long long>(64, (h->groups.most + 31) / 32 * 32));
+        if (bs + sweep_stage_bytes(h->dtype, h->groups.words, h->groups.n_groups, (int)n_ops) <= cap)
+            s.words = (uint32_t)h->groups.words;
+    } else if (s.form == 1) {
+        s.blocks = 16;
+        s.threads = 512;
+    } else {
+        // one block per SM where that covers an operator's pairs: fewer arrivals at each barrier
+        // (24 qubits, 25,000 pairs: 0.152 / 0.170 ms with one, 0.169 / 0.196 with two; 26 qubits,
+        // 130,000: 0.215 / 0.281 and 0.181 / 0.236)
+        s.threads = 256;
+        s.blocks = sweep_grid_blocks(h->dtype, adjoint, h->sm_count, avg < 60000 ? 1 : h->sweep_bps);
+        if (s.blocks <= 0) s.form = -1;
+    }
+    return s;
+}
+
+// One launch for a whole sector sweep (forward on psi, or reverse from psi and lambda with
+// the gradient sums [L][warps] in h->partials); false (nothing launched) where it is refused:
+// the caller then launches per op.
+static bool sweep_once(sv_handle h, const SweepShape &s, bool adjoint, void *psi, const void *lam, void *work, long long init) {
+    if (s.form < 0 || !h->sweep_buf) return false;
+    if (s.form == 2 && (!h->kerr || cudaMemsetAsync(h->sweep_buf, 0, sizeof(unsigned int), h->stream) != cudaSuccess)) {
         cudaGetLastError();
         return false;
     }
-    const cudaError_t e = launch_sweep_l(buf, h->dtype, adjoint, (const uint32_t *)h->lists.buf, h->lists.dinfo,
-                                         (const double *)((const uint8_t *)h->sweep_buf + 256), (int)L, h->Da, h->Db,
-                                         grid,
-                                         (unsigned int *)h->sweep_buf, h->kerr, (uint32_t)h->wait_polls, partial,
-                                         h->stream);
+    const cudaError_t e =
+        launch_sweep(psi, lam, h->dtype, adjoint, s.form, s.blocks, s.threads, s.words, h->groups.buf, h->groups.dgroups,
+                     h->groups.n_groups, (const uint8_t *)h->sweep_buf + 256, h->groups.n_ops, h->Da, h->Db, init, work,
+                     (unsigned int *)h->sweep_buf, h->kerr, (uint32_t)h->wait_polls, h->partials, h->stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     h->launches++;
-    cudaMemcpyAsync(h->hkerr, h->kerr, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+    if (s.form == 2) cudaMemcpyAsync(h->hkerr, h->kerr, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
     return true;
 }
 
-static sv_status forward(sv_handle h, const std::vector<OpDesc> &ops, bool checkpoints) {
+// U_L ... U_1 on psi; from_ref: on the handle's reference, written first.
+static sv_status forward(sv_handle h, const std::vector<OpDesc> &ops, bool checkpoints, bool from_ref) {
     const int64_t C = h->ckpt_interval;
-    if (h->storage == 1 && !ops.empty()) {
-        SV_TRY(ensure_op_lists(h, ops, h->lists));
-        SV_TRY(ensure_kerr(h));
+    if (h->storage == 1 && !ops.empty() && h->sweep_mode && !(checkpoints && C > 0 && (size_t)C < ops.size())) {
+        // one launch for the whole sweep (checkpoint copies would be due in its middle)
+        SV_TRY(ensure_groups(h, ops));
         SV_TRY(upload_sweep_angles(h, ops));
-        // one launch for the whole sweep unless checkpoint copies are due in the middle
-        if (!(checkpoints && C > 0 && (size_t)C < ops.size()) &&
-            sweep_once(h, false, h->psi, ops.size(), sweep_grid(h->dtype, false, h->Db, h->sm_count, h->sweep_bps),
-                       nullptr))
+        const SweepShape s = sweep_shape(h, false, ops.size());
+        if (s.form == 2) SV_TRY(ensure_kerr(h));
+        const bool det = from_ref && h->ref_kind == 1;  // written by the sweep itself
+        if (from_ref && !det) SV_TRY(prepare_reference(h));
+        if (sweep_once(h, s, false, h->psi, nullptr, nullptr, det ? (long long)compact_index(h, h->ref_det) : -1))
             return SV_OK;
+        from_ref = det;
     }
+    if (from_ref) SV_TRY(prepare_reference(h));
+    if (h->storage == 1 && !ops.empty()) SV_TRY(ensure_op_lists(h, ops, h->lists));
     const uint32_t *L = (const uint32_t *)h->lists.buf;
     const int G = sector_grid(h->Db, h->sm_count, h->sect_bps);
     for (size_t k = 0; k < ops.size(); ++k) {
@@ -1218,19 +1331,42 @@ static bool core_wanted(sv_handle h) {
 static void drop_core(sv_handle h) {
     if (!h->core) return;
     h->launches += h->core->launches;
+    if (h->core_map) cudaFree(h->core_map);
+    h->core_map = nullptr;
     destroy_handle(h->core);
     h->core = nullptr;
     h->core_cur = 0;
     h->core_ref = false;
 }
 
-// The storage-space spreads of the handle's strings (NULL in sector storage: same order).
-static sv_status core_spreads(sv_handle h, const uint32_t **sa, const uint32_t **sb) {
-    *sa = *sb = nullptr;
-    if (h->storage == 1) return SV_OK;
-    SV_TRY(ensure_strings(h));
-    *sa = h->str_sa_s;
-    *sb = h->str_sb_s;
+// Where the core's strings lie in the handle's vector: string pair (a, b) at *ca[a] + *cb[b]; kept on
+// the device while the handle's layout stays.
+static sv_status core_places(sv_handle h, const uint32_t **ca, const uint32_t **cb) {
+    sv_handle c = h->core;
+    SV_TRY(ensure_strings(c));
+    if (!h->core_map || memcmp(h->core_map_perm, h->perm, sizeof h->perm) != 0) {
+        const int N = h->n / 2;
+        std::vector<uint32_t> m((size_t)c->Da + c->Db);
+        if (h->storage == 1) SV_TRY(ensure_strings(h));
+        for (int spin = 0; spin < 2; ++spin) {
+            const std::vector<uint16_t> &str = spin ? c->h_strb : c->h_stra;
+            for (size_t i = 0; i < str.size(); ++i) {
+                uint32_t at = 0;
+                if (h->storage == 1) {
+                    at = spin ? (uint32_t)h->h_rb[str[i]] * (uint32_t)h->Da : h->h_ra[str[i]];
+                } else {
+                    for (int p = 0; p < N; ++p) at |= (uint32_t)((str[i] >> p) & 1u) << h->perm[2 * p + spin];
+                }
+                m[(spin ? (size_t)c->Da : 0) + i] = at;
+            }
+        }
+        if (!h->core_map) SV_TRY(dev_alloc(c, (void **)&h->core_map, m.size() * sizeof(uint32_t), "core addresses"));
+        SV_CUDA(h, cudaMemcpyAsync(h->core_map, m.data(), m.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, h->stream));
+        SV_CUDA(h, cudaStreamSynchronize(h->stream));  // the host vector goes out of scope
+        memcpy(h->core_map_perm, h->perm, sizeof h->perm);
+    }
+    *ca = h->core_map;
+    *cb = h->core_map + c->Da;
     return SV_OK;
 }
 
@@ -1265,10 +1401,9 @@ static sv_status ensure_core(sv_handle h) {
     c->ref_kind = h->ref_kind;
     c->ref_det = h->ref_det;
     if (h->ref_kind == 2 && !h->core_ref) {
-        SV_TRY(ensure_strings(c));
         if (!c->ref_vec) SV_TRY(dev_alloc(c, &c->ref_vec, vec_bytes(c), "reference copy"));
         const uint32_t *sa, *sb;
-        SV_TRY(core_spreads(h, &sa, &sb));
+        SV_TRY(core_places(h, &sa, &sb));
         SV_CUDA(c, launch_core_move(h->ref_vec, h->dtype, c->ref_vec, c->dtype, false, sa, sb, c->Da, c->Db, c->sm_count,
                                     h->stream));
         c->launches++;
@@ -1281,7 +1416,7 @@ static sv_status ensure_core(sv_handle h) {
 static sv_status core_publish(sv_handle h) {
     sv_handle c = h->core;
     const uint32_t *sa, *sb;
-    SV_TRY(core_spreads(h, &sa, &sb));
+    SV_TRY(core_places(h, &sa, &sb));
     if (h->storage == 0 && (!h->psi_clean || h->exposed))
         SV_CUDA(h, cudaMemsetAsync(h->psi, 0, vec_bytes(h), h->stream));
     SV_CUDA(h, launch_core_move(h->psi, h->dtype, c->psi, c->dtype, true, sa, sb, c->Da, c->Db, h->sm_count, h->stream));
@@ -1388,15 +1523,17 @@ static sv_status autotune_impl(sv_handle h, sv_ham_handle ham, const std::vector
             if (d[j].nbits == 4 && d[j].pos[0] >= 4) { k = j; break; }
         // sector storage with whole-sweep launches: the two sweeps themselves are timed, on
         // copies (blocks per SM 1, 2, 4, 8); else one rotation and one adjoint step
-        const bool sweeps = h->storage == 1 && h->sweep_mode && h->ckpt_interval <= 0 && adj;
+        bool sweeps = h->storage == 1 && h->sweep_mode && h->ckpt_interval <= 0 && adj;
         const int cands_op[] = {4, 8, 16, 32}, cands_sw[] = {1, 2, 4, 8};
         int best_b = 8;
         float best_t = -1.f;
         if (h->storage == 1) SV_TRY(ensure_op_lists(h, d, h->lists));
-        SV_TRY(ensure_partials(h, (size_t)h->sm_count * 32 * (sweeps ? d.size() : 1)));
+        SV_TRY(ensure_partials(h, (size_t)h->sm_count * 64 * (sweeps ? d.size() : 1)));
         if (sweeps) {
+            SV_TRY(ensure_groups(h, d));
             SV_TRY(ensure_kerr(h));
             SV_TRY(upload_sweep_angles(h, d));
+            sweeps = sweep_shape(h, false, d.size()).form == 2;  // blocks per SM: the grid form's choice alone
         }
         // sector storage: the adjoint step as sv_energy_grad runs it (interleaved unless checkpoints resync psi)
         bool inter = h->storage == 1 && adj && h->ckpt_interval <= 0;
@@ -1408,15 +1545,17 @@ static sv_status autotune_impl(sv_handle h, sv_ham_handle ham, const std::vector
             SV_CUDA(h, launch_interleave(h->lam, h->saved, h->dtype, h->CLbuf, (size_t)h->Da * h->Db, h->sm_count,
                                          h->stream));
         }
+        const int sweep_bps = h->sweep_bps;
         for (int ci = 0; ci < 4; ++ci) {
             const int b = (sweeps && inter) ? cands_sw[ci] : cands_op[ci];
             float t;
             if (sweeps && inter) {
-                const int Gf = sweep_grid(h->dtype, false, h->Db, h->sm_count, b),
-                          Gr = sweep_grid(h->dtype, true, h->Db, h->sm_count, b);
+                h->sweep_bps = b;
+                const SweepShape sf = sweep_shape(h, false, d.size()), sr = sweep_shape(h, true, d.size());
+                h->sweep_bps = sweep_bps;
                 t = time_best(h, e0, e1, [&]() -> sv_status {
-                    if (!sweep_once(h, false, h->lam, d.size(), Gf, nullptr) ||
-                        !sweep_once(h, true, h->CLbuf, d.size(), Gr, h->partials))
+                    if (!sweep_once(h, sf, false, h->lam, nullptr, nullptr, -1) ||
+                        !sweep_once(h, sr, true, h->lam, h->saved, h->CLbuf, -1))
                         return fail(h, SV_ERR_CUDA, "autotune: whole-sweep launch refused");
                     return SV_OK;
                 });
@@ -1502,7 +1641,7 @@ extern "C" {
 const char *sv_version(void) { return "sv-gb300 0.1 (sm_103a)"; }
 
 uint32_t sv_check_status(void) {
-    const uint32_t a = check_word_sector(), b = check_word_rows(), c = check_word_abtc(), d = check_word_pool();
+    const uint32_t a = check_word_sector() | check_word_sweep(), b = check_word_rows(), c = check_word_abtc(), d = check_word_pool();
     return (a & 0xFFu) | ((b & 0xFFu) << 8) | ((c & 0xFFu) << 16) | ((d & 0x0Fu) << 24) |
            ((a | b | c | d) & 0x80000000u);
 }
@@ -1596,6 +1735,7 @@ static void destroy_handle(sv_handle h) {
     if (h->hkerr) cudaFreeHost(h->hkerr);
     dev_free(h, h->lists.buf, h->lists.bytes);
     dev_free(h, h->pool_lists.buf, h->pool_lists.bytes);
+    dev_free(h, h->groups.buf, h->groups.bytes);
     dev_free(h, h->rdm_lists.buf, h->rdm_lists.bytes);
     dev_free(h, h->CLbuf, h->CLbuf_bytes);
     dev_free(h, h->sweep_buf, h->sweep_bytes);
@@ -1884,10 +2024,10 @@ sv_status sv_apply_ansatz(sv_handle h, const sv_excitation *ops, int n_ops, cons
     }
     if (core && ensure_core(h) == SV_OK && h->core_cur != 0) {
         sv_handle c = h->core;
-        if (h->core_cur == 1) SV_TRY(core_status(h, prepare_reference(c)));
+        const bool ref = h->core_cur == 1;
         h->core_cur = 0;  // until psi is written
         c->prepared = true;
-        SV_TRY(core_status(h, forward(c, d, false)));
+        SV_TRY(core_status(h, forward(c, d, false, ref)));
         h->at_ref = false;
         if (move) {
             for (int q = 0; q < 32; ++q) h->perm[q] = q < h->n ? np[q] : q;
@@ -1908,7 +2048,7 @@ sv_status sv_apply_ansatz(sv_handle h, const sv_excitation *ops, int n_ops, cons
     }
     h->at_ref = false;
     h->core_cur = 0;
-    SV_TRY(forward(h, d, false));
+    SV_TRY(forward(h, d, false, false));
     return SV_OK;
 }
 
@@ -1970,10 +2110,10 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
     h->prepared = false;
     h->tc_timed = 0;
     SV_TRY(mark(h, 0, "sv_energy_grad: reference"));
-    SV_TRY(prepare_reference(h));
-    h->prepared = true;
+    if (!sect) SV_TRY(prepare_reference(h));
     SV_TRY(mark(h, 1, "sv_energy_grad: forward sweep"));
-    SV_TRY(forward(h, d, true));
+    SV_TRY(forward(h, d, true, sect));  // sector storage: the reference is written with the sweep
+    h->prepared = true;
     SV_TRY(mark(h, 2, "sv_energy_grad: working copy"));
     if (h->outer) SV_TRY(core_publish(h->outer));
     // The reverse sweep un-applies the ops to a working copy of psi(theta), so that psi
@@ -1982,9 +2122,23 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
     // allocated under the byte cap, the sweep runs on psi and psi(theta) is recomputed.
     const int64_t C = h->ckpt_interval;
     bool inter = sect && C <= 0 && L > 0;
-    if (inter && ensure_clbuf(h) != SV_OK) {
+    SweepShape shape;
+    if (inter && h->sweep_mode) {  // a whole sweep: it interleaves psi and lambda itself
+        SV_TRY(ensure_groups(h, d));
+        SV_TRY(upload_sweep_angles(h, d));
+        shape = sweep_shape(h, true, L);
+        if (shape.form == 2) SV_TRY(ensure_kerr(h));
+        if (shape.form >= 0 &&
+            ensure_partials(h, std::max<size_t>((size_t)shape.warps() * L, std::max<size_t>((size_t)G * L, need))) != SV_OK) {
+            cudaGetLastError();
+            shape.form = -1;
+            SV_TRY(ensure_partials(h, std::max<size_t>((size_t)G * L, need)));
+        }
+    }
+    if (inter && shape.form != 0 && ensure_clbuf(h) != SV_OK) {
         cudaGetLastError();
         inter = false;
+        shape.form = -1;
     }
     // dense storage: psi(theta) and lambda interleaved by amplitude in the adjoint pair
     // buffer (k_adjoint_i), where it exists, checkpoints do not resynchronise the working
@@ -2013,22 +2167,16 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
         SV_TRY(expectation(h, ham, T, h->lam, c, 0));
     }
     SV_TRY(mark(h, 4, "sv_energy_grad: reverse sweep"));
-    // reverse sweep
-    if (inter) {
+    // reverse sweep: sector storage in one launch where it can, else one launch per op (gradient partials [L][G])
+    const bool swept = inter && shape.form >= 0 && sweep_once(h, shape, true, h->psi, h->lam, h->CLbuf, -1);
+    if (inter && !swept) {
+        SV_TRY(ensure_clbuf(h));
+        SV_TRY(ensure_op_lists(h, d, h->lists));
         SV_CUDA(h, launch_interleave(h->psi, h->lam, h->dtype, h->CLbuf, (size_t)h->Da * h->Db, h->sm_count,
                                      h->stream));
         h->launches++;
-    }
-    // sector storage: the reverse sweep in one launch where it can (gradient partials
-    // [L][Gs], Gs its grid), else one launch per op ([L][G])
-    int Gred = G;
-    bool swept = false;
-    if (inter) {
-        const int Gs = sweep_grid(h->dtype, true, h->Db, h->sm_count, h->sweep_bps);
-        if (Gs > 0 && Gs <= G && sweep_once(h, true, h->CLbuf, L, Gs, h->partials)) {
-            swept = true;
-            Gred = Gs;
-        }
+    } else if (sect && !swept && L > 0) {
+        SV_TRY(ensure_op_lists(h, d, h->lists));
     }
     for (size_t kk = swept ? 0 : L; kk-- > 0;) {
         if (inter) {
@@ -2056,14 +2204,14 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
                 SV_CUDA(h, cudaMemcpyAsync(wpsi, h->ckpt[j], vec_bytes(h), cudaMemcpyDeviceToDevice, h->stream));
         }
     }
-    SV_CUDA(h, launch_reduce_rows(h->partials, (int)L, Gred, h->dout + 2, h->stream));
+    if (swept) SV_CUDA(h, launch_sweep_grad(h->partials, h->dtype, (int)L, shape.warps(), h->dout + 2, h->stream));
+    else SV_CUDA(h, launch_reduce_rows(h->partials, (int)L, G, h->dout + 2, h->stream));
     h->launches++;
     SV_TRY(mark(h, 5, "sv_energy_grad: restore"));
     SV_CUDA(h, cudaMemcpyAsync(h->hpinned, h->dout, (2 + L) * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     // leave psi(theta) in the handle (only a sweep on psi itself took it away)
     if (!inter && !dint && wpsi == h->psi) {
-        SV_TRY(prepare_reference(h));
-        SV_TRY(forward(h, d, false));
+        SV_TRY(forward(h, d, false, true));
     }
     SV_TRY(mark(h, 6, nullptr));
     SV_CUDA(h, cudaStreamSynchronize(h->stream));

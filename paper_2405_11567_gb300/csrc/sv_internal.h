@@ -217,6 +217,18 @@ struct OpLists {
     const int *dinfo = nullptr; // their device copy (inside buf)
 };
 
+// The steps of a whole sector sweep, two operators to a step (k_sweep.cu), kept on the device:
+// the lists, then the plans they are built from, then the groups.
+struct SweepGroups {
+    void *buf = nullptr;
+    size_t bytes = 0;
+    std::vector<uint32_t> key;  // sector counts and every op's masks they were built for
+    const void *dgroups = nullptr;
+    int n_groups = 0, n_ops = 0;
+    uint64_t words = 0;         // list entries (8 bytes each)
+    long long most = 0, all = 0;  // pairs of the largest operator, and of all of them
+};
+
 struct sv_ctx {
     int n = 0;
     sv_dtype dtype = SV_C64;
@@ -245,6 +257,8 @@ struct sv_ctx {
     // written from it before a call returns.
     sv_ctx *core = nullptr, *outer = nullptr;  // outer: the handle a core serves
     int core_cur = 0;          // what the core holds of the state in psi: 0 nothing, 1 that it is the reference, 2 psi
+    uint32_t *core_map = nullptr;  // where the core's strings lie in psi (alpha, then beta), in layout
+    int core_map_perm[32] = {};    // core_map_perm
     bool core_ref = false;     // the core's copy of a stored reference is current
     bool exposed = false;      // psi's address is known outside the library: it may be written there
     bool psi_clean = false;    // dense psi is zero outside the (na, nb) sector in layout perm
@@ -267,6 +281,7 @@ struct sv_ctx {
     // per-op alpha / beta pair lists (k_build_lists): the ansatz's (sector storage
     // rotations and adjoint steps) and the screened pool's
     OpLists lists, pool_lists;
+    SweepGroups groups;        // the ansatz's steps for whole sector sweeps
     OpLists rdm_lists;         // the 1-RDM's alpha-pair lists (one per orbital pair p < q)
     void *CLbuf = nullptr;     // compact amplitudes and sigma interleaved [Db][Da][2] (screening)
     size_t CLbuf_bytes = 0;

@@ -144,3 +144,50 @@ def test_a_written_state_is_read_from_its_vector(storage):
     E2, g2 = st.energy_grad(ham, p["ops"], p["theta"])
     assert abs(E2 - Eref) <= 1e-12 and np.max(np.abs(g2 - gref)) <= 1e-11
     assert np.max(np.abs(st.state() - psi)) <= 1e-13
+
+
+def _overlapping_ops(n):
+    """Every ordered pair of operators that share flip-mask bits in every way: disjoint, one
+    orbital shared, the same masks with other "from" patterns, a single inside a double."""
+    base = [(1, 0, -1, 4, -1), (1, 4, -1, 0, -1), (1, 1, -1, 5, -1), (1, 2, -1, 6, -1), (2, 0, 1, 4, 5), (2, 0, 5, 1, 4),
+            (2, 0, 2, 4, 6), (2, 2, 3, 6, 7), (2, 0, 3, 4, 7), (2, 1, 3, 5, 7), (4, 0, 1, 4, 7), (3, 2, -1, 4, -1)]
+    base = [op for op in base if max(op[1:]) < n]
+    return np.array([op for a in base for b in base for op in (a, b)], np.int32)
+
+
+@pytest.mark.parametrize("dtype", ["c128", "c64", "r64", "r32"])
+@pytest.mark.parametrize("n,na,nb", [(8, 2, 2), (10, 3, 2), (16, 4, 4), (22, 5, 4)])
+def test_paired_steps_match_single_operators(n, na, nb, dtype):
+    """Whole sweeps, two operators to a step, in the block (8, 10 qubits), the cluster (16) and
+    the grid form (22), against one launch per operator (SV_OPT_SECTOR_SWEEP = 0), for every way
+    in which a step's two masks can overlap, an odd number of operators and operators without a
+    pair: the same states and gradients, within the rounding of each pair's rotation, whose
+    operands are the same."""
+    rng = np.random.default_rng(n)
+    ops = _overlapping_ops(n)
+    if n > 16:
+        ops = ops[:61]
+    elif n == 16:
+        ops = np.vstack([inputs.adapt_list(inputs.uccsd_pool(n, 8), 40, rng), ops[:101]])
+    theta = rng.normal(0, 0.4, len(ops))
+    theta[3] = 2.0                                       # cos < 0: not three shears
+    h, eri, e_nuc = inputs.synthetic_integrals(n // 2, rng)
+    ham = sv.Hamiltonian(h, eri, e_nuc)
+    dense = inputs.random_sector_state(n, na, nb, rng)
+    if dtype.startswith("r"):
+        dense = dense.real / np.linalg.norm(dense.real)
+    out = []
+    for mode, polls in ((0, 1 << 22), (1, 1 << 22), (1, 1000)):    # 1000 polls: the grid form at every size
+        st = sv.StateVector(n, dtype, sector=(na, nb))
+        st.set_option(sv.SV_OPT_SECTOR_SWEEP, mode)
+        st.set_option(sv.SV_OPT_WAIT_POLLS, polls)
+        st.prepare_state(dense.astype(NP[dtype]), na, nb)
+        E, g = st.energy_grad(ham, ops, theta)
+        out.append((E, g, st.state()))
+        st.close()
+    eps = 2.3e-16 if dtype in ("c128", "r64") else 1.2e-7
+    scale = np.max(np.abs(out[0][1])) + 1.0
+    for E, g, psi in out[1:]:
+        assert np.max(np.abs(psi - out[0][2])) <= 4 * len(ops) * eps
+        assert abs(E - out[0][0]) <= 64 * len(ops) * eps
+        assert np.max(np.abs(g - out[0][1])) <= 64 * len(ops) * eps * scale
