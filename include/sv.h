@@ -279,9 +279,11 @@ typedef struct {
 } sv_instance;
 
 /* Plan a batch: tables, integrals and operators of every instance move to the
- * device once; states are kept per block in compact (N_alpha, N_beta)-sector form.
- * Work is ordered by estimated cost (largest first) and taken by the blocks of one
- * persistent kernel.  cuda_stream may be NULL (the plan then owns a stream; the
+ * device once, and what is the same for every angle (pair lists, same-spin matrices) is
+ * built there; states are kept in compact (N_alpha, N_beta)-sector form, in real
+ * amplitudes (every instance starts from a determinant).  Work is ordered by estimated
+ * cost (largest first) and taken by the blocks of one persistent kernel, small instances
+ * by parts of a block.  cuda_stream may be NULL (the plan then owns a stream; the
  * launch is captured in a CUDA graph, which the legacy default stream cannot
  * hold).  No counterpart in the paper beyond running many emulations; the
  * batched configuration of this library's workload list. */
@@ -307,8 +309,8 @@ uint64_t sv_batch_launch_count(sv_batch_handle b);
 
 /* Autotuner for the persistent batched launch: times the captured launch (angles
  * up, kernel, results down) at the angles theta (as for sv_batch_energy_grad) with
- * 256, 512 and 1024 threads per block and 1, 2 or 4 blocks per SM (at most 2048
- * threads per SM; grids capped by the instance count) and keeps the fastest for later
+ * 256 and 384 threads per block and 1, 2 or 4 blocks per SM (grids capped by the
+ * instance count) and keeps the fastest for later
  * calls; *grid_out (may be NULL) receives the grid.  Each instance runs whole in one
  * block with fixed-order sums, so results depend on the block size only through the
  * order of those sums (rounding) and reruns with one choice are bit-identical.  No

@@ -72,12 +72,6 @@ __device__ __forceinline__ R eri4(const SigmaTables<R> &A, int p, int q, int r, 
     return A.eri[((p * N + q) * N + r) * N + s];
 }
 
-template <typename R>
-__device__ __forceinline__ void fma_c(cplx<R> &acc, R v, const cplx<R> &c) {
-    acc.x += v * c.x;
-    acc.y += v * c.y;
-}
-
 // Orbital-order part of the Jordan-Wigner sign of a same-spin double p1<p2 -> q1<q2
 // taken as -(a+_q1 a_p2)(a+_q2 a_p1): the string-dependent part is the parity of the
 // prefix-parity word over the four orbitals.
@@ -85,19 +79,19 @@ __device__ __forceinline__ uint32_t double_order_sign(int p1, int p2, int q1, in
     return (uint32_t)((p1 < q2) ^ (q2 < p2) ^ (p1 < q1) ^ (p2 < q1));
 }
 
-// sigma at (rank a = Ia, rank b = Ib) for amplitudes C ([Db][Da]); c0 = C[Ib][Ia].
+// sigma at (rank a = Ia, rank b = Ib) for real amplitudes C ([Db][Da]); c0 = C[Ib][Ia].
 // Signs from prefix-parity words (bit u = parity of the bits below u): with
 // interleaved spin-orbitals the bits of x strictly between 2p and 2q are the alpha
 // orbitals strictly between p and q and the beta orbitals in [min, max), so an alpha
 // excitation's sign is the parity of pp(a) ^ pp(b) over its orbitals (plus an
 // orbital-order term), and a beta excitation's that of pp(b) ^ pp(a) ^ a.
 template <typename R>
-__device__ __forceinline__ cplx<R> sigma_at(const SigmaTables<R> &A, const cplx<R> *__restrict__ C, int Ia, int Ib,
-                                            cplx<R> c0) {
+__device__ __forceinline__ R sigma_at(const SigmaTables<R> &A, const R *__restrict__ C, int Ia, int Ib,
+                                            R c0) {
     const int N = A.N, Da = A.Da;
     const uint32_t b = A.strb[Ib], xb = A.sb[Ib];
     const uint32_t eb = ~b & A.maskN;
-    const cplx<R> *row = C + (size_t)Ib * Da;
+    const R *row = C + (size_t)Ib * Da;
     const uint32_t a = A.stra[Ia], xa = A.sa[Ia], x = xa | xb;
     const uint32_t ea = ~a & A.maskN;
     const uint32_t ppa = prefix_parity(a), ppb = prefix_parity(b);
@@ -109,7 +103,7 @@ __device__ __forceinline__ cplx<R> sigma_at(const SigmaTables<R> &A, const cplx<
         d += A.hdiag[k];
         for (uint32_t o2 = o & (o - 1u); o2; o2 &= o2 - 1u) d += A.Jp[k * A.n + __ffs(o2) - 1];
     }
-    cplx<R> acc = mk<R>((R)d * c0.x, (R)d * c0.y);
+    R acc = (R)d * c0;
     // alpha singles p -> q (partner in this row)
     for (uint32_t o = a; o; o &= o - 1u) {
         const int p = __ffs(o) - 1;
@@ -118,7 +112,7 @@ __device__ __forceinline__ cplx<R> sigma_at(const SigmaTables<R> &A, const cplx<
             const uint32_t m = (1u << p) | (1u << q);
             R v = single_value<R>(A, p, q, a, b);
             if ((uint32_t)par(PPa & m) ^ (uint32_t)(p < q)) v = -v;
-            fma_c<R>(acc, v, row[A.ra[a ^ m]]);
+            acc += v * row[A.ra[a ^ m]];
         }
     }
     // alpha-alpha doubles (p1<p2 occupied -> q1<q2 empty), partner in this row
@@ -133,7 +127,7 @@ __device__ __forceinline__ cplx<R> sigma_at(const SigmaTables<R> &A, const cplx<
                     const uint32_t m = (1u << p1) | (1u << p2) | (1u << q1) | (1u << q2);
                     R v = eri4<R>(A, q1, p1, q2, p2) - eri4<R>(A, q1, p2, q2, p1);
                     if ((uint32_t)par(PPa & m) ^ double_order_sign(p1, p2, q1, q2)) v = -v;
-                    fma_c<R>(acc, v, row[A.ra[a ^ m]]);
+                    acc += v * row[A.ra[a ^ m]];
                 }
             }
         }
@@ -146,7 +140,7 @@ __device__ __forceinline__ cplx<R> sigma_at(const SigmaTables<R> &A, const cplx<
             const uint32_t m = (1u << r) | (1u << s);
             R v = single_value<R>(A, r, s, b, a);
             if ((uint32_t)par(PPb & m) ^ (uint32_t)(r < s)) v = -v;
-            fma_c<R>(acc, v, C[(size_t)A.rb[b ^ m] * Da + Ia]);
+            acc += v * C[(size_t)A.rb[b ^ m] * Da + Ia];
         }
     }
     // beta-beta doubles
@@ -161,7 +155,7 @@ __device__ __forceinline__ cplx<R> sigma_at(const SigmaTables<R> &A, const cplx<
                     const uint32_t m = (1u << r1) | (1u << r2) | (1u << s1) | (1u << s2);
                     R v = eri4<R>(A, s1, r1, s2, r2) - eri4<R>(A, s1, r2, s2, r1);
                     if ((uint32_t)par(PPb & m) ^ double_order_sign(r1, r2, s1, s2)) v = -v;
-                    fma_c<R>(acc, v, C[(size_t)A.rb[b ^ m] * Da + Ia]);
+                    acc += v * C[(size_t)A.rb[b ^ m] * Da + Ia];
                 }
             }
         }
@@ -173,7 +167,7 @@ __device__ __forceinline__ cplx<R> sigma_at(const SigmaTables<R> &A, const cplx<
         for (uint32_t e = eb; e; e &= e - 1u) {
             const int s = __ffs(e) - 1;
             const uint32_t mb = (1u << r) | (1u << s);
-            const cplx<R> *prow = C + (size_t)A.rb[b ^ mb] * Da;
+            const R *prow = C + (size_t)A.rb[b ^ mb] * Da;
             const uint32_t sb = (uint32_t)par(PPb & mb) ^ (uint32_t)(r < s);
             const uint32_t PPx = ppa ^ prefix_parity(b ^ mb);  // alpha parity word on x'
             const R *er = A.eri + s * N + r;                   // (qp|sr) at er[(q N + p) N^2]
@@ -184,7 +178,7 @@ __device__ __forceinline__ cplx<R> sigma_at(const SigmaTables<R> &A, const cplx<
                     const uint32_t m = (1u << p) | (1u << q);
                     R v = er[(q * N + p) * N * N];
                     if (sb ^ (uint32_t)par(PPx & m) ^ (uint32_t)(p < q)) v = -v;
-                    fma_c<R>(acc, v, prow[A.ra[a ^ m]]);
+                    acc += v * prow[A.ra[a ^ m]];
                 }
             }
         }

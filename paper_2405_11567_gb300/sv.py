@@ -401,13 +401,14 @@ class Batch:
         self.dtype = dtype_code(dtype)
         self.sizes = [len(p["ops"]) for p in problems]
         self.n_inst = len(problems)
-        self.total_ops = int(sum(self.sizes))
+        self.starts = [0] + np.cumsum(self.sizes).tolist()
+        self.total_ops = self.starts[-1]
         self.handle = sv_batch_create(problems, self.dtype, stream)
 
     def energy_grad(self, theta_concat):
         """(E per instance, list of gradient arrays per instance)."""
         e, g = sv_batch_energy_grad(self.handle, theta_concat, self.n_inst, self.total_ops)
-        return e, np.split(g, np.cumsum(self.sizes)[:-1])
+        return e, [g[i:j] for i, j in zip(self.starts, self.starts[1:])]
 
     def set_time_limit(self, ms):
         sv_batch_set_time_limit(self.handle, ms)
