@@ -328,7 +328,7 @@ typedef enum {
     SV_OPT_MAX_BYTES = 2,           /* cap on device bytes this handle may allocate
                                        (0 = no cap); checkpoints are dropped to fit */
     SV_OPT_EXPECT_VARIANT = 3,      /* 0 auto (= 5 for complex64 / real float32 states
-                                       of at least 2^20 sector determinants whose
+                                       of at least 2^14 sector determinants whose
                                        same-spin couplings fill at least 5% of a string
                                        space of at most 4096 strings, where variant 5's
                                        limits hold and its planes take at most 16 GiB

@@ -129,29 +129,31 @@ __device__ __forceinline__ uint64_t ab_desc(uint32_t addr) {
     return d;
 }
 
-// The twelve (P = 2) or six MMAs of one K block in stage S: per plane the six piece products
+// The twelve MMAs of one K block in stage S: per plane the six piece products
 // (A piece, B piece) = (0,0) (0,1) (1,0) (0,2) (1,1) (2,0) into the plane's accumulator
 // (columns dacc + plane kAbMaxN).  Every operand is a compile-time offset from the
 // loop-invariant tensor-memory base and B descriptor, so the issuing thread spends a
 // few instructions per MMA; `first` starts the accumulation (the unit's first K block).
-constexpr int kAbStageBytes = 3 * kAbMaxN * kAbKc * 2;  // B ring stage: three pieces of 64 rows x 16 K
-template <int P, int S>
+// PAIR (real states): the two planes are two partner rows, each with B rows of its own.
+constexpr int kAbBBytes = 3 * kAbMaxN * kAbKc * 2;  // one partner row's B of a K block: three pieces of 64 rows x 16 K
+template <bool PAIR> constexpr int kAbStageBytes = (PAIR ? 2 : 1) * kAbBBytes;
+template <bool PAIR, bool SPLIT, int S>
 __device__ __forceinline__ void ab_mma_stage(uint32_t tmem, uint64_t d0, uint32_t dacc, uint32_t idesc, uint32_t first) {
     constexpr int pa[6] = {0, 0, 1, 0, 1, 2}, pbk[6] = {0, 1, 0, 2, 1, 0};
-    constexpr uint32_t kPieceD = (kAbMaxN * kAbKc * 2) >> 4, kStageD = kAbStageBytes >> 4;
+    constexpr uint32_t kPieceD = (kAbMaxN * kAbKc * 2) >> 4, kStageD = kAbStageBytes<PAIR> >> 4;
     #pragma unroll
-    for (int pl = 0; pl < P; ++pl) {
+    for (int pl = 0; pl < 2; ++pl) {
         #pragma unroll
         for (int x = 0; x < 6; ++x) {
             // A from tensor memory (lanes = tile rows, two K per column), B from shared memory;
             // B descriptor: that of the ring's start plus the byte offset in 16-byte units (the
             // start-address field does not carry: shared addresses < 256 KB)
             const uint32_t ta = tmem + (uint32_t)(kAbABase + S * kAbAStage + (pl * 3 + pa[x]) * kAbACols);
-            const uint64_t db = d0 + (uint64_t)(S * kStageD + pbk[x] * kPieceD);
-            const uint32_t acc = x > 0 ? 1u : first ^ 1u;
+            const uint64_t db = d0 + (uint64_t)(S * kStageD + (PAIR ? pl * (kAbBBytes >> 4) : 0) + pbk[x] * kPieceD);
+            const uint32_t acc = x > (SPLIT ? 1 : 0) ? 1u : first ^ 1u;  // the first into an accumulator starts it
             asm volatile(
                 "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, q;\n\t}\n" ::"r"(dacc + (uint32_t)(pl * kAbMaxN)),
+                "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, q;\n\t}\n" ::"r"(dacc + (uint32_t)(pl * kAbMaxN + (SPLIT && x > 0 ? kAbAccCols : 0))),
                 "r"(ta), "l"(db), "r"(idesc), "r"(acc)
                 : "memory");
         }
@@ -183,7 +185,8 @@ __device__ __forceinline__ uint32_t ab_between(int i, int j) {
 }  // namespace
 
 struct AbTcArgs {
-    const uint32_t *Xi;       // [Db][ldi][3]: per amplitude of X = phi C, words (re_k | im_k << 16), k = 1, 2, 3
+    const uint32_t *Xi;       // [rows][ldi][3]: per amplitude of X = phi C, words (re_k | im_k << 16), k = 1, 2, 3;
+                              // PAIR: (row 2 m | row 2 m + 1 << 16) of the pair m
     int ldi;                  // row stride of Xi in amplitudes (a multiple of 4: 16-byte rows)
     const uint16_t *stra, *strb, *ra;
     const uint16_t *Bp;       // pieces [3][rowsB][256] of the B table (rows: N^2 integral rows, Db own rows, a zero row)
@@ -193,6 +196,7 @@ struct AbTcArgs {
     int ldh;                  // row stride of H (floats, a multiple of 32: 128-byte rows)
     size_t hplane;
     int Da, Db, N, na, nb, ncols, nK, units;
+    int rows;                 // partner rows (PAIR: pairs of them) that the units of an alpha tile take
     uint32_t maskN;
     int *err;
     uint32_t spins;           // mbarrier polls (each with a short sleep) before a wait gives up
@@ -204,8 +208,20 @@ struct AbTcArgs {
 // per row, so the builders' 8-byte reads of 16 consecutive rows hit distinct bank pairs.
 __host__ __device__ __forceinline__ int ab_tstride(int nK) { return nK * kAbKc + 4; }
 
-template <int P>
+// PAIR: a real state.  Its amplitudes have one component, so a unit takes two partner rows in the
+// place of the two planes: the gathers through the table, the words staged and the tensor-memory
+// stores serve both, and only B is read twice.  At 30 qubits (real) 2.67 ms with one row to a unit,
+// 1.80 ms so.
+// SPLIT: the five small piece products have an accumulator of their own, in the columns of the second
+// buffer (the tensor core cuts every accumulation to float32, so one accumulator for all six loses six
+// times the bits; k_same_tc has the same split).  Without the second buffer the drain of a unit and the
+// next one's products take turns, so it serves sectors below 2^20 determinants, whose sums were float32
+// ones before: relative gradient errors over
+// 20 problems of 20 to 26 qubits (geometric mean) 2.8e-7 so, 3.0e-7 in the float32 split form and 3.5e-7
+// with one accumulator; 24 qubits 53 us and 51 us.
+template <bool PAIR, bool SPLIT>
 __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_tc(AbTcArgs g) {
+    constexpr int kBuf = SPLIT ? 1 : 2;  // accumulator buffers
     extern __shared__ uint8_t ab_smem[];
     __shared__ __align__(8) uint64_t full[kAbS], empty[kAbS], accf[2], acce[2], done;
     __shared__ uint32_t tmem_base;
@@ -213,7 +229,7 @@ __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_tc(AbTcArgs g) {
     __shared__ uint8_t s_kp[kAbMaxK], s_kq[kAbMaxK];
     // dynamic: stage ring of B (1024-aligned), the two staged X rows, the tile's table; the A
     // stages live in tensor memory (columns kAbABase + s kAbAStage + (plane 3 + piece) kAbACols)
-    constexpr int kStageBytes = kAbStageBytes;
+    constexpr int kStageBytes = kAbStageBytes<PAIR>, kCopies = PAIR ? 2 : 1, kSet = 6 * kAbMaxN;
     const uint32_t raw = su32(ab_smem), sbase = (raw + 1023u) & ~1023u;
     uint8_t *ring = ab_smem + (sbase - raw);
     // staged X rows: ldi amplitudes copied, then 4 zero amplitudes (what zero table entries read)
@@ -280,29 +296,33 @@ __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_tc(AbTcArgs g) {
         int cur_tile = -1, it = 0, gch = 0;
         // this thread's share of the B copies: entries i = tid + 256 k of (piece, row, core
         // column); shared-memory offsets fixed, global rows set per unit
-        int bdst[1], bsel[1];
+        int bdst[kCopies], bsel[kCopies], bset[kCopies];
         #pragma unroll
-        for (int k = 0; k < 1; ++k) {
+        for (int k = 0; k < kCopies; ++k) {
             const int i = tid + k * kAbBuild;
-            bsel[k] = i < ncolsP * 6 ? i : -1;
-            const int ii = bsel[k] < 0 ? 0 : i, piece = ii / (ncolsP * 2), rem = ii - piece * ncolsP * 2;
-            bdst[k] = piece * (ncolsP * kAbKc * 2) + (int)ab_off(rem >> 1, rem & 1);
+            bsel[k] = i < kSet * kCopies ? i % kSet : -1;
+            bset[k] = bsel[k] < 0 ? 0 : i / kSet;  // which of a pair's rows
+            const int ii = bsel[k] < 0 ? 0 : bsel[k], piece = ii / (ncolsP * 2), rem = ii - piece * ncolsP * 2;
+            bdst[k] = bset[k] * kAbBBytes + piece * (ncolsP * kAbKc * 2) + (int)ab_off(rem >> 1, rem & 1);
         }
-        const uint16_t *bsrc[1] = {g.Bp};
-        int brow[1];
-        #pragma unroll
-        for (int k = 0; k < 1; ++k) {
+        const uint16_t *bsrc[kCopies];
+        int brow[kCopies];
+        // the B-table row of this thread's column for a unit's partner row (a pair's second row may not exist: zeros)
+        auto row_of = [&](int u, int k) {
             const int ii = bsel[k] < 0 ? 0 : bsel[k], rem = ii - (ii / (ncolsP * 2)) * ncolsP * 2;
-            brow[k] = g.rowB[(size_t)((int)blockIdx.x % g.Db) * kAbMaxN + (rem >> 1)];
-        }
-        stage_row((int)blockIdx.x % g.Db, 0);
+            const int bp = PAIR ? 2 * (u % g.rows) + bset[k] : u % g.rows;
+            return bp < g.Db ? (int)g.rowB[(size_t)bp * kAbMaxN + (rem >> 1)] : N * N + g.Db;
+        };
+        #pragma unroll
+        for (int k = 0; k < kCopies; ++k) brow[k] = row_of((int)blockIdx.x, k);
+        stage_row((int)blockIdx.x % g.rows, 0);
         for (int u = blockIdx.x; u < g.units; u += gridDim.x, ++it) {
-            const int atile = u / g.Db, buf = it & 1;
+            const int atile = u / g.rows, buf = it & 1;
             asm volatile("cp.async.wait_all;" ::: "memory");
             // this unit's row has landed; every builder is done with the previous unit
             if (builders_any(tid == 0 && s_fail)) break;
             const int un = u + (int)gridDim.x;  // the next unit
-            if (un < g.units) stage_row(un % g.Db, buf ^ 1);
+            if (un < g.units) stage_row(un % g.rows, buf ^ 1);
             if (atile != cur_tile) {
                 // the tile's table: per row and kappa, the word offset in a row buffer of the
                 // partner amplitude (3 J; 3 ldi, a zero amplitude, where the entry is zero)
@@ -329,19 +349,19 @@ __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_tc(AbTcArgs g) {
             }
             // this unit's B rows (read one unit ahead from the per-partner-row table)
             #pragma unroll
-            for (int k = 0; k < 1; ++k) {
+            for (int k = 0; k < kCopies; ++k) {
                 const int ii = bsel[k] < 0 ? 0 : bsel[k], piece = ii / (ncolsP * 2), rem = ii - piece * ncolsP * 2;
                 bsrc[k] = g.Bp + (size_t)piece * g.pb + (size_t)brow[k] * 256 + (rem & 1) * 8;
-                if (un < g.units) brow[k] = g.rowB[(size_t)(un % g.Db) * kAbMaxN + (rem >> 1)];
+                if (un < g.units) brow[k] = row_of(un, k);
             }
             const uint32_t *xr = xrow + (size_t)buf * xstride;
             const uint16_t *trow = tbl + r * tstride + hf * kAbKpt;
             for (int c = 0; c < g.nK; ++c, ++gch) {
                 const int s = gch % kAbS;
                 // B rows of this K block into registers (ncolsP rows x 2 core columns x 3 pieces)
-                uint4 bv[1];
+                uint4 bv[kCopies];
                 #pragma unroll
-                for (int k = 0; k < 1; ++k)
+                for (int k = 0; k < kCopies; ++k)
                     if (bsel[k] >= 0) bv[k] = *reinterpret_cast<const uint4 *>(bsrc[k] + c * kAbKc);
                 // this thread's 8 K entries of row r: three words each (pieces 1..3, re | im << 16),
                 // sign bits flipped by the entry's sign
@@ -377,7 +397,7 @@ __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_tc(AbTcArgs g) {
                 // A: this thread's row (its tensor-memory lane) and 4 K = 2 columns of each piece
                 __syncwarp();
                 #pragma unroll
-                for (int pl = 0; pl < P; ++pl) {
+                for (int pl = 0; pl < 2; ++pl) {
                     const uint32_t sel = pl ? 0x7632u : 0x5410u;  // the im or the re halves of two words
                     #pragma unroll
                     for (int pc = 0; pc < 3; ++pc) {
@@ -389,7 +409,7 @@ __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_tc(AbTcArgs g) {
                     }
                 }
                 #pragma unroll
-                for (int k = 0; k < 1; ++k)
+                for (int k = 0; k < kCopies; ++k)
                     if (bsel[k] >= 0) *reinterpret_cast<uint4 *>(st + bdst[k]) = bv[k];
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // B, for the MMAs' reads
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");   // A written
@@ -405,20 +425,22 @@ __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_tc(AbTcArgs g) {
         const int quarter = warp & 3, r = quarter * 32 + (tid & 31), eh = (warp - kAbBuild / 32 - 1) >> 2;
         int it = 0;
         for (int u = blockIdx.x; u < g.units; u += gridDim.x, ++it) {
-            const int atile = u / g.Db, bp = u - atile * g.Db, t = it & 1, ia = atile * kAbM + r;
+            const int atile = u / g.rows, bu = u - atile * g.rows, t = it % kBuf, ia = atile * kAbM + r;
             bool bad = false;
             if (tid == kAbBuild + 32) {
-                if (!ab_wait(su32(&accf[t]), (uint32_t)((it >> 1) & 1), g.spins)) s_fail = 1;
+                if (!ab_wait(su32(&accf[t]), (uint32_t)((it / kBuf) & 1), g.spins)) s_fail = 1;
                 bad = s_fail != 0;
             }
             if (epi_any(bad)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const bool ok_row = ia < g.Da;
             #pragma unroll
-            for (int pl = 0; pl < P; ++pl) {
+            for (int pl = 0; pl < 2; ++pl) {
+                const int bp = PAIR ? 2 * bu + pl : bu;
+                if (PAIR && bp >= g.Db) break;  // the whole warp
                 const uint32_t tbase =
                     tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(t * kAbAccCols + pl * kAbMaxN);
-                float *Hp = g.H + (size_t)pl * g.hplane + (size_t)bp * g.ncols * g.ldh + ia;
+                float *Hp = g.H + (PAIR ? 0 : (size_t)pl * g.hplane) + (size_t)bp * g.ncols * g.ldh + ia;
                 for (int c = 16 * eh; c < g.ncols; c += 32) {
                     uint32_t v[16];
                     asm volatile(
@@ -429,7 +451,21 @@ __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_tc(AbTcArgs g) {
                           "=r"(v[15])
                         : "r"(tbase + (uint32_t)c)
                         : "memory");
+                    uint32_t w[16];
+                    if constexpr (SPLIT)
+                        asm volatile(
+                            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+                            "%15}, [%16];"
+                            : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]),
+                              "=r"(w[7]), "=r"(w[8]), "=r"(w[9]), "=r"(w[10]), "=r"(w[11]), "=r"(w[12]), "=r"(w[13]),
+                              "=r"(w[14]), "=r"(w[15])
+                            : "r"(tbase + (uint32_t)(c + kAbAccCols))
+                            : "memory");
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if constexpr (SPLIT) {
+                        #pragma unroll
+                        for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(w[j]));
+                    }
                     if (ok_row) {
                         #pragma unroll
                         for (int j = 0; j < 16; ++j)
@@ -449,8 +485,8 @@ __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_tc(AbTcArgs g) {
         int gch = 0, it = 0;
         bool stop = false;
         for (int u = blockIdx.x; u < g.units && !stop; u += gridDim.x, ++it) {
-            const int t = it & 1;
-            if (it >= 2 && !ab_wait(su32(&acce[t]), (uint32_t)(((it >> 1) - 1) & 1), g.spins)) { s_fail = 1; break; }
+            const int t = it % kBuf;
+            if (it >= kBuf && !ab_wait(su32(&acce[t]), (uint32_t)((it / kBuf - 1) & 1), g.spins)) { s_fail = 1; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             for (int c = 0; c < g.nK; ++c, ++gch) {
                 const int s = gch % kAbS;
@@ -463,10 +499,10 @@ __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_tc(AbTcArgs g) {
                 const uint32_t dacc = tmem + (uint32_t)(t * kAbAccCols), first = c == 0 ? 1u : 0u;
                 static_assert(kAbS == 4, "one case per stage");
                 switch (s) {
-                    case 0: ab_mma_stage<P, 0>(tmem, d0, dacc, idesc, first); break;
-                    case 1: ab_mma_stage<P, 1>(tmem, d0, dacc, idesc, first); break;
-                    case 2: ab_mma_stage<P, 2>(tmem, d0, dacc, idesc, first); break;
-                    default: ab_mma_stage<P, 3>(tmem, d0, dacc, idesc, first); break;
+                    case 0: ab_mma_stage<PAIR, SPLIT, 0>(tmem, d0, dacc, idesc, first); break;
+                    case 1: ab_mma_stage<PAIR, SPLIT, 1>(tmem, d0, dacc, idesc, first); break;
+                    case 2: ab_mma_stage<PAIR, SPLIT, 2>(tmem, d0, dacc, idesc, first); break;
+                    default: ab_mma_stage<PAIR, SPLIT, 3>(tmem, d0, dacc, idesc, first); break;
                 }
                 ab_commit(su32(&empty[s]));
             }
@@ -536,8 +572,8 @@ __global__ void __launch_bounds__(kAbMaxN) k_ab_rows(const uint16_t *__restrict_
     rowB[(size_t)bp * kAbMaxN + t] = (uint16_t)row;
 }
 
-size_t ab_tc_smem(int Da, int N) {
-    const size_t stage = 3 * kAbMaxN * kAbKc * 2;
+size_t ab_tc_smem(int planes, int Da, int N) {
+    const size_t stage = planes == 1 ? kAbStageBytes<true> : kAbStageBytes<false>;
     const int nK = (N * (N + 1) / 2 + kAbKc - 1) / kAbKc;
     const size_t ldi = ((size_t)Da + 3) / 4 * 4;
     return 1024 + kAbS * stage + 2 * (ldi + 4) * 12 + (size_t)kAbM * ab_tstride(nK) * 2;
@@ -567,11 +603,10 @@ cudaError_t launch_ab_table(const float *eri, const float *Jt, const uint16_t *s
 // Whether the tensor-core alpha-beta form applies: N <= 16, D <= 4096 per spin, at most
 // 64 columns, and its shared memory fits.
 bool ab_tc_fits(int planes, int Da, int Db, int na, int nb, int N) {
-    (void)planes;
     (void)na;
     if (N > 16 || N < 1 || Da > 4096 || Db > 4096 || Da < 1 || Db < 1) return false;
     if (nb * (N - nb) + 1 > kAbMaxN) return false;
-    return ab_tc_smem(Da, N) <= 227 * 1024 - 1024;
+    return ab_tc_smem(planes, Da, N) <= 227 * 1024 - 1024;
 }
 
 // Row stride (amplitudes) of the interleaved X pieces the kernel reads.
@@ -582,8 +617,8 @@ int ab_xi_ld(int Da) { return (Da + 3) / 4 * 4; }
 // of 128 strings).
 int ab_h_ld(int Da) { return (Da + 31) / 32 * 32; }
 
-// H = the per-partner-row products (see above); Xi [Db][ab_xi_ld(Da)][3] the phased
-// amplitudes as bf16 pieces (phase kernel); Bp the B table pieces; H planes
+// H = the per-partner-row products (see above); Xi [rows][ab_xi_ld(Da)][3] the phased
+// amplitudes as bf16 pieces (phase kernel), rows Db or, for real states, pairs of rows; Bp the B table pieces; H planes
 // [planes][Db][ncols][ab_h_ld(Da)] (hplane elements apart); rowB the column table of
 // launch_ab_table.
 // spins: polls of each bounded wait; stall: the test hook of AbTcArgs.
@@ -598,23 +633,20 @@ cudaError_t launch_ab_tc(const uint32_t *Xi, int planes, const uint16_t *stra, c
     g.hplane = hplane; g.ldh = ab_h_ld(Da); g.Da = Da; g.Db = Db; g.N = N; g.na = na; g.nb = nb;
     g.ncols = nb * (N - nb) + 1;
     g.nK = (N * (N + 1) / 2 + kAbKc - 1) / kAbKc;
-    g.units = ((Da + kAbM - 1) / kAbM) * Db;
+    g.rows = planes == 1 ? (Db + 1) / 2 : Db;
+    g.units = ((Da + kAbM - 1) / kAbM) * g.rows;
     g.maskN = (1u << N) - 1u;
     g.err = err;
     g.spins = spins;
     g.stall = stall;
     const int grid = g.units < sm_count ? g.units : sm_count;
-    const size_t sm = ab_tc_smem(Da, N);
-    cudaError_t e;
-    if (planes == 2) {
-        e = cudaFuncSetAttribute(k_ab_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        k_ab_tc<2><<<grid, kAbThreadsTc, sm, st>>>(g);
-    } else {
-        e = cudaFuncSetAttribute(k_ab_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        k_ab_tc<1><<<grid, kAbThreadsTc, sm, st>>>(g);
-    }
+    const size_t sm = ab_tc_smem(planes, Da, N);
+    const bool split = (long long)Da * Db < 1 << 20;
+    auto *kernel = planes == 2 ? (split ? k_ab_tc<false, true> : k_ab_tc<false, false>)
+                               : (split ? k_ab_tc<true, true> : k_ab_tc<true, false>);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    kernel<<<grid, kAbThreadsTc, sm, st>>>(g);
     return cudaGetLastError();
 }
 

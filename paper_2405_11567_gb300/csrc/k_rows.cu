@@ -822,7 +822,8 @@ __device__ __forceinline__ void bf16x3(float v, uint16_t *p, size_t piece) {
 
 // With Xp (tensor-core form) the planes are written as three bf16 pieces at stride px
 // instead of float32 X.  With Xi (variant 5) also, per amplitude, the three words
-// (re_k | im_k << 16), k = 1..3, at Xi[(Ib ldi + Ia) 3 + k - 1].
+// (re_k | im_k << 16), k = 1..3, at Xi[(Ib ldi + Ia) 3 + k - 1]; for real states the halves of
+// a word are rows 2 m and 2 m + 1, at Xi[(m ldi + Ia) 3 + k - 1].
 __device__ __forceinline__ void bf16x3_u(float v, uint32_t &p1, uint32_t &p2, uint32_t &p3) {
     const __nv_bfloat16 a = __float2bfloat16_rn(v);
     const float r = v - __bfloat162float(a);
@@ -853,13 +854,21 @@ __global__ void __launch_bounds__(kThreads) k_phase_planar(const Amp *__restrict
                 bf16x3(xi, Xp + plane + xo + Ia, px);
             }
             if (Xi) {
-                uint32_t r1, r2, r3, i1, i2, i3;
+                uint32_t r1, r2, r3;
                 bf16x3_u(xr, r1, r2, r3);
-                bf16x3_u(xi, i1, i2, i3);
-                uint32_t *w = Xi + ((size_t)Ib * ldi + Ia) * 3;
-                w[0] = r1 | (i1 << 16);
-                w[1] = r2 | (i2 << 16);
-                w[2] = r3 | (i3 << 16);
+                if constexpr (AmpT<Amp>::kCplx) {
+                    uint32_t i1, i2, i3;
+                    bf16x3_u(xi, i1, i2, i3);
+                    uint32_t *w = Xi + ((size_t)Ib * ldi + Ia) * 3;
+                    w[0] = r1 | (i1 << 16);
+                    w[1] = r2 | (i2 << 16);
+                    w[2] = r3 | (i3 << 16);
+                } else {
+                    uint16_t *w = reinterpret_cast<uint16_t *>(Xi + ((size_t)(Ib >> 1) * ldi + Ia) * 3) + (Ib & 1);
+                    w[0] = (uint16_t)r1;
+                    w[2] = (uint16_t)r2;
+                    w[4] = (uint16_t)r3;
+                }
             }
         }
     }
@@ -1103,7 +1112,7 @@ static cudaError_t launch_ab_k(const RowArgs<ff> &A, int K, size_t smem, cudaStr
 
 cudaError_t launch_same_tc(const uint16_t *M, size_t pm, const uint16_t *X, size_t px, uint16_t *Xt, size_t pt,
                            float *G, int planes, int Da, int Db, int lda, int ldb, int *err, uint32_t spins, int stall,
-                           cudaStream_t st);
+                           int sm_count, cudaStream_t st);
 cudaError_t launch_ab_tc(const uint32_t *Xi, int planes, const uint16_t *stra, const uint16_t *strb,
                          const uint16_t *ra, const uint16_t *Bp, size_t pb, const uint16_t *rowB, float *H,
                          size_t hplane, int Da, int Db,
@@ -1122,7 +1131,7 @@ static cudaError_t launch_same_t(RowArgs<Amp> A, const RowTables &T, int dtype, 
         if (e != cudaSuccess) return e;
         if (g.ev && (e = cudaEventRecord(g.ev[0], st)) != cudaSuccess) return e;
         e = launch_same_tc(g.Mp, g.pm, g.Xp, g.px, g.Xtp, g.pt, g.G, g.planes, T.Da, T.Db, g.lda, g.ldb, g.err,
-                           g.spins, g.stall & 1, st);
+                           g.spins, g.stall & 1, sm_count, st);
         if (e != cudaSuccess) return e;
         if (g.ev && (e = cudaEventRecord(g.ev[1], st)) != cudaSuccess) return e;
         A.same_gemm = 1;

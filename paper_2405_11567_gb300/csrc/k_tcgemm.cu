@@ -32,13 +32,24 @@ namespace {
 
 constexpr int kTcThreads = 128;
 constexpr int kTcM = 128;                              // alpha strings per tile (tensor-memory lanes)
-constexpr int kTcN = 256;                              // beta strings per tile (tensor-memory columns)
 constexpr int kTcKb = 32;                              // K (bf16 elements, 64 bytes) per stage
 constexpr int kTcABytes = kTcM * kTcKb * 2;            // one piece of A in one stage
-constexpr int kTcBBytes = kTcN * kTcKb * 2;            // one piece of B in one stage
-constexpr int kTcStageBytes = 3 * kTcABytes + 3 * kTcBBytes;
-constexpr int kTcStages = 3;                           // 3 x 72 KB
-constexpr int kTcSmem = kTcStages * kTcStageBytes + 1024;  // + alignment of the ring to 1024 bytes
+constexpr int kTcCols = 512;                           // tensor-memory columns: every accumulator
+
+// A tile of TN beta strings.  The tensor core cuts each accumulation to float32, and a sum keeps
+// losing bits at the rate of its largest terms; so the five small piece products have an accumulator
+// of their own and the first pieces' product x1 y1 the rest, K blocks in turn: one with TN = 256,
+// three with TN = 128.  Relative gradient error at 24 qubits: 2.1e-6 to 2.8e-6 with one accumulator
+// for all six, 0.7e-6 to 1.2e-6 with TN = 256.  TN = 128 serves sectors of few tiles (launch_same_tc),
+// where it also has twice the blocks.
+template <int TN>
+struct TcTile {
+    static constexpr int kMain = kTcCols / TN - 1;                      // accumulators of x1 y1
+    static constexpr int kBBytes = TN * kTcKb * 2;                      // one piece of B in one stage
+    static constexpr int kStageBytes = 3 * kTcABytes + 3 * kBBytes;
+    static constexpr int kStages = TN == 256 ? 3 : 4;                   // 3 x 72 KB, 4 x 48 KB
+    static constexpr int kSmem = kStages * kStageBytes + 1024;          // + alignment of the ring to 1024 bytes
+};
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -100,9 +111,12 @@ struct TcOut {
 // Tensor maps (innermost first): ma {K = Da, rows Da, piece}, mb {K = Db, rows Db, piece},
 // x {K = Da, rows Db, plane, piece}, xt {K = Db, rows Da, plane, piece}; box {32, rows of a
 // tile, 1, 1}.
+template <int TN>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_same_tc(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb,
               const __grid_constant__ CUtensorMap x, const __grid_constant__ CUtensorMap xt, TcOut g) {
+    constexpr int kTcN = TN, kMain = TcTile<TN>::kMain, kTcBBytes = TcTile<TN>::kBBytes,
+                  kTcStageBytes = TcTile<TN>::kStageBytes, kTcStages = TcTile<TN>::kStages;
     extern __shared__ uint8_t tc_smem[];
     __shared__ __align__(8) uint64_t full[kTcStages], empty[kTcStages], done;
     __shared__ uint32_t tmem_base;
@@ -112,7 +126,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int n0 = blockIdx.x * kTcN, m0 = blockIdx.y * kTcM, p = blockIdx.z;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "n"(kTcN)
+                     "n"(kTcCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -178,11 +192,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const uint32_t a = base + pa[t] * kTcABytes, b = base + 3 * kTcABytes + pb[t] * kTcBBytes;
                 #pragma unroll
                 for (int ks = 0; ks < kTcKb / 16; ++ks) {  // K = 16 per instruction: 32 bytes into the 64-byte rows
-                    const uint32_t acc = (it > 0 || t > 0 || ks > 0) ? 1u : 0u;
+                    // the first into an accumulator starts it
+                    const uint32_t acc = t == 0 ? (it >= kMain || ks > 0) : (it > 0 || t > 1 || ks > 0);
+                    const uint32_t d = tmem + (uint32_t)((t == 0 ? it % kMain : kMain) * kTcN);
                     const uint64_t da = tc_desc(a + ks * 32), db = tc_desc(b + ks * 32);
                     asm volatile(
                         "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
-                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n\t}\n" ::"r"(tmem),
+                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n\t}\n" ::"r"(d),
                         "l"(da), "l"(db), "r"(idesc), "r"(acc)
                         : "memory");
                 }
@@ -213,19 +229,25 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const int m = m0 + warp * 32 + lane;  // this thread's tensor-memory lane: alpha string a
         #pragma unroll 1
         for (int c = 0; c < kTcN; c += 8) {
-            uint32_t v[8];
+            uint32_t v[kMain + 1][8];
             const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c;
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                           "=r"(v[7])
-                         : "r"(taddr)
-                         : "memory");
+            #pragma unroll
+            for (int x2 = 0; x2 <= kMain; ++x2)
+                asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                             : "=r"(v[x2][0]), "=r"(v[x2][1]), "=r"(v[x2][2]), "=r"(v[x2][3]), "=r"(v[x2][4]),
+                               "=r"(v[x2][5]), "=r"(v[x2][6]), "=r"(v[x2][7])
+                             : "r"(taddr + (uint32_t)(x2 * kTcN))
+                             : "memory");
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
             if (m < g.Da) {
                 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int n = n0 + c + j;
-                    if (n < g.Db) g.G[((size_t)p * g.Db + n) * g.Da + m] = __uint_as_float(v[j]);
+                    float sum = __uint_as_float(v[kMain][j]);  // the small products first
+                    #pragma unroll
+                    for (int x2 = 0; x2 < kMain; ++x2)
+                        if (x2 < nIt) sum += __uint_as_float(v[x2][j]);  // (started: one per K block)
+                    if (n < g.Db) g.G[((size_t)p * g.Db + n) * g.Da + m] = sum;
                 }
             }
         }
@@ -234,7 +256,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTcN) : "memory");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTcCols) : "memory");
 }
 
 // Three bf16 pieces of n floats (x1 = bf16(x), x2 = bf16(x - x1), x3 = bf16(x - x1 - x2)),
@@ -313,16 +335,10 @@ bool encode_map(CUtensorMap *m, const void *base, int rank, const uint64_t *dims
 // spins: polls of each bounded wait; stall: the test hook of TcOut.
 cudaError_t launch_same_tc(const uint16_t *M, size_t pm, const uint16_t *X, size_t px, uint16_t *Xt, size_t pt,
                            float *G, int planes, int Da, int Db, int lda, int ldb, int *err, uint32_t spins, int stall,
-                           cudaStream_t st) {
+                           int sm_count, cudaStream_t st) {
     if (Da < 1 || Db < 1 || lda % 8 || ldb % 8 || pm % 8 || px % 8 || pt % 8 || spins < 1 || ((uintptr_t)M & 15) ||
         ((uintptr_t)X & 15) || ((uintptr_t)Xt & 15))
         return cudaErrorInvalidValue;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_same_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
     k_transpose_pieces<<<dim3((Da + 31) / 32, (Db + 31) / 32, 3 * planes), dim3(32, 8), 0, st>>>(X, Xt, Da, Db, lda,
                                                                                                  ldb, px, pt);
     cudaError_t e = cudaGetLastError();
@@ -335,12 +351,25 @@ cudaError_t launch_same_tc(const uint16_t *M, size_t pm, const uint16_t *X, size
                    sx[3] = {(uint64_t)lda * 2, (uint64_t)Db * lda * 2, (uint64_t)px * 2};
     const uint64_t dt[4] = {(uint64_t)Db, (uint64_t)Da, P, 3},
                    stt[3] = {(uint64_t)ldb * 2, (uint64_t)Da * ldb * 2, (uint64_t)pt * 2};
-    if (!encode_map(&ma, M, 3, dma, sma, kTcM) || !encode_map(&mb, M + (size_t)Da * lda, 3, dmb, smb, kTcN) ||
-        !encode_map(&mx, X, 4, dx, sx, kTcN) || !encode_map(&mt, Xt, 4, dt, stt, kTcM))
+    // narrow tiles while every one of them has an SM: 24 qubits (495 strings, real) 46 us wide with the
+    // transposes, 35 us narrow; at 28 qubits (2,002) 256 narrow tiles would take two rounds of the SMs
+    const int tm = (Da + kTcM - 1) / kTcM;
+    const bool narrow = (long long)((Db + 127) / 128) * tm * planes <= sm_count;
+    const uint32_t tn = narrow ? 128 : 256;
+    if (!encode_map(&ma, M, 3, dma, sma, kTcM) || !encode_map(&mb, M + (size_t)Da * lda, 3, dmb, smb, tn) ||
+        !encode_map(&mx, X, 4, dx, sx, tn) || !encode_map(&mt, Xt, 4, dt, stt, kTcM))
         return cudaErrorInvalidValue;
     const TcOut g{G, Da, Db, err, spins, stall};
-    k_same_tc<<<dim3((Db + kTcN - 1) / kTcN, (Da + kTcM - 1) / kTcM, planes), kTcThreads, kTcSmem, st>>>(ma, mb, mx,
-                                                                                                       mt, g);
+    const dim3 grid((Db + tn - 1) / tn, tm, planes);
+    if (narrow) {
+        e = cudaFuncSetAttribute(k_same_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcTile<128>::kSmem);
+        if (e != cudaSuccess) return e;
+        k_same_tc<128><<<grid, kTcThreads, TcTile<128>::kSmem, st>>>(ma, mb, mx, mt, g);
+    } else {
+        e = cudaFuncSetAttribute(k_same_tc<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcTile<256>::kSmem);
+        if (e != cudaSuccess) return e;
+        k_same_tc<256><<<grid, kTcThreads, TcTile<256>::kSmem, st>>>(ma, mb, mx, mt, g);
+    }
     return cudaGetLastError();
 }
 

@@ -948,9 +948,12 @@ static int row_chunk(sv_handle h, const RowTables &R) {
 // Whether the string-row expectation takes the same-spin products (variant 4):
 // single-precision states whose split form fits and whose strings number at most
 // 4096 per spin (matrices up to 64 MB).  Automatic choice (variant 0): where the
-// sector has at least 2^20 determinants and every string at least 5% of the strings
+// sector has at least 2^14 determinants and every string at least 5% of the strings
 // of its spin as same-spin partners (singles and doubles), so that the dense
-// products do at most 20 times the multiplies of the sparse sums.
+// products do at most 20 times the multiplies of the sparse sums.  Measured, variants
+// 3 / 5 in us (real float32): 14,400 determinants 62 / 65, 63,504 158 / 86, 108,900
+// 248 / 115, 245,025 435 / 149, 627,264 1223 / 299 (complex64: 44,100 144 / 89, 245,025
+// 529 / 173); variant 4 alone 73, 128, 179, 361, 689.
 static bool use_same_gemm(sv_handle h, int K) {
     if (!single_prec(h->dtype) || K == 0 || h->Da > 4096 || h->Db > 4096) return false;
     if (h->expect_variant == 4 || h->expect_variant == 5) return true;
@@ -961,7 +964,7 @@ static bool use_same_gemm(sv_handle h, int K) {
         const long ns = (long)ne * (N - ne), nd = c2(ne) * c2(N - ne);
         return (double)(ns + nd) / (double)D;
     };
-    return (double)h->Da * h->Db >= (double)(1 << 20) && dens(h->na, h->Da) >= 0.05 && dens(h->nb, h->Db) >= 0.05;
+    return (double)h->Da * h->Db >= (double)(1 << 14) && dens(h->na, h->Da) >= 0.05 && dens(h->nb, h->Db) >= 0.05;
 }
 
 // Whether the same-spin product form also takes the alpha-beta part as tensor-core
