@@ -14,7 +14,7 @@
 //                over the op's pairs (alpha list x beta list, built by k_build_lists)
 //   k_adjoint_l  g += s (Re conj(lam[x']) psi[x] - Re conj(lam[x]) psi[x']), then U^dagger
 //                on psi and lambda (float64 per block, fixed-order sums)
-//   k_rdm_rows   one block per beta string: every density-matrix element's share
+//   k_rdm_rows   groups of rows, then of columns: every density-matrix element's share
 // with s = (-1)^popc(x & sm), the Jordan-Wigner sign (sm = 0 for qubit
 // excitations).
 #include <cstring>
@@ -289,129 +289,205 @@ __device__ __forceinline__ ff warp_sum(ff v) {
     return v;
 }
 
-// Density matrix by rows: a block takes beta strings (rows) Ib = blockIdx.x,
-// blockIdx.x + gridDim.x, ...; for each row
-//   norm and alpha occupations   sum_a |C[b][a]|^2 (a_p)                (all warps)
-//   beta occupations             the row norm when b holds p
-//   alpha pairs p < q            sum over a with q in a, p not in a of
-//                                conj(C[b][a']) C[b][a] (-1)^popc(x & between(2p, 2q)), a' = a - q + p
-//                                (those a from the pair's list, built once per sector)
-//   beta pairs p < q (b holds q, not p)
-//                                sum_a conj(C[b'][a]) C[b][a] (-1)^popc(x & between(2p+1, 2q+1))
-// (x = spread(a) | spread(b)), in the element order norm, n occupations
-// (j = 2p + sigma), alpha pairs, beta pairs.  Each pair element belongs to one warp
-// (pairs dealt round-robin to the warps), which sums it over the row with its lanes
-// and one warp reduction; the norm and occupations are summed by every warp over a
-// share of the row.  Each warp writes its sums to its own shared slots; after each row
-// the block adds them (the owner's slot for a pair element, the warps in order for the
-// others) into float64 running sums, written to partial[e][blockIdx.x] at the end:
-// fixed-order sums.
-template <typename A>
-__global__ void __launch_bounds__(kThreads) k_rdm_rows(const A *__restrict__ C, SectTabs T, int N,
-                                                       const uint32_t *__restrict__ alist,
-                                                       const int4 *__restrict__ ainfo,
-                                                       double *__restrict__ partial) {
+// Density matrix by rows.  A block takes RW rows b of C at a time (alpha pairs), then RW columns a
+// (beta pairs), and holds them in shared memory string by string, so that one list entry serves RW
+// products and a string's amplitudes are one or two 16-byte words:
+//   norm (alpha part) and the spin's occupations   sum |C|^2 (string holds p)
+//   pairs p < q   sum over the strings x with q, without p of
+//                 conj(C[x']) C[x] (-1)^popc(spread(x) & between), x' = x - q + p (the pair's list),
+//                 times each row's own sign (-1)^popc(spread(other string) & between)
+// in the element order norm, n occupations (j = 2p + sigma), alpha pairs, beta pairs.  Each pair belongs
+// to one warp.  Its lanes' sums are reduced row by row (row_sums) and added, in float64, to the pair's
+// slot of that row; the occupations are summed in float-float (float64 for float64 rows).  partial[e]
+// [blockIdx.x] at the end: fixed-order sums.
+// Bound by shared memory (16-byte words at list order: four cycles a warp and more where strings share
+// a bank); float-float states by the FP32 pipe.  One row to a warp's pass, from L1, with the list read
+// again for every row: 30 qubits (5, 5) float32 900 us, float64 1,250; so: 230 and 590 (28 qubits float32
+// 478 and 153, 24 qubits 45 and 27).
+template <typename R> struct RdmSum { using T = R; };
+template <> struct RdmSum<float> { using T = ff; };
+__device__ __forceinline__ void sum_to(ff &acc, float w) {
+    float s, e;
+    two_sum(acc.hi, w, s, e);
+    acc = ff_make(s, acc.lo + e);
+}
+__device__ __forceinline__ void sum_to(ff &acc, ff w) { acc += w; }
+__device__ __forceinline__ void sum_to(double &acc, double w) { acc += w; }
+template <typename T> __device__ __forceinline__ T lane_xor(T v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ ff lane_xor(ff v, int o) {
+    return ff_make(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
+}
+// Sums v[r] over the lanes, each of the RW sums on 32 / RW lanes: lane l returns that of r = l RW / 32.
+template <int RW, typename R>
+__device__ __forceinline__ R row_sums(R (&v)[RW], int lane) {
+    int o = 16;
+    #pragma unroll
+    for (int h = RW / 2; h > 0; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+        #pragma unroll
+        for (int j = 0; j < h; ++j) {
+            const R send = up ? v[j] : v[j + h], keep = up ? v[j + h] : v[j];
+            v[j] = keep + lane_xor(send, o);
+        }
+    }
+    for (; o > 0; o >>= 1) v[0] += lane_xor(v[0], o);
+    return v[0];
+}
+
+__device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ ff mad(ff a, ff b, ff c) { return ff_fma(a, b, c); }
+
+constexpr int kRdmThreads = 512;
+// NV: 16-byte words to a string, RW = 16 NV / sizeof(A) rows.  Two, which halve the list reads, while
+// the rows still make two groups per SM and two blocks fit on it; one below and above that.  At most
+// 64 registers: two blocks (30 qubits float32 272 us with one, 229 with two).
+template <typename A, int NV> constexpr int kRdmRows = 16 * NV / (int)sizeof(A);
+template <typename A, int NV>
+__global__ void __launch_bounds__(kRdmThreads, 2) k_rdm_rows(const A *__restrict__ C, SectTabs T, int N,
+                                                          const uint32_t *__restrict__ lists,
+                                                          const int4 *__restrict__ info,
+                                                          double *__restrict__ partial) {
     using R = real_of<A>;
-    extern __shared__ double rdm_s[];  // [2 n_el] running sums, then [kThreads/32][2 n_el] warp slots
-    const int n = 2 * N, npair = N * (N - 1) / 2, n_el = 1 + n + 2 * npair, W = 2 * n_el;
-    constexpr int NW = kThreads / 32;
-    double *acc = rdm_s, *slot = rdm_s + W;
+    using S = typename RdmSum<R>::T;
+    constexpr int RW = kRdmRows<A, NV>, NC = AmpT<A>::kCplx ? 2 : 1, NW = kRdmThreads / 32;
+    struct alignas(16) Word { A v[RW / NV]; };
+    extern __shared__ __align__(16) uint8_t rdm_s[];  // [strings][RW] amplitudes, then the pairs' float64 slots
+    __shared__ double s_occ[NW][17];
+    const int n = 2 * N, npair = N * (N - 1) / 2, Dm = T.Da > T.Db ? T.Da : T.Db;
+    Word *buf = reinterpret_cast<Word *>(rdm_s);
+    double *slot = reinterpret_cast<double *>(buf + (size_t)Dm * NV);  // [2 npair][RW][NC]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double *my = slot + warp * W;
-    for (int i = threadIdx.x; i < W; i += blockDim.x) acc[i] = 0.0;
-    for (int Ib = blockIdx.x; Ib < T.Db; Ib += gridDim.x) {
-        const uint32_t b = T.strb[Ib], xb = T.sb[Ib];
-        const A *row = C + (size_t)Ib * T.Da;
-        // norm and alpha occupations (every warp, a share of the row)
-        R nrm = 0, occ[16];
-        #pragma unroll
-        for (int p = 0; p < 16; ++p) occ[p] = 0;
-        for (int Ia = threadIdx.x; Ia < T.Da; Ia += blockDim.x) {
-            const A c = row[Ia];
-            const R w = re_dot(c, c);
-            const uint32_t a = T.stra[Ia];
-            nrm += w;
-            #pragma unroll
-            for (int p = 0; p < 16; ++p)
-                if ((a >> p) & 1u) occ[p] += w;
+    for (int i = threadIdx.x; i < 2 * npair * RW * NC; i += kRdmThreads) slot[i] = 0.0;
+    auto put = [&](int e, double v) {
+        partial[(size_t)(2 * e) * gridDim.x + blockIdx.x] = v;
+        partial[(size_t)(2 * e + 1) * gridDim.x + blockIdx.x] = 0.0;
+    };
+    const int na_items = (T.Db + RW - 1) / RW, nb_items = (T.Da + RW - 1) / RW;
+    int item = blockIdx.x;  // row groups, then column groups
+    for (int s = 0; s < 2; ++s) {
+        const int D = s ? T.Db : T.Da, rows = s ? T.Da : T.Db;  // strings of the pairs' spin; rows of them
+        const uint16_t *str = s ? T.strb : T.stra;
+        const uint32_t *other = s ? T.sa : T.sb;
+        const int first = s ? na_items : 0, last = s ? na_items + nb_items : na_items;
+        if (item >= last) {  // no group of this pass
+            if (threadIdx.x < N) put(1 + 2 * threadIdx.x + s, 0.0);
+            if (threadIdx.x == 0 && s == 0) put(0, 0.0);
+            continue;
         }
-        nrm = warp_sum(nrm);
-        if (lane == 0) {
-            my[0] = to_double(nrm);
-            my[1] = 0.0;
-        }
-        #pragma unroll
-        for (int p = 0; p < 16; ++p) {
-            if (p >= N) break;
-            const R s = warp_sum(occ[p]);
-            if (lane == 0) {
-                my[2 * (1 + 2 * p)] = to_double(s);
-                my[2 * (1 + 2 * p) + 1] = 0.0;
-                my[2 * (2 + 2 * p)] = ((b >> p) & 1u) ? to_double(nrm) : 0.0;
-                my[2 * (2 + 2 * p) + 1] = 0.0;
-            }
-        }
-        // pair elements: element e = 1 + n + k (k = 0 .. 2 npair - 1; alpha pairs first) to warp k % NW
-        for (int k = warp; k < 2 * npair; k += NW) {
-            const int s = k >= npair, kk = s ? k - npair : k;
-            int p = 0, rem = kk;
-            while (rem >= N - 1 - p) {
-                rem -= N - 1 - p;
-                ++p;
-            }
-            const int q = p + 1 + rem, e = 1 + n + k;
-            const uint32_t m = (1u << p) | (1u << q), f = 1u << q;
-            const uint32_t bm = between(2 * p + s, 2 * q + s);
-            R re = 0, im = 0;
+        if (lane < 17) s_occ[warp][lane] = 0.0;
+        for (; item < last; item += (int)gridDim.x) {
+            const int r0 = (item - first) * RW;
+            __syncthreads();  // the last group's reads of buf are done
             if (s == 0) {
-                // the alpha strings holding q but not p, from the pair's list: entry =
-                // rank | parity of its alpha bits under bm << 15 | partner rank << 16
-                const int4 li = ainfo[kk];
-                const uint32_t *L = alist + li.x, rsg = (uint32_t)par(xb & bm);
-                for (int i = lane; i < li.y; i += 32) {
-                    const uint32_t ea = L[i];
-                    if (!(SV_IN_RANGE(ea & 0x7FFFu, T.Da, kChkRank) && SV_IN_RANGE(ea >> 16, T.Da, kChkRank)))
-                        continue;  // checked build: skip the entry
-                    const A u = row[ea & 0x7FFFu], v = row[ea >> 16];
-                    R ar = re_dot(v, u), ai = im_dot(v, u);  // conj(v) u
-                    if (((ea >> 15) & 1u) ^ rsg) { ar = -ar; ai = -ai; }
-                    re += ar;
-                    im += ai;
-                }
-            } else if ((b & m) == f) {
-                const uint32_t r2 = T.rb[b ^ m];
-                if (SV_IN_RANGE(r2, T.Db, kChkRank)) {  // checked build: a bad rank skips the partner row
-                    const A *row2 = C + (size_t)r2 * T.Da;
-                    for (int Ia = lane; Ia < T.Da; Ia += 32) {
-                        const A u = row[Ia], v = row2[Ia];
-                        R ar = re_dot(v, u), ai = im_dot(v, u);
-                        if (par((T.sa[Ia] | xb) & bm)) { ar = -ar; ai = -ai; }
-                        re += ar;
-                        im += ai;
+                for (int x = threadIdx.x; x < D; x += kRdmThreads) {
+                    #pragma unroll
+                    for (int w = 0; w < NV; ++w) {
+                        Word v;
+                        #pragma unroll
+                        for (int j = 0; j < RW / NV; ++j) {
+                            const int r = r0 + w * (RW / NV) + j;
+                            v.v[j] = r < rows ? C[(size_t)r * T.Da + x] : mka<A>(R(0), R(0));
+                        }
+                        buf[w * Dm + x] = v;
                     }
                 }
+            } else {
+                A *flat = reinterpret_cast<A *>(buf);
+                for (int i = threadIdx.x; i < D * RW; i += kRdmThreads) {
+                    constexpr int WV = RW / NV;
+                    const int j = i % RW, r = r0 + j;
+                    flat[((j / WV) * Dm + i / RW) * WV + j % WV] = r < rows ? C[(size_t)(i / RW) * T.Da + r] : mka<A>(R(0), R(0));
+                }
             }
-            re = warp_sum(re);
-            im = warp_sum(im);
-            if (lane == 0) {
-                my[2 * e] = to_double(re);
-                my[2 * e + 1] = to_double(im);
+            __syncthreads();
+            // this spin's occupations (and the norm)
+            S occ[16], nrm[1] = {S(0)};
+            #pragma unroll
+            for (int p = 0; p < 16; ++p) occ[p] = S(0);
+            for (int x = threadIdx.x; x < D; x += kRdmThreads) {
+                const uint32_t bits = str[x];
+                R w = R(0);
+                #pragma unroll
+                for (int k = 0; k < NV; ++k) {
+                    const Word v = buf[k * Dm + x];
+                    #pragma unroll
+                    for (int j = 0; j < RW / NV; ++j) w += re_dot(v.v[j], v.v[j]);
+                }
+                sum_to(nrm[0], w);
+                #pragma unroll
+                for (int p = 0; p < 16; ++p)
+                    if ((bits >> p) & 1u) sum_to(occ[p], w);
+            }
+            const S so = row_sums<16>(occ, lane), sn = row_sums<1>(nrm, lane);
+            if (lane % 2 == 0) s_occ[warp][lane / 2] += to_double(so);
+            if (lane == 0) s_occ[warp][16] += to_double(sn);
+            const uint32_t xo = lane * RW / 32 + r0 < rows ? other[lane * RW / 32 + r0] : 0u;  // this lane's row's string
+            // pair k of this spin to warp k % NW
+            int p = 0, q = 0;
+            for (int k = 0; k < npair; ++k) {
+                if (++q == N) { ++p; q = p + 1; }
+                if (k % NW != warp) continue;
+                // list entry: rank | parity of the string's own bits between << 15 | partner rank << 16
+                const int4 li = info[k];
+                const uint32_t *L = lists + (s ? li.z : li.x);
+                const int cnt = s ? li.w : li.y;
+                R acc[RW], ai[RW];
+                #pragma unroll
+                for (int j = 0; j < RW; ++j) acc[j] = ai[j] = R(0);
+                #pragma unroll 2
+                for (int i = lane; i < cnt; i += 32) {
+                    const uint32_t ea = L[i];
+                    if (!(SV_IN_RANGE(ea & 0x7FFFu, D, kChkRank) && SV_IN_RANGE(ea >> 16, D, kChkRank)))
+                        continue;  // checked build: skip the entry
+                    const bool neg = ((ea >> 15) & 1u) != 0u;
+                    #pragma unroll
+                    for (int w = 0; w < NV; ++w) {
+                        const Word wu = buf[w * Dm + (ea & 0x7FFFu)], wv = buf[w * Dm + (ea >> 16)];
+                        #pragma unroll
+                        for (int j = 0; j < RW / NV; ++j) {
+                            // conj(v) u, the sign on u
+                            const A v = wv.v[j], u0 = wu.v[j];
+                            const R ux = neg ? -re(u0) : re(u0);
+                            const int r = w * (RW / NV) + j;
+                            acc[r] = mad(re(v), ux, acc[r]);
+                            if constexpr (NC == 2) {
+                                const R uy = neg ? -im(u0) : im(u0);
+                                acc[r] = mad(im(v), uy, acc[r]);
+                                ai[r] = mad(re(v), uy, ai[r]);
+                                ai[r] = mad(-im(v), ux, ai[r]);
+                            }
+                        }
+                    }
+                }
+                const bool flip = par(xo & between(2 * p + s, 2 * q + s)) != 0;
+                double *my = slot + ((size_t)(s * npair + k) * RW + lane * RW / 32) * NC;
+                const R sr = row_sums<RW>(acc, lane);
+                if (lane % (32 / RW) == 0) my[0] += to_double(flip ? -sr : sr);
+                if constexpr (NC == 2) {
+                    const R si = row_sums<RW>(ai, lane);
+                    if (lane % (32 / RW) == 0) my[1] += to_double(flip ? -si : si);
+                }
             }
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < W; i += blockDim.x) {
-            const int e = i >> 1;
+        if (threadIdx.x < 17) {
             double t = 0.0;
-            if (e < 1 + n) {
-                for (int w = 0; w < NW; ++w) t += slot[w * W + i];
-            } else {
-                t = slot[((e - 1 - n) % NW) * W + i];
-            }
-            acc[i] += t;
+            for (int w = 0; w < NW; ++w) t += s_occ[w][threadIdx.x];
+            if (threadIdx.x < N) put(1 + 2 * threadIdx.x + s, t);
+            if (threadIdx.x == 16 && s == 0) put(0, t);
         }
         __syncthreads();
     }
-    for (int i = threadIdx.x; i < W; i += blockDim.x) partial[(size_t)i * gridDim.x + blockIdx.x] = acc[i];
+    for (int e = threadIdx.x; e < 2 * npair; e += kRdmThreads) {
+        double re = 0.0, im = 0.0;
+        for (int r = 0; r < RW; ++r) {
+            re += slot[((size_t)e * RW + r) * NC];
+            if constexpr (NC == 2) im += slot[((size_t)e * RW + r) * NC + 1];
+        }
+        partial[(size_t)(2 * (1 + n + e)) * gridDim.x + blockIdx.x] = re;
+        partial[(size_t)(2 * (1 + n + e) + 1) * gridDim.x + blockIdx.x] = im;
+    }
 }
 
 // out[i] = C[idx[i]] or 0 when idx[i] is 0xFFFFFFFF (a basis state outside the sector)
@@ -569,34 +645,56 @@ cudaError_t launch_adjoint_li(void *CL, int dtype, const uint32_t *al, int na_l,
 
 int rdm_rows_elements(int n) { return 1 + n + (n / 2) * (n / 2 - 1); }
 
-int rdm_rows_grid(int Db, int sm_count, int bps) {
+// Blocks: at most bps per SM, and no more than rows.
+int rdm_rows_grid(int rows, int sm_count, int bps) {
     const int cap = sm_count * (bps > 0 ? bps : 4);
-    return Db < cap ? Db : cap;
+    return rows < cap ? rows : cap;
 }
 
+namespace {
+
+template <typename A, int NV>
+cudaError_t rdm_rows_nv(const void *C, const SectTabs &T, int N, int grid, const uint32_t *lists, const int *info,
+                        double *partial, cudaStream_t st) {
+    constexpr int RW = kRdmRows<A, NV>, NC = AmpT<A>::kCplx ? 2 : 1;
+    const size_t smem = (size_t)(T.Da > T.Db ? T.Da : T.Db) * 16 * NV + sizeof(double) * (size_t)N * (N - 1) * RW * NC;
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_rdm_rows<A, NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_rdm_rows<A, NV><<<grid, kRdmThreads, smem, st>>>((const A *)C, T, N, lists, (const int4 *)info, partial);
+    return cudaGetLastError();
+}
+
+template <typename A>
+cudaError_t rdm_rows_of(const void *C, const SectTabs &T, int N, int grid, const uint32_t *lists, const int *info,
+                        double *partial, int sm_count, cudaStream_t st) {
+    const int Dm = T.Da > T.Db ? T.Da : T.Db;
+    // two words: up to two blocks per SM by shared memory (about 100 KB each)
+    if (Dm <= 3 * 1024 && Dm / kRdmRows<A, 2> >= 2 * sm_count)
+        return rdm_rows_nv<A, 2>(C, T, N, grid, lists, info, partial, st);
+    return rdm_rows_nv<A, 1>(C, T, N, grid, lists, info, partial, st);  // at most 12,870 strings: 214 KB
+}
+
+}  // namespace
+
 // partial: [2 n_el][grid] doubles (n_el = rdm_rows_elements(n)), reduced by launch_reduce_rows.
-// alist / ainfo: the alpha-pair lists (one list op per pair p < q in (p, q) order with flip
-// mask {p, q}, "from" pattern {q} and sign mask between(2p, 2q)) and their int4 records.
+// lists / info: the pair lists and their int4 records, one list op per pair p < q in (p, q) order (for
+// each spin flip mask {p, q}, "from" pattern {q}, sign mask the orbitals between).
 // ff_form: C holds the float-float form of a float64 state (ffc for complex128, ff for
 // float64), as launch_to_ff writes it.
 cudaError_t launch_rdm_rows(const void *C, int dtype, int ff_form, int n, const uint32_t *sa, const uint32_t *sb,
                             const uint16_t *stra, const uint16_t *strb, const uint16_t *ra, const uint16_t *rb, int Da,
-                            int Db, int grid, const uint32_t *alist, const int *ainfo, double *partial,
+                            int Db, int grid, const uint32_t *lists, const int *info, double *partial, int sm_count,
                             cudaStream_t st) {
-    SectTabs T = tabs(sa, sb, stra, strb, ra, rb, Da, Db);
-    const size_t smem = sizeof(double) * 2 * rdm_rows_elements(n) * (1 + kThreads / 32);  // <= 40 KB (n <= 32)
+    const SectTabs T = tabs(sa, sb, stra, strb, ra, rb, Da, Db);
     if (ff_form) {
-        if (dtype == SV_C128)
-            k_rdm_rows<ffc><<<grid, kThreads, smem, st>>>((const ffc *)C, T, n / 2, alist, (const int4 *)ainfo, partial);
-        else if (dtype == SV_R64)
-            k_rdm_rows<ff><<<grid, kThreads, smem, st>>>((const ff *)C, T, n / 2, alist, (const int4 *)ainfo, partial);
-        else
-            return cudaErrorInvalidValue;  // single-precision states have no float-float form
-        return cudaGetLastError();
+        if (dtype == SV_C128) return rdm_rows_of<ffc>(C, T, n / 2, grid, lists, info, partial, sm_count, st);
+        if (dtype == SV_R64) return rdm_rows_of<ff>(C, T, n / 2, grid, lists, info, partial, sm_count, st);
+        return cudaErrorInvalidValue;  // single-precision states have no float-float form
     }
-    SV_DISPATCH_AMP(dtype, k_rdm_rows<A><<<grid, kThreads, smem, st>>>((const A *)C, T, n / 2, alist,
-                                                                       (const int4 *)ainfo, partial));
-    return cudaGetLastError();
+    cudaError_t e = cudaErrorInvalidValue;
+    SV_DISPATCH_AMP(dtype, e = rdm_rows_of<A>(C, T, n / 2, grid, lists, info, partial, sm_count, st));
+    return e;
 }
 
 cudaError_t launch_gather_c(const void *psi, int dtype, const uint32_t *idx, int count, void *out, cudaStream_t st) {

@@ -78,11 +78,11 @@ cudaError_t launch_adjoint_li(void *CL, int dtype, const uint32_t *al, int na_l,
 cudaError_t launch_adjoint_l(void *psi, void *lam, int dtype, const uint32_t *al, int na_l, const uint32_t *bl,
                              int nb_l, int Da, double c, double s, int grid, double *partial, cudaStream_t st);
 int rdm_rows_elements(int n);
-int rdm_rows_grid(int Db, int sm_count, int bps);
+int rdm_rows_grid(int rows, int sm_count, int bps);
 cudaError_t launch_to_ff(const void *C, int dtype, size_t count, void *out, int sm_count, cudaStream_t st);
 cudaError_t launch_rdm_rows(const void *C, int dtype, int ff_form, int n, const uint32_t *sa, const uint32_t *sb,
                             const uint16_t *stra, const uint16_t *strb, const uint16_t *ra, const uint16_t *rb, int Da,
-                            int Db, int grid, const uint32_t *alist, const int *ainfo, double *partial,
+                            int Db, int grid, const uint32_t *lists, const int *info, double *partial, int sm_count,
                             cudaStream_t st);
 cudaError_t launch_gather_c(const void *psi, int dtype, const uint32_t *idx, int count, void *out, cudaStream_t st);
 cudaError_t launch_core_move(void *handle_vec, int dtype, void *core_vec, int core_dtype, bool publish,
@@ -731,21 +731,24 @@ struct L2FetchScope {
     L2FetchScope &operator=(const L2FetchScope &) = delete;
 };
 
-// The 1-RDM's alpha-pair lists: for each orbital pair p < q (in (p, q) order) the alpha
-// strings holding q but not p with their partners (q -> p) and the parity of their alpha
-// bits strictly between spin-orbitals 2p and 2q; kept while the sector is unchanged.
+// The 1-RDM's pair lists: for each orbital pair p < q (in (p, q) order) the alpha strings
+// holding q but not p with their partners (q -> p) and the parity of their bits strictly between
+// p and q, and the beta strings likewise: one list op of both spins' masks (an alpha string has
+// even spin-orbitals only, a beta string odd ones).  Kept while the sector is unchanged.
 static sv_status ensure_rdm_lists(sv_handle h) {
     const int N = h->n / 2;
     std::vector<OpDesc> ops;
     for (int p = 0; p < N; ++p)
         for (int q = p + 1; q < N; ++q) {
             OpDesc d;
-            d.m = (1u << (2 * p)) | (1u << (2 * q));
-            d.from = 1u << (2 * q);
-            d.sm = ((1u << (2 * q)) - 1u) & ~((2u << (2 * p)) - 1u);
-            d.nbits = 2;
+            d.m = (3u << (2 * p)) | (3u << (2 * q));
+            d.from = 3u << (2 * q);
+            d.sm = ((1u << (2 * q)) - 1u) & ~((4u << (2 * p)) - 1u);
+            d.nbits = 4;
             d.pos[0] = 2 * p;
-            d.pos[1] = 2 * q;
+            d.pos[1] = 2 * p + 1;
+            d.pos[2] = 2 * q;
+            d.pos[3] = 2 * q + 1;
             ops.push_back(d);
         }
     if (ops.empty()) {
@@ -1611,18 +1614,18 @@ static sv_status autotune_impl(sv_handle h, sv_ham_handle ham, const std::vector
         }
         const int n_el = rdm_rows_elements(h->n);
         const int cands[] = {2, 4, 8, 16};
-        SV_TRY(ensure_partials(h, (size_t)2 * n_el * rdm_rows_grid(h->Db, h->sm_count, 16)));
+        SV_TRY(ensure_partials(h, (size_t)2 * n_el * rdm_rows_grid(std::max(h->Da, h->Db), h->sm_count, 16)));
         const void *src = nullptr;
         int ff_form = 0;
         SV_TRY(rdm_input(h, Cm, &src, &ff_form));
         int best_b = 4;
         float best_t = -1.f;
         for (int b : cands) {
-            const int grid = rdm_rows_grid(h->Db, h->sm_count, b);
+            const int grid = rdm_rows_grid(std::max(h->Da, h->Db), h->sm_count, b);
             const float t = time_best(h, e0, e1, [&]() -> sv_status {
                 SV_CUDA(h, launch_rdm_rows(src, h->dtype, ff_form, h->n, h->str_sa, h->str_sb, h->str_a, h->str_b,
                                            h->rank_a, h->rank_b, h->Da, h->Db, grid, (const uint32_t *)h->rdm_lists.buf,
-                                           h->rdm_lists.dinfo, h->partials, h->stream));
+                                           h->rdm_lists.dinfo, h->partials, h->sm_count, h->stream));
                 return SV_OK;
             });
             if (t < 0.f) return fail(h, SV_ERR_CUDA, "autotune: 1-RDM candidate failed");
@@ -2360,7 +2363,7 @@ static sv_status rdm1_run(sv_handle h, double *re_out, double *im_out) {
         SV_TRY(ensure_strings(h));
         SV_TRY(ensure_rdm_lists(h));
         const int n_el = rdm_rows_elements(h->n);
-        const int grid = rdm_rows_grid(h->Db, h->sm_count, h->rdm_bps);
+        const int grid = rdm_rows_grid(std::max(h->Da, h->Db), h->sm_count, h->rdm_bps);
         SV_TRY(ensure_partials(h, (size_t)2 * n_el * grid));
         SV_TRY(ensure_out(h, 2 * (size_t)n_el));
         SV_TRY(mark(h, 0, "sv_rdm1"));
@@ -2376,7 +2379,7 @@ static sv_status rdm1_run(sv_handle h, double *re_out, double *im_out) {
         SV_TRY(rdm_input(h, Cm, &src, &ff_form));
         SV_CUDA(h, launch_rdm_rows(src, h->dtype, ff_form, h->n, h->str_sa, h->str_sb, h->str_a, h->str_b, h->rank_a,
                                    h->rank_b, h->Da, h->Db, grid, (const uint32_t *)h->rdm_lists.buf,
-                                   h->rdm_lists.dinfo, h->partials, h->stream));
+                                   h->rdm_lists.dinfo, h->partials, h->sm_count, h->stream));
         h->launches++;
         SV_CUDA(h, launch_reduce_rows(h->partials, 2 * n_el, grid, h->dout, h->stream));
         h->launches++;

@@ -282,7 +282,7 @@ struct sv_ctx {
     // rotations and adjoint steps) and the screened pool's
     OpLists lists, pool_lists;
     SweepGroups groups;        // the ansatz's steps for whole sector sweeps
-    OpLists rdm_lists;         // the 1-RDM's alpha-pair lists (one per orbital pair p < q)
+    OpLists rdm_lists;         // the 1-RDM's pair lists of both spins (per orbital pair p < q)
     void *CLbuf = nullptr;     // compact amplitudes and sigma interleaved [Db][Da][2] (screening)
     size_t CLbuf_bytes = 0;
     // reduction scratch

@@ -1,0 +1,39 @@
+"""The 1-RDM's row and column groups at the edges of their sizes: one and two words to a string,
+a last group that is not full, a spin without pairs (empty, full, one electron), unequal spins."""
+import numpy as np
+import pytest
+
+import oracle
+from oracle import route_a as A
+from paper_2405_11567_gb300 import inputs, sv
+
+pytestmark = pytest.mark.gpu
+
+# the parity suite's 1-RDM tolerance of each precision
+TOL = {"c128": 1e-12, "r64": 1e-12, "c64": 2e-6, "r32": 2e-6}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    from paper_2405_11567_gb300 import build
+    build.build()
+    sv.lib()
+
+
+# C(13, 6) = 1,716 strings take two words in float64, C(15, 5) = 3,003 in float32
+@pytest.mark.parametrize("variant", [0, 2])
+@pytest.mark.parametrize("dtype", ["c128", "r64", "c64", "r32"])
+@pytest.mark.parametrize("n,na,nb", [(4, 1, 0), (4, 2, 1), (6, 3, 1), (10, 2, 3), (14, 7, 1), (26, 6, 1), (30, 1, 5)])
+def test_rdm_groups(n, na, nb, dtype, variant):
+    rng = np.random.default_rng(100 * n + na)
+    occ = [2 * p for p in range(na)] + [2 * p + 1 for p in range(nb)]
+    pool = inputs.qeb_pool(n, 2 if n < 8 else 4)
+    ops = pool[rng.integers(0, len(pool), 150)]
+    theta = rng.normal(0, 0.7, len(ops))
+    sec = oracle.Sector(n, na, nb)
+    psi = A.apply_ansatz(sec, ops, theta, A.hf_state(sec, occ))
+    st = sv.StateVector(n, dtype, sector=(na, nb))
+    st.set_option(sv.SV_OPT_RDM_VARIANT, variant)
+    st.prepare_hf(occ)
+    st.apply_ansatz(ops, theta)
+    assert np.max(np.abs(st.rdm1() - A.rdm1(sec, psi))) <= TOL[dtype]
