@@ -479,6 +479,7 @@ __global__ void __launch_bounds__(kRdmThreads, 2) k_rdm_rows(const A *__restrict
         }
         __syncthreads();
     }
+    __syncthreads();  // (a block without groups: the slots were zeroed by other threads)
     for (int e = threadIdx.x; e < 2 * npair; e += kRdmThreads) {
         double re = 0.0, im = 0.0;
         for (int r = 0; r < RW; ++r) {

@@ -37,3 +37,26 @@ def test_rdm_groups(n, na, nb, dtype, variant):
     st.prepare_hf(occ)
     st.apply_ansatz(ops, theta)
     assert np.max(np.abs(st.rdm1() - A.rdm1(sec, psi))) <= TOL[dtype]
+
+
+def test_blocks_without_groups():
+    """More blocks than row and column groups: the idle blocks add zeros, whatever shared memory held."""
+    n, na, nb = 26, 6, 1
+    rng = np.random.default_rng(7)
+    pool = inputs.qeb_pool(n, 4)
+    ops = pool[rng.integers(0, len(pool), 60)]
+    theta = rng.normal(0, 0.7, len(ops))
+    occ = [2 * p for p in range(na)] + [1]
+    sec = oracle.Sector(n, na, nb)
+    ref = A.rdm1(sec, A.apply_ansatz(sec, ops, theta, A.hf_state(sec, occ)))
+    dirty = sv.StateVector(24, "r32", sector=(4, 4))  # its 1-RDM leaves other values in shared memory
+    dirty.prepare_hf(list(range(8)))
+    for bps in (1, 4, 16, 64):
+        st = sv.StateVector(n, "r64", sector=(na, nb))
+        st.set_option(sv.SV_OPT_RDM_BLOCKS_PER_SM, bps)
+        st.prepare_hf(occ)
+        st.apply_ansatz(ops, theta)
+        for _ in range(4):
+            dirty.rdm1()
+            assert np.max(np.abs(st.rdm1() - ref)) <= TOL["r64"]
+        st.close()
