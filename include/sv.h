@@ -368,7 +368,13 @@ typedef enum {
                                        FP32 pipe instead of GB300's much narrower FP64
                                        pipe; the amplitudes are converted once per call
                                        and sigma written back as float64 (two work
-                                       matrices of 16 Da Db bytes, complex) */
+                                       matrices of 16 Da Db bytes, complex).  Real float64
+                                       amplitudes (also a complex128 handle's with a real
+                                       reference) of a sector that would take variant 5 in
+                                       single precision: the same sums as integer products
+                                       of seven base-256 digits on the tensor cores,
+                                       accumulated exactly (planes of 8 bytes: 3.7 GB at 30
+                                       qubits; float-float where the memory cannot be had) */
     SV_OPT_RDM_VARIANT = 4,         /* 0 auto (3 for float64 states, else 2); 1 sector
                                        gather: one thread per sector determinant (dense
                                        storage only); 2 string rows: one block per beta

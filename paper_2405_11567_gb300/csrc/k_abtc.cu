@@ -45,89 +45,18 @@
 
 #include "sv_check.cuh"
 #include "sv_internal.h"
+#include "sv_tc.cuh"
 
 namespace svk {
 
 namespace {
 
-constexpr int kAbBuild = 512;                  // builder threads (16 warps): 4 per tile row
-constexpr int kAbKpt = 4;                      // K entries of a stage per builder thread (16 / 4)
-constexpr int kAbEpi = 256;                    // epilogue threads (8 warps: two per tensor-memory lane quarter)
-constexpr int kAbThreadsTc = kAbBuild + 32 + kAbEpi;  // builders, the MMA warp, the epilogue warps
-constexpr int kAbM = 128;                      // alpha strings per tile
-constexpr int kAbKc = 16;                      // K (orbitals and orbital pairs) per stage
 constexpr int kAbS = 4;                        // stages
-constexpr int kAbMaxK = 144;                   // N (N + 1) / 2 <= 136 for N <= 16, padded to 16
-constexpr int kAbMaxN = 64;                    // columns per accumulator: nb (N - nb) + 1 <= 51 within the limits
 constexpr int kAbACols = kAbKc / 2;            // tensor-memory columns of one bf16 piece of A (two K per column)
 constexpr int kAbAccCols = 2 * kAbMaxN;        // one accumulator: both planes
 constexpr int kAbAStage = 6 * kAbACols;        // A columns per stage: 2 planes x 3 pieces
 constexpr int kAbABase = 2 * kAbAccCols;       // first A column (after the two accumulators)
 static_assert(kAbABase + kAbS * kAbAStage <= 512, "tensor memory: accumulators and A stages in 512 columns");
-
-__device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// One poll: a try-wait that suspends the thread until the phase completes or at most
-// kAbPollNs nanoseconds have passed (a thread waiting here wakes as soon as the phase
-// completes, and takes no issue slots meanwhile).
-constexpr uint32_t kAbPollNs = 64;
-__device__ __forceinline__ bool ab_try(uint32_t mbar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(mbar), "r"(parity), "n"(kAbPollNs)
-        : "memory");
-    return ok != 0;
-}
-
-__device__ __forceinline__ bool ab_wait(uint32_t mbar, uint32_t parity, uint32_t spins) {
-    for (uint32_t it = 0; it < spins; ++it)
-        if (ab_try(mbar, parity)) return true;
-    return false;
-}
-
-__device__ __forceinline__ void ab_arrive(uint32_t mbar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
-}
-
-__device__ __forceinline__ void ab_commit(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
-}
-
-__device__ __forceinline__ void builders_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kAbBuild) : "memory"); }
-
-// Barrier over the builder warps (named barrier 1) or the epilogue warps (2) that also
-// returns, to every thread of the group, whether any of them passed `v` true: a
-// decision the whole group takes the same way.
-__device__ __forceinline__ bool builders_any(bool v) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}\n"
-        : "=r"(r)
-        : "r"((uint32_t)v), "n"(kAbBuild)
-        : "memory");
-    return r != 0;
-}
-__device__ __forceinline__ bool epi_any(bool v) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 2, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}\n"
-        : "=r"(r)
-        : "r"((uint32_t)v), "n"(kAbEpi)
-        : "memory");
-    return r != 0;
-}
-
-// Canonical no-swizzle K-major descriptor: K-adjacent core matrices 128 bytes apart,
-// adjacent 8-row groups 256 bytes apart (16 K elements = two 16-byte cores per row).
-__device__ __forceinline__ uint64_t ab_desc(uint32_t addr) {
-    uint64_t d = (uint64_t)((addr >> 4) & 0x3FFFu);
-    d |= (uint64_t)(128u >> 4) << 16;
-    d |= (uint64_t)(256u >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    return d;
-}
 
 // The twelve MMAs of one K block in stage S: per plane the six piece products
 // (A piece, B piece) = (0,0) (0,1) (1,0) (0,2) (1,1) (2,0) into the plane's accumulator
@@ -160,9 +89,6 @@ __device__ __forceinline__ void ab_mma_stage(uint32_t tmem, uint64_t d0, uint32_
     }
 }
 
-// byte offset of (row r, 16-byte column kc) in a tile of 16 K
-__device__ __forceinline__ uint32_t ab_off(int r, int kc) { return (uint32_t)(((r >> 3) * 2 + kc) * 128 + (r & 7) * 16); }
-
 __device__ __forceinline__ void split3(float v, uint32_t &p1, uint32_t &p2, uint32_t &p3) {
     const __nv_bfloat16 a = __float2bfloat16_rn(v);
     const float r = v - __bfloat162float(a);
@@ -171,14 +97,6 @@ __device__ __forceinline__ void split3(float v, uint32_t &p1, uint32_t &p2, uint
     p1 = __bfloat16_as_ushort(a);
     p2 = __bfloat16_as_ushort(b);
     p3 = __bfloat16_as_ushort(c);
-}
-
-__device__ __forceinline__ int ab_par(uint32_t x) { return __popc(x) & 1; }
-
-// bits strictly between i and j
-__device__ __forceinline__ uint32_t ab_between(int i, int j) {
-    const int lo = min(i, j), hi = max(i, j);
-    return ((1u << hi) - 1u) & ~((1u << (lo + 1)) - 1u);
 }
 
 
@@ -203,10 +121,6 @@ struct AbTcArgs {
     int stall;                // test hook: the builders stage and write nothing, so the MMA issuer's
                               // and the epilogue's first waits run out with nothing in flight
 };
-
-// K entries per tile row in the table (nK * 16) plus 4: an odd number of 8-byte words
-// per row, so the builders' 8-byte reads of 16 consecutive rows hit distinct bank pairs.
-__host__ __device__ __forceinline__ int ab_tstride(int nK) { return nK * kAbKc + 4; }
 
 // PAIR: a real state.  Its amplitudes have one component, so a unit takes two partner rows in the
 // place of the two planes: the gathers through the table, the words staged and the tensor-memory
@@ -587,17 +501,21 @@ size_t ab_table_rows(int N, int Db) { return (size_t)N * N + Db + 1; }
 // Elements of the per-partner-row column table (uint16) that launch_ab_table writes.
 size_t ab_rowb_elems(int Db) { return (size_t)Db * kAbMaxN; }
 
+// The column table [Db][64] of the sector with nb beta electrons.
+cudaError_t launch_ab_rows(const uint16_t *strb, int N, int nb, int Db, uint16_t *rowB, cudaStream_t st) {
+    if (nb * (N - nb) + 1 > kAbMaxN) return cudaSuccess;  // more columns than the products take: no column table
+    k_ab_rows<<<Db, kAbMaxN, 0, st>>>(strb, N, nb, Db, rowB);
+    return cudaGetLastError();
+}
+
 // The B table pieces and, where rowB is given, the column table [Db][64] of the sector
 // with nb beta electrons (two launches).
 cudaError_t launch_ab_table(const float *eri, const float *Jt, const uint16_t *strb, int N, int nb, int Db,
                             uint16_t *Bp, size_t pb, uint16_t *rowB, cudaStream_t st) {
     if (N * N > 256 || nb < 0 || nb > N) return cudaErrorInvalidValue;
     k_ab_table<<<(unsigned)ab_table_rows(N, Db), 256, 0, st>>>(eri, Jt, strb, N, Db, Bp, pb);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !rowB) return e;
-    if (nb * (N - nb) + 1 > kAbMaxN) return cudaSuccess;  // more columns than k_ab_tc takes: no column table
-    k_ab_rows<<<Db, kAbMaxN, 0, st>>>(strb, N, nb, Db, rowB);
-    return cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess || !rowB ? e : launch_ab_rows(strb, N, nb, Db, rowB, st);
 }
 
 // Whether the tensor-core alpha-beta form applies: N <= 16, D <= 4096 per spin, at most

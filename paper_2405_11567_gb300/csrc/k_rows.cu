@@ -757,8 +757,9 @@ __global__ void __launch_bounds__(kAbThreads, 1) k_sigma_ab(RowArgs<Amp> A) {
 // Block I < Da builds alpha row I of Ma, block Da + I beta row I of Mb; thread 0 also
 // writes the string's one-spin diagonal energy sum_k h_kk + sum_{k<l} [kk|ll]-[kl|lk]
 // (spin-orbital tables hdiag, Jp) to dA / dB.  Ma and Mb must be zeroed before.
-__global__ void __launch_bounds__(128) k_same_mats(SigmaTables<float> T, float *__restrict__ Ma,
-                                                    float *__restrict__ Mb, double *__restrict__ dA,
+template <typename R>
+__global__ void __launch_bounds__(128) k_same_mats(SigmaTables<R> T, R *__restrict__ Ma,
+                                                    R *__restrict__ Mb, double *__restrict__ dA,
                                                     double *__restrict__ dB, int lda, int ldb) {
     __shared__ uint8_t occ[kMaxOrb], emp[kMaxOrb];
     __shared__ int s_no, s_ne;
@@ -766,7 +767,7 @@ __global__ void __launch_bounds__(128) k_same_mats(SigmaTables<float> T, float *
     const int I = beta ? (int)blockIdx.x - T.Da : (int)blockIdx.x, N = T.N, spin = beta;
     const uint16_t *rk = beta ? T.rb : T.ra;
     const uint32_t str = beta ? T.strb[I] : T.stra[I], pps = prefix_parity(str);
-    float *row = (beta ? Mb : Ma) + (size_t)I * (beta ? ldb : lda);
+    R *row = (beta ? Mb : Ma) + (size_t)I * (beta ? ldb : lda);
     if (threadIdx.x == 0) {
         int no = 0, ne = 0;
         for (int o = 0; o < N; ++o) {
@@ -786,13 +787,13 @@ __global__ void __launch_bounds__(128) k_same_mats(SigmaTables<float> T, float *
     __syncthreads();
     const int no = s_no, ne = s_ne, nsg = no * ne, npo = no * (no - 1) / 2, npe = ne * (ne - 1) / 2;
     for (int t = threadIdx.x; t < nsg + npo * npe; t += blockDim.x) {
-        float v;
+        R v;
         uint32_t m, sg;
         if (t < nsg) {
             const int p = occ[t / ne], q = emp[t % ne];
             m = (1u << p) | (1u << q);
             v = T.hm[q * N + p];
-            const float *dt = T.Dt + (q * N + p) * N;
+            const R *dt = T.Dt + (q * N + p) * N;
             for (uint32_t o = str; o; o &= o - 1u) v += dt[__ffs(o) - 1];
             sg = (uint32_t)par(pps & m) ^ (uint32_t)(p < q);
         } else {
@@ -801,7 +802,7 @@ __global__ void __launch_bounds__(128) k_same_mats(SigmaTables<float> T, float *
             while (ie >= ne - 1 - e1) ie -= ne - 1 - e1++;
             const int p1 = occ[i1], p2 = occ[i1 + 1 + io], q1 = emp[e1], q2 = emp[e1 + 1 + ie];
             m = (1u << p1) | (1u << p2) | (1u << q1) | (1u << q2);
-            v = eri4<float>(T, q1, p1, q2, p2) - eri4<float>(T, q1, p2, q2, p1);
+            v = eri4<R>(T, q1, p1, q2, p2) - eri4<R>(T, q1, p2, q2, p1);
             sg = (uint32_t)par(pps & m) ^ double_order_sign(p1, p2, q1, q2);
         }
         row[rk[str ^ m]] = sg ? -v : v;
@@ -1291,16 +1292,38 @@ cudaError_t launch_sigma_rows(const void *C, void *lam, void *lamc, int dtype, i
     return e;
 }
 
-// Ma [Da][lda], Mb [Db][ldb] (zeroed here, padding included), dA, dB of the sector for
-// single-precision tables.
+// Ma [Da][lda], Mb [Db][ldb] (zeroed here, padding included), dA, dB of the sector for tables of
+// real type R (float or double).
+template <typename R>
+static cudaError_t same_mats_t(int n, const RowTables &T, const double *hdiag, const double *Jp, R *Ma, R *Mb,
+                               double *dA, double *dB, int lda, int ldb, cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(Ma, 0, sizeof(R) * (size_t)T.Da * lda, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(Mb, 0, sizeof(R) * (size_t)T.Db * ldb, st);
+    if (e != cudaSuccess) return e;
+    RowArgs<R> A = row_args<R>(nullptr, nullptr, nullptr, n, T, hdiag, Jp, 0.0, nullptr);
+    k_same_mats<R><<<T.Da + T.Db, 128, 0, st>>>(A.T, Ma, Mb, dA, dB, lda, ldb);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_same_mats(int n, const RowTables &T, const double *hdiag, const double *Jp, float *Ma, float *Mb,
                              double *dA, double *dB, int lda, int ldb, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(Ma, 0, sizeof(float) * (size_t)T.Da * lda, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(Mb, 0, sizeof(float) * (size_t)T.Db * ldb, st);
-    if (e != cudaSuccess) return e;
-    RowArgs<float> A = row_args<float>(nullptr, nullptr, nullptr, n, T, hdiag, Jp, 0.0, nullptr);
-    k_same_mats<<<T.Da + T.Db, 128, 0, st>>>(A.T, Ma, Mb, dA, dB, lda, ldb);
-    return cudaGetLastError();
+    return same_mats_t<float>(n, T, hdiag, Jp, Ma, Mb, dA, dB, lda, ldb, st);
+}
+cudaError_t launch_same_mats(int n, const RowTables &T, const double *hdiag, const double *Jp, double *Ma, double *Mb,
+                             double *dA, double *dB, int lda, int ldb, cudaStream_t st) {
+    return same_mats_t<double>(n, T, hdiag, Jp, Ma, Mb, dA, dB, lda, ldb, st);
+}
+
+cudaError_t launch_sigma_digits(const SigmaTables<double> &T, const double *C, double *lam, double *lamc,
+                                const uint32_t *sa_s, const uint32_t *sb_s, int Db, int nb, const SameDigits &g,
+                                double *partial, int sm_count, cudaStream_t st);
+
+// The digit products (k_digits.cu) for a real float64 state; partial: 2 Db doubles.
+cudaError_t launch_sigma_rows_digits(const void *C, void *lam, void *lamc, int n, const RowTables &T,
+                                     const double *hdiag, const double *Jp, double e_shift, double *partial, int nb,
+                                     const SameDigits &g, int sm_count, cudaStream_t st) {
+    const RowArgs<double> A = row_args<double>(C, lam, lamc, n, T, hdiag, Jp, e_shift, partial);
+    return launch_sigma_digits(A.T, A.C, A.lam, A.lamc, A.sa_s, A.sb_s, T.Db, nb, g, partial, sm_count, st);
 }
 
 // This unit's check word (checked build), for sv_check_status.

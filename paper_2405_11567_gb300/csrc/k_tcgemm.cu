@@ -25,14 +25,13 @@
 #include <cudaTypedefs.h>
 
 #include "sv_internal.h"
+#include "sv_tc.cuh"
 
 namespace svk {
 
 namespace {
 
 constexpr int kTcThreads = 128;
-constexpr int kTcM = 128;                              // alpha strings per tile (tensor-memory lanes)
-constexpr int kTcKb = 32;                              // K (bf16 elements, 64 bytes) per stage
 constexpr int kTcABytes = kTcM * kTcKb * 2;            // one piece of A in one stage
 constexpr int kTcCols = 512;                           // tensor-memory columns: every accumulator
 
@@ -50,55 +49,6 @@ struct TcTile {
     static constexpr int kStages = TN == 256 ? 3 : 4;                   // 3 x 72 KB, 4 x 48 KB
     static constexpr int kSmem = kStages * kStageBytes + 1024;          // + alignment of the ring to 1024 bytes
 };
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// Shared-memory matrix descriptor of a K-major operand tile with 64-byte swizzle: start
-// address, stride byte offset 512 (8 rows of 64 bytes), descriptor version 1, swizzle
-// mode 4 (64-byte).  The leading byte offset is unused for swizzled K-major tiles.
-__device__ __forceinline__ uint64_t tc_desc(uint32_t addr) {
-    uint64_t d = (uint64_t)((addr >> 4) & 0x3FFFu);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(512u >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)4 << 61;
-    return d;
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(mbar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, uint32_t spins) {
-    for (uint32_t it = 0; it < spins; ++it) {
-        if (mbar_try(mbar, parity)) return true;
-        __nanosleep(32);
-    }
-    return false;
-}
-
-__device__ __forceinline__ void tma_3d(uint32_t dst, const CUtensorMap *map, int k, int row, int c3, uint32_t mbar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-        "[%5];" ::"r"(dst),
-        "l"((uint64_t)map), "r"(k), "r"(row), "r"(c3), "r"(mbar)
-        : "memory");
-}
-
-__device__ __forceinline__ void tma_4d(uint32_t dst, const CUtensorMap *map, int k, int row, int p, int c,
-                                       uint32_t mbar) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-        "%5}], [%6];" ::"r"(dst),
-        "l"((uint64_t)map), "r"(k), "r"(row), "r"(p), "r"(c), "r"(mbar)
-        : "memory");
-}
 
 struct TcOut {
     float *G;  // [P][Db][Da]
@@ -294,35 +244,6 @@ __global__ void __launch_bounds__(256) k_transpose_pieces(const uint16_t *__rest
         const int a = a0 + i, b = b0 + threadIdx.x;
         if (a < Da && b < Db) Xtp[(size_t)a * ldb + b] = t[threadIdx.x][i];
     }
-}
-
-// cuTensorMapEncodeTiled from the driver (through the runtime's entry-point query, so
-// the library links no driver library).
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            return nullptr;
-        fn = (PFN_cuTensorMapEncodeTiled_v12000)f;
-    }
-    return fn;
-}
-
-// A bf16 tensor map of `rank` dims (innermost first) with byte strides of dims 1.., box
-// {kTcKb, rows, 1, 1}, 64-byte swizzle, zero fill.
-bool encode_map(CUtensorMap *m, const void *base, int rank, const uint64_t *dims, const uint64_t *strides,
-                uint32_t rows) {
-    PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
-    if (!fn) return false;
-    const cuuint32_t box[4] = {(cuuint32_t)kTcKb, rows, 1, 1}, es[4] = {1, 1, 1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void *>(base),
-              (const cuuint64_t *)dims, (const cuuint64_t *)strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace

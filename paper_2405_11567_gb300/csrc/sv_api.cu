@@ -111,6 +111,16 @@ size_t ab_rowb_elems(int Db);
 cudaError_t launch_ab_table(const float *eri, const float *Jt, const uint16_t *strb, int N, int nb, int Db, uint16_t *Bp,
                             size_t pb, uint16_t *rowB, cudaStream_t st);
 bool ab_tc_fits(int planes, int Da, int Db, int na, int nb, int N);
+bool digits_fit(int Da, int Db, int nb, int N);
+cudaError_t launch_same_mats(int n, const RowTables &T, const double *hdiag, const double *Jp, double *Ma, double *Mb,
+                             double *dA, double *dB, int lda, int ldb, cudaStream_t st);
+cudaError_t launch_ham_digits(const double *M, size_t nm, uint16_t *Mp, const double *eri, const double *Jt,
+                              const uint16_t *strb, int N, int Db, double *B64, uint16_t *Bp, unsigned int *maxw,
+                              int sm_count, cudaStream_t st);
+cudaError_t launch_ab_rows(const uint16_t *strb, int N, int nb, int Db, uint16_t *rowB, cudaStream_t st);
+cudaError_t launch_sigma_rows_digits(const void *C, void *lam, void *lamc, int n, const RowTables &T,
+                                     const double *hdiag, const double *Jp, double e_shift, double *partial, int nb,
+                                     const SameDigits &g, int sm_count, cudaStream_t st);
 int ab_xi_ld(int Da);
 int ab_h_ld(int Da);
 int sigma_ab_chunk(int dtype, const RowTables &T, int nb, int want);
@@ -137,6 +147,7 @@ uint32_t check_word_sector();
 uint32_t check_word_sweep();
 uint32_t check_word_rows();
 uint32_t check_word_abtc();
+uint32_t check_word_digits();
 uint32_t check_word_pool();
 }  // namespace svk
 
@@ -515,6 +526,8 @@ static sv_status upload_tables(sv_handle h, sv_ham_handle ham, DevTables &T) {
     SV_TRY(up(&T.hm_r, hm.data(), hm.size() * sizeof(R)));
     SV_TRY(up(&T.Dt, Dt.data(), Dt.size() * sizeof(R)));
     SV_TRY(up(&T.Jt, Jt.data(), Jt.size() * sizeof(R)));
+    for (double v : ham->eri) T.eri_max = std::max(T.eri_max, std::isfinite(v) ? std::fabs(v) : HUGE_VAL);
+    for (double v : ham->h) T.h_max = std::max(T.h_max, std::isfinite(v) ? std::fabs(v) : HUGE_VAL);
     // same-spin doubles p1 < p2 -> q1 < q2 by pairs, W2[(p1,p2)][(q1,q2)] =
     // s0 ((q1p1|q2p2) - (q1p2|q2p1)), with the orbital-order part of the
     // Jordan-Wigner sign, s0 = (-1)^([p1<q2] + [q2<p2] + [p1<q1] + [p2<q1]), folded in;
@@ -948,6 +961,18 @@ static int row_chunk(sv_handle h, const RowTables &R) {
     return sigma_ab_chunk(h->dtype, R, h->nb, (int)h->ab_chunk);
 }
 
+// Whether every string has at least 5% of its spin's strings as same-spin partners (singles and
+// doubles), so that dense products do at most 20 times the multiplies of the sparse sums.
+static bool dense_couplings(sv_handle h) {
+    const int N = h->n / 2;
+    auto c2 = [](long x) { return x * (x - 1) / 2; };
+    auto dens = [&](int ne, int D) {
+        const long ns = (long)ne * (N - ne), nd = c2(ne) * c2(N - ne);
+        return (double)(ns + nd) / (double)D;
+    };
+    return dens(h->na, h->Da) >= 0.05 && dens(h->nb, h->Db) >= 0.05;
+}
+
 // Whether the string-row expectation takes the same-spin products (variant 4):
 // single-precision states whose split form fits and whose strings number at most
 // 4096 per spin (matrices up to 64 MB).  Automatic choice (variant 0): where the
@@ -961,13 +986,7 @@ static bool use_same_gemm(sv_handle h, int K) {
     if (!single_prec(h->dtype) || K == 0 || h->Da > 4096 || h->Db > 4096) return false;
     if (h->expect_variant == 4 || h->expect_variant == 5) return true;
     if (h->expect_variant != 0) return false;
-    const int N = h->n / 2;
-    auto c2 = [](long x) { return x * (x - 1) / 2; };
-    auto dens = [&](int ne, int D) {
-        const long ns = (long)ne * (N - ne), nd = c2(ne) * c2(N - ne);
-        return (double)(ns + nd) / (double)D;
-    };
-    return (double)h->Da * h->Db >= (double)(1 << 14) && dens(h->na, h->Da) >= 0.05 && dens(h->nb, h->Db) >= 0.05;
+    return (double)h->Da * h->Db >= (double)(1 << 14) && dense_couplings(h);
 }
 
 // Whether the same-spin product form also takes the alpha-beta part as tensor-core
@@ -1168,8 +1187,144 @@ static sv_status rdm_input(sv_handle h, const void *Cm, const void **src, int *f
     return SV_OK;
 }
 
+// The digit products' memory for a sector: [Ma | Mb] (float64), the one-spin diagonals, their digits
+// and the alpha-beta table's, its rows and its float64 values, their largest words (mats, built once per Hamiltonian and sector); the digits of X
+// and its transpose, the records, G and the largest amplitude's word (work); H.
+struct DigitBytes {
+    size_t lda, ldb, ldh, nm, rowsB, ncols;
+    size_t dof, sof, bof, rbo, vof, wof, mats;  // offsets in mats
+    size_t tof, iof, gof, mof, work;        // offsets in work
+    size_t hplane;
+    explicit DigitBytes(sv_handle h) {
+        auto r = [](size_t b) { return (b + 255) / 256 * 256; };
+        const size_t Da = (size_t)h->Da, Db = (size_t)h->Db;
+        const int N = h->n / 2;
+        lda = (Da + 7) / 8 * 8;
+        ldb = (Db + 7) / 8 * 8;
+        ldh = ab_h_ld((int)Da);
+        nm = Da * lda + Db * ldb;
+        rowsB = ab_table_rows(N, (int)Db);
+        ncols = (size_t)h->nb * (N - h->nb) + 1;
+        dof = r(nm * sizeof(double));
+        sof = dof + r((Da + Db) * sizeof(double));
+        bof = sof + r(7 * nm * 2);
+        rbo = bof + r(7 * rowsB * 256 * 2);
+        vof = rbo + r(ab_rowb_elems((int)Db) * 2);
+        wof = vof + r(rowsB * 256 * sizeof(double));
+        mats = wof + 256;
+        tof = r(7 * Db * lda * 2);
+        iof = tof + r(7 * Da * ldb * 2);
+        gof = iof + r(Db * (Da + 4) * 16);
+        mof = gof + r(2 * Da * Db * 8);
+        work = mof + 256;
+        hplane = Db * ncols * ldh;
+    }
+};
+
+// Whether the float-float expectation (variant 6, or the automatic choice of float64 states) takes the
+// digit products (k_digits.cu): real float64 sectors of at least 2^14 determinants within their limits
+// and with dense same-spin couplings, finite integrals, planes H of at most 16 GiB, everything under the
+// handle's byte cap.  Measured, float-float / digits
+// in us: 44,100 determinants 173 / 100, 108,900 390 / 145, 245,025 668 / 222, 9,018,009 39,100 / 8,930.
+static bool use_digits(sv_handle h, const DevTables *T) {
+    if (h->dtype != SV_R64 || (h->expect_variant != 0 && h->expect_variant != 6)) return false;
+    if ((double)h->Da * h->Db < (double)(1 << 14) || !digits_fit(h->Da, h->Db, h->nb, h->n / 2) || !dense_couplings(h))
+        return false;
+    if (!(T->eri_max < 1e100 && T->h_max < 1e100)) return false;
+    const DigitBytes B(h);
+    const size_t hb = B.hplane * 8;
+    if (hb > (16ull << 30)) return false;
+    if (h->max_bytes <= 0) return true;
+    const double held = (double)h->sg_mats_bytes + (double)h->sg_buf_bytes + (double)h->ab_H_bytes;
+    return (double)h->bytes_owned - held + (double)B.mats + (double)B.work + (double)hb <= (double)h->max_bytes;
+}
+
+// The digit products' operands (an allocation's status where the memory cannot be had).
+static sv_status ensure_digits(sv_handle h, DevTables *T, const RowTables &R, SameDigits *g) {
+    SV_TRY(ensure_kerr(h));
+    const DigitBytes B(h);
+    const int N = h->n / 2;
+    auto hold = [&](void **p, size_t *have, size_t want, const char *what) -> sv_status {
+        if (*have >= want) return SV_OK;
+        dev_free(h, *p, *have);
+        *p = nullptr;
+        *have = 0;
+        const sv_status st = dev_alloc(h, p, want, what);
+        if (st == SV_OK) *have = want;
+        else cudaGetLastError();
+        return st;
+    };
+    SV_TRY(hold((void **)&h->ab_H, &h->ab_H_bytes, B.hplane * 8, "alpha-beta product planes"));
+    if (!h->sg_mats || h->sg_serial != T->serial || h->sg_na != h->na || h->sg_nb != h->nb) {
+        h->sg_serial = 0;
+        SV_TRY(hold(&h->sg_mats, &h->sg_mats_bytes, B.mats, "same-spin matrices"));
+        uint8_t *m = (uint8_t *)h->sg_mats;
+        double *Ma = (double *)m, *dA = (double *)(m + B.dof);
+        SV_CUDA(h, launch_same_mats(h->n, R, T->hdiag, T->Jp, Ma, Ma + (size_t)h->Da * B.lda, dA, dA + h->Da,
+                                    (int)B.lda, (int)B.ldb, h->stream));
+        SV_CUDA(h, launch_ham_digits(Ma, B.nm, (uint16_t *)(m + B.sof), (const double *)R.eri, (const double *)R.Jt,
+                                     h->str_b, N, h->Db, (double *)(m + B.vof), (uint16_t *)(m + B.bof),
+                                     (unsigned int *)(m + B.wof), h->sm_count, h->stream));
+        SV_CUDA(h, launch_ab_rows(h->str_b, N, h->nb, h->Db, (uint16_t *)(m + B.rbo), h->stream));
+        h->launches += 7;
+        h->sg_serial = T->serial;
+        h->sg_na = h->na;
+        h->sg_nb = h->nb;
+    }
+    const uint64_t geom = ((uint64_t)h->Da << 32) | ((uint64_t)h->Db << 3) | 1u;
+    if (h->sg_buf_bytes < B.work || h->sg_buf_geom != geom) {
+        h->sg_buf_geom = 0;
+        SV_TRY(hold(&h->sg_buf, &h->sg_buf_bytes, B.work, "same-spin product planes"));
+        SV_CUDA(h, cudaMemsetAsync(h->sg_buf, 0, B.work, h->stream));  // the row padding stays zero
+        h->sg_buf_geom = geom;
+    }
+    const uint8_t *m = (const uint8_t *)h->sg_mats;
+    uint8_t *w = (uint8_t *)h->sg_buf;
+    g->dA = (const double *)(m + B.dof);
+    g->dB = g->dA + h->Da;
+    g->Mp = (const uint16_t *)(m + B.sof);
+    g->pm = B.nm;
+    g->Bp = (const uint16_t *)(m + B.bof);
+    g->pb = B.rowsB * 256;
+    g->rowB = (const uint16_t *)(m + B.rbo);
+    g->Xp = (uint16_t *)w;
+    g->px = (size_t)h->Db * B.lda;
+    g->Xtp = (uint16_t *)(w + B.tof);
+    g->pt = (size_t)h->Da * B.ldb;
+    g->Xi = (uint32_t *)(w + B.iof);
+    g->G = (long long *)(w + B.gof);
+    g->maxw = (unsigned int *)(w + B.mof);
+    g->lda = (int)B.lda;
+    g->ldb = (int)B.ldb;
+    g->ldh = (int)B.ldh;
+    g->ncols = (int)B.ncols;
+    g->H = (long long *)h->ab_H;
+    g->hplane = B.hplane;
+    g->ham_maxw = (const unsigned int *)(m + B.wof);
+    g->err = h->kerr;
+    g->spins = (uint32_t)h->wait_polls;
+    g->stall = h->test_stall;
+    if (h->profile) {
+        for (cudaEvent_t &e : h->tcev)
+            if (!e) SV_CUDA(h, cudaEventCreate(&e));
+        g->ev = h->tcev;
+    }
+    return SV_OK;
+}
+
 static sv_status sigma_rows(sv_handle h, DevTables *T, const RowTables &R, const void *C, void *lam, void *lamc,
                             double e_shift) {
+    if (use_digits(h, T)) {
+        SameDigits g;
+        if (ensure_digits(h, T, R, &g) == SV_OK) {  // else the float-float sums below
+            SV_CUDA(h, launch_sigma_rows_digits(C, lam, lamc, h->n, R, T->hdiag, T->Jp, e_shift, h->partials, h->nb, g,
+                                                h->sm_count, h->stream));
+            h->launches += 6;
+            if (g.ev) h->tc_timed = 3;
+            SV_CUDA(h, cudaMemcpyAsync(h->hkerr, h->kerr, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+            return SV_OK;
+        }
+    }
     const int K = row_chunk(h, R);
     if (use_ff(h, K) && T->eri_ff) {
         const size_t r = ff_matrix_bytes(h);
@@ -1647,7 +1802,7 @@ extern "C" {
 const char *sv_version(void) { return "sv-gb300 0.1 (sm_103a)"; }
 
 uint32_t sv_check_status(void) {
-    const uint32_t a = check_word_sector() | check_word_sweep(), b = check_word_rows(), c = check_word_abtc(), d = check_word_pool();
+    const uint32_t a = check_word_sector() | check_word_sweep(), b = check_word_rows(), c = check_word_abtc() | check_word_digits(), d = check_word_pool();
     return (a & 0xFFu) | ((b & 0xFFu) << 8) | ((c & 0xFFu) << 16) | ((d & 0x0Fu) << 24) |
            ((a | b | c | d) & 0x80000000u);
 }

@@ -149,6 +149,26 @@ struct SameGemm {
     int ncols = 0, na = 0, nb = 0;
 };
 
+// Operands of the digit products (k_digits.cu; real float64 states).
+struct SameDigits {
+    const double *dA = nullptr, *dB = nullptr;   // one-spin diagonal energies per string
+    const uint16_t *Mp = nullptr;                // seven digits of [Ma | Mb], piece stride pm
+    uint16_t *Xp = nullptr, *Xtp = nullptr;      // digits of X = phi C [Db][lda] (px) and its transpose [Da][ldb] (pt)
+    size_t pm = 0, px = 0, pt = 0, pb = 0;
+    int lda = 0, ldb = 0, ldh = 0, ncols = 0;
+    uint32_t *Xi = nullptr;                      // digits of X as words [Db][4][Da rounded up]
+    long long *G = nullptr;                      // same-spin products [2][Db][Da], fixed point
+    const uint16_t *Bp = nullptr, *rowB = nullptr;  // digits of the alpha-beta integral table (piece stride pb), its rows
+    long long *H = nullptr;                      // alpha-beta products [Db][ncols][ldh], fixed point
+    size_t hplane = 0;                           // elements of H
+    unsigned int *maxw = nullptr;                // device: high word of the largest amplitude
+    const unsigned int *ham_maxw = nullptr;      // device: those of [Ma | Mb] and of the table
+    int *err = nullptr;
+    uint32_t spins = 1u << 22;
+    cudaEvent_t *ev = nullptr;                   // as in SameGemm
+    int stall = 0;
+};
+
 struct DevTables {
     uint64_t serial = 0;   // unique per table set (keys the per-handle same-spin matrices)
     int n = 0;
@@ -169,6 +189,7 @@ struct DevTables {
     void *W2 = nullptr;     // [NP][NP] same-spin doubles by (q1<q2, p1<p2) pairs
     // the same five tables as float-float pairs (float64 tables only; expectation variant 6)
     void *eri_ff = nullptr, *hm_ff = nullptr, *Dt_ff = nullptr, *Jt_ff = nullptr, *W2_ff = nullptr;
+    double eri_max = 0.0, h_max = 0.0;  // largest |(pq|rs)| and |h_pq|
     // tiled-pass schedule (k_expect.cu); empty until first needed
     struct Pass {
         uint32_t S;        // local qubit set (bit mask over storage positions)
