@@ -444,8 +444,9 @@ typedef enum {
                                        handle needs sv_prepare_hf / sv_prepare_state.
                                        1..2^30, default 2^22 */
     SV_OPT_TEST_STALL = 16,         /* failure-detection test hook, 0 (default) off: bit 0
-                                       makes k_same_tc's producer issue no copy, bit 1
-                                       makes k_ab_tc's builders stage and write nothing,
+                                       makes k_same_tc's (k_same_digits's) producer issue no
+                                       copy, bit 1 makes k_ab_tc's (k_ab_digits's) builders
+                                       stage and write nothing,
                                        so that the consumers' first bounded waits run out
                                        with no copy or MMA in flight (the path of a stuck
                                        producer).  No fault and no hang: the call reports
@@ -462,10 +463,10 @@ typedef enum {
                                        checkpoint copy falls inside the sweep and the
                                        device accepts the launch, else one launch per
                                        operator (0 always) */
-    SV_OPT_SWEEP_BLOCKS_PER_SM = 18,/* launch geometry of the whole-sweep launches: at most
-                                       this many blocks per SM, no more than can be
-                                       resident (1..64, default 2; sv_autotune times
-                                       1, 2, 4, 8) */
+    SV_OPT_SWEEP_BLOCKS_PER_SM = 18,/* launch geometry of the whole-sweep launches on the
+                                       grid: at most this many blocks per SM, no more than
+                                       can be resident, one where the operators are small
+                                       (1..64, default 2; sv_autotune times 1, 2, 4, 8) */
     SV_OPT_FULL_VECTOR = 19         /* 0 (default): the path runs on the sector's amplitudes
                                        alone, in real arithmetic where the reference is
                                        real (a determinant, or a stored state without
@@ -509,12 +510,12 @@ sv_status sv_autotune(sv_handle h, sv_ham_handle ham, const sv_excitation *ops, 
 
 /* Device time (ms) of each phase of the last sv_energy_grad / sv_rdm1 call,
  * measured with CUDA events on the handle's stream while SV_OPT_PROFILE is 1:
- * [0] reference preparation, [1] forward sweep (one rotation kernel per op),
- * [2] expectation (sigma and energy), [3] reverse sweep (one adjoint kernel per
- * op plus the gradient reduction), [4] restoring psi(theta), [5] the last
- * sv_rdm1; inside [2], for the tensor-core expectation forms (variants 4 and 5):
- * [6] the same-spin products (k_transpose_pieces + k_same_tc), [7] the
- * alpha-beta products (k_ab_tc, variant 5).  Writes min(n_out, SV_PHASES)
+ * [0] reference preparation, [1] forward sweep, [2] expectation (sigma and
+ * energy), [3] reverse sweep (with the gradient reduction), [4] restoring or
+ * publishing psi(theta), [5] the last
+ * sv_rdm1; inside [2], for the tensor-core expectation forms (variants 4, 5; digits):
+ * [6] the same-spin products with their transposes (k_same_tc, k_same_digits),
+ * [7] the alpha-beta products (k_ab_tc, variant 5; k_ab_digits).  Writes min(n_out, SV_PHASES)
  * values; phases not run are 0. */
 sv_status sv_phase_times(sv_handle h, double *ms_out, int n_out);
 

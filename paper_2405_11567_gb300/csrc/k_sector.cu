@@ -502,6 +502,7 @@ __global__ void k_gather_c(const A *__restrict__ psi, const uint32_t *__restrict
 // A handle's vector from its compute core's compact amplitudes (Out the handle's type, In the
 // core's: the same, or its real one): string pair (a, b) of the core, at ca[a] + cb[b] of the
 // vector (dense storage: the storage-space spreads; sector storage: the ranks in its order).
+// Without C, zeros.
 // Bound: dense, one partly written 32-byte DRAM sector per scattered amplitude.
 template <typename Out, typename In>
 __global__ void __launch_bounds__(kThreads) k_core_publish(const In *__restrict__ C, Out *__restrict__ psi,
@@ -512,7 +513,7 @@ __global__ void __launch_bounds__(kThreads) k_core_publish(const In *__restrict_
         const size_t row = (size_t)Ib * Da;
         const uint32_t xb = cb[Ib];
         for (int Ia = blockIdx.y * kThreads + threadIdx.x; Ia < Da; Ia += gridDim.y * kThreads) {
-            const In c = C[row + Ia];
+            const In c = C ? C[row + Ia] : In{};
             psi[xb + ca[Ia]] = mka<Out>((R)re(c), (R)im(c));
         }
     }
@@ -536,7 +537,7 @@ __global__ void __launch_bounds__(kThreads) k_core_gather(const In *__restrict__
 
 // ---------------------------------------------------------------- launchers
 
-// publish: core (core_dtype) -> handle (dtype); else the handle's vector -> core.
+// publish: core (core_dtype; NULL: zeros) -> handle (dtype); else the handle's vector -> core.
 cudaError_t launch_core_move(void *handle_vec, int dtype, void *core_vec, int core_dtype, bool publish,
                              const uint32_t *ca, const uint32_t *cb, int Da, int Db, int sm_count, cudaStream_t st) {
     if (Da <= 0 || Db <= 0) return cudaSuccess;

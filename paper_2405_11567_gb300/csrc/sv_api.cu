@@ -1953,6 +1953,25 @@ static void reference_changed(sv_handle h) {
     if (h->core) h->core->failed = false;
 }
 
+// The determinant reference in a whole vector that is zero outside the reference's sector (an earlier
+// state of it): zeros at the sector's amplitudes alone, where they are few: a partly written 32-byte
+// sector is read and written, 64 bytes to an amplitude.  30 qubits (9,018,009 of 2^30, complex64): the
+// memset of 8 GiB 1.14 ms, so 0.22; 24 qubits 49 and 25 us.
+static sv_status prepare_in_sector(sv_handle h) {
+    sv_handle c = h->core;
+    const uint32_t *sa, *sb;
+    if (h->storage != 0 || (double)c->Da * c->Db * 64.0 >= (double)vec_bytes(h)) return prepare_reference(h);
+    if (core_places(h, &sa, &sb) != SV_OK) {
+        cudaGetLastError();
+        return prepare_reference(h);
+    }
+    SV_CUDA(h, launch_core_move(h->psi, h->dtype, nullptr, h->dtype, true, sa, sb, c->Da, c->Db, h->sm_count, h->stream));
+    SV_CUDA(h, launch_set_basis(h->psi, h->dtype, map_bits(h->ref_det, h->perm), h->stream));
+    h->launches += 2;
+    h->psi_clean = true;
+    return SV_OK;
+}
+
 sv_status sv_prepare_hf(sv_handle h, const int32_t *occ, int n_occ) {
     if (!h) return fail(nullptr, SV_ERR_ARG, "NULL handle");
     if (n_occ < 0 || n_occ > h->n || (n_occ > 0 && !occ)) return fail(h, SV_ERR_ARG, "bad occupation list");
@@ -1968,6 +1987,8 @@ sv_status sv_prepare_hf(sv_handle h, const int32_t *occ, int n_occ) {
     if (h->storage == 1 && (na != h->na || nb != h->nb))
         return fail(h, SV_ERR_ARG, "determinant outside the handle's (n_alpha, n_beta) sector");
     DeviceGuard g(h->device);
+    const bool in_sector = h->prepared && !h->failed && h->psi_clean && !h->exposed && h->core &&
+                           na == h->na && nb == h->nb && na == h->core->na && nb == h->core->nb;
     h->failed = false;
     h->prepared = false;
     h->ref_kind = 1;
@@ -1976,7 +1997,7 @@ sv_status sv_prepare_hf(sv_handle h, const int32_t *occ, int n_occ) {
     h->na = na;
     h->nb = nb;
     reference_changed(h);
-    SV_TRY(prepare_reference(h));
+    SV_TRY(in_sector ? prepare_in_sector(h) : prepare_reference(h));
     h->prepared = true;
     h->at_ref = true;
     h->core_cur = 1;

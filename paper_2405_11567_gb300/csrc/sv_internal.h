@@ -330,10 +330,10 @@ struct sv_ctx {
     int l2_fetch = 32;         // context L2 fetch granularity during dense sweeps (0: leave it)
     int rev_inter = 1;         // dense reverse sweep on psi and lambda interleaved (k_adjoint_i) where it can
     bool lam_pair = false;     // lam's allocation holds two vectors: lam, then the working copy `saved`
-    int *kerr = nullptr;       // device flag of kernels with bounded waits (k_same_tc, k_ab_tc)
+    int *kerr = nullptr;       // device flag of kernels with bounded waits (k_same_tc, k_ab_tc, the digit kernels, k_sweep)
     int64_t wait_polls = 1 << 22;  // polls of each of their bounded waits (SV_OPT_WAIT_POLLS)
-    int test_stall = 0;        // SV_OPT_TEST_STALL: bit 0 k_same_tc, bit 1 k_ab_tc issue no copy / MMA
-    // sector storage, whole-sweep launches (k_sweep_rotate_l / k_sweep_adjoint_li): a barrier
+    int test_stall = 0;        // SV_OPT_TEST_STALL: bit 0 k_same_tc / k_same_digits, bit 1 k_ab_tc / k_ab_digits issue nothing
+    // sector storage, whole-sweep launches (k_sweep): a barrier
     // counter (first 256 bytes) and the ops' (cos, sin) on the device, their host staging
     void *sweep_buf = nullptr;
     size_t sweep_bytes = 0;

@@ -414,7 +414,7 @@ class Batch:
         sv_batch_set_time_limit(self.handle, ms)
 
     def autotune(self, theta_concat) -> int:
-        """Time the batched launch at 1-4 blocks per SM and keep the fastest grid (returned)."""
+        """Time the batched launch at each block count per SM that can be resident and keep the fastest grid (returned)."""
         return sv_batch_autotune(self.handle, theta_concat, self.total_ops)
 
     @property

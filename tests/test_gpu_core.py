@@ -191,3 +191,33 @@ def test_paired_steps_match_single_operators(n, na, nb, dtype):
         assert np.max(np.abs(psi - out[0][2])) <= 4 * len(ops) * eps
         assert abs(E - out[0][0]) <= 64 * len(ops) * eps
         assert np.max(np.abs(g - out[0][1])) <= 64 * len(ops) * eps * scale
+
+
+@pytest.mark.parametrize("dtype", ["c128", "c64", "r64", "r32"])
+def test_prepare_again_leaves_one_amplitude(dtype):
+    """A determinant prepared over an earlier state of the same sector (few of the vector's amplitudes),
+    of another sector, in a moved layout and after whole-vector calls: one amplitude, and its energy."""
+    n = 16
+    p = inputs.make_problem(n, 4, 20, seed=12)
+    ham = sv.Hamiltonian(p["h"], p["eri"], p["e_nuc"])
+    rng = np.random.default_rng(3)
+    st = sv.StateVector(n, dtype)
+    occs = [_occ(2, 2), _occ(2, 2), [0, 4, 3, 9], _occ(1, 2), _occ(2, 2), _occ(2, 2)]
+    for k, occ in enumerate(occs):
+        st.prepare_hf(occ)
+        if k == 3:
+            st.set_option(sv.SV_OPT_FULL_VECTOR, 1)
+        if k == 4:
+            st.set_option(sv.SV_OPT_FULL_VECTOR, 0)
+        st.energy_grad(ham, p["ops"], p["theta"])
+        if k == 1:
+            st.set_layout(rng.permutation(n))
+        st.prepare_hf(occ)
+        got = st.state()
+        x = sum(1 << j for j in occ)
+        assert np.count_nonzero(got) == 1 and got[x] == 1.0, k
+        sec = oracle.Sector(n, sum(j % 2 == 0 for j in occ), sum(j % 2 for j in occ))
+        assert abs(st.energy(ham) - A.energy(sec, p["h"], p["eri"], p["e_nuc"], A.hf_state(sec, occ))) <= TOL[
+            {"r64": "c128", "r32": "c64"}.get(dtype, dtype)][0]
+        st.apply_ansatz(p["ops"], p["theta"])
+    st.close()
