@@ -7,12 +7,13 @@ restore psi(theta) and take the spin-resolved 1-RDM.  Workload: 30 qubits
 (15 spatial orbitals, 10 electrons), seeded synthetic integrals shaped like the
 paper's molecules (config 5 of the workload list).
 
-Headline: the dense 2^30-amplitude complex64 state (8 GiB per vector, float64
-reductions), the state-vector method the metric is defined on; complex128 beside
-it.  Also timed: the same step in sector storage (only the C(15,5)^2 = 9,018,009
-amplitudes of the (5, 5) sector, 72 MB, a separate row with its own roofline), with
-real float32 amplitudes (the real-angle ansatz keeps psi real), and the batched
-small-instance launch (config 4).  L2 is flushed (a 256 MB write)
+Headline: a dense 2^30-amplitude complex64 handle (float64 reductions) as a user
+creates it; complex128 beside it.  Such a handle computes on the C(15,5)^2 =
+9,018,009 amplitudes of its (5, 5) sector, in real arithmetic while the reference is
+real, and publishes psi in its 8 GiB vector.  Also timed: the same step with every
+kernel on the whole vector (SV_OPT_FULL_VECTOR = 1: the sweeps against HBM), in
+sector storage, with real float32 amplitudes, and the batched small-instance launch
+(config 4).  L2 is flushed (a 256 MB write)
 before every timed step, outside its events.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
@@ -44,7 +45,9 @@ SIGMA_KERNELS = {
     4: "expectation: k_phase_planar + k_transpose_pieces + k_same_tc (same-spin products, tcgen05 bf16x3) "
        "+ k_sigma_ab + k_sigma_comb",
     5: "expectation: k_phase_planar + k_transpose_pieces + k_same_tc (same-spin products) + k_ab_tc "
-       "(alpha-beta products; both tcgen05 bf16x3) + k_sigma_comb (gathers the alpha-beta planes)"}
+       "(alpha-beta products; both tcgen05 bf16x3) + k_sigma_comb (gathers the alpha-beta planes)",
+    6: "expectation: k_max_word + k_phase_digits + k_transpose_digits + k_same_digits + k_ab_digits (exact integer "
+       "products, tcgen05 on bf16 digits) + k_comb_digits"}
 # Measured DRAM traffic lives in a small committed record written from ncu captures
 # (--record-traffic), keyed by a hash of the sources of the kernels it measured: a
 # record whose sources changed since is stale and the bench line reports null.
@@ -52,8 +55,8 @@ TRAFFIC_RECORDS = os.path.join(ROOT, "profiles", "traffic.json")
 CSRC = "paper_2405_11567_gb300/csrc/"
 TRAFFIC_SOURCES = {
     "dense_adjoint_c64": [CSRC + "k_state.cu", CSRC + "sv_device.cuh"],
-    "sector_sigma_c64": [CSRC + "k_rows.cu", CSRC + "k_tcgemm.cu", CSRC + "k_abtc.cu", CSRC + "sv_sigma.cuh",
-                         CSRC + "sv_device.cuh"],
+    "sector_sigma_c64": [CSRC + "k_rows.cu", CSRC + "k_tcgemm.cu", CSRC + "k_abtc.cu", CSRC + "sv_tc.cuh",
+                         CSRC + "sv_sigma.cuh", CSRC + "sv_device.cuh"],
 }
 GOLDEN = os.path.join(ROOT, "tests", "golden", "config5_oracle.json")
 FP64_NOMINAL_TFLOPS = 1.25  # GB300 FP64 rate, nominal
@@ -288,7 +291,8 @@ def workload_config(p):
             "n_qubits": p["n_qubits"], "n_electrons": p["n_elec"],
             "n_ops": int(len(p["ops"])), "seed": p["seed"],
             "step": "prepare_hf + energy_grad (forward, sigma, adjoint) + rdm1",
-            "storage": "dense 2^30 amplitudes (8 GiB per vector, complex64); sector storage timed beside it",
+            "storage": "dense 2^30 amplitudes (8 GiB, complex64; computed on its sector's, in real arithmetic); "
+                       "whole-vector and sector storage timed beside it",
             "l2": "flushed before every timed step (256 MB write outside the step's events)"}
 
 
@@ -342,9 +346,11 @@ def run_ours(args, rank, world, local_rank):
     peak, peak_kind = measured_peaks()
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")  # 256 MB > 126 MB of L2
 
-    def timed(dtype, sector):
+    def timed(dtype, sector, full=False):
         st = sv.StateVector(n, dtype, stream, sector=(p["na"], p["nb"]) if sector else None)
         st.set_option(sv.SV_OPT_PROFILE, 1)
+        if full:  # every kernel on the whole 2^n vector
+            st.set_option(sv.SV_OPT_FULL_VECTOR, 1)
         if args.expect_variant is not None:  # a fixed expectation form (profiling; with --no-autotune)
             st.set_option(sv.SV_OPT_EXPECT_VARIANT, args.expect_variant)
         outs = {}
@@ -484,6 +490,8 @@ def run_ours(args, rank, world, local_rank):
         return 0
     head = timed("c64", sector=False)
     head128 = None if args.no_c128 else timed("c128", sector=False)
+    full64 = None if args.no_full else timed("c64", sector=False, full=True)
+    full128 = None if (args.no_full or args.no_c128) else timed("c128", sector=False, full=True)
     s64 = None if args.no_sector else timed("c64", sector=True)
     s128 = None if (args.no_sector or args.no_c128) else timed("c128", sector=True)
     r32d = None if args.no_real else timed("r32", sector=False)
@@ -495,36 +503,7 @@ def run_ours(args, rank, world, local_rank):
     K = args.steps
     value = throughput(world, K, head["ms"])
     e2e = throughput(world, K, 1000.0 * head["t_host"])
-    # roofline of the dominant kernel (by phase time): algorithmic bytes per launch / mean launch time
-    rot_bytes = touched_bytes(p["ops"], n, 8)
-    kernels = {
-        "adjoint_step": dict(phase="reverse", mult=2.0,
-                             desc="fused adjoint step (k_adjoint_i: psi and lambda interleaved in one buffer): "
-                                  "psi and lambda pairs, read + write"),
-        "rotation": dict(phase="forward", mult=1.0, desc="excitation rotation (k_rotate): touched pairs, read + write"),
-    }
-    rows = {}
-    for name, kd in kernels.items():
-        t_launch = head["phases"][kd["phase"]] / L / 1000.0
-        per_launch = kd["mult"] * rot_bytes.sum() / L
-        a = per_launch / t_launch / 1e9
-        rows[name] = {"achieved_gbs": a, "frac": a / peak, "mean_launch_ms": t_launch * 1e3,
-                      "bytes_per_launch": per_launch, "launches_per_step": L, "desc": kd["desc"]}
-    dom = max(kernels, key=lambda k: head["phases"][kernels[k]["phase"]])
-    traffic, traffic_note = None, "no ncu record for the current kernel sources"
-    rec = traffic_record("dense_adjoint_c64")
-    if dom == "adjoint_step" and rec is not None and head["layout"] is not None:
-        # the record's DRAM / algorithmic ratio of each lowest-address-bit class, weighted by this ansatz's ops
-        ratio = rec["ratio_by_lowest_bit"]
-        tb = 2.0 * rot_bytes
-        cls = [lowest_bit_class(min(head["layout"][q] for q in op_qubits(op))) for op in p["ops"]]
-        traffic = float(sum(t * ratio[c] for t, c in zip(tb, cls)) / L)
-        traffic_note = "ncu DRAM bytes per launch by lowest-address-bit class (%s), weighted by this ansatz" % rec[
-            "capture"]
-    roof = {"bound": "hbm", "kernel": dom, "achieved": rows[dom]["achieved_gbs"], "peak": peak, "unit": "GB/s",
-            "frac": rows[dom]["frac"], "traffic": traffic, "traffic_note": traffic_note,
-            "peak_kind": "measured (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured"
-            else "fallback 6.8 TB/s"}
+    roof, kern = tensor_roofline(p, head["phases"])
     golden = load_golden()
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": args.warmup,
@@ -532,47 +511,39 @@ def run_ours(args, rank, world, local_rank):
         "dtype": "f32", "precision": "complex64 state, float64 reductions", "data": "synthetic",
         "config": workload_config(p),
         "roofline": roof,
-        "kernels": rows,
+        "kernels": kern,
         "phases_ms": head["phases"],
         "clocks": head["clocks"],
         "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": int(L * (20 + 8) + len(p["occ"]) * 4),
                 "d2h_bytes_per_step": int((1 + L) * 8 + 2 * 2 * p["n_orb"] ** 2 * 8)},
         "gpu_launches": int(head["launches"]),
         "autotune": head["tuned"],
-        "step_lower_bound": step_lower_bound(rot_bytes, n, 8, head["ms"] / K, peak),
+        "expectation_form": SIGMA_KERNELS.get(head["variant"] or 5, "expectation form %d" % head["variant"]),
     }
     if golden is not None:
         line["vs_oracle"] = vs_golden(head["out"], golden)
     if head128 is not None:
         v128 = throughput(world, K, head128["ms"])
-        fp64 = fp64_peak(torch)
         line["fp64_state"] = {"value": v128, "ms_per_step": head128["ms"] / K, "phases_ms": head128["phases"],
                               "clocks": head128["clocks"],
-                              "bound": fp64_rooflines(p, head128["phases"], fp64, peak, head128["variant"]),
-                              "expectation_form": head128["variant"],
+                              "expectation_form": SIGMA_KERNELS.get(head128["variant"] or 6,
+                                                                    "expectation form %d" % head128["variant"]),
+                              "tensor_kernels": digit_kernels(p, head128["phases"]),
                               "vs_oracle": vs_golden(head128["out"], golden) if golden is not None else None}
         line["speedup_fp32_over_fp64"] = value / v128
-        line["speedup_bounds"] = {
-            "complex64": "HBM: the sweeps move their bytes at %.2f (reverse) / %.2f (forward) of the copy peak"
-                         % (rows["adjoint_step"]["frac"], rows["rotation"]["frac"]),
-            "complex128": "the sweeps on the FP64 pipe (fp64_state.bound: FP64 flops / time against the "
-                          "measured FP64 rate), the expectation in float-float arithmetic on the FP32 pipe; the "
-                          "byte ratio alone would give 2x"}
         line["fp32_vs_fp64"] = {
             "abs_dE": abs(head["out"]["E"] - head128["out"]["E"]),
             "max_abs_dg": float(np.max(np.abs(head["out"]["g"] - head128["out"]["g"]))),
             "max_abs_drdm": float(np.max(np.abs(head["out"]["rdm"] - head128["out"]["rdm"]))),
             "E_fp64": head128["out"]["E"]}
+    if full64 is not None:
+        line["full_vector"] = full_vector_row(p, full64, full128, world, K, L, n, peak, peak_kind, torch)
     if s64 is not None:
         line["sector_storage"] = sector_row(p, s64, s128, head, head128, world, K, L, golden)
     if r32d is not None:
-        # real-amplitude float32 state (the real-angle ansatz keeps psi real): half the bytes per amplitude
-        rb4 = touched_bytes(p["ops"], n, 4)
-        t_adj = r32d["phases"]["reverse"] / L / 1000.0
-        a = 2.0 * rb4.sum() / L / t_adj / 1e9
         real = {"state": "real float32 amplitudes, float64 reductions",
                 "dense": {"value": throughput(world, K, r32d["ms"]), "ms_per_step": r32d["ms"] / K,
-                          "phases_ms": r32d["phases"], "adjoint_step_gbs": a, "adjoint_step_frac": a / peak,
+                          "phases_ms": r32d["phases"],
                           "abs_dE_vs_c64": abs(r32d["out"]["E"] - head["out"]["E"]),
                           "max_abs_dg_vs_c64": float(np.max(np.abs(r32d["out"]["g"] - head["out"]["g"])))}}
         if r32s is not None:
@@ -636,6 +607,48 @@ def fp64_peak(torch):
     return 2.0 * 4096 ** 3 / (best / 1e3) / 1e12
 
 
+def full_vector_row(p, f64, f128, world, K, L, n, peak, peak_kind, torch):
+    """The step with every kernel on the whole 2^n vector (complex64, complex128 beside it): the sweeps' algorithmic
+    bytes per launch over their mean launch time against HBM, complex128's against the FP64 pipe too."""
+    rot_bytes = touched_bytes(p["ops"], n, 8)
+    kernels = {
+        "adjoint_step": dict(phase="reverse", mult=2.0,
+                             desc="fused adjoint step (k_adjoint_i: psi and lambda interleaved in one buffer): "
+                                  "psi and lambda pairs, read + write"),
+        "rotation": dict(phase="forward", mult=1.0, desc="excitation rotation (k_rotate): touched pairs, read + write"),
+    }
+    rows = {}
+    for name, kd in kernels.items():
+        t_launch = f64["phases"][kd["phase"]] / L / 1000.0
+        per_launch = kd["mult"] * rot_bytes.sum() / L
+        a = per_launch / t_launch / 1e9
+        rows[name] = {"achieved_gbs": a, "frac": a / peak, "mean_launch_ms": t_launch * 1e3,
+                      "bytes_per_launch": per_launch, "launches_per_step": L, "desc": kd["desc"]}
+    dom = max(kernels, key=lambda k: f64["phases"][kernels[k]["phase"]])
+    traffic, traffic_note = None, "no ncu record for the current kernel sources"
+    rec = traffic_record("dense_adjoint_c64")
+    if dom == "adjoint_step" and rec is not None and f64["layout"] is not None:
+        # the record's DRAM / algorithmic ratio of each lowest-address-bit class, weighted by this ansatz's ops
+        ratio = rec["ratio_by_lowest_bit"]
+        tb = 2.0 * rot_bytes
+        cls = [lowest_bit_class(min(f64["layout"][q] for q in op_qubits(op))) for op in p["ops"]]
+        traffic = float(sum(t * ratio[c] for t, c in zip(tb, cls)) / L)
+        traffic_note = "ncu DRAM bytes per launch by lowest-address-bit class (%s), weighted by this ansatz" % rec[
+            "capture"]
+    out = {"value": throughput(world, K, f64["ms"]), "unit": UNIT, "ms_per_step": f64["ms"] / K,
+           "phases_ms": f64["phases"], "clocks": f64["clocks"], "gpu_launches": int(f64["launches"]), "kernels": rows,
+           "roofline": {"bound": "hbm", "kernel": dom, "achieved": rows[dom]["achieved_gbs"], "peak": peak,
+                        "unit": "GB/s", "frac": rows[dom]["frac"], "traffic": traffic, "traffic_note": traffic_note,
+                        "peak_kind": "measured (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured"
+                        else "fallback 6.8 TB/s"},
+           "step_lower_bound": step_lower_bound(rot_bytes, n, 8, f64["ms"] / K, peak)}
+    if f128 is not None:
+        out["fp64_state"] = {"value": throughput(world, K, f128["ms"]), "ms_per_step": f128["ms"] / K,
+                             "phases_ms": f128["phases"],
+                             "bound": fp64_rooflines(p, f128["phases"], fp64_peak(torch), peak, f128["variant"])}
+    return out
+
+
 def fp64_rooflines(p, phases, fp64_tflops, hbm_peak, variant=None):
     """complex128 sweeps against the FP64 pipe and HBM: FP64 flops per amplitude pair = 12 in the rotation
     (three shears of the real and imaginary parts, six FMAs) and 32 in the adjoint step (two rotations plus
@@ -681,10 +694,11 @@ def fp32_ops_peak(sm_mhz=2070.0):
     return 152 * 128 * sm_mhz * 1e6 / 1e12
 
 
-def mma_flops(p, planes=2):
-    """bf16 tensor-core flops the two tcgen05 kernels issue per sigma: k_same_tc, tiles of 128 x 256 over
-    K blocks of 32 (both products, six piece products); k_ab_tc, units of 128 alpha strings x one partner beta
-    string, N = 64 columns over K blocks of 16 (six piece products per plane)."""
+def mma_flops(p, planes=1):
+    """bf16 tensor-core flops the two tcgen05 kernels issue per float32 sigma (planes = 1: real amplitudes, also a
+    complex handle's with a real reference): k_same_tc, tiles of 128 x 256 over K blocks of 32 (both products, six
+    piece products); k_ab_tc, units of 128 alpha strings x one partner beta string, N = 64 columns over K blocks of
+    16 (six piece products)."""
     from math import comb
     N, na, nb = p["n_orb"], p["na"], p["nb"]
     Da, Db = comb(N, na), comb(N, nb)
@@ -695,50 +709,71 @@ def mma_flops(p, planes=2):
     return same, ab
 
 
+def digit_kernels(p, ph):
+    """The float64 expectation's integer products: 28 digit products of 128 x 64 x 16 per K block."""
+    from math import comb
+    N, na, nb = p["n_orb"], p["na"], p["nb"]
+    Da, Db = comb(N, na), comb(N, nb)
+    cdiv = lambda a, b: (a + b - 1) // b  # noqa: E731
+    flop = {"k_same_digits": cdiv(Db, 64) * cdiv(Da, 128) * (cdiv(Da, 32) + cdiv(Db, 32)) * 28 * 2.0 * 128 * 64 * 32,
+            "k_ab_digits": cdiv(Da, 128) * Db * cdiv(N * (N + 1) // 2, 16) * 28 * 2.0 * 128 * 64 * 16}
+    return _kernel_rows({"k_same_digits": (flop["k_same_digits"], ph.get("same_products", 0), "includes k_transpose_digits"),
+                         "k_ab_digits": (flop["k_ab_digits"], ph.get("ab_products", 0), None)})
+
+
+def _kernel_rows(kernels):
+    out = {}
+    for name, (flop, ms, note) in kernels.items():
+        if ms > 0:
+            out[name] = {"mma_tflop": flop / 1e12, "ms": ms, "achieved_tflops": flop / (ms / 1e3) / 1e12}
+            if note:
+                out[name]["note"] = note
+    return out
+
+
+def tensor_roofline(p, ph):
+    """(roofline of the step's dominant tensor-core kernel against the measured bf16 peak, both kernels' rows)."""
+    peaks = measured_tensor_peaks()
+    same, ab = mma_flops(p)
+    kern = _kernel_rows({"k_same_tc": (same, ph.get("same_products", 0), "includes k_transpose_pieces"),
+                         "k_ab_tc": (ab, ph.get("ab_products", 0), None)})
+    if not kern:
+        return None, kern
+    dom = max(kern, key=lambda k: kern[k]["ms"])
+    rec = traffic_record("sector_sigma_c64")
+    return {"bound": "tensor", "kernel": dom, "achieved": kern[dom]["achieved_tflops"],
+            "peak": peaks["bf16_tflops"], "unit": "TFLOP/s", "frac": kern[dom]["achieved_tflops"] /
+            peaks["bf16_tflops"], "peak_kind": peaks["kind"],
+            "traffic": (rec["bytes_per_launch"].get(dom) if rec else None),
+            "traffic_note": ("ncu DRAM bytes of one launch (%s)" % rec["capture"]) if rec else
+            "no ncu record for the current kernel sources",
+            "algorithmic": "bf16 MMA flops issued per launch (six bf16 piece products per float32 product)"}, kern
+
+
 def sector_row(p, s64, s128, head, head128, world, K, L, golden):
     """Sector storage (the state is 0.84% of 2^30 amplitudes and L2-resident): its own row, with the
     tensor-core expectation kernels against the tensor pipe's measured bf16 peak."""
     D, per = sigma_terms(p)
-    useful = 4.0 * D * per  # complex amplitude x real matrix element = 2 FMA per connection
+    useful = 2.0 * D * per  # real amplitude (the reference is real) x real matrix element = 1 FMA per connection
     ph = s64["phases"]
-    peaks = measured_tensor_peaks()
-    same, ab = mma_flops(p)
-    kern = {}
-    if ph.get("same_products", 0) > 0:
-        kern["k_same_tc"] = {"mma_tflop": same / 1e12, "ms": ph["same_products"],
-                             "achieved_tflops": same / (ph["same_products"] / 1e3) / 1e12,
-                             "note": "includes k_transpose_pieces"}
-    if ph.get("ab_products", 0) > 0:
-        kern["k_ab_tc"] = {"mma_tflop": ab / 1e12, "ms": ph["ab_products"],
-                           "achieved_tflops": ab / (ph["ab_products"] / 1e3) / 1e12}
-    roof = None
-    if kern:
-        dom = max(kern, key=lambda k: kern[k]["ms"])
-        rec = traffic_record("sector_sigma_c64")
-        roof = {"bound": "tensor", "kernel": dom, "achieved": kern[dom]["achieved_tflops"],
-                "peak": peaks["bf16_tflops"], "unit": "TFLOP/s", "frac": kern[dom]["achieved_tflops"] /
-                peaks["bf16_tflops"], "peak_kind": peaks["kind"],
-                "traffic": (rec["bytes_per_launch"].get(dom) if rec else None),
-                "traffic_note": ("ncu DRAM bytes of one launch (%s)" % rec["capture"]) if rec else
-                "no ncu record for the current kernel sources",
-                "algorithmic": "bf16 MMA flops issued per launch (six bf16 piece products per float32 product)"}
+    roof, kern = tensor_roofline(p, ph)
     t_sig = ph["expectation"] / 1000.0
-    sb = sector_touched_bytes(p["ops"], p["n_orb"], p["na"], p["nb"], 8)
+    sb = sector_touched_bytes(p["ops"], p["n_orb"], p["na"], p["nb"], 4)
     t_rot = ph["forward"] / L / 1000.0
     t_adj = ph["reverse"] / L / 1000.0
     rec = traffic_record("sector_sigma_c64")
     sect = {"storage": "sector: C(15,5)^2 = 9,018,009 amplitudes (72 MB complex64), L2-resident",
             "value": throughput(world, K, s64["ms"]), "unit": UNIT, "ms_per_step": s64["ms"] / K,
             "phases_ms": ph, "clocks": s64["clocks"], "gpu_launches": int(s64["launches"]),
-            "expectation_form": SIGMA_KERNELS.get(s64["variant"], "expectation form %d" % s64["variant"]),
+            "expectation_form": SIGMA_KERNELS.get(s64["variant"] or 5, "expectation form %d" % s64["variant"]),
             "roofline": roof, "tensor_kernels": kern,
             "useful": {"tflops": useful / t_sig / 1e12, "gflop": useful / 1e9,
-                       "algorithmic": "%d determinants x %d connections x 4 flops of sparse work per sigma"
+                       "algorithmic": "%d determinants x %d connections x 2 flops of sparse work per sigma"
                                       % (D, per)},
             "sigma_traffic_bytes": rec["bytes_per_sigma"] if rec else None,
-            "kernels": {"rotation_l": {"algorithmic_gbs": sb.sum() / L / t_rot / 1e9, "mean_launch_ms": t_rot * 1e3},
-                        "adjoint_l": {"algorithmic_gbs": 2.0 * sb.sum() / L / t_adj / 1e9,
-                                      "mean_launch_ms": t_adj * 1e3}},
+            "sweeps": {"forward": {"algorithmic_gbs": sb.sum() / L / t_rot / 1e9, "us_per_operator": t_rot * 1e6},
+                       "reverse": {"algorithmic_gbs": 2.0 * sb.sum() / L / t_adj / 1e9,
+                                   "us_per_operator": t_adj * 1e6}},
             "autotune": s64["tuned"],
             "abs_dE_vs_dense_c64": abs(s64["out"]["E"] - head["out"]["E"]),
             "max_abs_dg_vs_dense_c64": float(np.max(np.abs(s64["out"]["g"] - head["out"]["g"])))}
@@ -801,9 +836,9 @@ def per_config_rows(args, stream, peak, rbatch):
     from oracle import route_a as A
     from paper_2405_11567_gb300 import inputs, sv
     out = {"cores": oracle.num_threads()}
-    roofs = {1: "launch latency: 4 KiB state, 15 one-launch operators (microseconds each)",
-             2: "launch latency / L2: 1 MiB state, 198 operators",
-             3: "L2 / HBM: 128 MiB (complex64) and 256 MiB (complex128) vectors against a 126 MB L2"}
+    roofs = {1: "launch latency (the whole sweep is one launch)",
+             2: "latency of one block's operator steps (14,400 amplitudes) and launch latency",
+             3: "latency of a cluster's operator steps (245,025 amplitudes) and the expectation's tensor-core products"}
     for cid, dtypes in ((1, ("c128",)), (2, ("c128",)), (3, ("c64", "c128"))):
         p = inputs.config_problem(cid)
         n, L = p["n_qubits"], len(p["ops"])
@@ -878,10 +913,6 @@ def per_config_rows(args, stream, peak, rbatch):
                     res[name]["max_abs_dg_vs_oracle"] = float(np.max(np.abs(r[1] - g_o)))
                     if with_rdm:
                         res[name]["max_abs_drdm_vs_oracle"] = float(np.max(np.abs(r[2] - rdm_o)))
-            if cid == 3 and "energy_grad" in res:
-                tb = touched_bytes(p["ops"], n, 8 if dtype == "c64" else 16).sum()
-                res["sweeps_algorithmic_gbs"] = 3.0 * tb / (res["energy_grad"]["ms"] / 1e3) / 1e9
-                res["sweeps_frac_of_hbm_peak"] = res["sweeps_algorithmic_gbs"] / peak
             row["gpu"][dtype] = res
             st.close()
         ham.close()
@@ -937,6 +968,7 @@ def op_profile(args):
     out = {}
     for dtype in ("c64", "c128"):
         st = sv.StateVector(n, dtype, stream)
+        st.set_option(sv.SV_OPT_FULL_VECTOR, 1)
         st.prepare_hf(p["occ"])
         st.energy_grad(ham, p["ops"], p["theta"])          # picks the automatic layout
         lay = st.layout()
@@ -978,6 +1010,7 @@ def traffic_probe(args):
     n, L = p["n_qubits"], len(p["ops"])
     ham = sv.Hamiltonian(p["h"], p["eri"], p["e_nuc"])
     st = sv.StateVector(n, "c64")
+    st.set_option(sv.SV_OPT_FULL_VECTOR, 1)
     st.prepare_hf(p["occ"])
     st.energy_grad(ham, p["ops"], p["theta"])
     torch.cuda.synchronize()
@@ -1077,6 +1110,7 @@ def main():
     ap.add_argument("--no-c128", action="store_true", help="skip the complex128 comparison run")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-batch", action="store_true", help="skip the batched (config 4) timing")
+    ap.add_argument("--no-full", action="store_true", help="skip the whole-vector timing (SV_OPT_FULL_VECTOR)")
     ap.add_argument("--no-sector", action="store_true", help="skip the sector-storage timing")
     ap.add_argument("--no-autotune", action="store_true", help="keep the default launch choices")
     ap.add_argument("--no-real", action="store_true", help="skip the real-amplitude (float32) timing")
