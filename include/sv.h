@@ -370,8 +370,8 @@ typedef enum {
                                        and sigma written back as float64 (two work
                                        matrices of 16 Da Db bytes, complex).  Real float64
                                        amplitudes (also a complex128 handle's with a real
-                                       reference) of a sector that would take variant 5 in
-                                       single precision: the same sums as integer products
+                                       reference) of a sector of at least 2^12 determinants
+                                       that meets variant 5's limits and couplings: the same sums as integer products
                                        of seven base-256 digits on the tensor cores,
                                        accumulated exactly (planes of 8 bytes: 3.7 GB at 30
                                        qubits; float-float where the memory cannot be had) */

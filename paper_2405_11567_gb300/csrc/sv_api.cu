@@ -1222,13 +1222,14 @@ struct DigitBytes {
 };
 
 // Whether the float-float expectation (variant 6, or the automatic choice of float64 states) takes the
-// digit products (k_digits.cu): real float64 sectors of at least 2^14 determinants within their limits
+// digit products (k_digits.cu): real float64 sectors of at least 2^12 determinants within their limits
 // and with dense same-spin couplings, finite integrals, planes H of at most 16 GiB, everything under the
 // handle's byte cap.  Measured, float-float / digits
-// in us: 44,100 determinants 173 / 100, 108,900 390 / 145, 245,025 668 / 222, 9,018,009 39,100 / 8,930.
+// in us: 3,136 determinants 63.9 / 66.0, 4,356 78.0 / 74.1, 4,900 71.0 / 70.5, 7,056 76.2 / 69.7, 15,876
+// 94 / 74, 44,100 173 / 100, 108,900 390 / 145, 245,025 668 / 222, 9,018,009 39,100 / 8,550.
 static bool use_digits(sv_handle h, const DevTables *T) {
     if (h->dtype != SV_R64 || (h->expect_variant != 0 && h->expect_variant != 6)) return false;
-    if ((double)h->Da * h->Db < (double)(1 << 14) || !digits_fit(h->Da, h->Db, h->nb, h->n / 2) || !dense_couplings(h))
+    if ((double)h->Da * h->Db < (double)(1 << 12) || !digits_fit(h->Da, h->Db, h->nb, h->n / 2) || !dense_couplings(h))
         return false;
     if (!(T->eri_max < 1e100 && T->h_max < 1e100)) return false;
     const DigitBytes B(h);
