@@ -8,7 +8,7 @@
 //   x = 2^(e - 7) sum_i d_i 2^(-8 i),  -128 <= d_i <= 127,  error at most 2^(e - 56).
 // A digit fits bf16's eight-bit significand, and so does d_i 2^(-8 i); a product of digits has at most 15
 // bits, so float32 accumulation in tensor memory of the products of one level i + j is exact while the
-// sum stays below 2^24: always for the alpha-beta products (at most 56 nonzero entries of A, 7 pairs), and
+// sum stays below 2^24: always for the alpha-beta products (at most 60 nonzero entries of A, 7 pairs), and
 // for the same-spin products (at most 501) always in levels 0 and 1, in the others unless hundreds of
 // trailing digits conspire (a random sum is 2^18).  (This is the scheme of Ootomo, Ozaki and Yokota,
 // "DGEMM on integer matrix multiplication unit", 2024, with bf16 digits.)  The 28 products of levels 0 to
@@ -22,11 +22,11 @@
 //   k_max_word       the largest amplitude's exponent
 //   k_phase_digits   digits of X = phi C, as planes [7][Db][lda] (same-spin products, TMA) and as words of
 //                    two digits [Db][4][ldx] (alpha-beta products, gathers)
-//   k_same_digits    G[0] = Ma X and G[1] = X Mb^T (tiles of 128 x 80; the two products side by side)
+//   k_same_digits    G[0] = Ma X and G[1] = X Mb^T (tiles of 128 x 64; the two products side by side)
 //   k_ab_digits      H[b'][j][a], the per-partner-row products of k_abtc.cu
 //   k_comb_digits    sigma, the row's energy and norm
-// 30 qubits (3,003 strings per spin): 39.1 ms in float-float (k_sigma_ab 22.95, k_sigma_same 16.0), 8.9 so
-// (k_same_digits 2.45, k_ab_digits 5.1, the rest 1.4); 24 qubits (495) 668 and 222 us.
+// 30 qubits (3,003 strings per spin): 39.1 ms in float-float (k_sigma_ab 22.95, k_sigma_same 16.0), 8.6 so
+// (k_same_digits 2.45, k_ab_digits 5.1, the rest 1.05); 24 qubits (495) 668 and 216 us.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -158,8 +158,8 @@ __global__ void __launch_bounds__(256) k_ab_table64(const double *__restrict__ e
 __device__ __forceinline__ long long level(uint32_t w, int s) { return (long long)__float2int_rn(__uint_as_float(w) * __uint_as_float((uint32_t)(127 + s) << 23)); }
 
 // The same of a sum below 2^22 in magnitude, without a conversion (their rate is a sixteenth of an
-// addition's): 1.5 2^23 more, it is its own mantissa.  Alpha-beta levels 0 to 3: at most 56 nonzero
-// entries of A within the limits (N = 14, 7 electrons), four pairs, 2^14 a product: 2^21.9.
+// addition's): 1.5 2^23 more, it is its own mantissa.  Alpha-beta levels 0 to 3: at most 60 nonzero
+// entries of A within the limits (N = 15, 10 electrons), four pairs, 2^14 a product: 2^21.9.
 __device__ __forceinline__ int small_level(uint32_t w, int s) {
     return __float_as_int(fmaf(__uint_as_float(w), __uint_as_float((uint32_t)(127 + s) << 23), 12582912.f)) - 0x4B400000;
 }
@@ -253,22 +253,22 @@ __global__ void __launch_bounds__(kDsThreads, 1)
             const uint64_t da = tc_desc(sb + (uint32_t)(s * kDsStage)),
                            db = tc_desc(sb + (uint32_t)(s * kDsStage + kDg * kDsABytes));
             if (elect_one()) {
-            #pragma unroll
-            for (int l = 0; l < kDg; ++l)
                 #pragma unroll
-                for (int i = 0; i <= l; ++i)
+                for (int l = 0; l < kDg; ++l)
                     #pragma unroll
-                    for (int ks = 0; ks < kTcKb / 16; ++ks) {
-                        // the first into an accumulator starts it
-                        const uint32_t acc = (i == 0 && ks == 0) ? (uint32_t)(it > 0) : 1u;
-                        // (start addresses in 16-byte units; the field does not carry: below 256 KB)
-                        asm volatile(
-                            "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
-                            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n\t}\n" ::"r"(tm + (uint32_t)(l * kDsN)),
-                            "l"(da + (uint64_t)((i * kDsABytes + ks * 32) >> 4)),
-                            "l"(db + (uint64_t)(((l - i) * kDsBBytes + ks * 32) >> 4)), "r"(idesc), "r"(acc)
-                            : "memory");
-                    }
+                    for (int i = 0; i <= l; ++i)
+                        #pragma unroll
+                        for (int ks = 0; ks < kTcKb / 16; ++ks) {
+                            // the first into an accumulator starts it
+                            const uint32_t acc = (i == 0 && ks == 0) ? (uint32_t)(it > 0) : 1u;
+                            // (start addresses in 16-byte units; the field does not carry: below 256 KB)
+                            asm volatile(
+                                "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
+                                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n\t}\n" ::"r"(tm + (uint32_t)(l * kDsN)),
+                                "l"(da + (uint64_t)((i * kDsABytes + ks * 32) >> 4)),
+                                "l"(db + (uint64_t)(((l - i) * kDsBBytes + ks * 32) >> 4)), "r"(idesc), "r"(acc)
+                                : "memory");
+                        }
                 ab_commit(smem_u32(&empty[s]));
             }
             __syncwarp();
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(kDsThreads, 1)
 
 constexpr int kDbS = 2;                                      // stages
 constexpr int kDbAcc = 6;                                    // accumulators: levels 0 to 4, and 5 with 6
-constexpr int kHUnit = 43;                                   // H in units of 2^-43: 56 products of 2^14 fit int64
+constexpr int kHUnit = 43;                                   // H in units of 2^-43: 60 products of 2^14 fit int64
 constexpr int kDbACols = kAbKc / 2;                          // tensor-memory columns of a digit of A
 constexpr int kDbAStage = kDg * kDbACols;
 constexpr int kDbABase = kDbAcc * kAbMaxN;                   // first A column, after the accumulators

@@ -1325,6 +1325,15 @@ static sv_status sigma_rows(sv_handle h, DevTables *T, const RowTables &R, const
             SV_CUDA(h, cudaMemcpyAsync(h->hkerr, h->kerr, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
             return SV_OK;
         }
+        // memory that could not all be had is given back
+        dev_free(h, h->ab_H, h->ab_H_bytes);
+        dev_free(h, h->sg_mats, h->sg_mats_bytes);
+        dev_free(h, h->sg_buf, h->sg_buf_bytes);
+        h->ab_H = nullptr;
+        h->sg_mats = h->sg_buf = nullptr;
+        h->ab_H_bytes = h->sg_mats_bytes = h->sg_buf_bytes = 0;
+        h->sg_serial = h->sg_buf_geom = 0;
+        cudaGetLastError();
     }
     const int K = row_chunk(h, R);
     if (use_ff(h, K) && T->eri_ff) {
