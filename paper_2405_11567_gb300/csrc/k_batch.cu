@@ -79,8 +79,8 @@ struct BatchInst {
 // Largest string count per spin for which an instance's sigma runs from per-block
 // dense same-spin matrices and excitation tables (matrices of kBatchSmax^2 values).
 constexpr int kBatchSmax = 512;
-// Dynamic shared memory of the launch at most (its static part stays below 2 KB, the block
-// limit is 227 KB).
+// Dynamic shared memory of the launch at most (its static part, 1,280 bytes, stays below 2 KB; the
+// block limit is 227 KB).
 constexpr size_t kBatchSmemCap = 224 * 1024;
 // Determinants of an instance that may run on a part of a block: the state and the integrals of the
 // largest take less than a quarter of the shared memory.
@@ -1109,38 +1109,43 @@ sv_status capture(sv_batch *b) {
     const BatchArgs<R> a = batch_args<R>(b);
     cudaStream_t st = b->stream;
     cudaError_t e = cudaSuccess;
-    if (b->smem > 48 * 1024) {  // dynamic shared memory above the default limit
-        e = b->threads == 384 ? cudaFuncSetAttribute(k_batch<R, 384>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem)
-                              : cudaFuncSetAttribute(k_batch<R, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return bfail(SV_ERR_CUDA, std::string("batch shared memory: ") + cudaGetErrorString(e));
-        }
+    // The limit on dynamic shared memory, always and to the same value: the default one is 48 KB less the kernel's
+    // static part, and a value of this batch's own would lower that of another thread's batch.
+    e = b->threads == 384 ? cudaFuncSetAttribute(k_batch<R, 384>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmemCap)
+                          : cudaFuncSetAttribute(k_batch<R, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmemCap);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return bfail(SV_ERR_CUDA, std::string("batch shared memory: ") + cudaGetErrorString(e));
     }
     e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return bfail(SV_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e));
-    cudaMemcpyAsync(b->d_theta, b->h_cs, std::max<long long>(b->total_ops, 1) * sizeof(double), cudaMemcpyHostToDevice,
-                    st);
+    // the first of its nodes that is refused ends the capture: a graph without it would return what is in d_out
+    auto add = [&](cudaError_t x) {
+        if (e == cudaSuccess) e = x;
+    };
+    add(cudaMemcpyAsync(b->d_theta, b->h_cs, std::max<long long>(b->total_ops, 1) * sizeof(double), cudaMemcpyHostToDevice, st));
     if (b->total_ops > 0) {
         const long long g = std::min<long long>((b->total_ops + kThreads - 1) / kThreads, (long long)b->sm_count * 4);
         k_batch_sincos<R><<<(int)g, kThreads, 0, st>>>(b->d_theta, (Angle<R> *)b->d_cs, b->total_ops);
+        add(cudaGetLastError());
     }
-    cudaMemsetAsync(b->d_ctrl, 0, 4 * sizeof(int), st);
+    add(cudaMemsetAsync(b->d_ctrl, 0, 4 * sizeof(int), st));
     if (b->threads == 384) k_batch<R, 384><<<b->grid, 384, b->smem, st>>>(a);
     else k_batch<R, 256><<<b->grid, 256, b->smem, st>>>(a);
-    cudaMemcpyAsync(b->h_out, b->d_out, std::max<long long>(b->total_out, 1) * sizeof(double), cudaMemcpyDeviceToHost,
-                    st);
-    cudaMemcpyAsync(b->h_ctrl, b->d_ctrl, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
-    e = cudaStreamEndCapture(st, &b->graph);
+    add(cudaGetLastError());
+    add(cudaMemcpyAsync(b->h_out, b->d_out, std::max<long long>(b->total_out, 1) * sizeof(double), cudaMemcpyDeviceToHost, st));
+    add(cudaMemcpyAsync(b->h_ctrl, b->d_ctrl, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+    cudaGraph_t graph = nullptr;
+    const cudaError_t end = cudaStreamEndCapture(st, &graph);
+    add(end);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, graph, 0);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        return bfail(SV_ERR_CUDA, std::string("capture end: ") + cudaGetErrorString(e));
+        if (graph) cudaGraphDestroy(graph);
+        b->exec = nullptr;
+        return bfail(SV_ERR_CUDA, std::string("batch capture: ") + cudaGetErrorString(e));
     }
-    e = cudaGraphInstantiate(&b->exec, b->graph, 0);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return bfail(SV_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-    }
+    b->graph = graph;
     return SV_OK;
 }
 

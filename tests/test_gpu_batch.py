@@ -128,3 +128,22 @@ def test_batch_generic_path_for_large_string_spaces(dtype):
         Er, gr = _oracle(q)
         assert abs(E[k] - Er) <= tE, (k, E[k], Er)
         assert np.max(np.abs(g[k] - gr)) <= tg, k
+
+
+@pytest.mark.parametrize("dtype,n,na,nb,n_ops", [("c128", 16, 2, 4, 20), ("c128", 18, 2, 2, 103), ("c64", 16, 2, 2, 217)])
+def test_batch_shared_memory_just_below_48_kb(dtype, n, na, nb, n_ops):
+    """Dynamic shared memory of 48,896, 48,448 and 48,336 bytes: below 48 KB, but with the kernel's own
+    static part above the launch limit that holds until it is raised."""
+    p = inputs.make_problem(n, 4, 4, seed=31)
+    pool = inputs.uccsd_pool(n, 4)
+    p["ops"] = np.ascontiguousarray(pool[np.arange(n_ops) % len(pool)])
+    p["theta"] = np.random.default_rng(n_ops).normal(0.0, 0.05, n_ops)
+    p["occ"] = [2 * k for k in range(na)] + [2 * k + 1 for k in range(nb)]
+    p["na"], p["nb"] = na, nb
+    b = sv.Batch([p, p], dtype)
+    E, g = b.energy_grad(np.concatenate([p["theta"], p["theta"]]))
+    Er, gr = _oracle(p)
+    tE, tg = TOL[dtype]
+    for k in range(2):
+        assert abs(E[k] - Er) <= tE and np.max(np.abs(g[k] - gr)) <= tg
+    b.close()
