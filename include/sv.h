@@ -431,17 +431,21 @@ typedef enum {
                                        adjoint vector, checkpoints or the record-scan
                                        expectation); 0 two separate vectors */
     SV_OPT_WAIT_POLLS = 15,         /* polls of each bounded wait before a kernel gives up
-                                       (a poll: in k_ab_tc an mbarrier try-wait that
-                                       suspends the thread for at most 64 ns; in k_same_tc
-                                       a try-wait and a 32 ns sleep; at a grid barrier a
-                                       read of its counter and a 32 ns sleep): the
-                                       tensor-core expectation kernels' mbarrier waits
-                                       (variants 4 and 5: the kernel then waits, bounded,
-                                       for its copies and MMAs in flight, frees its
-                                       tensor memory and returns) and the grid barriers
-                                       of the whole-sweep launches (SV_OPT_SECTOR_SWEEP);
-                                       the call then fails with SV_ERR_CUDA and the
-                                       handle needs sv_prepare_hf / sv_prepare_state.
+                                       (a poll: in k_ab_tc and k_ab_digits an mbarrier
+                                       try-wait that suspends the thread for at most 64 ns;
+                                       in k_same_tc and k_same_digits that or a try-wait
+                                       and a 32 ns sleep; at a grid barrier a read of its
+                                       counter, without a sleep): the tensor-core
+                                       expectation kernels' mbarrier waits
+                                       (variants 4 and 5, the digit products: the kernel
+                                       then waits, bounded, for its copies and MMAs in
+                                       flight, frees its tensor memory and returns) and the
+                                       grid barriers of the whole-sweep launches
+                                       (SV_OPT_SECTOR_SWEEP); the call then fails with
+                                       SV_ERR_CUDA (after sv_apply_ansatz, which returns
+                                       before its kernels have run: the next call that
+                                       returns a value or the state's address does) and
+                                       the handle needs sv_prepare_hf / sv_prepare_state.
                                        1..2^30, default 2^22 */
     SV_OPT_TEST_STALL = 16,         /* failure-detection test hook, 0 (default) off: bit 0
                                        makes k_same_tc's (k_same_digits's) producer issue no

@@ -250,8 +250,15 @@ static sv_status ensure_lam(sv_handle h) {
     return SV_OK;
 }
 
-// The device flag of kernels with bounded waits and its pinned host copy.
+// The device flag of kernels with bounded waits and its pinned host copy.  A core sets its handle's:
+// psi is published from it before its kernels have run, so whoever reads psi looks there.
 static sv_status ensure_kerr(sv_handle h) {
+    if (h->outer) {
+        SV_TRY(ensure_kerr(h->outer));
+        h->kerr = h->outer->kerr;
+        h->hkerr = h->outer->hkerr;
+        return SV_OK;
+    }
     if (!h->kerr) {
         SV_TRY(dev_alloc(h, (void **)&h->kerr, 16, "kernel error flag"));
         SV_CUDA(h, cudaMemsetAsync(h->kerr, 0, sizeof(int), h->stream));
@@ -264,6 +271,34 @@ static sv_status ensure_kerr(sv_handle h) {
         }
         *h->hkerr = 0;
     }
+    return SV_OK;
+}
+
+// Queues the flag's copy to the host, after a kernel with bounded waits.
+static cudaError_t fetch_kernel_flag(sv_handle h) {
+    (h->outer ? h->outer : h)->wait_pending = true;
+    return cudaMemcpyAsync(h->hkerr, h->kerr, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+}
+
+// After a stream synchronisation, in every call that returns what such a kernel may have written: a bounded
+// wait ran out (k_same_tc, k_ab_tc, the digit kernels, k_sweep), in the handle's kernels or its core's.
+static sv_status check_kernel_flag(sv_handle h) {
+    sv_handle o = h->outer ? h->outer : h;
+    o->wait_pending = false;
+    if (!o->hkerr || !*o->hkerr) return SV_OK;
+    *o->hkerr = 0;
+    cudaMemsetAsync(o->kerr, 0, sizeof(int), o->stream);
+    h->failed = o->failed = true;
+    return fail(h, SV_ERR_CUDA, "a bounded wait ran out (tensor-core products or a sweep's grid barrier)");
+}
+
+// Where the state is about to be written anew: what an earlier kernel that no call has looked at did to it
+// does not matter, so its flag goes, in stream order (that kernel may still be running).
+static sv_status clear_kernel_flag(sv_handle h) {
+    if (!h->wait_pending || !h->kerr || !h->hkerr) return SV_OK;
+    SV_CUDA(h, cudaMemsetAsync(h->kerr, 0, sizeof(int), h->stream));
+    SV_CUDA(h, cudaMemcpyAsync(h->hkerr, h->kerr, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    h->wait_pending = false;
     return SV_OK;
 }
 
@@ -896,7 +931,7 @@ static bool sweep_once(sv_handle h, const SweepShape &s, bool adjoint, void *psi
         return false;
     }
     h->launches++;
-    if (s.form == 2) cudaMemcpyAsync(h->hkerr, h->kerr, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+    if (s.form == 2 && fetch_kernel_flag(h) != cudaSuccess) cudaGetLastError();
     return true;
 }
 
@@ -1131,17 +1166,6 @@ static sv_status ensure_same_gemm(sv_handle h, DevTables *T, const RowTables &R,
     return SV_OK;
 }
 
-// After a stream synchronisation: a kernel whose bounded wait ran out (k_same_tc, k_ab_tc).
-static sv_status check_kernel_flag(sv_handle h) {
-    if (h->hkerr && *h->hkerr) {
-        *h->hkerr = 0;
-        if (h->kerr) cudaMemsetAsync(h->kerr, 0, sizeof(int), h->stream);
-        h->failed = true;
-        return fail(h, SV_ERR_CUDA, "a bounded wait ran out (tensor-core products or a sweep's grid barrier)");
-    }
-    return SV_OK;
-}
-
 // The string-row expectation (sigma into lam at storage addresses, or into lamc in
 // compact form), with or without the same-spin products; counts the launches.
 // Whether the expectation takes the float-float split form (variant 6): float64 states
@@ -1322,7 +1346,7 @@ static sv_status sigma_rows(sv_handle h, DevTables *T, const RowTables &R, const
                                                 h->sm_count, h->stream));
             h->launches += 6;
             if (g.ev) h->tc_timed = 3;
-            SV_CUDA(h, cudaMemcpyAsync(h->hkerr, h->kerr, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+            SV_CUDA(h, fetch_kernel_flag(h));
             return SV_OK;
         }
         // memory that could not all be had is given back
@@ -1362,7 +1386,7 @@ static sv_status sigma_rows(sv_handle h, DevTables *T, const RowTables &R, const
     h->launches += sg ? 5 : (K ? 2 : 1);
     if (sg && g.ev) h->tc_timed = 1 | (g.abtc ? 2 : 0);
     if (sg)
-        SV_CUDA(h, cudaMemcpyAsync(h->hkerr, h->kerr, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+        SV_CUDA(h, fetch_kernel_flag(h));
     return SV_OK;
 }
 
@@ -1902,8 +1926,10 @@ static void destroy_handle(sv_handle h) {
     dev_free(h, h->sg_mats, h->sg_mats_bytes);
     dev_free(h, h->sg_buf, h->sg_buf_bytes);
     dev_free(h, h->ab_H, h->ab_H_bytes);
-    dev_free(h, h->kerr, 16);
-    if (h->hkerr) cudaFreeHost(h->hkerr);
+    if (!h->outer) {
+        dev_free(h, h->kerr, 16);
+        if (h->hkerr) cudaFreeHost(h->hkerr);
+    }
     dev_free(h, h->lists.buf, h->lists.bytes);
     dev_free(h, h->pool_lists.buf, h->pool_lists.bytes);
     dev_free(h, h->groups.buf, h->groups.bytes);
@@ -1956,11 +1982,12 @@ sv_status sv_destroy(sv_handle h) {
 
 
 // A new reference: nothing that the core holds is current.
-static void reference_changed(sv_handle h) {
+static sv_status reference_changed(sv_handle h) {
     h->core_cur = 0;
     h->core_ref = false;
     h->psi_clean = false;
     if (h->core) h->core->failed = false;
+    return clear_kernel_flag(h);
 }
 
 // The determinant reference in a whole vector that is zero outside the reference's sector (an earlier
@@ -2006,7 +2033,7 @@ sv_status sv_prepare_hf(sv_handle h, const int32_t *occ, int n_occ) {
     h->ref_real = true;
     h->na = na;
     h->nb = nb;
-    reference_changed(h);
+    SV_TRY(reference_changed(h));
     SV_TRY(in_sector ? prepare_in_sector(h) : prepare_reference(h));
     h->prepared = true;
     h->at_ref = true;
@@ -2049,7 +2076,7 @@ sv_status sv_prepare_state(sv_handle h, const void *amplitudes_host, int n_alpha
     h->failed = false;
     h->prepared = false;
     h->at_ref = false;
-    reference_changed(h);
+    SV_TRY(reference_changed(h));
     if (!h->ref_vec) SV_TRY(dev_alloc(h, &h->ref_vec, vec_bytes(h), "reference copy"));
     if (h->storage == 1) {
         // host order is the dense qubit-order vector: keep its sector entries in C[rank(b)][rank(a)] order
@@ -2097,6 +2124,7 @@ sv_status sv_get_state(sv_handle h, void *amplitudes_host) {
         std::vector<uint8_t> comp(vec_bytes(h));
         SV_CUDA(h, cudaMemcpyAsync(comp.data(), h->psi, comp.size(), cudaMemcpyDeviceToHost, h->stream));
         SV_CUDA(h, cudaStreamSynchronize(h->stream));
+        SV_TRY(check_kernel_flag(h));
         memset(amplitudes_host, 0, (size_t)h->dim * h->amp_bytes);
         const int N = h->n / 2;
         for (int Ib = 0; Ib < h->Db; ++Ib)
@@ -2123,7 +2151,7 @@ sv_status sv_get_state(sv_handle h, void *amplitudes_host) {
     }
     SV_CUDA(h, cudaMemcpyAsync(amplitudes_host, src, vec_bytes(h), cudaMemcpyDeviceToHost, h->stream));
     SV_CUDA(h, cudaStreamSynchronize(h->stream));
-    return SV_OK;
+    return check_kernel_flag(h);
 }
 
 sv_status sv_get_amplitudes(sv_handle h, const uint64_t *basis, int count, void *amplitudes_host) {
@@ -2151,11 +2179,16 @@ sv_status sv_get_amplitudes(sv_handle h, const uint64_t *basis, int count, void 
     SV_CUDA(h, cudaMemcpyAsync(amplitudes_host, d_out, (size_t)count * h->amp_bytes, cudaMemcpyDeviceToHost,
                                h->stream));
     SV_CUDA(h, cudaStreamSynchronize(h->stream));
-    return SV_OK;
+    return check_kernel_flag(h);
 }
 
 sv_status sv_state_device_ptr(sv_handle h, void **psi_dev) {
     if (!h || !psi_dev) return fail(h, SV_ERR_ARG, "NULL argument");
+    if (h->wait_pending) {  // nothing will tell a reader on the device that a sweep gave up
+        DeviceGuard g(h->device);
+        SV_CUDA(h, cudaStreamSynchronize(h->stream));
+        SV_TRY(check_kernel_flag(h));
+    }
     h->at_ref = false;  // the caller may write the state through the pointer
     h->exposed = true;
     *psi_dev = h->psi;
@@ -2434,6 +2467,7 @@ sv_status sv_energy_grad(sv_handle h, sv_ham_handle ham, const sv_excitation *op
     SV_TRY(build_ops(h, ops, n_ops, theta, d, core ? kIdentity : nullptr));  // validates in any layout
     h->at_ref = false;
     DeviceGuard g(h->device);
+    SV_TRY(clear_kernel_flag(h));  // psi is written from the reference
     int np[32];
     const bool lay = h->layout_auto && n_ops > 0 && h->storage == 0;
     if (lay) layout_from_ops(h->n, ops, n_ops, np);
@@ -2596,6 +2630,7 @@ static sv_status rdm1_run(sv_handle h, double *re_out, double *im_out) {
                                    h->stream));
         SV_CUDA(h, cudaStreamSynchronize(h->stream));
     }
+    SV_TRY(check_kernel_flag(h));
     if (h->profile) h->phase_ms[5] = elapsed(h, 0, 7);
     const int n = h->n, N = n / 2;
     const double *o = h->hpinned;
@@ -2653,6 +2688,10 @@ sv_status sv_autotune(sv_handle h, sv_ham_handle ham, const sv_excitation *ops, 
     const sv_status st = r == h ? autotune_impl(h, ham, d, e0, e1) : core_status(h, autotune_impl(r, ham, d, e0, e1));
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    if (st == SV_OK) {
+        SV_CUDA(h, cudaStreamSynchronize(h->stream));
+        SV_TRY(check_kernel_flag(h));
+    }
     if (r != h && st == SV_OK) {  // the choices are the handle's
         h->expect_variant = r->expect_variant;
         h->ab_chunk = r->ab_chunk / (r->dtype == h->dtype ? 1 : 2);

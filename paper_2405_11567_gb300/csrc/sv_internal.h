@@ -343,7 +343,8 @@ struct sv_ctx {
     // expectation variant 6: the compact amplitudes and sigma as float-float matrices
     void *ffbuf = nullptr;
     size_t ffbuf_bytes = 0;
-    int *hkerr = nullptr;      // its pinned host copy, checked after stream synchronisations
+    int *hkerr = nullptr;      // its pinned host copy, checked after stream synchronisations (a core: its handle's two)
+    bool wait_pending = false; // a kernel with bounded waits runs whose flag no synchronising call has looked at
     // same-spin products (expectation variant 4): matrices for one table set and sector,
     // and the phased-psi / product planes
     void *sg_mats = nullptr;

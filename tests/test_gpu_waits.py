@@ -1,5 +1,5 @@
 """Failure detection without a GPU fault: the bounded waits of the tensor-core
-expectation kernels (k_same_tc, k_ab_tc).
+expectation kernels (k_same_tc, k_ab_tc) and of a sweep's grid barriers.
 
 A test hook (SV_OPT_TEST_STALL) makes a kernel's producer issue nothing -- no copy,
 no tensor-memory store, no MMA -- so its consumers' first mbarrier waits run out
@@ -72,3 +72,70 @@ def test_wait_options_validated():
             st.set_option(opt, bad)
         assert e.value.status == 1
     assert st.option(sv.SV_OPT_WAIT_POLLS) == 1 << 22 and st.option(sv.SV_OPT_TEST_STALL) == 0
+
+
+@pytest.mark.parametrize("storage,dtype", [("dense", "c128"), ("dense", "r32"), ("sector", "c64"), ("sector", "r64")])
+@pytest.mark.parametrize("reader", ["state", "amplitudes", "rdm1", "energy", "energy_full_vector", "pool", "address"])
+def test_a_sweep_that_gave_up_is_reported_by_the_next_reader(storage, dtype, reader):
+    """One poll per barrier wait: sv_apply_ansatz's sweep stops in the middle, after the call has returned.
+    Whatever reads the state next reports it; a state prepared again, or an evaluation from the reference,
+    does not see the old flag."""
+    p = inputs.config_problem(2)
+    n = p["n_qubits"]
+    sec = oracle.Sector(n, p["na"], p["nb"])
+    psi0 = A.hf_state(sec, p["occ"])
+    Eref, gref = A.energy_grad(sec, p["h"], p["eri"], p["e_nuc"], p["ops"], p["theta"], psi0)
+    want = A.apply_ansatz(sec, p["ops"], p["theta"], psi0)
+    at = sec.dets.astype(np.uint64)
+    ham = sv.Hamiltonian(p["h"], p["eri"], p["e_nuc"])
+    st = sv.StateVector(n, dtype, sector=(p["na"], p["nb"]) if storage == "sector" else None)
+
+    def read():
+        if reader == "state":
+            return st.state()
+        if reader == "amplitudes":
+            return st.amplitudes(at[:9])
+        if reader == "rdm1":
+            return st.rdm1()
+        if reader == "pool":
+            return st.pool_gradients(ham, p["ops"][:5])
+        if reader == "address":
+            return sv.sv_state_device_ptr(st.handle)
+        return st.energy(ham)
+
+    def fail():
+        st.set_option(sv.SV_OPT_WAIT_POLLS, 1)
+        st.prepare_hf(p["occ"])
+        st.apply_ansatz(p["ops"], p["theta"])
+        st.set_option(sv.SV_OPT_WAIT_POLLS, 1 << 22)
+
+    tE, tg, ta = (1e-10, 1e-9, 1e-12) if dtype in ("c128", "r64") else (1e-5, 1e-5, 2e-6)
+
+    def good():
+        E, g = st.energy_grad(ham, p["ops"], p["theta"])
+        assert abs(E - Eref) <= tE and np.max(np.abs(g - gref)) <= tg
+        assert np.max(np.abs(st.amplitudes(at) - want)) <= ta
+
+    fail()
+    if reader == "energy_full_vector":
+        st.set_option(sv.SV_OPT_FULL_VECTOR, 1)
+    with pytest.raises(sv.SvError) as e:
+        read()
+    assert e.value.status == 3 and "bounded wait" in str(e.value)
+    with pytest.raises(sv.SvError) as e2:
+        st.state()
+    assert e2.value.status == 5
+    st.set_option(sv.SV_OPT_FULL_VECTOR, 0)
+    st.prepare_hf(p["occ"])
+    read()
+    good()
+    fail()
+    st.prepare_hf(p["occ"])              # over a flag that nobody has read
+    read()
+    st.apply_ansatz(p["ops"], p["theta"])
+    assert reader == "address" or abs(st.energy(ham) - Eref) <= tE
+    assert np.max(np.abs(st.amplitudes(at) - want)) <= ta
+    fail()
+    good()                               # from the reference
+    st.close()
+    ham.close()
