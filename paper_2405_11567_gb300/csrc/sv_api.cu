@@ -1016,7 +1016,8 @@ static bool dense_couplings(sv_handle h) {
 // products do at most 20 times the multiplies of the sparse sums.  Measured, variants
 // 3 / 5 in us (real float32): 14,400 determinants 62 / 65, 63,504 158 / 86, 108,900
 // 248 / 115, 245,025 435 / 149, 627,264 1223 / 299 (complex64: 44,100 144 / 89, 245,025
-// 529 / 173); variant 4 alone 73, 128, 179, 361, 689.
+// 529 / 173); variant 4 alone 73, 128, 179, 361, 689.  Variant 3 where its memory cannot be had
+// (sigma_rows).
 static bool use_same_gemm(sv_handle h, int K) {
     if (!single_prec(h->dtype) || K == 0 || h->Da > 4096 || h->Db > 4096) return false;
     if (h->expect_variant == 4 || h->expect_variant == 5) return true;
@@ -1337,6 +1338,18 @@ static sv_status ensure_digits(sv_handle h, DevTables *T, const RowTables &R, Sa
     return SV_OK;
 }
 
+// Gives back what the product forms of the expectation hold (all of it is built anew on demand).
+static void drop_products(sv_handle h) {
+    dev_free(h, h->ab_H, h->ab_H_bytes);
+    dev_free(h, h->sg_mats, h->sg_mats_bytes);
+    dev_free(h, h->sg_buf, h->sg_buf_bytes);
+    h->ab_H = nullptr;
+    h->sg_mats = h->sg_buf = nullptr;
+    h->ab_H_bytes = h->sg_mats_bytes = h->sg_buf_bytes = 0;
+    h->sg_serial = h->sg_buf_geom = 0;
+    cudaGetLastError();
+}
+
 static sv_status sigma_rows(sv_handle h, DevTables *T, const RowTables &R, const void *C, void *lam, void *lamc,
                             double e_shift) {
     if (use_digits(h, T)) {
@@ -1349,15 +1362,7 @@ static sv_status sigma_rows(sv_handle h, DevTables *T, const RowTables &R, const
             SV_CUDA(h, fetch_kernel_flag(h));
             return SV_OK;
         }
-        // memory that could not all be had is given back
-        dev_free(h, h->ab_H, h->ab_H_bytes);
-        dev_free(h, h->sg_mats, h->sg_mats_bytes);
-        dev_free(h, h->sg_buf, h->sg_buf_bytes);
-        h->ab_H = nullptr;
-        h->sg_mats = h->sg_buf = nullptr;
-        h->ab_H_bytes = h->sg_mats_bytes = h->sg_buf_bytes = 0;
-        h->sg_serial = h->sg_buf_geom = 0;
-        cudaGetLastError();
+        drop_products(h);  // memory that could not all be had is given back
     }
     const int K = row_chunk(h, R);
     if (use_ff(h, K) && T->eri_ff) {
@@ -1379,8 +1384,16 @@ static sv_status sigma_rows(sv_handle h, DevTables *T, const RowTables &R, const
         }
     }
     SameGemm g;
-    const bool sg = use_same_gemm(h, K);
-    if (sg) SV_TRY(ensure_same_gemm(h, T, R, &g));
+    bool sg = use_same_gemm(h, K);
+    if (sg) {
+        const sv_status st = ensure_same_gemm(h, T, R, &g);
+        if (st == SV_ERR_OOM && h->expect_variant == 0) {  // the automatic choice: the sparse sums, which need none of it
+            drop_products(h);
+            sg = false;
+        } else if (st != SV_OK) {
+            return st;
+        }
+    }
     SV_CUDA(h, launch_sigma_rows(C, lam, lamc, h->dtype, h->n, R, T->hdiag, T->Jp, e_shift, h->partials, K,
                                  h->stream, sg ? &g : nullptr, h->sm_count));
     h->launches += sg ? 5 : (K ? 2 : 1);

@@ -1,0 +1,78 @@
+"""Device memory that runs short (SV_OPT_MAX_BYTES): whatever a handle keeps to be faster -- product planes,
+sweep steps -- gives way, so a cap under which the plainest forms run is enough for every default call,
+with the same results."""
+import numpy as np
+import pytest
+
+from paper_2405_11567_gb300 import inputs, sv
+
+pytestmark = pytest.mark.gpu
+
+# energy, gradient, 1-RDM: the parity suite's tolerances of each precision
+TOL = {"c128": (1e-10, 1e-9, 1e-12), "r64": (1e-10, 1e-9, 1e-12), "c64": (1e-5, 1e-5, 2e-6), "r32": (1e-5, 1e-5, 2e-6)}
+PLAIN = {sv.SV_OPT_EXPECT_VARIANT: 3, sv.SV_OPT_SECTOR_SWEEP: 0}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    from paper_2405_11567_gb300 import build
+    build.build()
+    sv.lib()
+
+
+def _problem(n, ne):
+    p = inputs.make_problem(n, ne, 60, seed=n)
+    return p, sv.Hamiltonian(p["h"], p["eri"], p["e_nuc"])
+
+
+def _run(n, ne, dtype, cap, options, calls):
+    """The results of calls(state) on a capped handle, None where one was refused for memory."""
+    st = None
+    try:
+        st = sv.StateVector(n, dtype, sector=(ne // 2, ne // 2))
+        st.set_option(sv.SV_OPT_MAX_BYTES, cap)
+        for opt, value in options.items():
+            st.set_option(opt, value)
+        return calls(st)
+    except sv.SvError as e:
+        assert e.status == 2, e
+        return None
+    finally:
+        if st is not None:
+            st.close()
+
+
+def _least_cap(run):
+    """The least cap (to 2 KB) under which run(cap) is accepted."""
+    lo, hi = 0, 256 << 20
+    assert run(hi) is not None
+    while hi - lo > 2048:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if run(mid) is not None else (mid, hi)
+    return hi
+
+
+def _check(got, want, tol, why):
+    assert got is not None, why
+    for (x, t), y in zip(got, want):
+        assert np.max(np.abs(np.asarray(x) - np.asarray(y[0]))) <= tol[t], why
+
+
+@pytest.mark.parametrize("dtype", ["r32", "c64"])
+@pytest.mark.parametrize("n,ne", [(20, 10), (22, 8)])
+def test_products_that_do_not_fit_leave_the_sparse_sums(n, ne, dtype):
+    """63,504 and 108,900 determinants: the automatic choice is the tensor-core products."""
+    p, ham = _problem(n, ne)
+
+    def calls(st):
+        st.prepare_hf(p["occ"])
+        st.apply_ansatz(p["ops"], p["theta"])
+        return [(st.energy(ham), 0)]
+
+    plain = lambda cap: _run(n, ne, dtype, cap, PLAIN, calls)
+    least = _least_cap(plain)
+    want = plain(0)
+    for factor in (1.0, 1.1, 1.5, 2.5, 6.0, 20.0):
+        got = _run(n, ne, dtype, int(least * factor), {sv.SV_OPT_SECTOR_SWEEP: 0}, calls)
+        _check(got, want, TOL[dtype], factor)
+    ham.close()
