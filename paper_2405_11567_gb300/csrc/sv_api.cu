@@ -191,14 +191,23 @@ struct DeviceGuard {
 
 // ---------------------------------------------------------------- buffers
 
-static sv_status dev_alloc(sv_handle h, void **p, size_t bytes, const char *what) {
+static bool give_back(sv_handle h);
+
+// `optional`: for what a call can do without: nothing that the handle keeps gives way to it.
+static sv_status dev_alloc(sv_handle h, void **p, size_t bytes, const char *what, bool optional = false) {
     *p = nullptr;
+    while (!optional && h->max_bytes > 0 && h->bytes_owned + bytes > (uint64_t)h->max_bytes && give_back(h)) {
+    }
     if (h->max_bytes > 0 && h->bytes_owned + bytes > (uint64_t)h->max_bytes)
         return fail(h, SV_ERR_OOM, std::string("device byte cap reached allocating ") + what);
     cudaError_t e = cudaMalloc(p, bytes);
-    if (e != cudaSuccess) {
+    while (e != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
+        if (e == cudaErrorMemoryAllocation && !optional && give_back(h)) {
+            e = cudaMalloc(p, bytes);
+            continue;
+        }
         return fail(h, SV_ERR_OOM, std::string("cudaMalloc failed for ") + what + ": " + cudaGetErrorString(e));
     }
     h->bytes_owned += bytes;
@@ -236,7 +245,7 @@ static sv_status ensure_lam(sv_handle h) {
     if (h->lam) return SV_OK;
     if (h->storage == 0 && !h->saved) {
         void *p = nullptr;
-        if (dev_alloc(h, &p, 2 * vec_bytes(h), "adjoint vector and working copy") == SV_OK) {
+        if (dev_alloc(h, &p, 2 * vec_bytes(h), "adjoint vector and working copy", true) == SV_OK) {
             h->lam = p;
             h->own_lam = true;
             h->lam_pair = true;
@@ -873,6 +882,26 @@ static sv_status ensure_groups(sv_handle h, const std::vector<OpDesc> &ops) {
     return SV_OK;
 }
 
+// Gives back what a whole sweep keeps (built anew on demand; sweep_once launches nothing without it).
+static void drop_sweep(sv_handle h) {
+    dev_free(h, h->groups.buf, h->groups.bytes);
+    dev_free(h, h->sweep_buf, h->sweep_bytes);
+    h->groups = SweepGroups();
+    h->sweep_buf = nullptr;
+    h->sweep_bytes = 0;
+}
+
+// Memory that is short: what the handle, its core or the handle that a core serves keeps only to be faster
+// gives way to an allocation that the call needs (cudaFree waits for the kernels that use it).  False: none left.
+static bool give_back(sv_handle h) {
+    for (sv_handle o : {h, (sv_handle)h->core, (sv_handle)h->outer})
+        if (o && o->groups.buf) {
+            drop_sweep(o);
+            return true;
+        }
+    return false;
+}
+
 // Form and geometry of a whole sweep over h->groups (k_sweep): -1 where none runs.
 struct SweepShape {
     int form = -1, blocks = 0, threads = 0;
@@ -917,7 +946,7 @@ static SweepShape sweep_shape(sv_handle h, bool adjoint, size_t n_ops) {
 // the gradient sums [L][warps] in h->partials); false (nothing launched) where it is refused:
 // the caller then launches per op.
 static bool sweep_once(sv_handle h, const SweepShape &s, bool adjoint, void *psi, const void *lam, void *work, long long init) {
-    if (s.form < 0 || !h->sweep_buf) return false;
+    if (s.form < 0 || !h->groups.buf || !h->sweep_buf) return false;
     if (s.form == 2 && (!h->kerr || cudaMemsetAsync(h->sweep_buf, 0, sizeof(unsigned int), h->stream) != cudaSuccess)) {
         cudaGetLastError();
         return false;
@@ -935,15 +964,31 @@ static bool sweep_once(sv_handle h, const SweepShape &s, bool adjoint, void *psi
     return true;
 }
 
+// The steps, angles and flag of a whole sweep over ops and its form; form -1 where the memory for them
+// cannot be had (a list entry takes twice the bytes of the per-operator lists'): one launch per op then.
+static sv_status prepare_sweep(sv_handle h, bool adjoint, const std::vector<OpDesc> &ops, SweepShape *s) {
+    *s = SweepShape();
+    sv_status st = ensure_groups(h, ops);
+    if (st == SV_OK) st = upload_sweep_angles(h, ops);
+    if (st == SV_OK) {
+        *s = sweep_shape(h, adjoint, ops.size());
+        if (s->form == 2) st = ensure_kerr(h);
+    }
+    if (st != SV_OK && st != SV_ERR_OOM) return st;
+    if (st != SV_OK || !h->groups.buf) {
+        drop_sweep(h);
+        *s = SweepShape();
+    }
+    return SV_OK;
+}
+
 // U_L ... U_1 on psi; from_ref: on the handle's reference, written first.
 static sv_status forward(sv_handle h, const std::vector<OpDesc> &ops, bool checkpoints, bool from_ref) {
     const int64_t C = h->ckpt_interval;
     if (h->storage == 1 && !ops.empty() && h->sweep_mode && !(checkpoints && C > 0 && (size_t)C < ops.size())) {
         // one launch for the whole sweep (checkpoint copies would be due in its middle)
-        SV_TRY(ensure_groups(h, ops));
-        SV_TRY(upload_sweep_angles(h, ops));
-        const SweepShape s = sweep_shape(h, false, ops.size());
-        if (s.form == 2) SV_TRY(ensure_kerr(h));
+        SweepShape s;
+        SV_TRY(prepare_sweep(h, false, ops, &s));
         const bool det = from_ref && h->ref_kind == 1;  // written by the sweep itself
         if (from_ref && !det) SV_TRY(prepare_reference(h));
         if (sweep_once(h, s, false, h->psi, nullptr, nullptr, det ? (long long)compact_index(h, h->ref_det) : -1))
@@ -982,7 +1027,7 @@ static void plan_checkpoints(sv_handle h, size_t L) {
     }
     while (h->ckpt.size() < want) {
         void *p = nullptr;
-        if (dev_alloc(h, &p, vec_bytes(h), "checkpoint") != SV_OK) {
+        if (dev_alloc(h, &p, vec_bytes(h), "checkpoint", true) != SV_OK) {
             cudaGetLastError();
             break;  // fewer checkpoints: the reverse sweep uncomputes instead
         }
@@ -1720,7 +1765,7 @@ static sv_status autotune_impl(sv_handle h, sv_ham_handle ham, const std::vector
     if (!d.empty()) {
         if (!h->saved) {  // as in sv_energy_grad: optional under the byte cap
             void *p = nullptr;
-            if (dev_alloc(h, &p, vec_bytes(h), "saved final state") == SV_OK) h->saved = p;
+            if (dev_alloc(h, &p, vec_bytes(h), "saved final state", true) == SV_OK) h->saved = p;
             else cudaGetLastError();
         }
         const bool adj = h->saved != nullptr;  // without it only the rotation is timed
@@ -2326,7 +2371,7 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
     // state buffers first (so the byte cap drops checkpoints, not required scratch)
     if (!h->saved) {
         void *p = nullptr;
-        if (dev_alloc(h, &p, vec_bytes(h), "saved final state") == SV_OK) h->saved = p;
+        if (dev_alloc(h, &p, vec_bytes(h), "saved final state", true) == SV_OK) h->saved = p;
         else cudaGetLastError();
     }
     const bool sect = h->storage == 1;
@@ -2362,16 +2407,14 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
     bool inter = sect && C <= 0 && L > 0;
     SweepShape shape;
     if (inter && h->sweep_mode) {  // a whole sweep: it interleaves psi and lambda itself
-        SV_TRY(ensure_groups(h, d));
-        SV_TRY(upload_sweep_angles(h, d));
-        shape = sweep_shape(h, true, L);
-        if (shape.form == 2) SV_TRY(ensure_kerr(h));
+        SV_TRY(prepare_sweep(h, true, d, &shape));
         if (shape.form >= 0 &&
             ensure_partials(h, std::max<size_t>((size_t)shape.warps() * L, std::max<size_t>((size_t)G * L, need))) != SV_OK) {
             cudaGetLastError();
             shape.form = -1;
             SV_TRY(ensure_partials(h, std::max<size_t>((size_t)G * L, need)));
         }
+        if (!h->groups.buf) shape.form = -1;
     }
     if (inter && shape.form != 0 && ensure_clbuf(h) != SV_OK) {
         cudaGetLastError();
@@ -2407,8 +2450,15 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
     SV_TRY(mark(h, 4, "sv_energy_grad: reverse sweep"));
     // reverse sweep: sector storage in one launch where it can, else one launch per op (gradient partials [L][G])
     const bool swept = inter && shape.form >= 0 && sweep_once(h, shape, true, h->psi, h->lam, h->CLbuf, -1);
+    if (inter && !swept && ensure_clbuf(h) != SV_OK) {  // (the block form holds none; its launch was refused)
+        cudaGetLastError();
+        inter = false;
+        if (h->saved) {
+            wpsi = h->saved;
+            SV_CUDA(h, cudaMemcpyAsync(wpsi, h->psi, vec_bytes(h), cudaMemcpyDeviceToDevice, h->stream));
+        }
+    }
     if (inter && !swept) {
-        SV_TRY(ensure_clbuf(h));
         SV_TRY(ensure_op_lists(h, d, h->lists));
         SV_CUDA(h, launch_interleave(h->psi, h->lam, h->dtype, h->CLbuf, (size_t)h->Da * h->Db, h->sm_count,
                                      h->stream));

@@ -76,3 +76,29 @@ def test_products_that_do_not_fit_leave_the_sparse_sums(n, ne, dtype):
         got = _run(n, ne, dtype, int(least * factor), {sv.SV_OPT_SECTOR_SWEEP: 0}, calls)
         _check(got, want, TOL[dtype], factor)
     ham.close()
+
+
+@pytest.mark.parametrize("dtype", ["r32", "r64", "c128"])
+@pytest.mark.parametrize("call", ["apply", "energy_grad"])
+def test_sweep_steps_that_do_not_fit_leave_one_launch_per_operator(call, dtype):
+    """A list of 600 operators over few determinants: the lists weigh more than the vectors."""
+    p, ham = _problem(16, 4)
+    pool = inputs.uccsd_pool(16, 4)
+    ops = np.ascontiguousarray(pool[np.arange(600) % len(pool)])
+    theta = np.random.default_rng(6).normal(0.0, 0.05, len(ops))
+
+    def calls(st):
+        st.prepare_hf(p["occ"])
+        if call == "apply":
+            st.apply_ansatz(ops, theta)
+            return [(st.state(), 2)]
+        E, g = st.energy_grad(ham, ops, theta)
+        return [(E, 0), (g, 1), (st.state(), 2)]
+
+    plain = lambda cap: _run(16, 4, dtype, cap, PLAIN, calls)
+    least = _least_cap(plain)
+    want = plain(0)
+    for factor in (1.0, 1.02, 1.1, 1.3, 1.6, 2.0, 3.0):
+        got = _run(16, 4, dtype, int(least * factor), {sv.SV_OPT_EXPECT_VARIANT: 3}, calls)
+        _check(got, want, TOL[dtype], factor)
+    ham.close()
