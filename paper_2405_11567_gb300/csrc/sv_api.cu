@@ -886,17 +886,46 @@ static sv_status ensure_groups(sv_handle h, const std::vector<OpDesc> &ops) {
 static void drop_sweep(sv_handle h) {
     dev_free(h, h->groups.buf, h->groups.bytes);
     dev_free(h, h->sweep_buf, h->sweep_bytes);
+    dev_free(h, h->sweep_part, h->sweep_part_bytes);
     h->groups = SweepGroups();
     h->sweep_buf = nullptr;
-    h->sweep_bytes = 0;
+    h->sweep_part = nullptr;
+    h->sweep_bytes = h->sweep_part_bytes = 0;
+}
+
+// Gives back what the product forms of the expectation hold (all of it is built anew on demand).
+static void drop_products(sv_handle h) {
+    dev_free(h, h->ab_H, h->ab_H_bytes);
+    dev_free(h, h->sg_mats, h->sg_mats_bytes);
+    dev_free(h, h->sg_buf, h->sg_buf_bytes);
+    h->ab_H = nullptr;
+    h->sg_mats = h->sg_buf = nullptr;
+    h->ab_H_bytes = h->sg_mats_bytes = h->sg_buf_bytes = 0;
+    h->sg_serial = h->sg_buf_geom = 0;
+    cudaGetLastError();
 }
 
 // Memory that is short: what the handle, its core or the handle that a core serves keeps only to be faster
 // gives way to an allocation that the call needs (cudaFree waits for the kernels that use it).  False: none left.
 static bool give_back(sv_handle h) {
-    for (sv_handle o : {h, (sv_handle)h->core, (sv_handle)h->outer})
+    const sv_handle all[] = {h, h->core, h->outer};
+    for (sv_handle o : all)
+        if (o && !o->products_held && (o->ab_H || o->sg_mats || o->sg_buf)) {
+            drop_products(o);
+            return true;
+        }
+    // an automatic choice's products do without them before the sweeps do
+    if (h->products_held && h->expect_variant == 0) return false;
+    for (sv_handle o : all)
         if (o && o->groups.buf) {
             drop_sweep(o);
+            return true;
+        }
+    for (sv_handle o : all)
+        if (o && o->ffbuf) {
+            dev_free(o, o->ffbuf, o->ffbuf_bytes);
+            o->ffbuf = nullptr;
+            o->ffbuf_bytes = 0;
             return true;
         }
     return false;
@@ -943,10 +972,10 @@ static SweepShape sweep_shape(sv_handle h, bool adjoint, size_t n_ops) {
 }
 
 // One launch for a whole sector sweep (forward on psi, or reverse from psi and lambda with
-// the gradient sums [L][warps] in h->partials); false (nothing launched) where it is refused:
+// the gradient sums [L][warps] in h->sweep_part); false (nothing launched) where it is refused:
 // the caller then launches per op.
 static bool sweep_once(sv_handle h, const SweepShape &s, bool adjoint, void *psi, const void *lam, void *work, long long init) {
-    if (s.form < 0 || !h->groups.buf || !h->sweep_buf) return false;
+    if (s.form < 0 || !h->groups.buf || !h->sweep_buf || (adjoint && !h->sweep_part)) return false;
     if (s.form == 2 && (!h->kerr || cudaMemsetAsync(h->sweep_buf, 0, sizeof(unsigned int), h->stream) != cudaSuccess)) {
         cudaGetLastError();
         return false;
@@ -954,7 +983,7 @@ static bool sweep_once(sv_handle h, const SweepShape &s, bool adjoint, void *psi
     const cudaError_t e =
         launch_sweep(psi, lam, h->dtype, adjoint, s.form, s.blocks, s.threads, s.words, h->groups.buf, h->groups.dgroups,
                      h->groups.n_groups, (const uint8_t *)h->sweep_buf + 256, h->groups.n_ops, h->Da, h->Db, init, work,
-                     (unsigned int *)h->sweep_buf, h->kerr, (uint32_t)h->wait_polls, h->partials, h->stream);
+                     (unsigned int *)h->sweep_buf, h->kerr, (uint32_t)h->wait_polls, h->sweep_part, h->stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return false;
@@ -964,7 +993,19 @@ static bool sweep_once(sv_handle h, const SweepShape &s, bool adjoint, void *psi
     return true;
 }
 
-// The steps, angles and flag of a whole sweep over ops and its form; form -1 where the memory for them
+// A reverse sweep's gradient sums [operators][warps].
+static sv_status ensure_sweep_part(sv_handle h, size_t doubles) {
+    const size_t need = doubles * sizeof(double);
+    if (h->sweep_part_bytes >= need) return SV_OK;
+    dev_free(h, h->sweep_part, h->sweep_part_bytes);
+    h->sweep_part = nullptr;
+    h->sweep_part_bytes = 0;
+    SV_TRY(dev_alloc(h, (void **)&h->sweep_part, need, "sweep gradient sums"));
+    h->sweep_part_bytes = need;
+    return SV_OK;
+}
+
+// The steps, angles, flag and sums of a whole sweep over ops and its form; form -1 where the memory for them
 // cannot be had (a list entry takes twice the bytes of the per-operator lists'): one launch per op then.
 static sv_status prepare_sweep(sv_handle h, bool adjoint, const std::vector<OpDesc> &ops, SweepShape *s) {
     *s = SweepShape();
@@ -973,6 +1014,7 @@ static sv_status prepare_sweep(sv_handle h, bool adjoint, const std::vector<OpDe
     if (st == SV_OK) {
         *s = sweep_shape(h, adjoint, ops.size());
         if (s->form == 2) st = ensure_kerr(h);
+        if (st == SV_OK && adjoint && s->form >= 0) st = ensure_sweep_part(h, (size_t)s->warps() * ops.size());
     }
     if (st != SV_OK && st != SV_ERR_OOM) return st;
     if (st != SV_OK || !h->groups.buf) {
@@ -1383,23 +1425,17 @@ static sv_status ensure_digits(sv_handle h, DevTables *T, const RowTables &R, Sa
     return SV_OK;
 }
 
-// Gives back what the product forms of the expectation hold (all of it is built anew on demand).
-static void drop_products(sv_handle h) {
-    dev_free(h, h->ab_H, h->ab_H_bytes);
-    dev_free(h, h->sg_mats, h->sg_mats_bytes);
-    dev_free(h, h->sg_buf, h->sg_buf_bytes);
-    h->ab_H = nullptr;
-    h->sg_mats = h->sg_buf = nullptr;
-    h->ab_H_bytes = h->sg_mats_bytes = h->sg_buf_bytes = 0;
-    h->sg_serial = h->sg_buf_geom = 0;
-    cudaGetLastError();
-}
-
 static sv_status sigma_rows(sv_handle h, DevTables *T, const RowTables &R, const void *C, void *lam, void *lamc,
                             double e_shift) {
+    auto held = [&](auto ensure) {  // one of its buffers does not give way to another
+        h->products_held = true;
+        const sv_status st = ensure();
+        h->products_held = false;
+        return st;
+    };
     if (use_digits(h, T)) {
         SameDigits g;
-        if (ensure_digits(h, T, R, &g) == SV_OK) {  // else the float-float sums below
+        if (held([&] { return ensure_digits(h, T, R, &g); }) == SV_OK) {  // else the float-float sums below
             SV_CUDA(h, launch_sigma_rows_digits(C, lam, lamc, h->n, R, T->hdiag, T->Jp, e_shift, h->partials, h->nb, g,
                                                 h->sm_count, h->stream));
             h->launches += 6;
@@ -1431,7 +1467,7 @@ static sv_status sigma_rows(sv_handle h, DevTables *T, const RowTables &R, const
     SameGemm g;
     bool sg = use_same_gemm(h, K);
     if (sg) {
-        const sv_status st = ensure_same_gemm(h, T, R, &g);
+        const sv_status st = held([&] { return ensure_same_gemm(h, T, R, &g); });
         if (st == SV_ERR_OOM && h->expect_variant == 0) {  // the automatic choice: the sparse sums, which need none of it
             drop_products(h);
             sg = false;
@@ -1781,12 +1817,12 @@ static sv_status autotune_impl(sv_handle h, sv_ham_handle ham, const std::vector
         int best_b = 8;
         float best_t = -1.f;
         if (h->storage == 1) SV_TRY(ensure_op_lists(h, d, h->lists));
-        SV_TRY(ensure_partials(h, (size_t)h->sm_count * 64 * (sweeps ? d.size() : 1)));
+        SV_TRY(ensure_partials(h, (size_t)h->sm_count * 64));
         if (sweeps) {
-            SV_TRY(ensure_groups(h, d));
-            SV_TRY(ensure_kerr(h));
-            SV_TRY(upload_sweep_angles(h, d));
-            sweeps = sweep_shape(h, false, d.size()).form == 2;  // blocks per SM: the grid form's choice alone
+            SweepShape s;
+            SV_TRY(prepare_sweep(h, false, d, &s));
+            sweeps = s.form == 2 &&  // blocks per SM: the grid form's choice alone
+                     ensure_sweep_part(h, (size_t)h->sm_count * 64 * d.size()) == SV_OK;
         }
         // sector storage: the adjoint step as sv_energy_grad runs it (interleaved unless checkpoints resync psi)
         bool inter = h->storage == 1 && adj && h->ckpt_interval <= 0;
@@ -1798,6 +1834,7 @@ static sv_status autotune_impl(sv_handle h, sv_ham_handle ham, const std::vector
             SV_CUDA(h, launch_interleave(h->lam, h->saved, h->dtype, h->CLbuf, (size_t)h->Da * h->Db, h->sm_count,
                                          h->stream));
         }
+        sweeps = sweeps && h->groups.buf;  // (else given back to the matrix above)
         const int sweep_bps = h->sweep_bps;
         for (int ci = 0; ci < 4; ++ci) {
             const int b = (sweeps && inter) ? cands_sw[ci] : cands_op[ci];
@@ -1990,10 +2027,9 @@ static void destroy_handle(sv_handle h) {
     }
     dev_free(h, h->lists.buf, h->lists.bytes);
     dev_free(h, h->pool_lists.buf, h->pool_lists.bytes);
-    dev_free(h, h->groups.buf, h->groups.bytes);
+    drop_sweep(h);
     dev_free(h, h->rdm_lists.buf, h->rdm_lists.bytes);
     dev_free(h, h->CLbuf, h->CLbuf_bytes);
-    dev_free(h, h->sweep_buf, h->sweep_bytes);
     dev_free(h, h->ffbuf, h->ffbuf_bytes);
     dev_free(h, h->partials, h->partials_cap * sizeof(double));
     dev_free(h, h->dout, h->dout_cap * sizeof(double));
@@ -2408,13 +2444,6 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
     SweepShape shape;
     if (inter && h->sweep_mode) {  // a whole sweep: it interleaves psi and lambda itself
         SV_TRY(prepare_sweep(h, true, d, &shape));
-        if (shape.form >= 0 &&
-            ensure_partials(h, std::max<size_t>((size_t)shape.warps() * L, std::max<size_t>((size_t)G * L, need))) != SV_OK) {
-            cudaGetLastError();
-            shape.form = -1;
-            SV_TRY(ensure_partials(h, std::max<size_t>((size_t)G * L, need)));
-        }
-        if (!h->groups.buf) shape.form = -1;
     }
     if (inter && shape.form != 0 && ensure_clbuf(h) != SV_OK) {
         cudaGetLastError();
@@ -2492,7 +2521,7 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
                 SV_CUDA(h, cudaMemcpyAsync(wpsi, h->ckpt[j], vec_bytes(h), cudaMemcpyDeviceToDevice, h->stream));
         }
     }
-    if (swept) SV_CUDA(h, launch_sweep_grad(h->partials, h->dtype, (int)L, shape.warps(), h->dout + 2, h->stream));
+    if (swept) SV_CUDA(h, launch_sweep_grad(h->sweep_part, h->dtype, (int)L, shape.warps(), h->dout + 2, h->stream));
     else SV_CUDA(h, launch_reduce_rows(h->partials, (int)L, G, h->dout + 2, h->stream));
     h->launches++;
     SV_TRY(mark(h, 5, "sv_energy_grad: restore"));

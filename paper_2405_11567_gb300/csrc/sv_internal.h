@@ -337,6 +337,8 @@ struct sv_ctx {
     // counter (first 256 bytes) and the ops' (cos, sin) on the device, their host staging
     void *sweep_buf = nullptr;
     size_t sweep_bytes = 0;
+    double *sweep_part = nullptr;  // a reverse sweep's gradient sums
+    size_t sweep_part_bytes = 0;
     std::vector<double> sweep_host;
     int sweep_mode = 1;        // SV_OPT_SECTOR_SWEEP: 1 one launch per sweep where possible, 0 one per op
     int sweep_bps = 2;         // SV_OPT_SWEEP_BLOCKS_PER_SM: blocks per SM of a whole-sweep launch
@@ -356,6 +358,7 @@ struct sv_ctx {
     uint64_t sg_buf_geom = 0;  // the planes' geometry (their row padding is zeroed when it changes)
     float *ab_H = nullptr;     // variant 5: the alpha-beta product planes
     size_t ab_H_bytes = 0;
+    bool products_held = false;  // these buffers are being gathered: none of them gives way to an allocation
     // storage layout: address bit perm[q] holds qubit q (identity by default);
     // layout_auto: sv_energy_grad picks it from its operator list
     int perm[32];

@@ -53,7 +53,7 @@ def _least_cap(run):
 
 
 def _check(got, want, tol, why):
-    assert got is not None, why
+    assert got is not None, ("refused", why)
     for (x, t), y in zip(got, want):
         assert np.max(np.abs(np.asarray(x) - np.asarray(y[0]))) <= tol[t], why
 
@@ -101,4 +101,32 @@ def test_sweep_steps_that_do_not_fit_leave_one_launch_per_operator(call, dtype):
     for factor in (1.0, 1.02, 1.1, 1.3, 1.6, 2.0, 3.0):
         got = _run(16, 4, dtype, int(least * factor), {sv.SV_OPT_EXPECT_VARIANT: 3}, calls)
         _check(got, want, TOL[dtype], factor)
+    ham.close()
+
+
+@pytest.mark.parametrize("dtype", ["r64", "r32", "c64"])
+def test_planes_give_way_to_later_calls(dtype):
+    """The expectation may take what a cap leaves; the 1-RDM, the pool, a checkpointed sweep and a longer list
+    after it are accepted wherever they are with the plain forms."""
+    n, ne = 20, 8
+    p, ham = _problem(n, ne)
+    pool = inputs.uccsd_pool(n, ne)
+    theta = np.random.default_rng(2).normal(0.0, 0.05, 400)
+
+    def calls(st):
+        st.prepare_hf(p["occ"])
+        E, g = st.energy_grad(ham, p["ops"], p["theta"])
+        out = [(E, 0), (g, 1), (st.rdm1(), 2)]
+        E, g = st.energy_grad(ham, pool[:400], theta)
+        out += [(E, 0), (g, 1), (st.rdm1(), 2)]
+        E, g = st.pool_gradients(ham, pool)
+        return out + [(E, 0), (g, 1)]
+
+    plain = lambda cap: _run(n, ne, dtype, cap, PLAIN, calls)
+    least = _least_cap(plain)
+    want = plain(0)
+    full = _run(n, ne, dtype, 0, {}, calls)
+    _check(full, want, TOL[dtype], "no cap")
+    for cap in range(least, 8 * least, max(least // 6, 1)):
+        _check(_run(n, ne, dtype, cap, {}, calls), want, TOL[dtype], cap)
     ham.close()
