@@ -742,6 +742,7 @@ static sv_status ensure_op_lists(sv_handle h, const std::vector<OpDesc> &ops, Op
         SV_TRY(dev_alloc(h, &cache.buf, lb + obb + ib, "operator pair lists"));
         cache.bytes = lb + obb + ib;
     }
+    cache.key.clear();  // until all of it is written: a call that fails halfway leaves no lists
     uint8_t *dops = (uint8_t *)cache.buf + lb;  // op records after the lists, then the int4 records
     int *dinfo = (int *)(dops + obb);
     SV_CUDA(h, cudaMemcpyAsync(dops, host.data(), ops.size() * ob, cudaMemcpyHostToDevice, h->stream));
@@ -864,6 +865,7 @@ static sv_status ensure_groups(sv_handle h, const std::vector<OpDesc> &ops) {
         SV_TRY(dev_alloc(h, &c.buf, need, "sweep steps"));
         c.bytes = need;
     }
+    c.key.clear();  // until all of it is written: a call that fails halfway leaves no steps of either list
     uint8_t *dp = (uint8_t *)c.buf + lb;
     SV_CUDA(h, cudaMemcpyAsync(dp, plans.data(), plans.size(), cudaMemcpyHostToDevice, h->stream));
     SV_CUDA(h, cudaMemcpyAsync(dp + pb, groups.data(), groups.size(), cudaMemcpyHostToDevice, h->stream));
