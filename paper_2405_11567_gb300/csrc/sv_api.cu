@@ -448,13 +448,15 @@ static sv_status ensure_sector(sv_handle h) {
 // ascending; their ranks; their spread over the even (odd) bit positions.
 static sv_status ensure_strings(sv_handle h) {
     if (h->str_sa && h->str_na == h->na && h->str_nb == h->nb) return SV_OK;
-    if (h->str_sa) {
-        for (void *p : {(void *)h->str_sa, (void *)h->str_sb, (void *)h->str_sa_s, (void *)h->str_sb_s,
-                        (void *)h->str_a, (void *)h->str_b, (void *)h->rank_a, (void *)h->rank_b})
-            cudaFree(p);
-        h->bytes_owned -= std::min<uint64_t>(h->bytes_owned, h->str_bytes);
-        h->str_sa = h->str_sb = h->str_sa_s = h->str_sb_s = nullptr;
-    }
+    // the old tables go first, and no sector has any until all of them are there
+    for (void *p : {(void *)h->str_sa, (void *)h->str_sb, (void *)h->str_sa_s, (void *)h->str_sb_s,
+                    (void *)h->str_a, (void *)h->str_b, (void *)h->rank_a, (void *)h->rank_b})
+        cudaFree(p);
+    h->bytes_owned -= std::min<uint64_t>(h->bytes_owned, h->str_bytes);
+    h->str_bytes = 0;
+    h->str_sa = h->str_sb = h->str_sa_s = h->str_sb_s = nullptr;
+    h->str_a = h->str_b = h->rank_a = h->rank_b = nullptr;
+    h->str_na = h->str_nb = -1;
     const int N = h->n / 2;
     // Ascending (the documented order of sector storage), but in a core with orbital 0 as the most
     // significant: an excitation p -> q touches runs of strings that agree on every orbital down to
@@ -493,10 +495,9 @@ static sv_status ensure_strings(sv_handle h) {
         spb[i] = x;
         spb_s[i] = map_bits(x, h->perm);
     }
-    size_t bytes = 0;
     auto up = [&](void **dst, const void *src, size_t nb) -> sv_status {
         SV_TRY(dev_alloc(h, dst, std::max<size_t>(nb, 16), "string tables"));
-        bytes += std::max<size_t>(nb, 16);
+        h->str_bytes += std::max<size_t>(nb, 16);
         SV_CUDA(h, cudaMemcpy(*dst, src, nb, cudaMemcpyHostToDevice));
         return SV_OK;
     };
@@ -508,24 +509,22 @@ static sv_status ensure_strings(sv_handle h) {
     SV_TRY(up((void **)&h->str_b, sb16.data(), sb16.size() * 2));
     SV_TRY(up((void **)&h->rank_a, ra.data(), ra.size() * 2));
     SV_TRY(up((void **)&h->rank_b, rb.data(), rb.size() * 2));
-    h->str_bytes = bytes;
     h->Da = (int)sa16.size();
     h->Db = (int)sb16.size();
-    h->str_na = h->na;
-    h->str_nb = h->nb;
     h->h_stra = sa16;
     h->h_strb = sb16;
     h->h_ra = ra;
     h->h_rb = rb;
-    if (h->storage == 1) return SV_OK;  // the state itself is the compact matrix
-    size_t cb = (size_t)h->Da * h->Db * h->amp_bytes;
-    if (h->Cbuf_bytes < cb) {
+    const size_t cb = (size_t)h->Da * h->Db * h->amp_bytes;
+    if (h->storage == 0 && h->Cbuf_bytes < cb) {  // (sector storage: the state itself is the compact matrix)
         dev_free(h, h->Cbuf, h->Cbuf_bytes);
         h->Cbuf = nullptr;
         h->Cbuf_bytes = 0;
         SV_TRY(dev_alloc(h, &h->Cbuf, std::max<size_t>(cb, 16), "compact sector amplitudes"));
         h->Cbuf_bytes = std::max<size_t>(cb, 16);
     }
+    h->str_na = h->na;
+    h->str_nb = h->nb;
     return SV_OK;
 }
 

@@ -130,3 +130,27 @@ def test_planes_give_way_to_later_calls(dtype):
     for cap in range(least, 8 * least, max(least // 6, 1)):
         _check(_run(n, ne, dtype, cap, {}, calls), want, TOL[dtype], cap)
     ham.close()
+
+
+def test_tables_that_do_not_fit_are_refused_again():
+    """A dense handle whose string tables or compact matrix do not fit is refused each time it asks, not only
+    the first, and serves a smaller sector in between."""
+    n = 16
+    p, ham = _problem(n, 8)
+    big, small = p["occ"], p["occ"][:2]
+    want = {}
+    base = 8 << n
+    for cap in [0] + list(range(base, base + 96 * 1024, 1536)):
+        st = sv.StateVector(n, "c64")
+        st.set_option(sv.SV_OPT_MAX_BYTES, cap)
+        st.set_option(sv.SV_OPT_EXPECT_VARIANT, 3)
+        for occ in (big, big, small, big, big, small):
+            st.prepare_hf(occ)
+            try:
+                E = st.energy(ham)
+            except sv.SvError as e:
+                assert e.status == 2 and cap, e
+                continue
+            assert abs(E - want.setdefault(len(occ), E)) <= 1e-5, cap
+        st.close()
+    ham.close()
