@@ -518,13 +518,15 @@ cudaError_t launch_ab_table(const float *eri, const float *Jt, const uint16_t *s
     return e != cudaSuccess || !rowB ? e : launch_ab_rows(strb, N, nb, Db, rowB, st);
 }
 
+constexpr size_t kAbTcSmemCap = 227 * 1024 - 1024;  // dynamic; the static part takes 400 bytes
+
 // Whether the tensor-core alpha-beta form applies: N <= 16, D <= 4096 per spin, at most
 // 64 columns, and its shared memory fits.
 bool ab_tc_fits(int planes, int Da, int Db, int na, int nb, int N) {
     (void)na;
     if (N > 16 || N < 1 || Da > 4096 || Db > 4096 || Da < 1 || Db < 1) return false;
     if (nb * (N - nb) + 1 > kAbMaxN) return false;
-    return ab_tc_smem(planes, Da, N) <= 227 * 1024 - 1024;
+    return ab_tc_smem(planes, Da, N) <= kAbTcSmemCap;
 }
 
 // Row stride (amplitudes) of the interleaved X pieces the kernel reads.
@@ -562,7 +564,7 @@ cudaError_t launch_ab_tc(const uint32_t *Xi, int planes, const uint16_t *stra, c
     const bool split = (long long)Da * Db < 1 << 20;
     auto *kernel = planes == 2 ? (split ? k_ab_tc<false, true> : k_ab_tc<false, false>)
                                : (split ? k_ab_tc<true, true> : k_ab_tc<true, false>);
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = allow_smem(kernel, kAbTcSmemCap);
     if (e != cudaSuccess) return e;
     kernel<<<grid, kAbThreadsTc, sm, st>>>(g);
     return cudaGetLastError();

@@ -1109,10 +1109,8 @@ sv_status capture(sv_batch *b) {
     const BatchArgs<R> a = batch_args<R>(b);
     cudaStream_t st = b->stream;
     cudaError_t e = cudaSuccess;
-    // The limit on dynamic shared memory, always and to the same value: the default one is 48 KB less the kernel's
-    // static part, and a value of this batch's own would lower that of another thread's batch.
-    e = b->threads == 384 ? cudaFuncSetAttribute(k_batch<R, 384>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmemCap)
-                          : cudaFuncSetAttribute(k_batch<R, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmemCap);
+    // always: the default limit on dynamic shared memory is 48 KB less the kernel's static part
+    e = b->threads == 384 ? allow_smem(k_batch<R, 384>, kBatchSmemCap) : allow_smem(k_batch<R, 256>, kBatchSmemCap);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return bfail(SV_ERR_CUDA, std::string("batch shared memory: ") + cudaGetErrorString(e));

@@ -643,6 +643,8 @@ __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_digits(DbArgs g) {
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
 
+constexpr size_t kDbSmemCap = 227 * 1024 - 1024;  // dynamic; the static part takes 352 bytes
+
 int digits_ldx(int Da) { return Da / 4 * 4 + 4; }  // a zero word at least after the last
 
 size_t ab_digits_smem(int Da, int N) {
@@ -748,7 +750,7 @@ __global__ void __launch_bounds__(kThreads) k_comb_digits(SigmaTables<double> T,
 bool digits_fit(int Da, int Db, int nb, int N) {
     if (N > 16 || N < 1 || Da > 4096 || Db > 4096 || Da < 1 || Db < 1 || nb < 0 || nb > N) return false;
     if (nb * (N - nb) + 1 > kAbMaxN) return false;
-    return ab_digits_smem(Da, N) <= 227 * 1024 - 1024;
+    return ab_digits_smem(Da, N) <= kDbSmemCap;
 }
 
 // The digits of [Ma | Mb] (nm float64 values) and of the B table; B64: room for the table's float64
@@ -800,8 +802,7 @@ cudaError_t launch_sigma_digits(const SigmaTables<double> &T, const double *C, d
     if (!map(&ma, g.Mp, Da, Da, g.lda, g.pm, kTcM) || !map(&mb, g.Mp + (size_t)Da * g.lda, Db, Db, g.ldb, g.pm, kDsN) ||
         !map(&mx, g.Xp, Da, Db, g.lda, g.px, kDsN) || !map(&mt, g.Xtp, Db, Da, g.ldb, g.pt, kTcM))
         return cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute(k_same_digits, cudaFuncAttributeMaxDynamicSharedMemorySize, kDsSmem)) != cudaSuccess)
-        return e;
+    if ((e = allow_smem(k_same_digits, kDsSmem)) != cudaSuccess) return e;
     k_same_digits<<<dim3((Db + kDsN - 1) / kDsN, (Da + kTcM - 1) / kTcM, 2), kDsThreads, kDsSmem, st>>>(
         ma, mb, mx, mt, DsOut{g.G, Da, Db, g.err, g.spins, g.stall & 1});
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -814,8 +815,7 @@ cudaError_t launch_sigma_digits(const SigmaTables<double> &T, const double *C, d
     a.units = (Da + kAbM - 1) / kAbM * Db;
     a.err = g.err; a.spins = g.spins; a.stall = (g.stall >> 1) & 1;
     const size_t sm = ab_digits_smem(Da, N);
-    if ((e = cudaFuncSetAttribute(k_ab_digits, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
-        return e;
+    if ((e = allow_smem(k_ab_digits, kDbSmemCap)) != cudaSuccess) return e;
     k_ab_digits<<<a.units < sm_count ? a.units : sm_count, kAbThreadsTc, sm, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (g.ev && (e = cudaEventRecord(g.ev[3], st)) != cudaSuccess) return e;

@@ -1077,7 +1077,7 @@ const int *sigma_ab_sizes(int dtype) { return kChunks[dtype & 3]; }
 
 template <typename Amp, int K>
 static cudaError_t launch_ab(const RowArgs<Amp> &A, size_t smem, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(k_sigma_ab<Amp, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_sigma_ab<Amp, K>, kAbSmemCap);
     if (e != cudaSuccess) return e;
     k_sigma_ab<Amp, K><<<A.Db, kAbThreads, smem, st>>>(A);
     return cudaGetLastError();
@@ -1164,12 +1164,12 @@ static cudaError_t launch_rows_t(const RowArgs<Amp> &A, const RowTables &T, int 
     if (e != cudaSuccess) return e;
     if (same_smem(dtype, T, true) <= kSameSmemCap) {
         const size_t smem = same_smem(dtype, T, true);
-        e = cudaFuncSetAttribute(k_sigma_same<Amp, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(k_sigma_same<Amp, true>, kSameSmemCap);
         if (e != cudaSuccess) return e;
         k_sigma_same<Amp, true><<<T.Db, kSameThreads, smem, st>>>(A);
     } else {
         const size_t smem = same_smem(dtype, T, false);
-        e = cudaFuncSetAttribute(k_sigma_same<Amp, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(k_sigma_same<Amp, false>, kSameSmemCap);
         if (e != cudaSuccess) return e;
         k_sigma_same<Amp, false><<<T.Db, kSameThreads, smem, st>>>(A);
     }
@@ -1231,12 +1231,12 @@ static cudaError_t launch_ff_t(const void *C, void *lam, void *lamc, int dtype, 
     if (e != cudaSuccess) return e;
     if (same_smem(dtype, Tf, true) <= kSameSmemCap) {
         const size_t smem = same_smem(dtype, Tf, true);
-        e = cudaFuncSetAttribute(k_sigma_same<F, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(k_sigma_same<F, true>, kSameSmemCap);
         if (e != cudaSuccess) return e;
         k_sigma_same<F, true><<<Tf.Db, kSameThreads, smem, st>>>(RA);
     } else {
         const size_t smem = same_smem(dtype, Tf, false);
-        e = cudaFuncSetAttribute(k_sigma_same<F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(k_sigma_same<F, false>, kSameSmemCap);
         if (e != cudaSuccess) return e;
         k_sigma_same<F, false><<<Tf.Db, kSameThreads, smem, st>>>(RA);
     }

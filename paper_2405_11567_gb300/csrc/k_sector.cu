@@ -655,13 +655,16 @@ int rdm_rows_grid(int rows, int sm_count, int bps) {
 
 namespace {
 
+// 12,870 strings of 16 bytes and the sums of 16 orbitals' pairs of four rows: 209 KB;
+// the static part takes 2,176 bytes.
+constexpr size_t kRdmSmemCap = 222 * 1024;
+
 template <typename A, int NV>
 cudaError_t rdm_rows_nv(const void *C, const SectTabs &T, int N, int grid, const uint32_t *lists, const int *info,
                         double *partial, cudaStream_t st) {
     constexpr int RW = kRdmRows<A, NV>, NC = AmpT<A>::kCplx ? 2 : 1;
     const size_t smem = (size_t)(T.Da > T.Db ? T.Da : T.Db) * 16 * NV + sizeof(double) * (size_t)N * (N - 1) * RW * NC;
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_rdm_rows<A, NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(k_rdm_rows<A, NV>, kRdmSmemCap);
     if (e != cudaSuccess) return e;
     k_rdm_rows<A, NV><<<grid, kRdmThreads, smem, st>>>((const A *)C, T, N, lists, (const int4 *)info, partial);
     return cudaGetLastError();

@@ -305,7 +305,7 @@ template <typename A, bool ADJ, int FORM>
 cudaError_t sweep_launch(A *psi, const A *lam, SweepPlan g, int blocks, int threads, size_t smem, cudaStream_t st) {
     auto *kernel = k_sweep<A, ADJ, FORM>;
     cudaError_t e = cudaSuccess;
-    if (FORM == kBlock) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (FORM == kBlock) e = allow_smem(kernel, kSweepSmemCap);
     if (FORM == kCluster) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};

@@ -951,7 +951,7 @@ static SweepShape sweep_shape(sv_handle h, bool adjoint, size_t n_ops) {
     // the block and cluster forms wait on hardware barriers: a caller who wants waits given up
     // after a few polls gets the grid form, whose waits SV_OPT_WAIT_POLLS bounds
     const bool hw = h->wait_polls >= 1024;
-    const size_t bs = sweep_block_smem(h->dtype, adjoint, h->Da, h->Db), cap = 226 * 1024;
+    const size_t bs = sweep_block_smem(h->dtype, adjoint, h->Da, h->Db), cap = kSweepSmemCap;
     s.form = hw && bs <= cap && avg <= 300 ? 0 : hw && avg <= 4000 ? 1 : 2;
     if (s.form == 0) {
         s.blocks = 1;

@@ -25,6 +25,17 @@ struct sv_ham;
 
 namespace svk {
 
+// Raises a kernel's limit on dynamic shared memory to `most`, the most that any launch of it takes (not what
+// this launch takes: the limit belongs to the process, and a smaller value would lower it under the launch
+// that another thread is about to make).
+template <typename K>
+inline cudaError_t allow_smem(K *kernel, size_t most) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
+// Shared memory of a sweep in one block (k_sweep's block form) at most.
+constexpr size_t kSweepSmemCap = 226 * 1024;
+
 // Bytes of one amplitude, and whether the state's arithmetic is single precision.
 inline size_t amp_size(int dtype) { return dtype == SV_C64 ? 8 : dtype == SV_C128 ? 16 : dtype == SV_R32 ? 4 : 8; }
 inline bool single_prec(int dtype) { return dtype == SV_C64 || dtype == SV_R32; }
