@@ -338,19 +338,22 @@ __device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a,
 __device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ ff mad(ff a, ff b, ff c) { return ff_fma(a, b, c); }
 
-constexpr int kRdmThreads = 512;
 // NV: 16-byte words to a string, RW = 16 NV / sizeof(A) rows.  Two, which halve the list reads, while
-// the rows still make two groups per SM and two blocks fit on it; one below and above that.  At most
-// 64 registers: two blocks (30 qubits float32 272 us with one, 229 with two).
+// the rows still make two groups per SM and two blocks fit on it, and for complex float64 amplitudes,
+// whose word holds one row alone (22 qubits 69 us with one, 48 with two); else one.  At most
+// 64 registers: two blocks (30 qubits float32 272 us with one, 229 with two).  NT threads: 512, but 256
+// up to kRdmFew strings, where a block's few lists leave half the warps idle at its barriers (8 qubits float32
+// 14.8 and 13.0 us, 18 qubits, 84 strings, no difference).
+constexpr int kRdmFew = 64;
 template <typename A, int NV> constexpr int kRdmRows = 16 * NV / (int)sizeof(A);
-template <typename A, int NV>
-__global__ void __launch_bounds__(kRdmThreads, 2) k_rdm_rows(const A *__restrict__ C, SectTabs T, int N,
+template <typename A, int NV, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_rdm_rows(const A *__restrict__ C, SectTabs T, int N,
                                                           const uint32_t *__restrict__ lists,
                                                           const int4 *__restrict__ info,
                                                           double *__restrict__ partial) {
     using R = real_of<A>;
     using S = typename RdmSum<R>::T;
-    constexpr int RW = kRdmRows<A, NV>, NC = AmpT<A>::kCplx ? 2 : 1, NW = kRdmThreads / 32;
+    constexpr int RW = kRdmRows<A, NV>, NC = AmpT<A>::kCplx ? 2 : 1, NW = NT / 32;
     struct alignas(16) Word { A v[RW / NV]; };
     extern __shared__ __align__(16) uint8_t rdm_s[];  // [strings][RW] amplitudes, then the pairs' float64 slots
     __shared__ double s_occ[NW][17];
@@ -358,7 +361,7 @@ __global__ void __launch_bounds__(kRdmThreads, 2) k_rdm_rows(const A *__restrict
     Word *buf = reinterpret_cast<Word *>(rdm_s);
     double *slot = reinterpret_cast<double *>(buf + (size_t)Dm * NV);  // [2 npair][RW][NC]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = threadIdx.x; i < 2 * npair * RW * NC; i += kRdmThreads) slot[i] = 0.0;
+    for (int i = threadIdx.x; i < 2 * npair * RW * NC; i += NT) slot[i] = 0.0;
     auto put = [&](int e, double v) {
         partial[(size_t)(2 * e) * gridDim.x + blockIdx.x] = v;
         partial[(size_t)(2 * e + 1) * gridDim.x + blockIdx.x] = 0.0;
@@ -380,7 +383,7 @@ __global__ void __launch_bounds__(kRdmThreads, 2) k_rdm_rows(const A *__restrict
             const int r0 = (item - first) * RW;
             __syncthreads();  // the last group's reads of buf are done
             if (s == 0) {
-                for (int x = threadIdx.x; x < D; x += kRdmThreads) {
+                for (int x = threadIdx.x; x < D; x += NT) {
                     #pragma unroll
                     for (int w = 0; w < NV; ++w) {
                         Word v;
@@ -394,7 +397,7 @@ __global__ void __launch_bounds__(kRdmThreads, 2) k_rdm_rows(const A *__restrict
                 }
             } else {
                 A *flat = reinterpret_cast<A *>(buf);
-                for (int i = threadIdx.x; i < D * RW; i += kRdmThreads) {
+                for (int i = threadIdx.x; i < D * RW; i += NT) {
                     constexpr int WV = RW / NV;
                     const int j = i % RW, r = r0 + j;
                     flat[((j / WV) * Dm + i / RW) * WV + j % WV] = r < rows ? C[(size_t)(i / RW) * T.Da + r] : mka<A>(R(0), R(0));
@@ -405,7 +408,7 @@ __global__ void __launch_bounds__(kRdmThreads, 2) k_rdm_rows(const A *__restrict
             S occ[16], nrm[1] = {S(0)};
             #pragma unroll
             for (int p = 0; p < 16; ++p) occ[p] = S(0);
-            for (int x = threadIdx.x; x < D; x += kRdmThreads) {
+            for (int x = threadIdx.x; x < D; x += NT) {
                 const uint32_t bits = str[x];
                 R w = R(0);
                 #pragma unroll
@@ -480,7 +483,7 @@ __global__ void __launch_bounds__(kRdmThreads, 2) k_rdm_rows(const A *__restrict
         __syncthreads();
     }
     __syncthreads();  // (a block without groups: the slots were zeroed by other threads)
-    for (int e = threadIdx.x; e < 2 * npair; e += kRdmThreads) {
+    for (int e = threadIdx.x; e < 2 * npair; e += NT) {
         double re = 0.0, im = 0.0;
         for (int r = 0; r < RW; ++r) {
             re += slot[((size_t)e * RW + r) * NC];
@@ -647,40 +650,47 @@ cudaError_t launch_adjoint_li(void *CL, int dtype, const uint32_t *al, int na_l,
 
 int rdm_rows_elements(int n) { return 1 + n + (n / 2) * (n / 2 - 1); }
 
-// Blocks: at most bps per SM, and no more than rows.
-int rdm_rows_grid(int rows, int sm_count, int bps) {
-    const int cap = sm_count * (bps > 0 ? bps : 4);
-    return rows < cap ? rows : cap;
-}
-
 namespace {
 
 // 12,870 strings of 16 bytes and the sums of 16 orbitals' pairs of four rows: 209 KB;
 // the static part takes 2,176 bytes.
 constexpr size_t kRdmSmemCap = 222 * 1024;
 
+// Words to a string of the sector's amplitudes (of `amp` bytes).
+int rdm_words(int amp, int Dm, int sm_count) {
+    if (amp == 16) return Dm <= 3 * 1024 ? 2 : 1;
+    return Dm <= 3 * 1024 && Dm * amp / 32 >= 2 * sm_count ? 2 : 1;  // two blocks per SM: about 100 KB each
+}
+
 template <typename A, int NV>
 cudaError_t rdm_rows_nv(const void *C, const SectTabs &T, int N, int grid, const uint32_t *lists, const int *info,
                         double *partial, cudaStream_t st) {
     constexpr int RW = kRdmRows<A, NV>, NC = AmpT<A>::kCplx ? 2 : 1;
     const size_t smem = (size_t)(T.Da > T.Db ? T.Da : T.Db) * 16 * NV + sizeof(double) * (size_t)N * (N - 1) * RW * NC;
-    const cudaError_t e = allow_smem(k_rdm_rows<A, NV>, kRdmSmemCap);
+    const bool few = (T.Da > T.Db ? T.Da : T.Db) <= kRdmFew;
+    const cudaError_t e = few ? allow_smem(k_rdm_rows<A, NV, 256>, kRdmSmemCap) : allow_smem(k_rdm_rows<A, NV, 512>, kRdmSmemCap);
     if (e != cudaSuccess) return e;
-    k_rdm_rows<A, NV><<<grid, kRdmThreads, smem, st>>>((const A *)C, T, N, lists, (const int4 *)info, partial);
+    if (few) k_rdm_rows<A, NV, 256><<<grid, 256, smem, st>>>((const A *)C, T, N, lists, (const int4 *)info, partial);
+    else k_rdm_rows<A, NV, 512><<<grid, 512, smem, st>>>((const A *)C, T, N, lists, (const int4 *)info, partial);
     return cudaGetLastError();
 }
 
 template <typename A>
 cudaError_t rdm_rows_of(const void *C, const SectTabs &T, int N, int grid, const uint32_t *lists, const int *info,
                         double *partial, int sm_count, cudaStream_t st) {
-    const int Dm = T.Da > T.Db ? T.Da : T.Db;
-    // two words: up to two blocks per SM by shared memory (about 100 KB each)
-    if (Dm <= 3 * 1024 && Dm / kRdmRows<A, 2> >= 2 * sm_count)
+    if (rdm_words((int)sizeof(A), T.Da > T.Db ? T.Da : T.Db, sm_count) == 2)
         return rdm_rows_nv<A, 2>(C, T, N, grid, lists, info, partial, st);
     return rdm_rows_nv<A, 1>(C, T, N, grid, lists, info, partial, st);  // at most 12,870 strings: 214 KB
 }
 
 }  // namespace
+
+// Blocks: one to a group of rows or columns, at most bps per SM.  (A float64 state's float-float form has its size.)
+int rdm_rows_grid(int dtype, int Da, int Db, int sm_count, int bps) {
+    const int amp = (int)amp_size(dtype), rw = 16 * rdm_words(amp, Da > Db ? Da : Db, sm_count) / amp;
+    const int cap = sm_count * (bps > 0 ? bps : 4), items = (Da + rw - 1) / rw + (Db + rw - 1) / rw;
+    return items < cap ? items : cap;
+}
 
 // partial: [2 n_el][grid] doubles (n_el = rdm_rows_elements(n)), reduced by launch_reduce_rows.
 // lists / info: the pair lists and their int4 records, one list op per pair p < q in (p, q) order (for

@@ -78,7 +78,7 @@ cudaError_t launch_adjoint_li(void *CL, int dtype, const uint32_t *al, int na_l,
 cudaError_t launch_adjoint_l(void *psi, void *lam, int dtype, const uint32_t *al, int na_l, const uint32_t *bl,
                              int nb_l, int Da, double c, double s, int grid, double *partial, cudaStream_t st);
 int rdm_rows_elements(int n);
-int rdm_rows_grid(int rows, int sm_count, int bps);
+int rdm_rows_grid(int dtype, int Da, int Db, int sm_count, int bps);
 cudaError_t launch_to_ff(const void *C, int dtype, size_t count, void *out, int sm_count, cudaStream_t st);
 cudaError_t launch_rdm_rows(const void *C, int dtype, int ff_form, int n, const uint32_t *sa, const uint32_t *sb,
                             const uint16_t *stra, const uint16_t *strb, const uint16_t *ra, const uint16_t *rb, int Da,
@@ -1899,14 +1899,14 @@ static sv_status autotune_impl(sv_handle h, sv_ham_handle ham, const std::vector
         }
         const int n_el = rdm_rows_elements(h->n);
         const int cands[] = {2, 4, 8, 16};
-        SV_TRY(ensure_partials(h, (size_t)2 * n_el * rdm_rows_grid(std::max(h->Da, h->Db), h->sm_count, 16)));
+        SV_TRY(ensure_partials(h, (size_t)2 * n_el * rdm_rows_grid(h->dtype, h->Da, h->Db, h->sm_count, 16)));
         const void *src = nullptr;
         int ff_form = 0;
         SV_TRY(rdm_input(h, Cm, &src, &ff_form));
         int best_b = 4;
         float best_t = -1.f;
         for (int b : cands) {
-            const int grid = rdm_rows_grid(std::max(h->Da, h->Db), h->sm_count, b);
+            const int grid = rdm_rows_grid(h->dtype, h->Da, h->Db, h->sm_count, b);
             const float t = time_best(h, e0, e1, [&]() -> sv_status {
                 SV_CUDA(h, launch_rdm_rows(src, h->dtype, ff_form, h->n, h->str_sa, h->str_sb, h->str_a, h->str_b,
                                            h->rank_a, h->rank_b, h->Da, h->Db, grid, (const uint32_t *)h->rdm_lists.buf,
@@ -2676,7 +2676,7 @@ static sv_status rdm1_run(sv_handle h, double *re_out, double *im_out) {
         SV_TRY(ensure_strings(h));
         SV_TRY(ensure_rdm_lists(h));
         const int n_el = rdm_rows_elements(h->n);
-        const int grid = rdm_rows_grid(std::max(h->Da, h->Db), h->sm_count, h->rdm_bps);
+        const int grid = rdm_rows_grid(h->dtype, h->Da, h->Db, h->sm_count, h->rdm_bps);
         SV_TRY(ensure_partials(h, (size_t)2 * n_el * grid));
         SV_TRY(ensure_out(h, 2 * (size_t)n_el));
         SV_TRY(mark(h, 0, "sv_rdm1"));

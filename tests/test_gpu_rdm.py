@@ -60,3 +60,18 @@ def test_blocks_without_groups():
             dirty.rdm1()
             assert np.max(np.abs(st.rdm1() - ref)) <= TOL["r64"]
         st.close()
+
+
+# complex amplitudes (two words to a string in float64), both sides of 64 strings (56, 70), rows left over
+@pytest.mark.parametrize("variant", [0, 2])
+@pytest.mark.parametrize("dtype", ["c128", "c64"])
+@pytest.mark.parametrize("n,na,nb", [(4, 2, 1), (10, 2, 3), (14, 7, 1), (16, 3, 3), (16, 4, 3), (20, 5, 4)])
+def test_rdm_groups_of_complex_states(n, na, nb, dtype, variant):
+    dense = inputs.random_sector_state(n, na, nb, np.random.default_rng(n + na))
+    sec = oracle.Sector(n, na, nb)
+    st = sv.StateVector(n, dtype, sector=(na, nb))
+    st.set_option(sv.SV_OPT_RDM_VARIANT, variant)
+    st.prepare_state(dense.astype(np.complex128 if dtype == "c128" else np.complex64), na, nb)
+    got = st.rdm1()
+    assert np.max(np.abs(got - A.rdm1(sec, dense[sec.dets.astype(np.int64)]))) <= TOL[dtype]
+    assert np.max(np.abs(got.imag)) > 0.0
