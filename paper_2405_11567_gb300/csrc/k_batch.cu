@@ -536,7 +536,7 @@ __device__ __noinline__ void run_blocked(const BatchArgs<R> &B, const BatchInst 
         team.sync();
         return true;
     };
-    run_steps<R, false, 1>(lists, groups, angles, I.n_groups, Da, (size_t)D, tid, NT, warp, nw, nullptr,
+    run_steps<R, false, 1>(lists, groups, angles, I.n_groups, Da, (size_t)D, tid, NT, warp, nw, 1, nullptr,
                            [&](uint32_t at) { return own[at].c; }, [&](uint32_t at, R v) { own[at].c = v; }, sync);
     team.sync();
     // phi of element (b, a), as a sign flip: the parity of the alpha string under the beta string's prefix parity
@@ -572,7 +572,7 @@ __device__ __noinline__ void run_blocked(const BatchArgs<R> &B, const BatchInst 
         sn += sum_value(red[2 * w + 1], (R)0);
     }
     if (tid == 0) B.out[I.out] = I.shift + se / sn;
-    run_steps<R, true, 1>(lists, groups, angles, I.n_groups, Da, (size_t)D, tid, NT, warp, nw, gsum,
+    run_steps<R, true, 1>(lists, groups, angles, I.n_groups, Da, (size_t)D, tid, NT, warp, nw, 1, gsum,
                           [&](uint32_t at) { return own[at]; }, [&](uint32_t at, const PairOf<R> &v) { own[at] = v; }, sync);
     team.sync();
     for (int k = tid; k < I.L; k += NT) {

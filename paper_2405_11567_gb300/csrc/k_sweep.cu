@@ -73,6 +73,7 @@ struct SweepPlan {
     unsigned int *bar;       // grid form: barrier arrivals, zero at launch
     int *err;
     uint32_t spins;
+    int once;                // 1 (run_steps)
     double *partial;         // reverse: [operators][warps] gradient sums (GradSum::bits)
 };
 
@@ -121,7 +122,7 @@ template <typename A, bool ADJ, int FORM>
 __global__ void __launch_bounds__(FORM == kGrid ? 256 : 512, FORM == kGrid ? 2 : 1) k_sweep(A *__restrict__ psi, const A *__restrict__ lam, SweepPlan g) {
     using R = real_of<A>;
     using P = std::conditional_t<ADJ, PairOf<A>, A>;
-        constexpr int kB = FORM == kGrid && sizeof(P) <= 8 ? 2 : 1;  // components of each operator in flight
+    constexpr int kB = FORM == kGrid && sizeof(P) <= 8 ? 2 : 1;  // components of each operator in flight
     extern __shared__ __align__(16) uint8_t sweep_smem[];
     __shared__ volatile int s_ok;
     P *own = reinterpret_cast<P *>(sweep_smem);
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(FORM == kGrid ? 256 : 512, FORM == kGrid ? 2 :
     };
     auto store = [&](uint32_t at, const P &p) { own[at] = p; };
     auto sync = [&](int n) { return step_sync<FORM>(g, (unsigned int)n, &s_ok); };
-    if (!run_steps<A, ADJ, kB>(lists, groups, angles, g.n_groups, g.Da, count, gt, T, gw, W, g.partial, load, store, sync)) return;
+    if (!run_steps<A, ADJ, kB>(lists, groups, angles, g.n_groups, g.Da, count, gt, T, gw, W, g.once, g.partial, load, store, sync)) return;
     if constexpr (FORM == kBlock && !ADJ) {
         __syncthreads();
         for (size_t e = tid; e < count; e += NT) psi[e] = own[e];
@@ -355,7 +356,7 @@ cudaError_t launch_sweep(void *psi, const void *lam, int dtype, bool adjoint, in
     SweepPlan g;
     g.lists = (const uint2 *)lists; g.groups = (const Group *)groups; g.angles = angles; g.n_ops = n_ops;
     g.n_groups = n_groups; g.Da = Da; g.Db = Db; g.words = words; g.init = init; g.work = work; g.bar = bar; g.err = err;
-    g.spins = spins; g.partial = partial;
+    g.spins = spins; g.once = 1; g.partial = partial;
     const size_t smem = form == kBlock ? sweep_block_smem(dtype, adjoint, Da, Db) +
                                              (words ? sweep_stage_bytes(dtype, words, n_groups, n_ops) : 0) : 0;
     cudaError_t e = cudaErrorInvalidValue;

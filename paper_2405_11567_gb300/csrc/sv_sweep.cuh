@@ -243,10 +243,15 @@ struct ListWalk {
 // A whole sweep's steps by T threads (this one number gt, of warp gw of W): amplitudes through
 // load(at) and store(at, value) (P: with lambda in reverse), sync(n) before step n (false: a wait
 // ran out, and so does this function return); gradient sums [operator][warp] into partial.
-// KB: components of each operator that a thread has in flight.
+// KB: components of each operator that a thread has in flight.  once: 1.  Forward rotations of real float64
+// amplitudes that a component may not have are loops of `once` turns, because a plain condition becomes
+// predicated or selected arithmetic: every warp then ran four or five rotations for the one or two that it had,
+// on the pipe that bounds it (30 qubits, 20 operators: 3.0 million FP64 instructions for 1.4; 200 operators 2.27 ms
+// so, 1.52 with the loops, 1.56 one operator to a step; 28 qubits 676 and 480 us, 16 qubits 115 and 102).  Complex
+// float64 gains nothing (22 qubits 195 and 197 us), and the reverse rotations branch by themselves.
 template <typename A, bool ADJ, int KB, class Load, class Store, class Sync>
 __device__ __forceinline__ bool run_steps(const uint2 *lists, const Group *groups, const Angle<real_of<A>> *angles, int n_groups,
-                                          int Da, size_t count, int gt, int T, int gw, int W, double *partial, Load load,
+                                          int Da, size_t count, int gt, int T, int gw, int W, int once, double *partial, Load load,
                                           Store store, Sync sync) {
     using R = real_of<A>;
     using P = std::conditional_t<ADJ, PairOf<A>, A>;
@@ -337,6 +342,14 @@ __device__ __forceinline__ bool run_steps(const uint2 *lists, const Group *group
                     if constexpr (ADJ) adjoint2<A>(u, x, a, neg, gs);
                     else rotate2<false, A>(u, x, a, neg);
                 };
+                auto turn_if = [&](bool c, P &u, P &x, const Angle<R> &a, uint32_t neg, GradSum<R> &gs) {
+                    if constexpr (!ADJ && std::is_same<A, double>::value) {
+                        #pragma unroll 1
+                        for (int r = c ? once : 0; r > 0; --r) turn(u, x, a, neg, gs);
+                    } else {
+                        if (c) turn(u, x, a, neg, gs);
+                    }
+                };
                 if (use[v]) {
                     // A from e0, and from e2 where o = 0 or e3 where o = mA; B from e0 (e1) where F (F') holds, else
                     // from e2 (e3).  With the two elements exchanged a rotation is that of the opposite sign.
@@ -344,11 +357,11 @@ __device__ __forceinline__ bool run_steps(const uint2 *lists, const Group *group
                     const uint32_t s0 = (sg[v] >> 1 ^ fl[v] ^ 1u) & 1u, s1 = (sg[v] >> 1 ^ G.cba ^ fl[v] >> 2 ^ 1u) & 1u;
                     auto opA = [&] {
                         turn(e[v][0], e[v][1], aA, a0, gA);
-                        if (a2[v]) turn(e[v][2], e[v][3], aA, a1, gA);
+                        turn_if(a2[v], e[v][2], e[v][3], aA, a1, gA);
                     };
                     auto opB = [&] {
-                        if (b0[v]) turn(e[v][0], e[v][2], aB, s0, gB);
-                        if (b1[v]) turn(e[v][1], e[v][3], aB, s1, gB);
+                        turn_if(b0[v], e[v][0], e[v][2], aB, s0, gB);
+                        turn_if(b1[v], e[v][1], e[v][3], aB, s1, gB);
                     };
                     if constexpr (ADJ) {
                         opB();
@@ -363,7 +376,7 @@ __device__ __forceinline__ bool run_steps(const uint2 *lists, const Group *group
                     if (b1[v] || a2[v]) store(at[v][3], e[v][3]);
                 }
                 if (useB[v]) {
-                    turn(p0[v], p1[v], aB, sq[v], gB);
+                    turn_if(true, p0[v], p1[v], aB, sq[v], gB);
                     store(q0[v], p0[v]);
                     store(q1[v], p1[v]);
                 }
