@@ -24,6 +24,8 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
+#include <type_traits>
+
 #include "sv_internal.h"
 #include "sv_tc.cuh"
 
@@ -38,15 +40,18 @@ constexpr int kTcCols = 512;                           // tensor-memory columns:
 // A tile of TN beta strings.  The tensor core cuts each accumulation to float32, and a sum keeps
 // losing bits at the rate of its largest terms; so the five small piece products have an accumulator
 // of their own and the first pieces' product x1 y1 the rest, K blocks in turn: one with TN = 256,
-// three with TN = 128.  Relative gradient error at 24 qubits: 2.1e-6 to 2.8e-6 with one accumulator
-// for all six, 0.7e-6 to 1.2e-6 with TN = 256.  TN = 128 serves sectors of few tiles (launch_same_tc),
-// where it also has twice the blocks.
+// three with 128, seven with 64.  Relative gradient error at 24 qubits: 2.1e-6 to 2.8e-6 with one
+// accumulator for all six, 0.7e-6 to 1.2e-6 with TN = 256.  The narrow tiles serve sectors of few tiles
+// (launch_same_tc), where they also have more blocks.  Against the sparse float32 sums (variant 3), whose
+// place these products take from 2^14 determinants, the error of a gradient (144 problems of 44,100 to
+// 627,264, geometric mean) is 0.92 of theirs with TN = 128 (1.09 at 511,225) and 0.83 with 64 (0.80 to 0.89
+// at each size).
 template <int TN>
 struct TcTile {
     static constexpr int kMain = kTcCols / TN - 1;                      // accumulators of x1 y1
     static constexpr int kBBytes = TN * kTcKb * 2;                      // one piece of B in one stage
     static constexpr int kStageBytes = 3 * kTcABytes + 3 * kBBytes;
-    static constexpr int kStages = TN == 256 ? 3 : 4;                   // 3 x 72 KB, 4 x 48 KB
+    static constexpr int kStages = TN == 256 ? 3 : TN == 128 ? 4 : 6;   // 3 x 72 KB, 4 x 48 KB, 6 x 36 KB
     static constexpr int kSmem = kStages * kStageBytes + 1024;          // + alignment of the ring to 1024 bytes
 };
 
@@ -272,26 +277,26 @@ cudaError_t launch_same_tc(const uint16_t *M, size_t pm, const uint16_t *X, size
                    sx[3] = {(uint64_t)lda * 2, (uint64_t)Db * lda * 2, (uint64_t)px * 2};
     const uint64_t dt[4] = {(uint64_t)Db, (uint64_t)Da, P, 3},
                    stt[3] = {(uint64_t)ldb * 2, (uint64_t)Da * ldb * 2, (uint64_t)pt * 2};
-    // narrow tiles while every one of them has an SM: 24 qubits (495 strings, real) 46 us wide with the
-    // transposes, 35 us narrow; at 28 qubits (2,002) 256 narrow tiles would take two rounds of the SMs
+    // the narrowest tiles of which every one has an SM: 24 qubits (495 strings, real) 46 us with 256, 35 with
+    // 128 and 33 with 64, the transposes included; 792 strings 61 us with 128, 49 with 64; at 28 qubits (2,002) 256
+    // tiles of 128 would take two rounds of the SMs
     const int tm = (Da + kTcM - 1) / kTcM;
-    const bool narrow = (long long)((Db + 127) / 128) * tm * planes <= sm_count;
-    const uint32_t tn = narrow ? 128 : 256;
+    auto fits = [&](int n) { return (long long)((Db + n - 1) / n) * tm * planes <= sm_count; };
+    const uint32_t tn = fits(64) ? 64 : fits(128) ? 128 : 256;
     if (!encode_map(&ma, M, 3, dma, sma, kTcM) || !encode_map(&mb, M + (size_t)Da * lda, 3, dmb, smb, tn) ||
         !encode_map(&mx, X, 4, dx, sx, tn) || !encode_map(&mt, Xt, 4, dt, stt, kTcM))
         return cudaErrorInvalidValue;
     const TcOut g{G, Da, Db, err, spins, stall};
     const dim3 grid((Db + tn - 1) / tn, tm, planes);
-    if (narrow) {
-        e = cudaFuncSetAttribute(k_same_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcTile<128>::kSmem);
-        if (e != cudaSuccess) return e;
-        k_same_tc<128><<<grid, kTcThreads, TcTile<128>::kSmem, st>>>(ma, mb, mx, mt, g);
-    } else {
-        e = cudaFuncSetAttribute(k_same_tc<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcTile<256>::kSmem);
-        if (e != cudaSuccess) return e;
-        k_same_tc<256><<<grid, kTcThreads, TcTile<256>::kSmem, st>>>(ma, mb, mx, mt, g);
-    }
-    return cudaGetLastError();
+    auto launch = [&](auto tile) -> cudaError_t {
+        constexpr int TN = decltype(tile)::value, smem = TcTile<TN>::kSmem;
+        if ((e = allow_smem(k_same_tc<TN>, smem)) != cudaSuccess) return e;
+        k_same_tc<TN><<<grid, kTcThreads, smem, st>>>(ma, mb, mx, mt, g);
+        return cudaGetLastError();
+    };
+    if (tn == 64) return launch(std::integral_constant<int, 64>());
+    if (tn == 128) return launch(std::integral_constant<int, 128>());
+    return launch(std::integral_constant<int, 256>());
 }
 
 // The three bf16 pieces of n floats (piece stride `piece` elements).
