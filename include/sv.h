@@ -26,8 +26,10 @@
  * basis index x (sv_create), or only the amplitudes of one (N_alpha, N_beta)
  * sector (sv_create_sector); complex amplitudes interleaved (re, im) in float
  * (SV_C64) or double (SV_C128), or real amplitudes (SV_R32, SV_R64).  Every
- * reduction (energy, gradient, norm, density matrix) is accumulated and returned
- * in float64 whatever the state precision.
+ * reduction (energy, gradient, norm, density matrix) is returned in float64 whatever
+ * the state precision, and accumulated in float64 or, from float32 terms, in two or
+ * three float32 words whose unevaluated sum has at least 48 bits (the 1-RDM's sums
+ * over one row group: in the amplitudes' own type).
  *
  * Ownership: the caller owns every host array passed in and out; the library
  * copies what it keeps.  Device buffers are owned by the library unless they

@@ -488,13 +488,48 @@ __device__ __noinline__ void sigma_blocked(const BatchArgs<R> &B, const BatchIns
     }
 }
 
-// A float32 sum with its rounding kept (hi + lo), or a float64 one: energies and norms without FP64
-// work for float32 states (products of float32 words are exact as such pairs).
-__device__ __forceinline__ void add_product(GradSum<float> &s, float x, float y) {
-    const float p = x * y;
-    s.v = s.v + ff(p, fmaf(x, y, -p));
-}
-__device__ __forceinline__ void add_product(GradSum<double> &s, double x, double y) { s.v = fma(x, y, s.v); }
+// Sums of products for the energy and the norm.  float32: no FP64 work, and no less than its precision: a
+// product is two words exactly, the sum three that pass their rounding on (about 72 bits).
+template <typename R> struct DotSum;
+template <> struct DotSum<float> {
+    float a = 0.f, b = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        float e, f;
+        two_sum(a, x, a, e);
+        two_sum(b, e, b, f);
+        c += f;
+    }
+    __device__ __forceinline__ void add(const DotSum &o) {
+        add(o.a);
+        add(o.b);
+        add(o.c);
+    }
+    __device__ __forceinline__ void add_product(float x, float y) {
+        const float p = x * y;
+        add(p);
+        add(fmaf(x, y, -p));
+    }
+    __device__ __forceinline__ DotSum xor_lane(int m) const {
+        DotSum o;
+        o.a = __shfl_xor_sync(0xffffffffu, a, m);
+        o.b = __shfl_xor_sync(0xffffffffu, b, m);
+        o.c = __shfl_xor_sync(0xffffffffu, c, m);
+        return o;
+    }
+    __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
+template <> struct DotSum<double> {
+    double a = 0.0;
+    __device__ __forceinline__ void add(const DotSum &o) { a += o.a; }
+    __device__ __forceinline__ void add_product(double x, double y) { a = fma(x, y, a); }
+    __device__ __forceinline__ DotSum xor_lane(int m) const {
+        DotSum o;
+        o.a = __shfl_xor_sync(0xffffffffu, a, m);
+        return o;
+    }
+    __device__ __forceinline__ double value() const { return a; }
+};
+// A gradient sum (GradSum::bits) as float64.
 __device__ __forceinline__ double sum_value(double bits, float) {
     return (double)__int_as_float(__double2hiint(bits)) + (double)__int_as_float(__double2loint(bits));
 }
@@ -548,28 +583,28 @@ __device__ __noinline__ void run_blocked(const BatchArgs<R> &B, const BatchInst 
     sigma_blocked<R, SM>(B, I, scratch, at, rest, team);
     team.sync();
     stage();  // sigma worked where the lists were
-    GradSum<R> e, n;
+    DotSum<R> e, n;
     for (int b = warp; b < I.Db; b += nw) {
         const uint32_t pb = prefix_parity(strb[b]);
         for (int a = lane; a < Da; a += 32) {
             const uint32_t f = parity32(stra[a] & pb);
             const PairOf<R> p = own[b * Da + a];
-            add_product(e, p.c, p.l);
-            add_product(n, p.c, p.c);
+            e.add_product(p.c, p.l);
+            n.add_product(p.c, p.c);
             own[b * Da + a] = PairOf<R>{flip(p.c, f), flip(p.l, f)};
         }
     }
     // energy (lower half warp) and norm (upper) in one tree, then the warps in order
-    GradSum<R> mine = lane < 16 ? e : n, other = lane < 16 ? n : e;
+    DotSum<R> mine = lane < 16 ? e : n, other = lane < 16 ? n : e;
     mine.add(other.xor_lane(16));
     #pragma unroll
     for (int o = 8; o > 0; o >>= 1) mine.add(mine.xor_lane(o));
-    if ((lane & 15) == 0) red[2 * warp + (lane >> 4)] = mine.bits();
+    if ((lane & 15) == 0) red[2 * warp + (lane >> 4)] = mine.value();
     team.sync();
     double se = 0.0, sn = 0.0;
     for (int w = 0; w < nw; ++w) {
-        se += sum_value(red[2 * w], (R)0);
-        sn += sum_value(red[2 * w + 1], (R)0);
+        se += red[2 * w];
+        sn += red[2 * w + 1];
     }
     if (tid == 0) B.out[I.out] = I.shift + se / sn;
     run_steps<R, true, 1>(lists, groups, angles, I.n_groups, Da, (size_t)D, tid, NT, warp, nw, 1, gsum,

@@ -6,9 +6,8 @@
 //   grid     every SM, amplitudes in L2, a counter in global memory; launched cooperatively, and
 //            each wait bounded: past the limit the block sets *err and stops
 // The reverse sweep works on psi and lambda interleaved (one access moves both) and takes the
-// gradient terms of both operators; each warp's sum leaves the chip (float32 states: as an
-// error-free sum of hi + lo words, since GB300 adds float64 at 1/64 of its float32 rate), and
-// k_sweep_grad adds the warps' in order.
+// gradient terms of both operators; each warp's sum leaves the chip (float32 states: as two words hi + lo,
+// 48 bits, since GB300 adds float64 at 1/64 of its float32 rate), and k_sweep_grad adds the warps' in order.
 #include <algorithm>
 #include <vector>
 

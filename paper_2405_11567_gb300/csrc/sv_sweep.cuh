@@ -132,7 +132,8 @@ struct alignas(2 * sizeof(A)) PairOf {
     A c, l;
 };
 
-// Sums of a thread's gradient terms: float32 terms error-free (hi + lo), float64 terms as they are.
+// Sums of a thread's gradient terms: float32 terms in two words (hi + lo, 48 bits: lo takes the rounding
+// of hi and rounds itself, at 2^-24 of a term's own rounding), float64 terms as they are.
 template <typename R> struct GradSum;
 template <> struct GradSum<float> {
     ff v = ff(0);
