@@ -46,7 +46,8 @@ SIGMA_KERNELS = {
        "+ k_sigma_ab + k_sigma_comb",
     5: "expectation: k_phase_planar + k_transpose_pieces + k_same_tc (same-spin products) + k_ab_tc "
        "(alpha-beta products; both tcgen05 bf16x3) + k_sigma_comb (gathers the alpha-beta planes)",
-    6: "expectation: k_max_word + k_phase_digits + k_transpose_digits + k_same_digits + k_ab_digits (exact integer "
+    6: "expectation: k_to_ff + k_sigma_ab + k_sigma_same (float-float)",
+    0: "expectation: k_max_word + k_phase_digits + k_transpose_digits + k_same_digits + k_ab_digits (exact integer "
        "products, tcgen05 on bf16 digits) + k_comb_digits"}
 # Measured DRAM traffic lives in a small committed record written from ncu captures
 # (--record-traffic), keyed by a hash of the sources of the kernels it measured: a
@@ -526,7 +527,7 @@ def run_ours(args, rank, world, local_rank):
         v128 = throughput(world, K, head128["ms"])
         line["fp64_state"] = {"value": v128, "ms_per_step": head128["ms"] / K, "phases_ms": head128["phases"],
                               "clocks": head128["clocks"],
-                              "expectation_form": SIGMA_KERNELS.get(head128["variant"] or 6,
+                              "expectation_form": SIGMA_KERNELS.get(head128["variant"],
                                                                     "expectation form %d" % head128["variant"]),
                               "tensor_kernels": digit_kernels(p, head128["phases"]),
                               "vs_oracle": vs_golden(head128["out"], golden) if golden is not None else None}

@@ -335,7 +335,9 @@ typedef enum {
                                        space of at most 4096 strings, where variant 5's
                                        limits hold and its planes take at most 16 GiB
                                        within the byte cap, else 4 for those states;
-                                       = 6 for complex128 / real float64 states where
+                                       the digit products, below, for real float64
+                                       states of at least 2^12; = 6 for other
+                                       complex128 / real float64 states where
                                        the split form's rows fit in shared memory (3
                                        when its two work matrices do not fit the byte
                                        cap); else 3 where its rows fit in shared
@@ -370,13 +372,24 @@ typedef enum {
                                        FP32 pipe instead of GB300's much narrower FP64
                                        pipe; the amplitudes are converted once per call
                                        and sigma written back as float64 (two work
-                                       matrices of 16 Da Db bytes, complex).  Real float64
-                                       amplitudes (also a complex128 handle's with a real
-                                       reference) of a sector of at least 2^12 determinants
-                                       that meets variant 5's limits and couplings: the same sums as integer products
-                                       of seven base-256 digits on the tensor cores,
-                                       accumulated exactly (planes of 8 bytes: 3.7 GB at 30
-                                       qubits; float-float where the memory cannot be had) */
+                                       matrices of 16 Da Db bytes, complex).
+                                       The digit products (0 alone chooses them): real
+                                       float64 amplitudes (also a complex128 handle's with
+                                       a real reference) of a sector of at least 2^12
+                                       determinants that meets variant 5's limits and
+                                       couplings; the same sums as integer products of
+                                       seven base-256 digits on the tensor cores (planes of
+                                       8 bytes: 3.7 GB at 30 qubits; 6 where the memory
+                                       cannot be had).  Every amplitude, matrix and table
+                                       element is a fixed-point number of 56 bits under the
+                                       largest of its kind, and the sums of the 28 leading
+                                       digit products are exact: an element of sigma is off
+                                       by about 2^-54 of the largest terms of a row,
+                                       whatever its own size (an amplitude of 2^-20 of the
+                                       largest has 36 bits), where 6 has 48 bits of each
+                                       term.  Energies and gradients come out closer with
+                                       the digits; a caller who needs small elements of
+                                       sigma to their own precision takes 6 or 3 */
     SV_OPT_RDM_VARIANT = 4,         /* 0 auto (3 for float64 states, else 2); 1 sector
                                        gather: one thread per sector determinant (dense
                                        storage only); 2 string rows: one block per beta
@@ -499,7 +512,7 @@ sv_status sv_get_option(sv_handle h, sv_option opt, int64_t *value);
 /* Autotuner: time, on this handle's device with CUDA events, the candidate launch
  * choices for the given Hamiltonian and ansatz (ops/theta as for sv_energy_grad)
  * and keep the fastest -- the expectation's form and partner-row chunk size
- * (SV_OPT_EXPECT_VARIANT 2 to 5, SV_OPT_AB_CHUNK), the rotation and adjoint kernels'
+ * (SV_OPT_EXPECT_VARIANT 2 to 6, or 0 where the digit products win, SV_OPT_AB_CHUNK), the rotation and adjoint kernels'
  * blocks per SM (4, 8, 16, 32; dense storage, or sector storage with one launch per
  * operator), the whole-sweep launches' (1, 2, 4, 8; sector storage,
  * SV_OPT_SWEEP_BLOCKS_PER_SM) and the 1-RDM's (2, 4, 8, 16).

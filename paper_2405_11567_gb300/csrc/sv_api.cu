@@ -1258,7 +1258,7 @@ static sv_status ensure_same_gemm(sv_handle h, DevTables *T, const RowTables &R,
 // The string-row expectation (sigma into lam at storage addresses, or into lamc in
 // compact form), with or without the same-spin products; counts the launches.
 // Whether the expectation takes the float-float split form (variant 6): float64 states
-// whose split form fits; the automatic choice (variant 0) for them.
+// whose split form fits; the automatic choice (variant 0) for them without the digit products.
 static bool use_ff(sv_handle h, int K) {
     if (single_prec(h->dtype) || K == 0) return false;
     return h->expect_variant == 6 || h->expect_variant == 0;
@@ -1334,14 +1334,14 @@ struct DigitBytes {
     }
 };
 
-// Whether the float-float expectation (variant 6, or the automatic choice of float64 states) takes the
-// digit products (k_digits.cu): real float64 sectors of at least 2^12 determinants within their limits
+// Whether the automatic choice of float64 states takes the digit products (k_digits.cu) where it would take
+// the float-float form (variant 6): real float64 sectors of at least 2^12 determinants within their limits
 // and with dense same-spin couplings, finite integrals, planes H of at most 16 GiB, everything under the
 // handle's byte cap.  Measured, float-float / digits
 // in us: 3,136 determinants 63.9 / 66.0, 4,356 78.0 / 74.1, 4,900 71.0 / 70.5, 7,056 76.2 / 69.7, 15,876
 // 94 / 74, 44,100 173 / 100, 108,900 390 / 145, 245,025 668 / 222, 9,018,009 39,100 / 8,550.
 static bool use_digits(sv_handle h, const DevTables *T) {
-    if (h->dtype != SV_R64 || (h->expect_variant != 0 && h->expect_variant != 6)) return false;
+    if (h->dtype != SV_R64 || h->expect_variant != 0) return false;
     if ((double)h->Da * h->Db < (double)(1 << 12) || !digits_fit(h->Da, h->Db, h->nb, h->n / 2) || !dense_couplings(h))
         return false;
     if (!(T->eri_max < 1e100 && T->h_max < 1e100)) return false;
@@ -1778,14 +1778,15 @@ static sv_status autotune_impl(sv_handle h, sv_ham_handle ham, const std::vector
         int64_t best_k = 0;
         float best_t = -1.f;
         // split form; same-spin products and the tensor-core alpha-beta form (single
-        // precision); the float-float split form (float64)
+        // precision); the float-float split form, and the digit products (the automatic
+        // choice, 0; float64)
         const bool sp = single_prec(h->dtype);
-        for (int i = -1; i < (sp ? 9 : 8); ++i) {
-            h->expect_variant = i < 0 ? 2 : (i < 4 ? 3 : (!sp ? 6 : (i < 8 ? 4 : 5)));
+        for (int i = -1; i < 9; ++i) {
+            h->expect_variant = i < 0 ? 2 : (i < 4 ? 3 : i < 8 ? (sp ? 4 : 6) : sp ? 5 : 0);
             h->ab_chunk = i < 0 ? 0 : (i < 8 ? sizes[i & 3] : 0);
             if (i >= 0 && i < 8 && row_chunk(h, R) != sizes[i & 3]) continue;  // that size does not fit
             if (sp && i >= 4 && !use_same_gemm(h, row_chunk(h, R))) continue;
-            if (i == 8 && !use_ab_tc(h)) continue;
+            if (i == 8 && !(sp ? use_ab_tc(h) : use_digits(h, T))) continue;
             const float t = time_best(h, e0, e1, [&] { return expectation(h, ham, T, h->lam, c, 0); });
             if (t < 0.f) return fail(h, SV_ERR_CUDA, "autotune: expectation candidate failed");
             if (best_t < 0.f || t < best_t) {

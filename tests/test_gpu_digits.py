@@ -100,3 +100,28 @@ def test_bounded_wait_runs_out_reports_and_recovers(stall):
     st.prepare_hf(occ)
     assert abs(st.energy_grad(ham, ops, theta)[0] - Eref) <= TOL_E
     st.close()
+
+
+def test_float_float_can_be_chosen():
+    """Variant 6 is the float-float form also where the automatic choice is the digit products: it has a sigma
+    element of an amplitude 2^-44 of the largest, coupled to no other, to its own precision (48 bits a term).
+    The gradient of the single excitation from that determinant at zero angle is that element alone."""
+    n, na, nb = 20, 4, 4
+    p = inputs.make_problem(n, 8, 4, seed=5)
+    ham = sv.Hamiltonian(p["h"], p["eri"], p["e_nuc"])
+    bits = lambda orbs: sum((1 << 2 * q) | (1 << (2 * q + 1)) for q in orbs)  # noqa: E731
+    psi = np.zeros(1 << n)
+    psi[bits(range(4))] = 1.0
+    psi[bits(range(6, 10))] = 0.7 * 2.0 ** -44      # eight excitations away
+    op = np.array([(1, 12, -1, 10, -1)], np.int32)  # alpha, orbital 6 -> 5
+    g = {}
+    for variant in (0, 3, 6):
+        st = sv.StateVector(n, "r64", sector=(na, nb))
+        st.set_option(sv.SV_OPT_EXPECT_VARIANT, variant)
+        st.prepare_state(psi, na, nb)
+        g[variant] = st.energy_grad(ham, op, [0.0])[1][0]
+        st.close()
+    assert abs(g[3]) > 1e-30
+    assert abs(g[6] - g[3]) <= 1e-12 * abs(g[3])     # some tens of terms of 2^-47
+    assert abs(g[0] - g[3]) <= 2.0 ** -90            # an absolute 2^-52 of the largest, times the amplitude
+    ham.close()
