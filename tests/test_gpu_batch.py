@@ -147,3 +147,58 @@ def test_batch_shared_memory_just_below_48_kb(dtype, n, na, nb, n_ops):
     for k in range(2):
         assert abs(E[k] - Er) <= tE and np.max(np.abs(g[k] - gr)) <= tg
     b.close()
+
+
+def _small(n, ne, n_ops, seed):
+    p = inputs.make_problem(n, ne, 4, seed=seed)
+    pool = inputs.uccsd_pool(n, ne)
+    rng = np.random.default_rng(seed)
+    p["ops"] = np.ascontiguousarray(pool[rng.integers(0, len(pool), n_ops)])
+    p["theta"] = rng.normal(0.0, 0.2, n_ops)
+    return p
+
+
+def _check(probs, E, g, dtype, picked):
+    tE, tg = TOL[dtype]
+    for k in picked:
+        Er, gr = _oracle(probs[k])
+        assert abs(E[k] - Er) <= tE, (k, probs[k]["n_qubits"])
+        assert np.max(np.abs(g[k] - gr), initial=0.0) <= tg, (k, probs[k]["n_qubits"])
+
+
+@pytest.mark.parametrize("dtype", ["c128", "c64"])
+@pytest.mark.parametrize("big", [False, True])
+@pytest.mark.parametrize("count", [310, 620])
+def test_batch_of_teams(count, big, dtype):
+    """Small instances on half (310: at least two to an SM) and quarter blocks (620: four), alone and behind
+    one that takes a whole block: every distinct problem against the oracle, copies of one bit for bit."""
+    base = [_small(4, 2, 3, 1), _small(8, 2, 9, 2), _small(8, 4, 20, 3), _small(10, 4, 25, 4), _small(12, 4, 7, 5),
+            dict(_small(12, 6, 30, 6)), _small(10, 4, 0, 7)]
+    probs = ([_small(18, 6, 30, 8)] if big else []) + [base[k % len(base)] for k in range(count)]
+    b = sv.Batch(probs, dtype)
+    theta = np.concatenate([p["theta"] for p in probs])
+    first = int(big)
+    for again in range(2):
+        E, g = b.energy_grad(theta)
+        _check(probs, E, g, dtype, range(first + len(base)))
+        for k in range(first, len(probs)):
+            j = first + (k - first) % len(base)
+            assert E[k] == E[j] and np.array_equal(g[k], g[j]), k
+        if not again:
+            b.autotune(theta)          # shared memory planned for one thread count, run with another
+    b.close()
+
+
+@pytest.mark.parametrize("dtype", ["c128", "c64"])
+@pytest.mark.parametrize("n,ne,n_ops", [(12, 6, 1500), (18, 6, 1200)])
+def test_batch_lists_that_do_not_fit(n, ne, n_ops, dtype):
+    """Operator lists longer than the shared memory beside the state: read from global memory; a batch of
+    one, and one whose quarter blocks have little each."""
+    p = _small(n, ne, n_ops, 40)
+    for copies in (1, 610 if n == 12 else 2):
+        b = sv.Batch([p] * copies, dtype)
+        E, g = b.energy_grad(np.concatenate([p["theta"]] * copies))
+        _check([p], E, g, dtype, [0])
+        for k in range(1, copies):
+            assert E[k] == E[0] and np.array_equal(g[k], g[0])
+        b.close()
