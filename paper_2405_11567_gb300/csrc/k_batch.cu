@@ -50,7 +50,6 @@ int plan_groups(const OpDesc *ops, int n_ops, int N, int na, int nb, std::vector
 struct BatchOp {
     uint32_t m, from, sm;  // qubit-space flip mask, "from" pattern, sign mask
     uint32_t mab;          // low 16 bits: alpha-string flip mask, high 16: beta-string flip mask
-    uint32_t fab;          // the same for the "from" pattern
 };
 
 struct BatchInst {
@@ -1012,12 +1011,7 @@ sv_status build_plan(sv_batch *b, int n_inst, const sv_instance *inst) {
                 if ((d.m >> (2 * p)) & 1u) ma |= 1u << p;
                 if ((d.m >> (2 * p + 1)) & 1u) mb |= 1u << p;
             }
-            uint32_t fa = 0, fb = 0;
-            for (int p = 0; p < N; ++p) {
-                if ((d.from >> (2 * p)) & 1u) fa |= 1u << p;
-                if ((d.from >> (2 * p + 1)) & 1u) fb |= 1u << p;
-            }
-            hops.push_back(BatchOp{d.m, d.from, d.sm, ma | (mb << 16), fa | (fb << 16)});
+            hops.push_back(BatchOp{d.m, d.from, d.sm, ma | (mb << 16)});
             descs.push_back(d);
         }
         if (I.fast) {
