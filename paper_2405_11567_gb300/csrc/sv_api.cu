@@ -214,6 +214,21 @@ static sv_status dev_alloc(sv_handle h, void **p, size_t bytes, const char *what
     return SV_OK;
 }
 
+// For a buffer that grows with a list an operator at a time: half as much again where that can be had, so that
+// not every call allocates.
+static sv_status dev_alloc_growing(sv_handle h, void **p, size_t bytes, size_t *have, const char *what) {
+    const size_t more = bytes + bytes / 2;
+    sv_status st = dev_alloc(h, p, more, what, true);
+    if (st == SV_OK) {
+        *have = more;
+        return st;
+    }
+    cudaGetLastError();
+    st = dev_alloc(h, p, bytes, what);
+    *have = st == SV_OK ? bytes : 0;
+    return st;
+}
+
 static void dev_free(sv_handle h, void *p, size_t bytes) {
     if (!p) return;
     cudaFree(p);
@@ -1001,9 +1016,7 @@ static sv_status ensure_sweep_part(sv_handle h, size_t doubles) {
     dev_free(h, h->sweep_part, h->sweep_part_bytes);
     h->sweep_part = nullptr;
     h->sweep_part_bytes = 0;
-    SV_TRY(dev_alloc(h, (void **)&h->sweep_part, need, "sweep gradient sums"));
-    h->sweep_part_bytes = need;
-    return SV_OK;
+    return dev_alloc_growing(h, (void **)&h->sweep_part, need, &h->sweep_part_bytes, "sweep gradient sums");
 }
 
 // The steps, angles, flag and sums of a whole sweep over ops and its form; form -1 where the memory for them
@@ -2426,7 +2439,10 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
         SV_TRY(ensure_strings(h));
         need = 3 * (size_t)h->Db;
     }
-    SV_TRY(ensure_partials(h, std::max<size_t>((size_t)G * std::max<size_t>(L, 1), need)));
+    // (where one launch per operator runs: its gradient sums [L][G])
+    const size_t per_op = (size_t)G * std::max<size_t>(L, 1);
+    const bool whole = sect && h->sweep_mode && h->ckpt_interval <= 0 && L > 0;
+    SV_TRY(ensure_partials(h, whole ? need : std::max<size_t>(per_op, need)));
     plan_checkpoints(h, L);
     h->prepared = false;
     h->tc_timed = 0;
@@ -2444,9 +2460,7 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
     const int64_t C = h->ckpt_interval;
     bool inter = sect && C <= 0 && L > 0;
     SweepShape shape;
-    if (inter && h->sweep_mode) {  // a whole sweep: it interleaves psi and lambda itself
-        SV_TRY(prepare_sweep(h, true, d, &shape));
-    }
+    if (whole) SV_TRY(prepare_sweep(h, true, d, &shape));  // it interleaves psi and lambda itself
     if (inter && shape.form != 0 && ensure_clbuf(h) != SV_OK) {
         cudaGetLastError();
         inter = false;
@@ -2489,6 +2503,7 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
             SV_CUDA(h, cudaMemcpyAsync(wpsi, h->psi, vec_bytes(h), cudaMemcpyDeviceToDevice, h->stream));
         }
     }
+    if (!swept) SV_TRY(ensure_partials(h, per_op));
     if (inter && !swept) {
         SV_TRY(ensure_op_lists(h, d, h->lists));
         SV_CUDA(h, launch_interleave(h->psi, h->lam, h->dtype, h->CLbuf, (size_t)h->Da * h->Db, h->sm_count,
