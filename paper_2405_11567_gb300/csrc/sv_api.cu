@@ -464,10 +464,7 @@ static sv_status ensure_sector(sv_handle h) {
 static sv_status ensure_strings(sv_handle h) {
     if (h->str_sa && h->str_na == h->na && h->str_nb == h->nb) return SV_OK;
     // the old tables go first, and no sector has any until all of them are there
-    for (void *p : {(void *)h->str_sa, (void *)h->str_sb, (void *)h->str_sa_s, (void *)h->str_sb_s,
-                    (void *)h->str_a, (void *)h->str_b, (void *)h->rank_a, (void *)h->rank_b})
-        cudaFree(p);
-    h->bytes_owned -= std::min<uint64_t>(h->bytes_owned, h->str_bytes);
+    dev_free(h, h->str_sa, h->str_bytes);
     h->str_bytes = 0;
     h->str_sa = h->str_sb = h->str_sa_s = h->str_sb_s = nullptr;
     h->str_a = h->str_b = h->rank_a = h->rank_b = nullptr;
@@ -510,20 +507,37 @@ static sv_status ensure_strings(sv_handle h) {
         spb[i] = x;
         spb_s[i] = map_bits(x, h->perm);
     }
-    auto up = [&](void **dst, const void *src, size_t nb) -> sv_status {
-        SV_TRY(dev_alloc(h, dst, std::max<size_t>(nb, 16), "string tables"));
-        h->str_bytes += std::max<size_t>(nb, 16);
-        SV_CUDA(h, cudaMemcpy(*dst, src, nb, cudaMemcpyHostToDevice));
-        return SV_OK;
+    // one allocation and one copy for all eight (a new problem makes them first thing; eight of each took longer
+    // than an evaluation at 8 qubits)
+    std::vector<uint8_t> host;
+    size_t at[8];
+    int n_tab = 0;
+    auto put = [&](const void *src, size_t nb) {
+        at[n_tab++] = host.size();
+        host.insert(host.end(), (const uint8_t *)src, (const uint8_t *)src + nb);
+        host.resize((host.size() + 15) / 16 * 16);
     };
-    SV_TRY(up((void **)&h->str_sa, spa.data(), spa.size() * 4));
-    SV_TRY(up((void **)&h->str_sb, spb.data(), spb.size() * 4));
-    SV_TRY(up((void **)&h->str_sa_s, spa_s.data(), spa_s.size() * 4));
-    SV_TRY(up((void **)&h->str_sb_s, spb_s.data(), spb_s.size() * 4));
-    SV_TRY(up((void **)&h->str_a, sa16.data(), sa16.size() * 2));
-    SV_TRY(up((void **)&h->str_b, sb16.data(), sb16.size() * 2));
-    SV_TRY(up((void **)&h->rank_a, ra.data(), ra.size() * 2));
-    SV_TRY(up((void **)&h->rank_b, rb.data(), rb.size() * 2));
+    put(spa.data(), spa.size() * 4);
+    put(spb.data(), spb.size() * 4);
+    put(spa_s.data(), spa_s.size() * 4);
+    put(spb_s.data(), spb_s.size() * 4);
+    put(sa16.data(), sa16.size() * 2);
+    put(sb16.data(), sb16.size() * 2);
+    put(ra.data(), ra.size() * 2);
+    put(rb.data(), rb.size() * 2);
+    void *tab = nullptr;
+    SV_TRY(dev_alloc(h, &tab, host.size(), "string tables"));
+    h->str_bytes = host.size();
+    h->str_sa = (uint32_t *)tab;  // (the allocation's start: freed by it)
+    SV_CUDA(h, cudaMemcpy(tab, host.data(), host.size(), cudaMemcpyHostToDevice));
+    auto where = [&](int t) { return (uint8_t *)tab + at[t]; };
+    h->str_sb = (uint32_t *)where(1);
+    h->str_sa_s = (uint32_t *)where(2);
+    h->str_sb_s = (uint32_t *)where(3);
+    h->str_a = (uint16_t *)where(4);
+    h->str_b = (uint16_t *)where(5);
+    h->rank_a = (uint16_t *)where(6);
+    h->rank_b = (uint16_t *)where(7);
     h->Da = (int)sa16.size();
     h->Db = (int)sb16.size();
     h->h_stra = sa16;
@@ -2028,9 +2042,7 @@ static void destroy_handle(sv_handle h) {
     if (!h->lam_pair) dev_free(h, h->saved, vec_bytes(h));
     for (void *p : h->ckpt) dev_free(h, p, vec_bytes(h));
     dev_free(h, h->sector, h->sector_len * sizeof(uint32_t));
-    for (void *p : {(void *)h->str_sa, (void *)h->str_sb, (void *)h->str_sa_s, (void *)h->str_sb_s,
-                    (void *)h->str_a, (void *)h->str_b, (void *)h->rank_a, (void *)h->rank_b})
-        if (p) cudaFree(p);
+    dev_free(h, h->str_sa, h->str_bytes);
     dev_free(h, h->Cbuf, h->Cbuf_bytes);
     dev_free(h, h->Lbuf, h->Lbuf_bytes);
     dev_free(h, h->sg_mats, h->sg_mats_bytes);
