@@ -214,17 +214,18 @@ static sv_status dev_alloc(sv_handle h, void **p, size_t bytes, const char *what
     return SV_OK;
 }
 
-// For a buffer that grows with a list an operator at a time: half as much again where that can be had, so that
-// not every call allocates.
+// For a buffer that grows with a list an operator at a time: half as much again where that can be had (under a byte
+// cap it could be what a later buffer needs), so that not every call allocates.
 static sv_status dev_alloc_growing(sv_handle h, void **p, size_t bytes, size_t *have, const char *what) {
     const size_t more = bytes + bytes / 2;
-    sv_status st = dev_alloc(h, p, more, what, true);
-    if (st == SV_OK) {
-        *have = more;
-        return st;
+    if (h->max_bytes <= 0) {
+        if (dev_alloc(h, p, more, what, true) == SV_OK) {
+            *have = more;
+            return SV_OK;
+        }
+        cudaGetLastError();
     }
-    cudaGetLastError();
-    st = dev_alloc(h, p, bytes, what);
+    const sv_status st = dev_alloc(h, p, bytes, what);
     *have = st == SV_OK ? bytes : 0;
     return st;
 }
@@ -860,6 +861,7 @@ static sv_status upload_sweep_angles(sv_handle h, const std::vector<OpDesc> &ops
     if (!ops.empty())
         SV_CUDA(h, cudaMemcpyAsync((uint8_t *)h->sweep_buf + 256, h->sweep_host.data(), one * ops.size(),
                                    cudaMemcpyHostToDevice, h->stream));
+    h->sweep_fresh = true;
     return SV_OK;
 }
 
@@ -890,18 +892,23 @@ static sv_status ensure_groups(sv_handle h, const std::vector<OpDesc> &ops) {
         c.buf = nullptr;
         c.bytes = 0;
         c.key.clear();
-        SV_TRY(dev_alloc(h, &c.buf, need, "sweep steps"));
-        c.bytes = need;
+        SV_TRY(dev_alloc_growing(h, &c.buf, need, &c.bytes, "sweep steps"));
     }
     c.key.clear();  // until all of it is written: a call that fails halfway leaves no steps of either list
     uint8_t *dp = (uint8_t *)c.buf + lb;
-    SV_CUDA(h, cudaMemcpyAsync(dp, plans.data(), plans.size(), cudaMemcpyHostToDevice, h->stream));
-    SV_CUDA(h, cudaMemcpyAsync(dp + pb, groups.data(), groups.size(), cudaMemcpyHostToDevice, h->stream));
+    // one copy, from memory that stays as it is until the copy is done (no wait for the stream: a call on a new
+    // list goes on to its sweep)
+    if (h->groups_copied) SV_CUDA(h, cudaEventSynchronize(h->groups_copied));
+    else SV_CUDA(h, cudaEventCreateWithFlags(&h->groups_copied, cudaEventDisableTiming));
+    h->groups_host.assign(pb + groups.size(), 0);
+    std::copy(plans.begin(), plans.end(), h->groups_host.begin());
+    std::copy(groups.begin(), groups.end(), h->groups_host.begin() + pb);
+    SV_CUDA(h, cudaMemcpyAsync(dp, h->groups_host.data(), h->groups_host.size(), cudaMemcpyHostToDevice, h->stream));
+    SV_CUDA(h, cudaEventRecord(h->groups_copied, h->stream));
     SV_CUDA(h, launch_build_groups(dp, n, h->str_sa, h->str_sb, h->str_a, h->str_b, h->rank_a, h->rank_b, h->Da, h->Db,
                                    single_prec(h->dtype) ? 0 : 1, c.buf,
                                    h->stream));
     h->launches++;
-    SV_CUDA(h, cudaStreamSynchronize(h->stream));  // the host staging vectors go out of scope
     c.key = key;
     c.dgroups = dp + pb;
     c.n_groups = n;
@@ -918,6 +925,7 @@ static void drop_sweep(sv_handle h) {
     dev_free(h, h->sweep_buf, h->sweep_bytes);
     dev_free(h, h->sweep_part, h->sweep_part_bytes);
     h->groups = SweepGroups();
+    h->sweep_fresh = false;
     h->sweep_buf = nullptr;
     h->sweep_part = nullptr;
     h->sweep_bytes = h->sweep_part_bytes = 0;
@@ -1038,7 +1046,7 @@ static sv_status ensure_sweep_part(sv_handle h, size_t doubles) {
 static sv_status prepare_sweep(sv_handle h, bool adjoint, const std::vector<OpDesc> &ops, SweepShape *s) {
     *s = SweepShape();
     sv_status st = ensure_groups(h, ops);
-    if (st == SV_OK) st = upload_sweep_angles(h, ops);
+    if (st == SV_OK && !(adjoint && h->sweep_fresh && h->sweep_buf)) st = upload_sweep_angles(h, ops);
     if (st == SV_OK) {
         *s = sweep_shape(h, adjoint, ops.size());
         if (s->form == 2) st = ensure_kerr(h);
@@ -2061,6 +2069,7 @@ static void destroy_handle(sv_handle h) {
     dev_free(h, h->partials, h->partials_cap * sizeof(double));
     dev_free(h, h->dout, h->dout_cap * sizeof(double));
     if (h->hpinned) cudaFreeHost(h->hpinned);
+    if (h->groups_copied) cudaEventDestroy(h->groups_copied);
     for (cudaEvent_t e : h->ev)
         if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : h->tcev)
@@ -2451,13 +2460,15 @@ static sv_status energy_grad_run(sv_handle h, sv_ham_handle ham, const std::vect
         SV_TRY(ensure_strings(h));
         need = 3 * (size_t)h->Db;
     }
-    // (where one launch per operator runs: its gradient sums [L][G])
+    // where one launch per operator runs, its gradient sums [L][G]; under a byte cap in any case, before checkpoints
+    // and the sweep's own buffers take their place
     const size_t per_op = (size_t)G * std::max<size_t>(L, 1);
     const bool whole = sect && h->sweep_mode && h->ckpt_interval <= 0 && L > 0;
-    SV_TRY(ensure_partials(h, whole ? need : std::max<size_t>(per_op, need)));
+    SV_TRY(ensure_partials(h, whole && h->max_bytes <= 0 ? need : std::max<size_t>(per_op, need)));
     plan_checkpoints(h, L);
     h->prepared = false;
     h->tc_timed = 0;
+    h->sweep_fresh = false;
     SV_TRY(mark(h, 0, "sv_energy_grad: reference"));
     if (!sect) SV_TRY(prepare_reference(h));
     SV_TRY(mark(h, 1, "sv_energy_grad: forward sweep"));

@@ -314,6 +314,8 @@ struct sv_ctx {
     // rotations and adjoint steps) and the screened pool's
     OpLists lists, pool_lists;
     SweepGroups groups;        // the ansatz's steps for whole sector sweeps
+    std::vector<uint8_t> groups_host;     // their plans and groups on the way to the device
+    cudaEvent_t groups_copied = nullptr;  // when they are there
     OpLists rdm_lists;         // the 1-RDM's pair lists of both spins (per orbital pair p < q)
     void *CLbuf = nullptr;     // compact amplitudes and sigma interleaved [Db][Da][2] (screening)
     size_t CLbuf_bytes = 0;
@@ -348,6 +350,7 @@ struct sv_ctx {
     // counter (first 256 bytes) and the ops' (cos, sin) on the device, their host staging
     void *sweep_buf = nullptr;
     size_t sweep_bytes = 0;
+    bool sweep_fresh = false;  // sweep_buf holds the angles of the evaluation that runs (its reverse sweep takes them)
     double *sweep_part = nullptr;  // a reverse sweep's gradient sums
     size_t sweep_part_bytes = 0;
     std::vector<double> sweep_host;
