@@ -362,17 +362,20 @@ static sv_status ensure_out(sv_handle h, size_t doubles) {
         h->dout_cap = doubles;
     }
     if (h->hpinned_cap < doubles) {
+        // 8 KB at least: an energy, a short gradient and a small 1-RDM in one allocation (each growth of pinned memory
+        // takes about 0.3 ms)
+        const size_t cap = std::max<size_t>(doubles + doubles / 2, 1024);
         if (h->hpinned) cudaFreeHost(h->hpinned);
         h->hpinned = nullptr;
         h->hpinned_cap = 0;
         void *p = nullptr;
-        cudaError_t e = cudaMallocHost(&p, doubles * sizeof(double));
+        cudaError_t e = cudaMallocHost(&p, cap * sizeof(double));
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(h, SV_ERR_OOM, "pinned host staging allocation failed");
         }
         h->hpinned = (double *)p;
-        h->hpinned_cap = doubles;
+        h->hpinned_cap = cap;
     }
     return SV_OK;
 }
