@@ -44,6 +44,8 @@
 #include <cuda_runtime.h>
 
 #include "sv_check.cuh"
+#include <type_traits>
+
 #include "sv_internal.h"
 #include "sv_tc.cuh"
 
@@ -66,23 +68,24 @@ static_assert(kAbABase + kAbS * kAbAStage <= 512, "tensor memory: accumulators a
 // PAIR (real states): the two planes are two partner rows, each with B rows of its own.
 constexpr int kAbBBytes = 3 * kAbMaxN * kAbKc * 2;  // one partner row's B of a K block: three pieces of 64 rows x 16 K
 template <bool PAIR> constexpr int kAbStageBytes = (PAIR ? 2 : 1) * kAbBBytes;
-template <bool PAIR, bool SPLIT, int S>
+// FROM, TO: of the products, these; SECOND: into the second accumulator (SPLIT).
+template <bool PAIR, int S, int FROM, int TO, bool SECOND>
 __device__ __forceinline__ void ab_mma_stage(uint32_t tmem, uint64_t d0, uint32_t dacc, uint32_t idesc, uint32_t first) {
     constexpr int pa[6] = {0, 0, 1, 0, 1, 2}, pbk[6] = {0, 1, 0, 2, 1, 0};
     constexpr uint32_t kPieceD = (kAbMaxN * kAbKc * 2) >> 4, kStageD = kAbStageBytes<PAIR> >> 4;
     #pragma unroll
     for (int pl = 0; pl < 2; ++pl) {
         #pragma unroll
-        for (int x = 0; x < 6; ++x) {
+        for (int x = FROM; x < TO; ++x) {
             // A from tensor memory (lanes = tile rows, two K per column), B from shared memory;
             // B descriptor: that of the ring's start plus the byte offset in 16-byte units (the
             // start-address field does not carry: shared addresses < 256 KB)
             const uint32_t ta = tmem + (uint32_t)(kAbABase + S * kAbAStage + (pl * 3 + pa[x]) * kAbACols);
             const uint64_t db = d0 + (uint64_t)(S * kStageD + (PAIR ? pl * (kAbBBytes >> 4) : 0) + pbk[x] * kPieceD);
-            const uint32_t acc = x > (SPLIT ? 1 : 0) ? 1u : first ^ 1u;  // the first into an accumulator starts it
+            const uint32_t acc = x > FROM ? 1u : first ^ 1u;  // the first into an accumulator starts it
             asm volatile(
                 "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, q;\n\t}\n" ::"r"(dacc + (uint32_t)(pl * kAbMaxN + (SPLIT && x > 0 ? kAbAccCols : 0))),
+                "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, q;\n\t}\n" ::"r"(dacc + (uint32_t)(pl * kAbMaxN + (SECOND ? kAbAccCols : 0))),
                 "r"(ta), "l"(db), "r"(idesc), "r"(acc)
                 : "memory");
         }
@@ -128,11 +131,15 @@ struct AbTcArgs {
 // 1.80 ms so.
 // SPLIT: the five small piece products have an accumulator of their own, in the columns of the second
 // buffer (the tensor core cuts every accumulation to float32, so one accumulator for all six loses six
-// times the bits; k_same_tc has the same split).  Without the second buffer the drain of a unit and the
+// times the bits; k_same_tc has the same split), and x1 y1 of the unit's last K blocks, up to half of them and two,
+// follows the last small products there, so that the other accumulator is cut less often: a common factor of sigma
+// off by 1.06e-7 / 1.40e-7 at 24 / 26 qubits (8 electrons), 0.54e-7 / 0.95e-7 so, k_same_tc's narrow tiles
+// included.  Without the second buffer the drain of a unit and the
 // next one's products take turns, so it serves sectors below 2^20 determinants, whose sums were float32
 // ones before: relative gradient errors over
-// 20 problems of 20 to 26 qubits (geometric mean) 2.8e-7 so, 3.0e-7 in the float32 split form and 3.5e-7
-// with one accumulator; 24 qubits 53 us and 51 us.
+// 20 problems of 20 to 26 qubits (geometric mean) 2.8e-7 with x1 y1 in one accumulator, 3.0e-7 in the float32 split
+// form and 3.5e-7 with all six in one; 24 qubits 51 us with one accumulator, 53 with the split, 55 with the late K
+// blocks, 26 qubits 117 and 121.
 template <bool PAIR, bool SPLIT>
 __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_tc(AbTcArgs g) {
     constexpr int kBuf = SPLIT ? 1 : 2;  // accumulator buffers
@@ -412,13 +419,41 @@ __global__ void __launch_bounds__(kAbThreadsTc, 1) k_ab_tc(AbTcArgs g) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t dacc = tmem + (uint32_t)(t * kAbAccCols), first = c == 0 ? 1u : 0u;
                 static_assert(kAbS == 4, "one case per stage");
-                switch (s) {
-                    case 0: ab_mma_stage<PAIR, SPLIT, 0>(tmem, d0, dacc, idesc, first); break;
-                    case 1: ab_mma_stage<PAIR, SPLIT, 1>(tmem, d0, dacc, idesc, first); break;
-                    case 2: ab_mma_stage<PAIR, SPLIT, 2>(tmem, d0, dacc, idesc, first); break;
-                    default: ab_mma_stage<PAIR, SPLIT, 3>(tmem, d0, dacc, idesc, first); break;
+                if constexpr (!SPLIT) {
+                    switch (s) {
+                        case 0: ab_mma_stage<PAIR, 0, 0, 6, false>(tmem, d0, dacc, idesc, first); break;
+                        case 1: ab_mma_stage<PAIR, 1, 0, 6, false>(tmem, d0, dacc, idesc, first); break;
+                        case 2: ab_mma_stage<PAIR, 2, 0, 6, false>(tmem, d0, dacc, idesc, first); break;
+                        default: ab_mma_stage<PAIR, 3, 0, 6, false>(tmem, d0, dacc, idesc, first); break;
+                    }
+                    ab_commit(su32(&empty[s]));
+                } else {
+                    // x1 y1 of the last `late` K blocks waits for the last small products and follows them into
+                    // their accumulator, so that neither sum is cut more often than it must be
+                    const int late = min(kAbS - 2, g.nK / 2);
+                    const bool now = c < g.nK - late;
+                    auto issue = [&](auto stage) {
+                        constexpr int S = decltype(stage)::value;
+                        ab_mma_stage<PAIR, S, 1, 6, true>(tmem, d0, dacc, idesc, first);
+                        if (now) ab_mma_stage<PAIR, S, 0, 1, false>(tmem, d0, dacc, idesc, first);
+                    };
+                    auto follow = [&](auto stage) { ab_mma_stage<PAIR, decltype(stage)::value, 0, 1, true>(tmem, d0, dacc, idesc, 0u); };
+                    auto by_stage = [&](int k, auto f) {
+                        switch (k) {
+                            case 0: f(std::integral_constant<int, 0>()); break;
+                            case 1: f(std::integral_constant<int, 1>()); break;
+                            case 2: f(std::integral_constant<int, 2>()); break;
+                            default: f(std::integral_constant<int, 3>()); break;
+                        }
+                    };
+                    by_stage(s, issue);
+                    if (now) ab_commit(su32(&empty[s]));
+                    if (c + 1 == g.nK)
+                        for (int b = late - 1; b >= 0; --b) {
+                            by_stage((gch - b) % kAbS, follow);
+                            ab_commit(su32(&empty[(gch - b) % kAbS]));
+                        }
                 }
-                ab_commit(su32(&empty[s]));
             }
             if (!stop) ab_commit(su32(&accf[t]));
         }

@@ -37,21 +37,21 @@ constexpr int kTcThreads = 128;
 constexpr int kTcABytes = kTcM * kTcKb * 2;            // one piece of A in one stage
 constexpr int kTcCols = 512;                           // tensor-memory columns: every accumulator
 
-// A tile of TN beta strings.  The tensor core cuts each accumulation to float32, and a sum keeps
-// losing bits at the rate of its largest terms; so the five small piece products have an accumulator
+// A tile of TN beta strings.  The tensor core cuts each accumulation to float32 (towards zero), and a sum
+// keeps losing bits at the rate of its largest terms; so the five small piece products have an accumulator
 // of their own and the first pieces' product x1 y1 the rest, K blocks in turn: one with TN = 256,
-// three with 128, seven with 64.  Relative gradient error at 24 qubits: 2.1e-6 to 2.8e-6 with one
-// accumulator for all six, 0.7e-6 to 1.2e-6 with TN = 256.  The narrow tiles serve sectors of few tiles
-// (launch_same_tc), where they also have more blocks.  Against the sparse float32 sums (variant 3), whose
-// place these products take from 2^14 determinants, the error of a gradient (144 problems of 44,100 to
-// 627,264, geometric mean) is 0.92 of theirs with TN = 128 (1.09 at 511,225) and 0.83 with 64 (0.80 to 0.89
-// at each size).
+// three with 128, seven with 64, fifteen with 32.  Relative gradient error at 24 qubits: 2.1e-6 to
+// 2.8e-6 with one accumulator for all six, 0.7e-6 to 1.2e-6 with TN = 256.  Against the sparse float32 sums
+// (variant 3), whose place these products take from 2^14 determinants, the error of variant 5's pool gradients at
+// 44,100 / 245,025 / 511,225 / 627,264 determinants (24 problems each, geometric mean) is 0.77 / 1.04 / 1.14 / 1.23
+// of theirs with TN = 128 or 64 as they fit, complex 627,264 1.95, and with TN = 32 (and k_ab_tc's split of
+// x1 y1) 0.70 / 0.81 / 0.92 / 0.93; of the gradient 0.81 over all.
 template <int TN>
 struct TcTile {
     static constexpr int kMain = kTcCols / TN - 1;                      // accumulators of x1 y1
     static constexpr int kBBytes = TN * kTcKb * 2;                      // one piece of B in one stage
     static constexpr int kStageBytes = 3 * kTcABytes + 3 * kBBytes;
-    static constexpr int kStages = TN == 256 ? 3 : TN == 128 ? 4 : 6;   // 3 x 72 KB, 4 x 48 KB, 6 x 36 KB
+    static constexpr int kStages = TN == 256 ? 3 : TN == 128 ? 4 : 6;   // 3 x 72 KB, 4 x 48 KB, 6 x 36 or 30 KB
     static constexpr int kSmem = kStages * kStageBytes + 1024;          // + alignment of the ring to 1024 bytes
 };
 
@@ -277,12 +277,13 @@ cudaError_t launch_same_tc(const uint16_t *M, size_t pm, const uint16_t *X, size
                    sx[3] = {(uint64_t)lda * 2, (uint64_t)Db * lda * 2, (uint64_t)px * 2};
     const uint64_t dt[4] = {(uint64_t)Db, (uint64_t)Da, P, 3},
                    stt[3] = {(uint64_t)ldb * 2, (uint64_t)Da * ldb * 2, (uint64_t)pt * 2};
-    // the narrowest tiles of which every one has an SM: 24 qubits (495 strings, real) 46 us with 256, 35 with
-    // 128 and 33 with 64, the transposes included; 792 strings 61 us with 128, 49 with 64; at 28 qubits (2,002) 256
-    // tiles of 128 would take two rounds of the SMs
+    // below 2^20 determinants, where the sparse float32 sums ran before these products, the tile that is as accurate
+    // as they are (above); from there the narrowest of which every tile has an SM (28 qubits, 2,002 strings: 256 tiles
+    // of 128 would take two rounds).  In us with the transposes, 32 and (one round) 64, 128 wide: 495 strings 31, 33,
+    // 35; 715 45, 45, 47; 792 82 (175 tiles), 49, 61
     const int tm = (Da + kTcM - 1) / kTcM;
     auto fits = [&](int n) { return (long long)((Db + n - 1) / n) * tm * planes <= sm_count; };
-    const uint32_t tn = fits(64) ? 64 : fits(128) ? 128 : 256;
+    const uint32_t tn = (long long)Da * Db < 1 << 20 ? 32 : fits(64) ? 64 : fits(128) ? 128 : 256;
     if (!encode_map(&ma, M, 3, dma, sma, kTcM) || !encode_map(&mb, M + (size_t)Da * lda, 3, dmb, smb, tn) ||
         !encode_map(&mx, X, 4, dx, sx, tn) || !encode_map(&mt, Xt, 4, dt, stt, kTcM))
         return cudaErrorInvalidValue;
@@ -294,6 +295,7 @@ cudaError_t launch_same_tc(const uint16_t *M, size_t pm, const uint16_t *X, size
         k_same_tc<TN><<<grid, kTcThreads, smem, st>>>(ma, mb, mx, mt, g);
         return cudaGetLastError();
     };
+    if (tn == 32) return launch(std::integral_constant<int, 32>());
     if (tn == 64) return launch(std::integral_constant<int, 64>());
     if (tn == 128) return launch(std::integral_constant<int, 128>());
     return launch(std::integral_constant<int, 256>());

@@ -1,5 +1,5 @@
 """The tensor-core products of single-precision states at the string counts where their tiles change width
-(64, 128 and 256 beta strings) and have ragged edges, against the float64 sums."""
+(32, 64, 128 and 256 beta strings) and have ragged edges, against the float64 sums."""
 import numpy as np
 import pytest
 
@@ -15,9 +15,10 @@ def _lib():
     sv.lib()
 
 
-# strings per spin and tile: 715 x 1,287 64; 1,287 x 1,287 and 2,002 x 1,001 128 (complex: 256); 2,002 x 2,002 256
+# strings per spin and tile: 330 x 165 (five K blocks: two follow the small products), 13 x 1,716 (a ragged edge on
+# few rows) and 792 x 792 32; 3,003 x 364 64; 1,287 x 1,287 and 2,002 x 1,001 128 (complex: 256); 2,002 x 2,002 256
 @pytest.mark.parametrize("dtype", ["r32", "c64"])
-@pytest.mark.parametrize("n,na,nb", [(26, 5, 4), (26, 5, 5), (28, 4, 5), (28, 5, 5)])
+@pytest.mark.parametrize("n,na,nb", [(22, 4, 3), (26, 1, 6), (24, 5, 5), (28, 6, 3), (26, 5, 5), (28, 4, 5), (28, 5, 5)])
 def test_products_at_every_tile_width(n, na, nb, dtype):
     rng = np.random.default_rng(n + nb)
     p = inputs.make_problem(n, 8, 4, seed=n)
