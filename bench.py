@@ -839,7 +839,7 @@ def per_config_rows(args, stream, peak, rbatch):
     out = {"cores": oracle.num_threads()}
     roofs = {1: "launch latency (the whole sweep is one launch)",
              2: "latency of one block's operator steps (14,400 amplitudes) and launch latency",
-             3: "latency of a cluster's operator steps (245,025 amplitudes) and the expectation's tensor-core products"}
+             3: "latency of a grid's operator steps (245,025 amplitudes) and the expectation's tensor-core products"}
     for cid, dtypes in ((1, ("c128",)), (2, ("c128",)), (3, ("c64", "c128"))):
         p = inputs.config_problem(cid)
         n, L = p["n_qubits"], len(p["ops"])

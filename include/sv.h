@@ -199,8 +199,10 @@ sv_status sv_ham_destroy(sv_ham_handle ham);
 /* ---- the hot path ---------------------------------------------------------- */
 
 /* psi <- U_L ... U_1 psi with U_k = exp(theta[k] (T_k - T_k^dagger)), ops[0] first.
- * cos/sin of theta are taken on the host in float64.  One kernel per operator (dense
- * storage; sector storage: one cooperative launch for the whole list, SV_OPT_SECTOR_SWEEP).
+ * cos/sin of theta are taken on the host in float64.  One launch for the whole list on the
+ * sector's amplitudes (SV_OPT_SECTOR_SWEEP), then, for a handle with a compute core
+ * (SV_OPT_FULL_VECTOR 0), one that writes its vector; one kernel per operator on the whole
+ * vector where that option or what it lists asks for it.
  * On a state still equal to the determinant sv_prepare_hf wrote, with SV_OPT_LAYOUT_AUTO
  * on, the storage layout first becomes the one the operator list prefers. */
 sv_status sv_apply_ansatz(sv_handle h, const sv_excitation *ops, int n_ops, const double *theta);
@@ -314,7 +316,8 @@ uint64_t sv_batch_launch_count(sv_batch_handle b);
  * 256 and 384 threads per block and 1, 2 or 4 blocks per SM (grids capped by the
  * instance count) and keeps the fastest for later
  * calls; *grid_out (may be NULL) receives the grid.  Each instance runs whole in one
- * block with fixed-order sums, so results depend on the block size only through the
+ * block, or (small ones in a large batch) in a half or a quarter of one, with fixed-order
+ * sums, so results depend on the block size and on that share only through the
  * order of those sums (rounding) and reruns with one choice are bit-identical.  No
  * counterpart in the paper. */
 sv_status sv_batch_autotune(sv_batch_handle b, const double *theta, int *grid_out);
@@ -328,7 +331,11 @@ typedef enum {
                                        sv_energy_grad and restore it in the reverse sweep
                                        (0 = none; default 0) */
     SV_OPT_MAX_BYTES = 2,           /* cap on device bytes this handle may allocate
-                                       (0 = no cap); checkpoints are dropped to fit */
+                                       (0 = no cap); checkpoints are dropped to fit, and
+                                       what is kept only to be faster (product planes, the
+                                       steps of whole sweeps, float-float matrices) gives
+                                       way to what a call needs: the sparse forms and one
+                                       launch per operator then run */
     SV_OPT_EXPECT_VARIANT = 3,      /* 0 auto (= 5 for complex64 / real float32 states
                                        of at least 2^14 sector determinants whose
                                        same-spin couplings fill at least 5% of a string
@@ -392,8 +399,9 @@ typedef enum {
                                        sigma to their own precision takes 6 or 3 */
     SV_OPT_RDM_VARIANT = 4,         /* 0 auto (3 for float64 states, else 2); 1 sector
                                        gather: one thread per sector determinant (dense
-                                       storage only); 2 string rows: one block per beta
-                                       string of the compact matrix, in the state's own
+                                       storage only); 2 string rows: groups of rows
+                                       and of columns of the compact matrix, one group of a
+                                       spin's strings to a block at a time, in the state's own
                                        arithmetic; 3 string rows in float-float arithmetic
                                        (float64 states, on the FP32 pipe: the compact
                                        matrix converted once per call into a work matrix
@@ -479,9 +487,9 @@ typedef enum {
                                        wait bounded by SV_OPT_WAIT_POLLS: past it the call
                                        fails with SV_ERR_CUDA; with a limit below 1024
                                        this form runs at every size); used where no
-                                       checkpoint copy falls inside the sweep and the
-                                       device accepts the launch, else one launch per
-                                       operator (0 always) */
+                                       checkpoint copy falls inside the sweep, the lists'
+                                       memory can be had and the device accepts the
+                                       launch, else one launch per operator (0 always) */
     SV_OPT_SWEEP_BLOCKS_PER_SM = 18,/* launch geometry of the whole-sweep launches on the
                                        grid: at most this many blocks per SM, no more than
                                        can be resident, one where the operators are small
