@@ -133,7 +133,7 @@ struct AbTcArgs {
 // buffer (the tensor core cuts every accumulation to float32, so one accumulator for all six loses six
 // times the bits; k_same_tc has the same split), and x1 y1 of the unit's last K blocks, up to half of them and two,
 // follows the last small products there, so that the other accumulator is cut less often: a common factor of sigma
-// off by 1.06e-7 / 1.40e-7 at 24 / 26 qubits (8 electrons), 0.54e-7 / 0.95e-7 so, k_same_tc's narrow tiles
+// off by 1.06e-7 / 1.40e-7 at 24 / 26 qubits (8 electrons), 0.58e-7 / 1.02e-7 so, k_same_tc's sides apart
 // included.  Without the second buffer the drain of a unit and the
 // next one's products take turns, so it serves sectors below 2^20 determinants, whose sums were float32
 // ones before: relative gradient errors over

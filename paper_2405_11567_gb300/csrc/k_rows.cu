@@ -884,7 +884,7 @@ __global__ void __launch_bounds__(kThreads) k_phase_planar(const Amp *__restrict
 // sum over the beta excitations r -> s of b (partner b') of
 // (-1)^popc(b & between(r, s)) H[b'][col(b', rs)][a], plus H[b][own][a], in a fixed
 // order, and added to G before the phase; the output is written, not added to.
-template <typename Amp, bool GATHER>
+template <typename Amp, bool GATHER, bool SIDES>
 __global__ void __launch_bounds__(kThreads) k_sigma_comb(RowArgs<Amp> A, SameGemm g) {
     using R = real_of<Amp>;
     __shared__ double xb[kMaxOrb];
@@ -936,6 +936,21 @@ __global__ void __launch_bounds__(kThreads) k_sigma_comb(RowArgs<Amp> A, SameGem
         const Amp c0 = A.C[off + Ia];
         float gr = g.G[off + Ia], gi = 0.f;
         if constexpr (AmpT<Amp>::kCplx) gi = g.G[plane + off + Ia];
+        // SIDES: the beta product apart, and the sums' rounding kept (er, ei): no less accurate than the sparse sums
+        float er = 0.f, ei = 0.f;
+        auto add = [](float &sum, float &err, float x) {
+            if constexpr (SIDES) {
+                float e;
+                two_sum(sum, x, sum, e);
+                err += e;
+            } else {
+                sum += x;
+            }
+        };
+        if constexpr (SIDES) {
+            add(gr, er, g.G[(AmpT<Amp>::kCplx ? 2 : 1) * plane + off + Ia]);
+            if constexpr (AmpT<Amp>::kCplx) add(gi, ei, g.G[3 * plane + off + Ia]);
+        }
         if constexpr (GATHER) {
             for (int j = 0; j < nh; ++j) {
                 if (!SV_IN_RANGE(s_hoff[j] + Ia, g.hplane, kChkPlane)) continue;  // checked build: skip the term
@@ -943,9 +958,13 @@ __global__ void __launch_bounds__(kThreads) k_sigma_comb(RowArgs<Amp> A, SameGem
                 float hr = hp[0], hi = 0.f;
                 if constexpr (AmpT<Amp>::kCplx) hi = hp[g.hplane];
                 if (s_hneg[j]) { hr = -hr; hi = -hi; }
-                gr += hr;
-                gi += hi;
+                add(gr, er, hr);
+                add(gi, ei, hi);
             }
+        }
+        if constexpr (SIDES) {
+            gr += er;
+            gi += ei;
         }
         Amp acc;
         if constexpr (AmpT<Amp>::kCplx)
@@ -1112,7 +1131,7 @@ static cudaError_t launch_ab_k(const RowArgs<ff> &A, int K, size_t smem, cudaStr
 }
 
 cudaError_t launch_same_tc(const uint16_t *M, size_t pm, const uint16_t *X, size_t px, uint16_t *Xt, size_t pt,
-                           float *G, int planes, int Da, int Db, int lda, int ldb, int *err, uint32_t spins, int stall,
+                           float *G, int planes, int sides, int Da, int Db, int lda, int ldb, int *err, uint32_t spins, int stall,
                            int sm_count, cudaStream_t st);
 cudaError_t launch_ab_tc(const uint32_t *Xi, int planes, const uint16_t *stra, const uint16_t *strb,
                          const uint16_t *ra, const uint16_t *Bp, size_t pb, const uint16_t *rowB, float *H,
@@ -1131,7 +1150,7 @@ static cudaError_t launch_same_t(RowArgs<Amp> A, const RowTables &T, int dtype, 
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         if (g.ev && (e = cudaEventRecord(g.ev[0], st)) != cudaSuccess) return e;
-        e = launch_same_tc(g.Mp, g.pm, g.Xp, g.px, g.Xtp, g.pt, g.G, g.planes, T.Da, T.Db, g.lda, g.ldb, g.err,
+        e = launch_same_tc(g.Mp, g.pm, g.Xp, g.px, g.Xtp, g.pt, g.G, g.planes, g.sides, T.Da, T.Db, g.lda, g.ldb, g.err,
                            g.spins, g.stall & 1, sm_count, st);
         if (e != cudaSuccess) return e;
         if (g.ev && (e = cudaEventRecord(g.ev[1], st)) != cudaSuccess) return e;
@@ -1142,11 +1161,13 @@ static cudaError_t launch_same_t(RowArgs<Amp> A, const RowTables &T, int dtype, 
                              g.nb, g.err, g.spins, (g.stall >> 1) & 1, sm_count, st);
             if (e != cudaSuccess) return e;
             if (g.ev && (e = cudaEventRecord(g.ev[3], st)) != cudaSuccess) return e;
-            k_sigma_comb<Amp, true><<<T.Db, kThreads, 0, st>>>(A, g);
+            if (g.sides == 2) k_sigma_comb<Amp, true, true><<<T.Db, kThreads, 0, st>>>(A, g);
+            else k_sigma_comb<Amp, true, false><<<T.Db, kThreads, 0, st>>>(A, g);
         } else {
             e = launch_ab_k(A, K, ab_smem(dtype, K, T), st);
             if (e != cudaSuccess) return e;
-            k_sigma_comb<Amp, false><<<T.Db, kThreads, 0, st>>>(A, g);
+            if (g.sides == 2) k_sigma_comb<Amp, false, true><<<T.Db, kThreads, 0, st>>>(A, g);
+            else k_sigma_comb<Amp, false, false><<<T.Db, kThreads, 0, st>>>(A, g);
         }
         return cudaGetLastError();
     }

@@ -9,6 +9,7 @@
 // (N), accumulates both products in the same tensor-memory tile:
 //   G[p][b][a] = sum_a' Ma[a][a'] X[p][b][a']          (K = D_alpha)
 //              + sum_b' Xt[p][a][b'] Mb[b][b']          (K = D_beta)
+// (sides = 2: one of the two, G of each side in planes of its own).
 // (Ma, Mb symmetric; Xt the transposed planes, so both operands of both products are
 // K-contiguous).  Operand tiles (rows x 32 bf16 of K, 64-byte rows) are moved by TMA
 // (cp.async.bulk.tensor, 64-byte swizzle; rows and K beyond the matrix read as zero)
@@ -41,11 +42,12 @@ constexpr int kTcCols = 512;                           // tensor-memory columns:
 // keeps losing bits at the rate of its largest terms; so the five small piece products have an accumulator
 // of their own and the first pieces' product x1 y1 the rest, K blocks in turn: one with TN = 256,
 // three with 128, seven with 64, fifteen with 32.  Relative gradient error at 24 qubits: 2.1e-6 to
-// 2.8e-6 with one accumulator for all six, 0.7e-6 to 1.2e-6 with TN = 256.  Against the sparse float32 sums
-// (variant 3), whose place these products take from 2^14 determinants, the error of variant 5's pool gradients at
-// 44,100 / 245,025 / 511,225 / 627,264 determinants (24 problems each, geometric mean) is 0.77 / 1.04 / 1.14 / 1.23
-// of theirs with TN = 128 or 64 as they fit, complex 627,264 1.95, and with TN = 32 (and k_ab_tc's split of
-// x1 y1) 0.70 / 0.81 / 0.92 / 0.93; of the gradient 0.81 over all.
+// 2.8e-6 with one accumulator for all six, 0.7e-6 to 1.2e-6 with TN = 256.  Below 2^20 determinants, where the
+// sparse float32 sums (variant 3) ran before, a CTA takes the alpha or the beta product alone (sides = 2: half as many
+// accumulations, and twice the CTAs), tiles are at most 64 wide, and k_sigma_comb adds up with the rounding kept.
+// The error of variant 5's pool gradients against the sparse sums' at 245,025 / 511,225 / 627,264 / 853,776
+// determinants (24 problems each, geometric mean): 1.04 / 1.14 / 1.23 / - with tiles of 128 and 64 as they fit
+// and both products in one CTA (complex, 627,264: 1.95), 0.69 / 0.87 / 0.93 / 0.97 so.
 template <int TN>
 struct TcTile {
     static constexpr int kMain = kTcCols / TN - 1;                      // accumulators of x1 y1
@@ -56,8 +58,9 @@ struct TcTile {
 };
 
 struct TcOut {
-    float *G;  // [P][Db][Da]
+    float *G;  // [sides][P][Db][Da]
     int Da, Db;
+    int planes, sides;  // sides = 2: the alpha and the beta product in CTAs (and planes) of their own
     int *err;
     uint32_t spins;  // mbarrier polls (each with a short sleep) before a wait gives up
     int stall;       // test hook: the producer issues no copy, so the MMA issuer's first wait runs out
@@ -78,7 +81,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __shared__ volatile int s_fail;
     __shared__ int s_issued, s_consumed;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int n0 = blockIdx.x * kTcN, m0 = blockIdx.y * kTcM, p = blockIdx.z;
+    const int n0 = blockIdx.x * kTcN, m0 = blockIdx.y * kTcM, side = blockIdx.z / g.planes, p = blockIdx.z - side * g.planes;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
                      "n"(kTcCols)
@@ -100,7 +103,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base, sbase = (smem_u32(tc_smem) + 1023u) & ~1023u;
-    const int nA = (g.Da + kTcKb - 1) / kTcKb, nB = (g.Db + kTcKb - 1) / kTcKb, nIt = nA + nB;
+    // K blocks first .. first + nIt of the alpha product's nA and the beta product's nB
+    const int nA = (g.Da + kTcKb - 1) / kTcKb, nB = (g.Db + kTcKb - 1) / kTcKb;
+    const int first = side ? nA : 0, nIt = side ? nB : g.sides == 2 ? nA : nA + nB;
     if (tid == 0) {
         // producer: K block it into stage it % kTcStages once the MMAs of block it - kTcStages are done
         int it = 0;
@@ -116,12 +121,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                          : "memory");
             #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                if (it < nA) {  // alpha side: A = Ma rows a, B = X[p] rows b, K = a'
-                    tma_3d(st + c * kTcABytes, &ma, it * kTcKb, m0, c, fb);
-                    tma_4d(st + 3 * kTcABytes + c * kTcBBytes, &x, it * kTcKb, n0, p, c, fb);
+                const int kb = first + it;
+                if (kb < nA) {  // alpha side: A = Ma rows a, B = X[p] rows b, K = a'
+                    tma_3d(st + c * kTcABytes, &ma, kb * kTcKb, m0, c, fb);
+                    tma_4d(st + 3 * kTcABytes + c * kTcBBytes, &x, kb * kTcKb, n0, p, c, fb);
                 } else {        // beta side: A = Xt[p] rows a, B = Mb rows b, K = b'
-                    tma_4d(st + c * kTcABytes, &xt, (it - nA) * kTcKb, m0, p, c, fb);
-                    tma_3d(st + 3 * kTcABytes + c * kTcBBytes, &mb, (it - nA) * kTcKb, n0, c, fb);
+                    tma_4d(st + c * kTcABytes, &xt, (kb - nA) * kTcKb, m0, p, c, fb);
+                    tma_3d(st + 3 * kTcABytes + c * kTcBBytes, &mb, (kb - nA) * kTcKb, n0, c, fb);
                 }
             }
         }
@@ -202,7 +208,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     #pragma unroll
                     for (int x2 = 0; x2 < kMain; ++x2)
                         if (x2 < nIt) sum += __uint_as_float(v[x2][j]);  // (started: one per K block)
-                    if (n < g.Db) g.G[((size_t)p * g.Db + n) * g.Da + m] = sum;
+                    if (n < g.Db) g.G[((size_t)blockIdx.z * g.Db + n) * g.Da + m] = sum;
                 }
             }
         }
@@ -260,8 +266,8 @@ __global__ void __launch_bounds__(256) k_transpose_pieces(const uint16_t *__rest
 // pointers 16-byte aligned and the piece strides multiples of 8 elements (TMA's rules).
 // spins: polls of each bounded wait; stall: the test hook of TcOut.
 cudaError_t launch_same_tc(const uint16_t *M, size_t pm, const uint16_t *X, size_t px, uint16_t *Xt, size_t pt,
-                           float *G, int planes, int Da, int Db, int lda, int ldb, int *err, uint32_t spins, int stall,
-                           int sm_count, cudaStream_t st) {
+                           float *G, int planes, int sides, int Da, int Db, int lda, int ldb, int *err, uint32_t spins,
+                           int stall, int sm_count, cudaStream_t st) {
     if (Da < 1 || Db < 1 || lda % 8 || ldb % 8 || pm % 8 || px % 8 || pt % 8 || spins < 1 || ((uintptr_t)M & 15) ||
         ((uintptr_t)X & 15) || ((uintptr_t)Xt & 15))
         return cudaErrorInvalidValue;
@@ -277,18 +283,17 @@ cudaError_t launch_same_tc(const uint16_t *M, size_t pm, const uint16_t *X, size
                    sx[3] = {(uint64_t)lda * 2, (uint64_t)Db * lda * 2, (uint64_t)px * 2};
     const uint64_t dt[4] = {(uint64_t)Db, (uint64_t)Da, P, 3},
                    stt[3] = {(uint64_t)ldb * 2, (uint64_t)Da * ldb * 2, (uint64_t)pt * 2};
-    // below 2^20 determinants, where the sparse float32 sums ran before these products, the tile that is as accurate
-    // as they are (above); from there the narrowest of which every tile has an SM (28 qubits, 2,002 strings: 256 tiles
-    // of 128 would take two rounds).  In us with the transposes, 32 and (one round) 64, 128 wide: 495 strings 31, 33,
-    // 35; 715 45, 45, 47; 792 82 (175 tiles), 49, 61
+    // the narrowest tiles of which every one has an SM, at most 64 wide with the sides apart.  In us with the
+    // transposes, sides apart and together with 128: 330 strings 19 and 29, 495 23 and 35, 715 33 and 47, 792 54 and 61,
+    // 924 58 and 55; sides together, 2,002 strings: 256 tiles of 128 would take two rounds
     const int tm = (Da + kTcM - 1) / kTcM;
-    auto fits = [&](int n) { return (long long)((Db + n - 1) / n) * tm * planes <= sm_count; };
-    const uint32_t tn = (long long)Da * Db < 1 << 20 ? 32 : fits(64) ? 64 : fits(128) ? 128 : 256;
+    auto fits = [&](int n) { return (long long)((Db + n - 1) / n) * tm * planes * sides <= sm_count; };
+    const uint32_t tn = sides == 2 ? (fits(32) ? 32 : 64) : fits(64) ? 64 : fits(128) ? 128 : 256;
     if (!encode_map(&ma, M, 3, dma, sma, kTcM) || !encode_map(&mb, M + (size_t)Da * lda, 3, dmb, smb, tn) ||
         !encode_map(&mx, X, 4, dx, sx, tn) || !encode_map(&mt, Xt, 4, dt, stt, kTcM))
         return cudaErrorInvalidValue;
-    const TcOut g{G, Da, Db, err, spins, stall};
-    const dim3 grid((Db + tn - 1) / tn, tm, planes);
+    const TcOut g{G, Da, Db, planes, sides, err, spins, stall};
+    const dim3 grid((Db + tn - 1) / tn, tm, planes * sides);
     auto launch = [&](auto tile) -> cudaError_t {
         constexpr int TN = decltype(tile)::value, smem = TcTile<TN>::kSmem;
         if ((e = allow_smem(k_same_tc<TN>, smem)) != cudaSuccess) return e;

@@ -1213,8 +1213,10 @@ static sv_status ensure_same_gemm(sv_handle h, DevTables *T, const RowTables &R,
     // X [planes][Db][lda], G [planes][Db][Da], Xt [planes][Da][ldb] (tensor-core form)
     // (each region rounded to 256 bytes: aligned starts for vector loads and TMA)
     // the three bf16 pieces of X and those of the transposes [planes][Da][ldb]; then G
-    // float32 [planes][Db][Da]
-    const size_t nx = (size_t)planes * Db * lda, nt = (size_t)planes * Da * ldb, ng = (size_t)planes * Db * Da;
+    // float32 [sides][planes][Db][Da]
+    const size_t nx = (size_t)planes * Db * lda, nt = (size_t)planes * Da * ldb;
+    const int sides = Da * Db < (1u << 20) ? 2 : 1;  // (k_same_tc's accuracy)
+    const size_t ng = (size_t)sides * planes * Db * Da;
     auto r256 = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t xb = r256(3 * nx * sizeof(uint16_t)), tb = r256(3 * nt * sizeof(uint16_t));
     // variant 5: then the phased amplitudes as interleaved bf16 pieces [Db][ldi][3] words
@@ -1246,6 +1248,7 @@ static sv_status ensure_same_gemm(sv_handle h, DevTables *T, const RowTables &R,
     g->pt = nt;
     g->G = (float *)(B + xb + tb);
     g->planes = planes;
+    g->sides = sides;
     g->lda = (int)lda;
     g->ldb = (int)ldb;
     g->err = h->kerr;

@@ -132,7 +132,8 @@ struct HostTables {
 struct SameGemm {
     const float *Ma = nullptr, *Mb = nullptr;  // [Da][Da], [Db][Db], symmetric
     const double *dA = nullptr, *dB = nullptr; // one-spin diagonal energies per string (float64)
-    float *G = nullptr;                        // same-spin sigma~ [planes][Db][Da]
+    float *G = nullptr;                        // same-spin sigma~ [sides][planes][Db][Da]
+    int sides = 1;                             // 2 (below 2^20 determinants): the alpha and the beta product apart
     // every operand as three bf16 pieces at a piece stride: [Ma | Mb] (Mp, pm), the
     // phased planes [planes][Db][lda] (Xp, px), their transposes [planes][Da][ldb] (Xtp, pt)
     const uint16_t *Mp = nullptr;

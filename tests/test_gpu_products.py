@@ -15,8 +15,9 @@ def _lib():
     sv.lib()
 
 
-# strings per spin and tile: 330 x 165 (five K blocks: two follow the small products), 13 x 1,716 (a ragged edge on
-# few rows) and 792 x 792 32; 3,003 x 364 64; 1,287 x 1,287 and 2,002 x 1,001 128 (complex: 256); 2,002 x 2,002 256
+# strings per spin and tile: below 2^20 determinants the alpha and the beta product in CTAs of their own, 330 x 165
+# (five K blocks: two follow the small products) and 13 x 1,716 (a ragged edge on few rows) 32, 792 x 792 64 in two
+# rounds; from there both in one, 3,003 x 364 64; 1,287 x 1,287 and 2,002 x 1,001 128 (complex: 256); 2,002 x 2,002 256
 @pytest.mark.parametrize("dtype", ["r32", "c64"])
 @pytest.mark.parametrize("n,na,nb", [(22, 4, 3), (26, 1, 6), (24, 5, 5), (28, 6, 3), (26, 5, 5), (28, 4, 5), (28, 5, 5)])
 def test_products_at_every_tile_width(n, na, nb, dtype):
