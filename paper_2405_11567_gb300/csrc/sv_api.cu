@@ -1140,9 +1140,9 @@ static bool dense_couplings(sv_handle h) {
 // sector has at least 2^14 determinants and every string at least 5% of the strings
 // of its spin as same-spin partners (singles and doubles), so that the dense
 // products do at most 20 times the multiplies of the sparse sums.  Measured, variants
-// 3 / 5 in us (real float32): 14,400 determinants 62 / 65, 63,504 158 / 86, 108,900
-// 248 / 115, 245,025 435 / 149, 627,264 1223 / 299 (complex64: 44,100 144 / 89, 245,025
-// 529 / 173); variant 4 alone 73, 128, 179, 361, 689.  Variant 3 where its memory cannot be had
+// 3 / 5 in us (real float32): 14,400 determinants 62 / 65, 63,504 158 / 77, 108,900
+// 248 / 98, 245,025 435 / 127, 627,264 1223 / 254 (complex64: 44,100 144 / 84, 245,025
+// 529 / 172); variant 4 alone, with wider tiles, 73, 128, 179, 361, 689.  Variant 3 where its memory cannot be had
 // (sigma_rows).
 static bool use_same_gemm(sv_handle h, int K) {
     if (!single_prec(h->dtype) || K == 0 || h->Da > 4096 || h->Db > 4096) return false;
