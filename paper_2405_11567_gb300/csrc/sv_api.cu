@@ -2605,7 +2605,13 @@ sv_status sv_energy_grad(sv_handle h, sv_ham_handle ham, const sv_excitation *op
     SV_TRY(build_ops(h, ops, n_ops, theta, d, core ? kIdentity : nullptr));  // validates in any layout
     h->at_ref = false;
     DeviceGuard g(h->device);
-    SV_TRY(clear_kernel_flag(h));  // psi is written from the reference
+    if (h->wait_pending) {
+        // an ansatz that nothing has read: psi is written from the reference, so one that gave up does not matter,
+        // but where this call is refused before that there is no state
+        SV_CUDA(h, cudaStreamSynchronize(h->stream));
+        if (*h->hkerr) h->prepared = false;
+        SV_TRY(clear_kernel_flag(h));
+    }
     int np[32];
     const bool lay = h->layout_auto && n_ops > 0 && h->storage == 0;
     if (lay) layout_from_ops(h->n, ops, n_ops, np);

@@ -139,3 +139,28 @@ def test_a_sweep_that_gave_up_is_reported_by_the_next_reader(storage, dtype, rea
     good()                               # from the reference
     st.close()
     ham.close()
+
+
+@pytest.mark.parametrize("dtype", ["r64", "c64"])
+def test_a_refused_evaluation_does_not_hide_a_sweep_that_gave_up(dtype):
+    """The evaluation would have written the state anew, but is refused for memory first: the state stays lost."""
+    p = inputs.config_problem(2)
+    ham = sv.Hamiltonian(p["h"], p["eri"], p["e_nuc"])
+    st = sv.StateVector(p["n_qubits"], dtype, sector=(p["na"], p["nb"]))
+    st.set_option(sv.SV_OPT_FULL_VECTOR, 1)
+    st.set_option(sv.SV_OPT_WAIT_POLLS, 1)
+    st.prepare_hf(p["occ"])
+    st.apply_ansatz(p["ops"], p["theta"])
+    st.set_option(sv.SV_OPT_WAIT_POLLS, 1 << 22)
+    st.set_option(sv.SV_OPT_MAX_BYTES, 1)
+    with pytest.raises(sv.SvError) as e:
+        st.energy_grad(ham, p["ops"], p["theta"])
+    assert e.value.status == 2
+    st.set_option(sv.SV_OPT_MAX_BYTES, 0)
+    with pytest.raises(sv.SvError) as e:
+        st.state()
+    assert e.value.status in (3, 5)
+    st.prepare_hf(p["occ"])
+    assert np.count_nonzero(st.state()) == 1
+    st.close()
+    ham.close()
